@@ -149,10 +149,9 @@ def _features(g, M, N, correlated):
     """Uniform features in [-1, 1], or correlated Gaussian ones scaled into it."""
     if not correlated:
         return torch.rand(M, N, generator=g, device="cuda") * 2 - 1
-    W = torch.randn(N, N, generator=g, device="cuda", dtype=torch.float64)
-    eye = torch.eye(N, device="cuda", dtype=torch.float64)
-    L = torch.linalg.cholesky(W @ W.T / N + 0.1 * eye).float()
-    X = torch.randn(M, N, generator=g, device="cuda") @ L.T
+    W = torch.randn(N, N, generator=g, device="cuda").double().cpu().numpy()
+    L = np.linalg.cholesky(W @ W.T / N + 0.1 * np.eye(N)).astype(np.float32)
+    X = torch.randn(M, N, generator=g, device="cuda") @ torch.from_numpy(L).cuda().T
     lo, hi = X.amin(0), X.amax(0)
     return (2 * (X - lo) / (hi - lo) - 1).clamp(-1, 1).contiguous()
 
