@@ -39,11 +39,12 @@
 //                = TMEM lane; warps 4-7 take the first half of the columns,
 //                8-11 the second), r = (y_m - a_0) - D, sse += r^2 in packed
 //                FP32 pairs, then added to an FP64 partial per (CTA, half).
-//   warps 12-15  expansion: each thread owns fixed pattern rows; per 8-column
-//                chunk (a table built once per launch says where the chunk
-//                starts in the feature / degree sequence) the basis
-//                recurrence runs in registers, is rounded to BF16 and stored
-//                in the K-major SWIZZLE_128B operand layout.
+//   warps 12-15  expansion: each thread owns fixed pattern rows; the basis
+//                recurrences run in registers, are rounded to the operand form
+//                and stored in the K-major SWIZZLE_128B operand layout: whole
+//                features at a time for degrees 1..10 (expand_stream.cuh),
+//                beyond them per 8-column chunk (a table built once per launch
+//                says where the chunk starts in the feature / degree sequence).
 // Expansion slots: the K-blocks of the tiles go, in order, into a ring of NS
 // K-block slots (use q = i * KB + kb takes slot q % NS); a slot is rewritten
 // as soon as the last MMA reading its previous use has completed. With
@@ -63,6 +64,7 @@
 #include <atomic>
 
 #include "basis.cuh"
+#include "expand_stream.cuh"
 #include "game_internal.cuh"
 #include "tc_common.cuh"
 #include "tc_ptx.cuh"
@@ -495,11 +497,43 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
   } else if (warp >= kBasisWarp0) {
     // ---------------- expansion (basis) ----------------
     const int bt = threadIdx.x - kBasisWarp0 * 32;
+    // staged features and degrees 1..10 stream whole features. Both sides, us
+    // per evaluation, chunk generator -> stream: bf16x3, M = 150,001, N = 17,
+    // trigonometric degree 5, P = 300: 187 -> 100; BF16, M = 50,000, N = 64,
+    // trigonometric degree 10, P = 512: 480 -> 238; FP8, M = 10^6, N = 32,
+    // Chebyshev degree 8, P = 1024: 488 -> 430.
+    const bool stream = (F != kFormBF16 || TRI || a.xstage) && stream_degree(a.d);
     for (int cid = bt; cid < KB * CPK; cid += kBasisThreads)
       tab[cid] = chunk_desc(cid, a.basis, a.d, a.Kp);
     if (F == kFormFP8)
       for (int k = bt; k < KB * 128; k += kBasisThreads) cs[k] = a.colinv[k];
     ptx::named_bar(1, kBasisThreads);
+    if (stream) {
+      StreamArgs sa;
+      sa.phi = ptx::smem_addr(phi);
+      sa.slot_bytes = (uint32_t)(NPHI * BN * 128);
+      sa.lo_off = (uint32_t)(BN * 128);
+      sa.phi_full0 = ptx::smem_addr(phi_full);
+      sa.phi_free0 = ptx::smem_addr(phi_free);
+      sa.x_full = ptx::smem_addr(x_full);
+      sa.x_empty = ptx::smem_addr(x_empty);
+      sa.xs = xs;
+      sa.cs = cs;
+      sa.xstride = XW;
+      sa.xblocks = xblocks;
+      sa.N = N;
+      sa.KB = KB;
+      sa.NS = NS;
+      // whole warps share a row pass and a group sequence
+      sa.RW = TRI ? 64 : BN >= 64 ? BN / 2 : 32;
+      sa.R = BN / sa.RW;
+      sa.QS = kBasisThreads / sa.RW;
+      sa.bt = bt;
+      sa.my_tiles = my_tiles;
+      sa.abort_flag = abort_flag;
+      sa.status = a.status;
+      stream_dispatch<F, false>(a.basis, a.d, sa);
+    }
     // thread -> rows r0 + RW * rr (rr < R) and 16-byte units q0, q0 + QS, ...:
     // BN = 128, 256: 128 rows per pass, R = BN / 128; BN = 192: 64 rows per
     // pass, R = 3, two unit groups; BN < 128: BN rows, R = 1, 128 / BN groups
@@ -812,7 +846,7 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
         }
       }
     }
-    for (int it = 0; it < my_tiles && ok && staged; ++it) {
+    for (int it = 0; it < my_tiles && ok && staged && !stream; ++it) {
       ok = wait_bar(ptx::smem_addr(x_full), it & 1, abort_flag, a.status);
       if (!ok) break;
       for (int kb = 0; kb < KB; ++kb) {

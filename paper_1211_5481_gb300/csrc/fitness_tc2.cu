@@ -39,6 +39,7 @@
 // even CTA its MMAs), and both CTAs meet at the final cluster barrier before
 // the pair's tensor memory is freed.
 #include "basis.cuh"
+#include "expand_stream.cuh"
 #include "game_internal.cuh"
 #include "tc_common.cuh"
 #include "tc_ptx.cuh"
@@ -446,6 +447,34 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       tab[cid] = chunk_desc(cid, a.basis, a.d, a.Kp);
     ptx::named_bar(1, kBasisThreads);
     const uint32_t phi_full_lead0 = ptx::mapa(ptx::smem_addr(phi_full), 0);
+    // (whole features at a time: see expand_stream.cuh; M = 10^6, N = 32,
+    // trigonometric degree 8, P = 1024: 2.58 -> 0.84 ms per evaluation)
+    const bool stream = a.xstage && stream_degree(a.d);
+    if (stream) {
+      StreamArgs sa;
+      sa.phi = ptx::smem_addr(phi);
+      sa.slot_bytes = kRows * 128;
+      sa.lo_off = 0;
+      sa.phi_full0 = phi_full_lead0;
+      sa.phi_free0 = ptx::smem_addr(phi_free);
+      sa.x_full = ptx::smem_addr(x_full);
+      sa.x_empty = ptx::smem_addr(x_empty);
+      sa.xs = xs;
+      sa.cs = nullptr;
+      sa.xstride = kRows;
+      sa.xblocks = 0;   // one block of 128 rows
+      sa.N = N;
+      sa.KB = KB;
+      sa.NS = NS;
+      sa.RW = kRows / 2;
+      sa.R = 2;
+      sa.QS = 2;
+      sa.bt = r0;
+      sa.my_tiles = my_tiles;
+      sa.abort_flag = abort_flag;
+      sa.status = a.status;
+      stream_dispatch<kFormBF16, true>(a.basis, a.d, sa);
+    }
     auto slot_free = [&](int q) -> bool {
       const int use = q / NS;
       return use == 0 ||
@@ -512,7 +541,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           publish(q);
         }
       }
-    } else {
+    } else if (!stream) {
       const float* xrow = xs + r0;   // block layout [N][128]
       for (int it = 0; it < my_tiles && ok; ++it) {
         ok = wait_bar(ptx::smem_addr(x_full), it & 1, abort_flag, a.status);
