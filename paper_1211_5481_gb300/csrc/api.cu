@@ -281,7 +281,8 @@ int ensure_colscales(game_ctx* h) {
 // tensor-core plan's chromosome tiles (paired-SM plans take them in pairs),
 // else whole tiles of 128.
 int padded_P(game_ctx* h, int P, int prec) {
-  if (prec == GAME_PREC_FP32 || prec == GAME_PREC_GRAM) return ceil_div(P, 128) * 128;
+  if (prec == GAME_PREC_GRAM) return ceil_div(P, 128) * 128;
+  if (prec == GAME_PREC_FP32) return plan_fp32(h->s, P, h->num_sms).Ppad;
   return plan_tc(h->s, P, h->num_sms, tc_form(prec)).C * 128;
 }
 
@@ -413,8 +414,8 @@ int eval_device(game_ctx* h, const float* dpop, int P, int prec, double* dfit,
     CK(launch_pack_fp32(dpop, P, Ppad, h->s, pl.Kc, h->popT, h->a0, h->st));
     stage_end(h, t0, kPack);
     t0 = stage_begin(h);
-    CK(launch_fitness_fp32(pl, h->s, h->Xt, h->y, h->popT, h->a0, P, Ppad, h->part, err,
-                           h->st));
+    CK(launch_fitness_fp32(pl, h->s, h->Xt, h->y, h->popT, h->a0, P, Ppad, h->part,
+                           h->status, err, h->st));
     stage_end(h, t0, kFitness);
     t0 = stage_begin(h);
     CK(launch_reduce(h->part, pl.grid_y, P, Ppad, rM, rerr, dfit, h->st));
@@ -931,7 +932,7 @@ int game_plan_info(game_t h, int32_t precision, int32_t P, int32_t* info) {
     const Fp32Plan pl = plan_fp32(h->s, P, h->num_sms);
     info[0] = GAME_KERNEL_FP32;
     info[1] = pl.BM;
-    info[6] = pl.grid_x * pl.grid_y;
+    info[6] = pl.cta_x * pl.grid_y;
     return GAME_OK;
   }
   const TcPlan pl = plan_tc(h->s, P, h->num_sms, tc_form(precision));

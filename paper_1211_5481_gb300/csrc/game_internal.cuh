@@ -74,12 +74,14 @@ cudaError_t launch_pack_fp32(const float* pop, int P, int Ppad, const Shape& s, 
 cudaError_t launch_replicate_tied(const float* pop, int P, const Shape& s, float* full,
                                   cudaStream_t st);
 // fitness_fp32.cu
-struct Fp32Plan { int BP, BM, Kc, grid_x, grid_y; };
+// grid_x: groups of 128 chromosomes; U: chromosomes per thread (16 U per CTA,
+// cta_x CTAs across the population); Ppad: columns popT, a0 and part need
+struct Fp32Plan { int BM, Kc, grid_x, grid_y, U, cta_x, Ppad; };
 Fp32Plan plan_fp32(const Shape& s, int P, int num_sms);
 // err: GAME_ERR_MAE sums absolute residuals, any other value squared ones
 cudaError_t launch_fitness_fp32(const Fp32Plan& pl, const Shape& s, const float* Xt,
                                 const float* y, const float* popT, const float* a0, int P,
-                                int Ppad, double* part, int err, cudaStream_t st);
+                                int Ppad, double* part, int* status, int err, cudaStream_t st);
 // fitness_tc.cu -- operand forms of the tensor-core contraction
 enum TcForm : int { kFormBF16 = 0, kFormBF16x3 = 1, kFormFP8 = 2 };
 // 16 KB gene blocks per (chromosome tile, K-block): hi and lo for bf16x3
