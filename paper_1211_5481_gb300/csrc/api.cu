@@ -114,10 +114,7 @@ struct game_ctx {
   float* uscale = nullptr;     // FP8: per-chromosome scales [cap_P]
   double* part = nullptr;
   // Gram form of the MSE (built once, at the first GAME_PREC_GRAM use)
-  double* G = nullptr;
-  double* gb = nullptr;
-  double* gyy = nullptr;
-  double* gpart = nullptr;    // re-scoring partial sums
+  GramDev gram{};
   // FP8 column scales of the expansion (computed once, at the first FP8 use)
   unsigned int* colmax = nullptr;
   float* colscale = nullptr;
@@ -220,34 +217,42 @@ Shape gram_shape(const game_ctx* h) {
 }
 
 int ensure_gram(game_ctx* h) {
-  if (h->G) return GAME_OK;
+  if (h->gram.G) return GAME_OK;
   const int K = h->Kg;
   const Shape gs = gram_shape(h);
   const int64_t rows = gram_chunk_rows(gs);
   double* phi = nullptr;
   double* part = nullptr;
-  if (dev_alloc(&h->G, (size_t)K * K) != cudaSuccess || dev_alloc(&h->gb, (size_t)K) != cudaSuccess ||
-      dev_alloc(&h->gyy, 1) != cudaSuccess ||
-      dev_alloc(&h->gpart, (size_t)gram_small_parts(gs) * kMaxRescore) != cudaSuccess ||
+  GramDev g{};
+  const size_t list = (size_t)gram_list(gs);
+  auto drop = [&]() {
+    dev_free(phi);
+    dev_free(part);
+    dev_free(g.G);
+    dev_free(g.b);
+    dev_free(g.yy);
+    dev_free(g.list);
+    dev_free(g.kk);
+  };
+  if (dev_alloc(&g.G, (size_t)K * K) != cudaSuccess || dev_alloc(&g.b, (size_t)K) != cudaSuccess ||
+      dev_alloc(&g.yy, 1) != cudaSuccess || dev_alloc(&g.list, list) != cudaSuccess ||
+      dev_alloc(&g.kk, gs.K <= 64 ? list : 1) != cudaSuccess ||
       dev_alloc(&phi, (size_t)rows * K) != cudaSuccess ||
       dev_alloc(&part, (size_t)gram_part_doubles(gs, h->num_sms)) != cudaSuccess) {
     cudaGetLastError();
-    dev_free(phi);
-    dev_free(part);
-    dev_free(h->G);
-    dev_free(h->gb);
-    dev_free(h->gyy);
-    dev_free(h->gpart);
-    h->G = nullptr;
-    h->gb = h->gyy = h->gpart = nullptr;
+    drop();
     return fail(GAME_ENOMEM, "Gram matrix");
   }
-  cudaError_t e = launch_gram_build(gs, h->Xt, h->y, h->G, h->gb, h->gyy, phi, part, h->num_sms,
-                                    h->st);
+  cudaError_t e = launch_gram_build(gs, h->Xt, h->y, g.G, g.b, g.yy, phi, part, h->num_sms, h->st);
+  if (e == cudaSuccess) e = launch_gram_list(gs, g, h->st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
+  if (e != cudaSuccess) {
+    drop();
+    return cuda_fail(e, "Gram build");
+  }
   dev_free(phi);
   dev_free(part);
-  if (e != cudaSuccess) return cuda_fail(e, "Gram build");
+  h->gram = g;
   return GAME_OK;
 }
 
@@ -398,8 +403,7 @@ int eval_device(game_ctx* h, const float* dpop, int P, int prec, double* dfit,
   cudaEvent_t t0;
   if (prec == GAME_PREC_GRAM) {
     t0 = stage_begin(h);
-    CK(launch_gram_fitness(gram_shape(h), dpop, P, nullptr, h->G, h->gb, h->gyy, dfit, err,
-                           h->st));
+    CK(launch_gram_fitness(gram_shape(h), dpop, P, nullptr, h->gram, dfit, err, h->st));
     stage_end(h, t0, kFitness);
     return GAME_OK;
   }
@@ -447,8 +451,7 @@ int rescore_device(game_ctx* h, const float* dpop, int P, int n, double* dfit) {
   if (rc) return rc;
   cudaEvent_t t0 = stage_begin(h);
   CK(launch_select_top(dfit, P, n, h->cand, h->st));
-  CK(launch_gram_rescore(gram_shape(h), dpop, n, h->cand, h->G, h->gb, h->gyy, h->gpart, dfit,
-                         h->prm.error, h->st));
+  CK(launch_gram_fitness(gram_shape(h), dpop, n, h->cand, h->gram, dfit, h->prm.error, h->st));
   stage_end(h, t0, kRescore);
   return GAME_OK;
 }
@@ -568,10 +571,14 @@ int setup_screening(game_ctx* h) {
   return rc;
 }
 
-int check_status(game_ctx* h) {
-  int st = 0;
-  CK(cudaMemcpyAsync(&st, h->status, sizeof(int), cudaMemcpyDeviceToHost, h->st));
+// Waits for the handle's work and reports its status word; gens_run: the
+// generations the last whole-generation launch ran (its second word).
+int check_status(game_ctx* h, int* gens_run = nullptr) {
+  int word[2] = {0, 0};
+  CK(cudaMemcpyAsync(word, h->status, sizeof(word), cudaMemcpyDeviceToHost, h->st));
   CK(cudaStreamSynchronize(h->st));
+  const int st = word[0];
+  if (gens_run) *gens_run = word[1];
   if (st != kDevOk) {
     CK(cudaMemsetAsync(h->status, 0, sizeof(int), h->st));
     CK(cudaStreamSynchronize(h->st));
@@ -717,10 +724,11 @@ void destroy_ctx(game_ctx* h) {
   dev_free(h->popA);
   dev_free(h->a0);
   dev_free(h->uscale);
-  dev_free(h->G);
-  dev_free(h->gb);
-  dev_free(h->gyy);
-  dev_free(h->gpart);
+  dev_free(h->gram.G);
+  dev_free(h->gram.b);
+  dev_free(h->gram.yy);
+  dev_free(h->gram.list);
+  dev_free(h->gram.kk);
   dev_free(h->colmax);
   dev_free(h->colscale);
   dev_free(h->colinv);
@@ -743,6 +751,24 @@ void destroy_ctx(game_ctx* h) {
   dev_free(h->sd.tstat);
   dev_free(h->sd.lfit);
   delete h;
+}
+
+// Small Gram-form runs take whole generations in one launch (gram_train.cu);
+// stage timing wants the separate kernels.
+bool whole_generations(game_ctx* h) {
+  return h->prm.precision == GAME_PREC_GRAM && !h->prm.surrogate && !h->timing && h->gram.G &&
+         gram_train_fits(ga_dev(h));
+}
+
+// Enqueues n such generations from the current state (with the stop rule when
+// asked: done0 generations of the training call ran before) into the other
+// population buffer; the caller advances cur and gen by what ran.
+int enqueue_generations(game_ctx* h, uint64_t seed, int n, int done0, bool stop) {
+  const int every = h->prm.check_every > 0 ? h->prm.check_every : 1;
+  CK(launch_gram_train(ga_dev(h), h->gram, h->s.M, h->prm.error, h->pop[h->cur],
+                       h->pop[h->cur ^ 1], h->fit, seed, (uint32_t)h->gen, n, done0,
+                       stop ? every : 0, h->prm.mse_threshold, h->status + 1, h->st));
+  return GAME_OK;
 }
 
 int copy_in(game_ctx* h, void* dst, const void* src, size_t bytes) {
@@ -1041,6 +1067,13 @@ int game_generation(game_t h, uint64_t seed) {
     stage_end(h, t0, kSurrogate);
     return rc;
   }
+  if (whole_generations(h)) {
+    rc = enqueue_generations(h, seed, 1, 0, false);
+    if (rc) return rc;
+    h->cur ^= 1;
+    h->gen += 1;
+    return GAME_OK;
+  }
   cudaEvent_t t0 = stage_begin(h);
   CK(launch_generation(ga_dev(h), h->pop[h->cur], h->fit, seed, (uint32_t)h->gen, h->plan,
                        h->pop[h->cur ^ 1], h->st));
@@ -1061,6 +1094,27 @@ int game_train(game_t h, int32_t generations, int32_t* generations_run) {
   if (generations_run) *generations_run = 0;
   const int every = h->prm.check_every > 0 ? h->prm.check_every : 1;
   const bool use_stop = h->prm.mse_threshold > 0.0;
+  if (h->fit_valid && whole_generations(h) && h->gen + generations < 0xFFFFFFFFll) {
+    // at most kGensPerLaunch at a time: a launch stays in the milliseconds
+    constexpr int kGensPerLaunch = 1000;
+    int done = 0;
+    while (done < generations) {
+      const int n = generations - done < kGensPerLaunch ? generations - done : kGensPerLaunch;
+      int rc = enqueue_generations(h, h->prm.seed, n, done, use_stop);
+      if (rc) return rc;
+      int ran = n;
+      if (use_stop) {
+        rc = check_status(h, &ran);
+        if (rc) return rc;
+      }
+      if (ran > 0) h->cur ^= 1;
+      h->gen += ran;
+      done += ran;
+      if (generations_run) *generations_run = done;
+      if (ran < n) break;
+    }
+    return use_stop ? GAME_OK : check_status(h);
+  }
   double* fit_h = nullptr;
   if (use_stop) {
     fit_h = new (std::nothrow) double[h->prm.P];
@@ -1325,9 +1379,9 @@ int game_gram(game_t h, double* G_out, double* b_out, double* yy_out) {
   int rc = ensure_gram(h);
   if (rc) return rc;
   const int K = h->Kg;
-  if (G_out) CK(cudaMemcpyAsync(G_out, h->G, (size_t)K * K * sizeof(double), cudaMemcpyDefault, h->st));
-  if (b_out) CK(cudaMemcpyAsync(b_out, h->gb, (size_t)K * sizeof(double), cudaMemcpyDefault, h->st));
-  if (yy_out) CK(cudaMemcpyAsync(yy_out, h->gyy, sizeof(double), cudaMemcpyDefault, h->st));
+  if (G_out) CK(cudaMemcpyAsync(G_out, h->gram.G, (size_t)K * K * sizeof(double), cudaMemcpyDefault, h->st));
+  if (b_out) CK(cudaMemcpyAsync(b_out, h->gram.b, (size_t)K * sizeof(double), cudaMemcpyDefault, h->st));
+  if (yy_out) CK(cudaMemcpyAsync(yy_out, h->gram.yy, sizeof(double), cudaMemcpyDefault, h->st));
   return check_status(h);
 }
 

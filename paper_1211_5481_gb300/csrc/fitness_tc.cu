@@ -488,7 +488,8 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
         ptx::tc_fence_before();
         ptx::mbar_arrive(ptx::smem_addr(&acc_empty[buf]));
         const float2 sp2 = ptx::f2_unpack(s2);
-        const double tile_sse = (double)sp2.x + (double)sp2.y + (double)s_tail;
+        double tile_sse = (double)sp2.x + (double)sp2.y;
+        if (s_tail != 0.f) tile_sse += (double)s_tail;   // (FP64 operations are scarce)
         part_row[chrom] = (it == 0) ? tile_sse : part_row[chrom] + tile_sse;
         ++acc_it;
       }

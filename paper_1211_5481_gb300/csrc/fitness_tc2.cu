@@ -435,7 +435,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive_cluster(acc_empty_lead0 + 8 * buf);
         const float2 sp2 = ptx::f2_unpack(s2);
-        const double tile_sse = (double)sp2.x + (double)sp2.y + (double)s_tail;
+        double tile_sse = (double)sp2.x + (double)sp2.y;
+        if (s_tail != 0.f) tile_sse += (double)s_tail;   // (FP64 operations are scarce)
         part_row[chrom] = (it == 0) ? tile_sse : part_row[chrom] + tile_sse;
         ++acc_it;
       }

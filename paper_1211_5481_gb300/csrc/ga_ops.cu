@@ -46,92 +46,15 @@ __global__ void init_population_kernel(uint64_t seed, int P, int K, float* __res
     pop[e] = ga::init_gene(seed, K, e);
 }
 
-__host__ __device__ inline int pow2_at_least(int P) {
-  int n2 = 1;
-  while (n2 < P) n2 <<= 1;
-  return n2;
-}
-
-// order[r] = the chromosome of rank r (order may be NULL: the result stays in
-// sidx): a bitonic sort of (rank key, index) over the next power of two
-// >= P, padded with keys above every chromosome; skey [n2] and sidx [n2] in
-// shared memory.
-__device__ void ranking_sort_body(int P, const double* __restrict__ fit, uint64_t* skey,
-                                  int* sidx, int* __restrict__ order) {
-  const int n2 = pow2_at_least(P);
-  for (int i = threadIdx.x; i < n2; i += kPlanThreads) {
-    skey[i] = i < P ? ga::rank_key(fit[i]) : ga::kKeyMax;
-    sidx[i] = i < P ? i : 0x7fffffff;
-  }
-  __syncthreads();
-  for (int k = 2; k <= n2; k <<= 1)
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int i = threadIdx.x; i < n2; i += kPlanThreads) {
-        const int l = i ^ j;
-        if (l <= i) continue;
-        const bool up = (i & k) == 0;   // ascending run
-        const bool swap = up ? ga::ranks_before(skey[l], sidx[l], skey[i], sidx[i])
-                             : ga::ranks_before(skey[i], sidx[i], skey[l], sidx[l]);
-        if (swap) {
-          const uint64_t tk = skey[i];
-          skey[i] = skey[l];
-          skey[l] = tk;
-          const int ti = sidx[i];
-          sidx[i] = sidx[l];
-          sidx[l] = ti;
-        }
-      }
-      __syncthreads();
-    }
-  if (order)
-    for (int i = threadIdx.x; i < P; i += kPlanThreads) order[i] = sidx[i];
-}
-
 __global__ void __launch_bounds__(kPlanThreads)
 ranking_order_kernel(int P, const double* __restrict__ fit, int* __restrict__ order) {
   extern __shared__ __align__(16) uint64_t skey[];
-  ranking_sort_body(P, fit, skey, reinterpret_cast<int*>(skey + pow2_at_least(P)), order);
-}
-
-// cum[p + 1] = sum_{j<=p} roulette_weight(fit[j]), cum[0] = 0: each thread
-// sums a contiguous chunk, an exclusive scan of the chunk sums gives its
-// offset (integers, so the result does not depend on the order).
-__device__ void roulette_cum_body(int P, const double* __restrict__ fit, uint64_t* cum) {
-  __shared__ uint64_t wsum[kPlanThreads / 32];
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int chunk = (P + kPlanThreads - 1) / kPlanThreads;
-  const int lo = min(P, tid * chunk), hi = min(P, lo + chunk);
-  uint64_t s = 0;
-  for (int p = lo; p < hi; ++p) s += ga::roulette_weight(fit[p]);
-  uint64_t inc = s;   // inclusive scan within the warp
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint64_t v = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += v;
-  }
-  if (lane == 31) wsum[wid] = inc;
-  __syncthreads();
-  if (wid == 0) {
-    uint64_t t = wsum[lane];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint64_t v = __shfl_up_sync(0xffffffffu, t, o);
-      if (lane >= o) t += v;
-    }
-    wsum[lane] = t;   // inclusive over warps
-  }
-  __syncthreads();
-  uint64_t run = (wid > 0 ? wsum[wid - 1] : 0) + inc - s;
-  for (int p = lo; p < hi; ++p) {
-    run += ga::roulette_weight(fit[p]);
-    cum[p + 1] = run;
-  }
-  if (tid == 0) cum[0] = 0;
+  ga::ranking_sort_body(P, fit, skey, reinterpret_cast<int*>(skey + ga::pow2_at_least(P)), order);
 }
 
 __global__ void __launch_bounds__(kPlanThreads)
 roulette_cum_kernel(int P, const double* __restrict__ fit, uint64_t* __restrict__ cum) {
-  roulette_cum_body(P, fit, cum);
+  ga::roulette_cum_body(P, fit, cum);
 }
 
 __global__ void __launch_bounds__(kPlanThreads)
@@ -156,25 +79,19 @@ __global__ void ga_breed_kernel(GaDev g_, const float* __restrict__ pop,
 constexpr int kFusedMax = 1024;
 constexpr int64_t kFusedGenes = 65536;
 
-__host__ __device__ inline int fused_table_bytes(const GaDev& ga) {
-  return ga.sel == GAME_SEL_RANKING    ? pow2_at_least(ga.P) * 12
-         : ga.sel == GAME_SEL_ROULETTE ? (ga.P + 1) * 8
-                                       : 0;
-}
-
 __global__ void __launch_bounds__(kPlanThreads)
 ga_fused_kernel(GaDev g_, const float* __restrict__ pop, const double* __restrict__ fit,
                 uint64_t seed, uint32_t g, float* __restrict__ next) {
   extern __shared__ __align__(16) uint64_t fsm[];
   GaDev ga = g_;
-  const int tb = (fused_table_bytes(g_) + 15) & ~15;
+  const int tb = (ga::table_bytes(g_) + 15) & ~15;
   int4* plan = reinterpret_cast<int4*>(reinterpret_cast<char*>(fsm) + tb);
   if (ga.sel == GAME_SEL_RANKING) {
-    int* sidx = reinterpret_cast<int*>(fsm + pow2_at_least(ga.P));
-    ranking_sort_body(ga.P, fit, fsm, sidx, nullptr);
+    int* sidx = reinterpret_cast<int*>(fsm + game::ga::pow2_at_least(ga.P));
+    game::ga::ranking_sort_body(ga.P, fit, fsm, sidx, nullptr);
     ga.order = sidx;
   } else if (ga.sel == GAME_SEL_ROULETTE) {
-    roulette_cum_body(ga.P, fit, fsm);
+    game::ga::roulette_cum_body(ga.P, fit, fsm);
     ga.cum = fsm;
   }
   __syncthreads();
@@ -210,7 +127,7 @@ cudaError_t launch_generation(const GaDev& ga, const float* pop, const double* f
                               cudaStream_t st) {
   if (ga.E > kMaxElites) return cudaErrorInvalidValue;
   if (ga.P <= kFusedMax && ga.Nout <= kFusedMax && (int64_t)ga.Nout * ga.K <= kFusedGenes) {
-    const int smem = ((fused_table_bytes(ga) + 15) & ~15) + ga.Nout * (int)sizeof(int4);
+    const int smem = ((ga::table_bytes(ga) + 15) & ~15) + ga.Nout * (int)sizeof(int4);
     ga_fused_kernel<<<1, kPlanThreads, smem, st>>>(ga, pop, fit, seed, g, next);
     return cudaGetLastError();
   }

@@ -224,17 +224,20 @@ int64_t gram_part_doubles(const Shape& s, int num_sms);
 cudaError_t launch_gram_build(const Shape& s, const float* Xt, const float* y, double* G,
                               double* b, double* yy, double* phi_chunk, double* part,
                               int num_sms, cudaStream_t st);
+// the Gram form of a training set, and what an evaluation reads of it: the
+// weighted entries of G in the order it takes them, b and yy
+struct GramDev {
+  double *G, *b, *yy;
+  double* list;    // [gram_list(s)]: K <= 64 pairs k1 <= k2, else 32-row steps
+  uint16_t* kk;    // K <= 64: [gram_list(s)] k1 | k2 << 8
+};
+int64_t gram_list(const Shape& s);
+cudaError_t launch_gram_list(const Shape& s, const GramDev& g, cudaStream_t st);
 // fit of the P chromosomes pop [P][K] (idx NULL), or of rows idx[0..P-1]
-// written to fit[idx[p]]; err GAME_ERR_MSE or GAME_ERR_RMSE
+// written to fit[idx[p]] (the elite re-scoring); err GAME_ERR_MSE or
+// GAME_ERR_RMSE
 cudaError_t launch_gram_fitness(const Shape& s, const float* pop, int P, const int* idx,
-                                const double* G, const double* b, const double* yy,
-                                double* fit, int err, cudaStream_t st);
-// the elite re-scoring: n <= kMaxRescore chromosomes pop rows idx[q], spread
-// over the GPU; part [gram_small_parts(s) * n] is scratch
-int gram_small_parts(const Shape& s);
-cudaError_t launch_gram_rescore(const Shape& s, const float* pop, int n, const int* idx,
-                                const double* G, const double* b, const double* yy,
-                                double* part, double* fit, int err, cudaStream_t st);
+                                const GramDev& g, double* fit, int err, cudaStream_t st);
 
 // predict.cu: Out(m) of chrom [Kg] in FP64 for M patterns of X (tiled: the
 // handle's [Mpad/128][N][128] layout, else row-major [M][N]) into out (may be
@@ -262,6 +265,15 @@ struct GaDev {
 };
 constexpr int kMaxRankingP = 16384;   // ranking sorts the population in shared memory
 cudaError_t launch_init_population(uint64_t seed, int P, int K, float* pop, cudaStream_t st);
+// gram_train.cu: up to `gens` generations of a small Gram-form run in one
+// launch, from pop_in and fit into pop_out (untouched if none runs) and fit;
+// every > 0: before generation n with (done0 + n) % every == 0 it stops if the
+// best fitness is below threshold. *done = generations run.
+bool gram_train_fits(const GaDev& g);
+cudaError_t launch_gram_train(const GaDev& g, const GramDev& gram, int64_t M, int err,
+                              const float* pop_in, float* pop_out, double* fit, uint64_t seed,
+                              uint32_t g0, int gens, int done0, int every, double threshold,
+                              int* done, cudaStream_t st);
 cudaError_t launch_generation(const GaDev& ga, const float* pop, const double* fit,
                               uint64_t seed, uint32_t g, int4* plan, float* next,
                               cudaStream_t st);

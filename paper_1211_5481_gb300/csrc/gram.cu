@@ -25,19 +25,19 @@
 // vec_accum_kernel / vec_add_kernel do the same for Phi^T y and y^T y over 64
 // row ranges. Every sum runs in a fixed order (chunks in sequence, ranges
 // in order, rows in order within a range), so G is reproducible.
-// The quadratic forms: quad_kernel, one CTA per 8 chromosomes, thread t owns
-// rows t, t + 256, ... of G a_p and reads G column-wise (G is symmetric, so
-// G[k2][k1] over k2 is a coalesced column read), then a fixed-order CTA sum.
+// The quadratic forms use G's symmetry, so a chromosome costs about K^2 / 2
+// FP64 multiply-adds (an SM issues two a cycle: the FP64 pipe bounds all of
+// this); quad_rows_kernel and quad_pairs_kernel (gram.cuh) below.
 #include <math_constants.h>
 
 #include "game_internal.cuh"
+#include "gram.cuh"
 
 namespace game {
 
 namespace {
 
 constexpr int kGT = 64;        // G tile
-constexpr int kQuadGroup = 8;  // chromosomes per quad CTA at most
 constexpr int kVecSplits = 64; // row splits of a chunk's b and y.y sums
 
 // Phi[r][k] for patterns m0 + r (r < mc), FP64; column 0 is 1.
@@ -114,14 +114,6 @@ __global__ void expand_tied_kernel(int64_t m0, int mc, int N, int d, int basis, 
       }
     }
   }
-}
-
-// The fitness from the Gram-form MSE, clamped at 0 (cancellation can leave
-// an exact fit a few ulps below zero): itself, or its square root for
-// GAME_ERR_RMSE.
-__device__ __forceinline__ double finish_error(double mse, int err) {
-  const double m = fmax(mse, 0.0);
-  return err == GAME_ERR_RMSE ? sqrt(m) : m;
 }
 
 // part[z][k1][k2] = sum over rows r of split z of Phi[r][k1] Phi[r][k2], for
@@ -228,135 +220,189 @@ __global__ void mirror_kernel(int K, double* __restrict__ G) {
   }
 }
 
-// fit_p = (yy - 2 a_p . b + a_p^T G a_p) / M for grp <= 8 chromosomes per CTA;
-// with idx, entry p is chromosome idx[p] (read from pop row idx[p], written to
-// fit[idx[p]]).
-__global__ void __launch_bounds__(256)
-quad_kernel(int P, int K, int64_t M, int grp, int err, const float* __restrict__ pop,
-            const int* __restrict__ idx, const double* __restrict__ G,
-            const double* __restrict__ b, const double* __restrict__ yy,
-            double* __restrict__ fit) {
-  extern __shared__ double as[];   // [8][K] genes of the group, FP64 (rows >= grp zero)
-  __shared__ double red[kQuadGroup][8];
-  const int p0 = blockIdx.x * grp;
-  const int ng = min(grp, P - p0);
-  for (int e = threadIdx.x; e < grp * K; e += 256) {
-    const int q = e / K, k = e % K;
-    const int64_t row = q < ng ? (idx ? idx[p0 + q] : p0 + q) : 0;
-    as[e] = q < ng ? (double)pop[row * K + k] : 0.0;
+// Pair list of a small form (K <= kPairK): entry e < K (K + 1) / 2 is the pair
+// k1 <= k2 in row order, with weight G[k1][k1] or 2 G[k1][k2].
+__global__ void pairs_kernel(int K, const double* __restrict__ G, double* __restrict__ Gp,
+                             uint16_t* __restrict__ kk) {
+  for (int e = threadIdx.x; e < K * K; e += blockDim.x) {
+    const int k1 = e / K, k2 = e % K;
+    if (k1 > k2) continue;
+    const int at = k1 * K - k1 * (k1 - 1) / 2 + (k2 - k1);
+    Gp[at] = k1 == k2 ? G[e] : 2.0 * G[e];
+    kk[at] = (uint16_t)(k1 | (k2 << 8));
+  }
+}
+
+// K <= kPairK: one warp per chromosome (quad_pairs in gram.cuh).
+constexpr int kPairWarps = 4;
+__global__ void __launch_bounds__(32 * kPairWarps)
+quad_pairs_kernel(int P, int K, double m, double rm, int err, const float* __restrict__ pop,
+                  const int* __restrict__ idx, const double* __restrict__ Gp,
+                  const uint16_t* __restrict__ kk, const double* __restrict__ b,
+                  const double* __restrict__ yy, double* __restrict__ fit) {
+  __shared__ double as[kPairWarps][kPairK];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int q = blockIdx.x * kPairWarps + warp;
+  if (q >= P) return;
+  const int p = idx ? idx[q] : q;
+  for (int k = lane; k < K; k += 32) as[warp][k] = (double)pop[(int64_t)p * K + k];
+  __syncwarp();
+  const double v = quad_pairs(K, as[warp], Gp, kk, b, lane);
+  if (lane == 0) fit[p] = finish_error(divide_by(*yy + v, m, rm), err);
+}
+
+// Larger K. Rows are taken in blocks of 32 (lane = row); block I needs the
+// columns k2 >= 32 I only: its own 32 x 32 square once, everything to the right
+// twice. The (block, column) steps of all blocks form one list, laid out once
+// per handle (steps_kernel: a step's 32 weighted entries of G side by side).
+constexpr int kAheadMax = 20;     // steps a warp loads ahead (the list is padded by them)
+__host__ __device__ inline int64_t row_steps(int K) {
+  const int64_t NB = (K + 31) / 32;
+  return NB * K - 16 * NB * (NB - 1);   // sum over I of (K - 32 I)
+}
+__global__ void steps_kernel(int K, const double* __restrict__ G, double* __restrict__ T) {
+  const int I = blockIdx.x, lane = threadIdx.x & 31;
+  const int64_t base = (int64_t)I * K - 16ll * I * (I - 1);
+  const int k1 = 32 * I + lane;
+  for (int c = blockIdx.y * 8 + (threadIdx.x >> 5); c < K - 32 * I; c += gridDim.y * 8) {
+    const double g = k1 < K ? G[(int64_t)(32 * I + c) * K + k1] : 0.0;
+    T[(base + c) * 32 + lane] = c < 32 ? g : 2.0 * g;
+  }
+}
+
+// The list is cut into kQuadRanges contiguous ranges; a warp takes a range at a
+// time for GRP chromosomes and leaves the range's sum per chromosome; the sums
+// are added in a fixed order. A cluster of S CTAs shares a group's ranges and
+// adds them in the leader's shared memory, so the result does not depend on S. With idx, entry q is chromosome idx[q].
+// Before, one CTA held 8 chromosomes and thread t the rows t, t + 256, ... of
+// the full square: at K = 257 the second pass served a single row, and 128
+// CTAs left 24 SMs idle. P = 1024, K = 257: 231 -> 85 us per
+// evaluation (the FP64 pipes, 1.0 TFLOP/s measured, need 68 us for half the
+// square); the 16 re-scored candidates with their selection: 45 -> 18.5 us.
+constexpr int kQuadWarps = 4;     // per CTA
+constexpr int kQuadRanges = 32;   // kQuadRanges / (S kQuadWarps) ranges per warp
+
+template <int GRP>
+__global__ void __launch_bounds__(32 * kQuadWarps)
+quad_rows_kernel(int P, int K, double m, double rm, int err, int S, const float* __restrict__ pop,
+                 const int* __restrict__ idx, const double* __restrict__ T,
+                 const double* __restrict__ b, const double* __restrict__ yy,
+                 double* __restrict__ fit) {
+  constexpr int kAhead = GRP >= 4 ? 8 : kAheadMax;   // loads in flight
+  extern __shared__ double as[];   // [K + kAheadMax][GRP] genes of the group (zero past the last)
+  __shared__ double red[kQuadRanges][GRP];   // the leader's: every range's sums
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (S > 1) ptx::cluster_arrive();   // the leader runs before anyone writes to it
+  const int rank = (int)(blockIdx.x % S), p0 = (int)(blockIdx.x / S) * GRP;
+  const int ng = min(GRP, P - p0);
+  {
+    // a thread's entries are one chromosome's genes (GRP divides the threads)
+    const int q = threadIdx.x % GRP;
+    const float* genes = q < ng ? pop + (int64_t)(idx ? idx[p0 + q] : p0 + q) * K : nullptr;
+#pragma unroll 4
+    for (int k = threadIdx.x / GRP; k < K; k += 32 * kQuadWarps / GRP)
+      as[k * GRP + q] = genes ? (double)genes[k] : 0.0;
   }
   __syncthreads();
-  double quad[kQuadGroup], lin[kQuadGroup];
+  if (S > 1) ptx::cluster_wait();
+  const int NB = (K + 31) / 32;
+  const int64_t steps = row_steps(K);
+  constexpr int kPer = kQuadRanges / kQuadWarps;
+  for (int j = 0; j < kPer / S; ++j) {
+    const int range = (rank * kQuadWarps + warp) * (kPer / S) + j;
+    int s = (int)(range * steps / kQuadRanges);
+    const int s1 = (int)((range + 1) * steps / kQuadRanges);
+    double v[GRP];
 #pragma unroll
-  for (int q = 0; q < kQuadGroup; ++q) {
-    quad[q] = 0.0;
-    lin[q] = 0.0;
-  }
-  for (int k1 = threadIdx.x; k1 < K; k1 += 256) {
-    double ga[kQuadGroup];
-#pragma unroll
-    for (int q = 0; q < kQuadGroup; ++q) ga[q] = 0.0;
-    for (int k2 = 0; k2 < K; ++k2) {
-      const double g = G[(int64_t)k2 * K + k1];   // = G[k1][k2]
-#pragma unroll
-      for (int q = 0; q < kQuadGroup; ++q)
-        if (q < grp) ga[q] = fma(g, as[q * K + k2], ga[q]);
+    for (int q = 0; q < GRP; ++q) v[q] = 0.0;
+    int I = 0, base = 0;   // block of step s and the block's first step
+    while (I + 1 < NB && s >= base + K - 32 * I) {
+      base += K - 32 * I;
+      ++I;
     }
-    const double bk = b[k1];
+    while (s < s1) {
+      const int k1 = I * 32 + lane;
+      const int end = base + K - 32 * I;   // the block's steps end
+      const int stop = end < s1 ? end : s1;
+      const double lin = s == base && k1 < K ? -2.0 * b[k1] : 0.0;
+      double h[GRP], h2[GRP];
 #pragma unroll
-    for (int q = 0; q < kQuadGroup; ++q)
-      if (q < grp) {
-        quad[q] = fma(as[q * K + k1], ga[q], quad[q]);
-        lin[q] = fma(as[q * K + k1], bk, lin[q]);
+      for (int q = 0; q < GRP; ++q) {
+        h[q] = lin;
+        h2[q] = 0.0;
       }
-  }
-  // fixed-order CTA sums: lanes by xor-butterfly, then the 8 warps in order
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+      int k2 = 32 * I + (s - base);
+      const double* t = T + (int64_t)s * 32 + lane;
+      for (; s < stop; s += kAhead, k2 += kAhead, t += kAhead * 32) {
+        double gv[kAhead];
 #pragma unroll
-  for (int q = 0; q < kQuadGroup; ++q) {
-    double v = quad[q] - 2.0 * lin[q];
+        for (int u = 0; u < kAhead; ++u) gv[u] = t[u * 32];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) red[q][warp] = v;
+        for (int u = 0; u < kAhead; ++u) {
+          if (GRP == 1) {
+            // few warps: straight-line code keeps all loads in flight; a step
+            // past the segment multiplies by zero (the list's entries are finite)
+#pragma unroll
+            for (int q = 0; q < GRP; ++q) {
+              const double av = s + u < stop ? as[(k2 + u) * GRP + q] : 0.0;
+              if (u & 1) h2[q] = fma(gv[u], av, h2[q]);
+              else h[q] = fma(gv[u], av, h[q]);
+            }
+          } else {
+            if (s + u >= stop) break;
+#pragma unroll
+            for (int q = 0; q < GRP; ++q) h[q] = fma(gv[u], as[(k2 + u) * GRP + q], h[q]);
+          }
+        }
+      }
+      s = stop;
+      if (k1 < K) {
+#pragma unroll
+        for (int q = 0; q < GRP; ++q)
+          v[q] = fma(as[k1 * GRP + q], GRP == 1 ? h[q] + h2[q] : h[q], v[q]);
+      }
+      base = end;
+      ++I;
+    }
+    // lane sums: each exchange halves the chromosomes a lane still holds
+    int n = GRP, q0 = 0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      if (n > 1) {
+        n >>= 1;
+        const bool up = (lane & o) != 0;
+        q0 += up ? n : 0;
+#pragma unroll
+        for (int q = 0; q < GRP / 2; ++q)
+          if (q < n) {
+            const double give = up ? v[q] : v[q + n];
+            const double keep = up ? v[q + n] : v[q];
+            v[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+          }
+      } else {
+        v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+      }
+    }
+    if ((lane & (32 / GRP - 1)) == 0) {
+      if (S > 1)
+        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(
+                         ptx::mapa(ptx::smem_addr(&red[range][q0]), 0)),
+                     "d"(v[0])
+                     : "memory");
+      else
+        red[range][q0] = v[0];
+    }
   }
-  __syncthreads();
-  if (threadIdx.x < ng) {
-    double s = 0.0;
-    for (int w = 0; w < 8; ++w) s += red[threadIdx.x][w];
+  if (S > 1) ptx::cluster_sync();
+  else __syncthreads();
+  if (rank == 0 && threadIdx.x < ng) {
+    double t[4] = {0.0, 0.0, 0.0, 0.0};   // ranges in four interleaved chains
+#pragma unroll
+    for (int r = 0; r < kQuadRanges; ++r) t[r & 3] += red[r][threadIdx.x];
     const int p = p0 + threadIdx.x;
-    fit[idx ? idx[p] : p] = finish_error((*yy + s) / (double)M, err);
+    const double sum = *yy + ((t[0] + t[1]) + (t[2] + t[3]));
+    fit[idx ? idx[p] : p] = finish_error(divide_by(sum, m, rm), err);
   }
-}
-
-// Few chromosomes (n <= kMaxRescore; the elite re-scoring): the K x K
-// products are spread over the whole GPU. CTA (bx, by) owns rows
-// k1 in [128 bx, 128 bx + 128) (one per thread) and the k2-range
-// [by ks, (by + 1) ks) of sum_k2 G[k1][k2] a_q[k2] (G read column-wise, as
-// G[k2][k1]); each thread forms a_q[k1] h_q (and, in split 0,
-// -2 a_q[k1] b[k1]); the CTA's sum per candidate (lanes by xor-butterfly,
-// warps in order) goes to part[by][bx][q]. quad_small_finish adds the parts
-// in order and writes fit[idx[q]] = (yy + sum) / M.
-constexpr int kSmallRows = 128;
-__global__ void __launch_bounds__(kSmallRows)
-quad_small_kernel(int n, int K, int ks, const float* __restrict__ pop, const int* __restrict__ idx,
-                  const double* __restrict__ G, const double* __restrict__ b,
-                  double* __restrict__ part) {
-  extern __shared__ double av[];   // [n][ks] genes of the k2-range
-  __shared__ double red[kMaxRescore][kSmallRows / 32];
-  const int k1 = blockIdx.x * kSmallRows + threadIdx.x;
-  const int k2lo = blockIdx.y * ks, k2hi = min(K, k2lo + ks);
-  const int len = k2hi - k2lo;
-  for (int e = threadIdx.x; e < n * ks; e += kSmallRows) {
-    const int q = e / ks, c = e % ks;
-    av[e] = c < len ? (double)pop[(int64_t)idx[q] * K + k2lo + c] : 0.0;
-  }
-  __syncthreads();
-  double h[kMaxRescore];
-#pragma unroll
-  for (int q = 0; q < kMaxRescore; ++q) h[q] = 0.0;
-  if (k1 < K) {
-    for (int c = 0; c < len; ++c) {
-      const double g = G[(int64_t)(k2lo + c) * K + k1];
-#pragma unroll
-      for (int q = 0; q < kMaxRescore; ++q)
-        if (q < n) h[q] = fma(g, av[q * ks + c], h[q]);
-    }
-  }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int q = 0; q < kMaxRescore; ++q) {
-    if (q >= n) break;
-    double v = 0.0;
-    if (k1 < K) {
-      const double ak = pop[(int64_t)idx[q] * K + k1];
-      v = ak * h[q];
-      if (blockIdx.y == 0) v -= 2.0 * ak * b[k1];
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) red[q][warp] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < n) {
-    double sum = 0.0;
-    for (int w = 0; w < kSmallRows / 32; ++w) sum += red[threadIdx.x][w];
-    part[((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * n + threadIdx.x] = sum;
-  }
-}
-
-// One warp per candidate q: lane l adds parts l, l + 32, ... in order, then
-// a fixed xor-butterfly.
-__global__ void quad_small_finish(int n, int nparts, int64_t M, int err,
-                                  const int* __restrict__ idx,
-                                  const double* __restrict__ part, const double* __restrict__ yy,
-                                  double* __restrict__ fit) {
-  const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (q >= n) return;
-  double s = 0.0;
-  for (int j = lane; j < nparts; j += 32) s += part[(int64_t)j * n + q];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) fit[idx[q]] = finish_error((*yy + s) / (double)M, err);
 }
 
 int blocks_for(int64_t n) {
@@ -428,47 +474,65 @@ cudaError_t launch_gram_build(const Shape& s, const float* Xt, const float* y, d
   return cudaGetLastError();
 }
 
-int gram_small_parts(const Shape& s) {
-  const int bx = (s.K + kSmallRows - 1) / kSmallRows;
-  int by = (304 + bx - 1) / bx;   // about two CTAs per SM over the grid
-  if (by > s.K) by = s.K;
-  return bx * by;
+int64_t gram_list(const Shape& s) {
+  return s.K <= kPairK ? (int64_t)s.K * (s.K + 1) / 2 : (row_steps(s.K) + kAheadMax) * 32;
 }
 
-cudaError_t launch_gram_rescore(const Shape& s, const float* pop, int n, const int* idx,
-                                const double* G, const double* b, const double* yy,
-                                double* part, double* fit, int err, cudaStream_t st) {
-  if (n < 1 || n > kMaxRescore) return cudaErrorInvalidValue;
-  const int bx = (s.K + kSmallRows - 1) / kSmallRows;
-  const int by = gram_small_parts(s) / bx;
-  const int ks = (s.K + by - 1) / by;
-  const size_t smem = (size_t)n * ks * sizeof(double);   // <= 16 x 410 x 8 at K = 4097
-  if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(
-        quad_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+cudaError_t launch_gram_list(const Shape& s, const GramDev& g, cudaStream_t st) {
+  if (s.K <= kPairK) {
+    pairs_kernel<<<1, 1024, 0, st>>>(s.K, g.G, g.list, g.kk);
+  } else {
+    const cudaError_t e =
+        cudaMemsetAsync(g.list, 0, (size_t)gram_list(s) * sizeof(double), st);
     if (e != cudaSuccess) return e;
+    steps_kernel<<<dim3((s.K + 31) / 32, 16), 256, 0, st>>>(s.K, g.G, g.list);
   }
-  quad_small_kernel<<<dim3(bx, by), kSmallRows, smem, st>>>(n, s.K, ks, pop, idx, G, b, part);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  quad_small_finish<<<1, 32 * n, 0, st>>>(n, bx * by, s.M, err, idx, part, yy, fit);
   return cudaGetLastError();
 }
+
+namespace {
+template <int GRP>
+cudaError_t launch_rows(const Shape& s, const float* pop, int P, const int* idx, const GramDev& g,
+                        double* fit, int err, int S, cudaStream_t st) {
+  const size_t smem = (size_t)GRP * (s.K + kAheadMax) * sizeof(double);
+  cudaError_t e = cudaFuncSetAttribute(quad_rows_kernel<GRP>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(ceil_div(P, GRP) * S));
+  cfg.blockDim = dim3(32 * kQuadWarps);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)S;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, quad_rows_kernel<GRP>, P, s.K, (double)s.M,
+                            1.0 / (double)s.M, err, S, pop, idx, (const double*)g.list,
+                            (const double*)g.b, (const double*)g.yy, fit);
+}
+}  // namespace
 
 cudaError_t launch_gram_fitness(const Shape& s, const float* pop, int P, const int* idx,
-                                const double* G, const double* b, const double* yy,
-                                double* fit, int err, cudaStream_t st) {
-  // as many chromosomes per CTA (<= 8) as fit in 200 KB of FP64 genes
-  int grp = (int)((200 * 1024) / ((size_t)s.K * sizeof(double)));
-  if (grp > kQuadGroup) grp = kQuadGroup;
-  if (grp < 1) grp = 1;
-  const size_t smem = (size_t)grp * s.K * sizeof(double);
-  cudaError_t e = cudaFuncSetAttribute(quad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       200 * 1024);
-  if (e != cudaSuccess) return e;
-  quad_kernel<<<(P + grp - 1) / grp, 256, smem, st>>>(P, s.K, s.M, grp, err, pop, idx, G, b,
-                                                       yy, fit);
-  return cudaGetLastError();
+                                const GramDev& g, double* fit, int err, cudaStream_t st) {
+  if (s.K <= kPairK) {
+    quad_pairs_kernel<<<ceil_div(P, kPairWarps), 32 * kPairWarps, 0, st>>>(
+        P, s.K, (double)s.M, 1.0 / (double)s.M, err, pop, idx, g.list, g.kk, g.b, g.yy, fit);
+    return cudaGetLastError();
+  }
+  // Four chromosomes share each entry where that still makes two CTAs per SM
+  // (152 SMs); else one each, every load of a range in flight. Cluster size: about six
+  // CTAs per SM, so the last SMs to finish are few. P = 1024, K = 257: 85 us
+  // with four chromosomes and S = 4, 90 with S = 8 or 2, 91 with eight
+  // chromosomes, 113 with one; P = 16: 12.4 us with one and S = 8, 18.5 with four.
+  constexpr int kSms = 152;
+  const int grp = (int64_t)ceil_div(P, 4) * 8 >= 2 * kSms ? 4 : 1;
+  int S = 1;
+  while (S < 8 && (int64_t)ceil_div(P, grp) * S < 6 * kSms) S <<= 1;
+  return grp == 4 ? launch_rows<4>(s, pop, P, idx, g, fit, err, S, st)
+                  : launch_rows<1>(s, pop, P, idx, g, fit, err, S, st);
 }
 
 }  // namespace game

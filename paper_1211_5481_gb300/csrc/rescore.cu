@@ -5,12 +5,20 @@
 // reduced value, so elitism (Section 3; 2 elites, Section 5) and the
 // tournaments rank the best candidates by accurate values.
 //
-// select_top_kernel, one CTA: each thread keeps the top 16 of its strided
-// elements in registers, each warp merges its lanes' lists, warp 0 merges the
-// 8 warps'. Fitness values are compared through order-preserving integer
-// keys (integer compares instead of the FP64 pipe).
+// Two kernels. select_rank_kernel: a warp per chromosome counts, 32 at a time,
+// the chromosomes that rank before it and gives up at n; the n that finish
+// write their own place, and no CTA waits for another. Latency bound: one pass
+// of the keys through shared memory, P / 32 ballots for the n best, a few for
+// all others. (Selection and re-evaluation of 16 candidates, K = 257: P = 1024
+// 45 -> 18.5 us, P = 2048 51 -> 22.6.) Above 16,384 chromosomes the launch of P
+// warps and the long counts cost more than select_top_kernel (one CTA: each
+// thread keeps the top 16 of its strided elements in registers, each warp
+// merges its lanes' lists, warp 0 merges the 8 warps'). Fitness values are
+// compared through order-preserving integer keys (integer compares instead of
+// the FP64 pipe).
 #include <math_constants.h>
 
+#include "ga_device.cuh"
 #include "game_internal.cuh"
 
 namespace game {
@@ -19,32 +27,7 @@ namespace {
 
 constexpr int kSelThreads = 256;
 
-// Fitness as an order-preserving unsigned key (NaN as +infinity, -0 as +0),
-// so the ranking runs on integer compares instead of the slow FP64 pipe.
-__device__ __forceinline__ uint64_t fit_key(double f) {
-  if (isnan(f)) f = CUDART_INF;
-  if (f == 0.0) f = 0.0;
-  const uint64_t u = (uint64_t)__double_as_longlong(f);
-  return (u >> 63) ? ~u : (u | 0x8000000000000000ull);
-}
-constexpr uint64_t kNoKey = ~0ull;
-
-__device__ __forceinline__ bool key_before(uint64_t fa, int a, uint64_t fb, int b) {
-  return fa < fb || (fa == fb && a < b);
-}
-
-// Warp-wide arg-min of (key, index); every lane receives the winner.
-__device__ __forceinline__ void warp_argmin(uint64_t& k, int& i) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const uint64_t ok = __shfl_xor_sync(0xffffffffu, k, o);
-    const int oi = __shfl_xor_sync(0xffffffffu, i, o);
-    if (key_before(ok, oi, k, i)) {
-      k = ok;
-      i = oi;
-    }
-  }
-}
+constexpr uint64_t kNoKey = ga::kKeyMax;
 
 // Sorted list of kMaxRescore (key, index) pairs held in registers.
 struct TopList {
@@ -58,12 +41,12 @@ struct TopList {
     }
   }
   __device__ __forceinline__ void insert(uint64_t key, int idx) {
-    if (!key_before(key, idx, k[kMaxRescore - 1], i[kMaxRescore - 1])) return;
+    if (!ga::ranks_before(key, idx, k[kMaxRescore - 1], i[kMaxRescore - 1])) return;
     k[kMaxRescore - 1] = key;
     i[kMaxRescore - 1] = idx;
 #pragma unroll
     for (int j = kMaxRescore - 1; j > 0; --j) {
-      if (key_before(k[j], i[j], k[j - 1], i[j - 1])) {
+      if (ga::ranks_before(k[j], i[j], k[j - 1], i[j - 1])) {
         const uint64_t tk = k[j];
         const int ti = i[j];
         k[j] = k[j - 1];
@@ -91,12 +74,12 @@ select_top_kernel(const double* __restrict__ fit, int P, int n, int* __restrict_
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   TopList L;
   L.clear();
-  for (int p = tid; p < P; p += kSelThreads) L.insert(fit_key(fit[p]), p);
+  for (int p = tid; p < P; p += kSelThreads) L.insert(ga::rank_key(fit[p]), p);
   // each warp: n rounds of arg-min over its lanes' list heads
   for (int r = 0; r < n; ++r) {
     uint64_t k = L.k[0];
     int i = L.i[0];
-    warp_argmin(k, i);
+    ga::warp_argmin(k, i);
     if (L.i[0] == i && i != 0x7fffffff) L.pop_front();
     if (lane == 0) {
       wk[warp][r] = k;
@@ -115,10 +98,35 @@ select_top_kernel(const double* __restrict__ fit, int P, int n, int* __restrict_
   for (int r = 0; r < n; ++r) {
     uint64_t k = L.k[0];
     int i = L.i[0];
-    warp_argmin(k, i);
+    ga::warp_argmin(k, i);
     if (L.i[0] == i && i != 0x7fffffff) L.pop_front();
     if (lane == 0) cand[r] = i;
   }
+}
+
+constexpr int kRankMax = 16384;
+constexpr int kRankWarps = 8;
+constexpr int kRankChunk = 2048;   // keys staged in shared memory at a time
+__global__ void __launch_bounds__(32 * kRankWarps)
+select_rank_kernel(const double* __restrict__ fit, int P, int n, int* __restrict__ cand) {
+  __shared__ uint64_t key[kRankChunk];
+  const int lane = threadIdx.x & 31;
+  const int i = blockIdx.x * kRankWarps + (threadIdx.x >> 5);
+  const uint64_t mine = i < P ? ga::rank_key(fit[i]) : kNoKey;
+  int before = i < P ? 0 : n;
+  for (int c0 = 0; c0 < P; c0 += kRankChunk) {
+    const int len = min(kRankChunk, P - c0);
+#pragma unroll 8
+    for (int k = threadIdx.x; k < len; k += 32 * kRankWarps) key[k] = ga::rank_key(fit[c0 + k]);
+    __syncthreads();
+    for (int k0 = 0; k0 < len && before < n; k0 += 32) {
+      const int k = k0 + lane;
+      const bool b = k < len && ga::ranks_before(key[k], c0 + k, mine, i);
+      before += __popc(__ballot_sync(0xffffffffu, b));
+    }
+    if (!__syncthreads_or(before < n)) break;
+  }
+  if (lane == 0 && before < n) cand[before] = i;
 }
 
 }  // namespace
@@ -126,7 +134,10 @@ select_top_kernel(const double* __restrict__ fit, int P, int n, int* __restrict_
 cudaError_t launch_select_top(const double* fit, int P, int n, int* cand, cudaStream_t st) {
   if (n < 1) return cudaSuccess;
   if (n > kMaxRescore || n > P) return cudaErrorInvalidValue;
-  select_top_kernel<<<1, kSelThreads, 0, st>>>(fit, P, n, cand);
+  if (P <= kRankMax)
+    select_rank_kernel<<<ceil_div(P, kRankWarps), 32 * kRankWarps, 0, st>>>(fit, P, n, cand);
+  else
+    select_top_kernel<<<1, kSelThreads, 0, st>>>(fit, P, n, cand);
   return cudaGetLastError();
 }
 
