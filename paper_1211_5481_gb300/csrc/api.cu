@@ -131,13 +131,17 @@ struct game_ctx {
   int4* oplan = nullptr;      // their plan [Nout]
   float* pred = nullptr;      // predictions of the children [kScreenMax]
   int* flag = nullptr;
-  int* pos = nullptr;
+  int* list = nullptr;        // the kept children, in slot order
   int last_n = 0;             // children screened by the last generation
   int* trust = nullptr;       // [2]: the trust check's verdict, the verdict the last screening used
   float* trust_r = nullptr;   // [1]: the trust check's last correlation
   float* rX[2] = {nullptr, nullptr};     // replay: the last two populations
   double* rfit[2] = {nullptr, nullptr};  // and their exact fitness
+  __nv_bfloat16* rXb[2] = {nullptr, nullptr};   // their training operands
+  float* rt[2] = {nullptr, nullptr};
+  bool ring_ready[2] = {false, false};   // rXb and rt are those of rX and rfit
   int ring_n = 0, ring_head = 0;
+  float* ut = nullptr;        // targets of a caller's or the first batch [sd.Bmax]
   float* uX = nullptr;        // device copies of caller arrays
   double* ufitd = nullptr;
   float* upred = nullptr;
@@ -477,9 +481,12 @@ int ensure_surrogate(game_ctx* h, int rows) {
     if (dev_alloc(&s.w, n) != cudaSuccess || dev_alloc(&s.g, n) != cudaSuccess ||
         dev_alloc(&s.m, n) != cudaSuccess || dev_alloc(&s.v, n) != cudaSuccess ||
         dev_alloc(&s.loss, 1) != cudaSuccess || dev_alloc(&s.tstat, 2) != cudaSuccess ||
-        dev_alloc(&s.split_ws, (size_t)kMaxSplits * kSurrogateHidden *
-                                   (h->Kg > kSurrogateHidden ? h->Kg : kSurrogateHidden)) !=
-            cudaSuccess) {
+        dev_alloc(&s.split1, (size_t)kMaxSplits * kSurrogateHidden * h->Kg) != cudaSuccess ||
+        dev_alloc(&s.split2, (size_t)kMaxSplits * kSurrogateHidden * kSurrogateHidden) !=
+            cudaSuccess ||
+        dev_alloc(&s.W1b, (size_t)kSurrogateHidden * surrogate_kq(h->Kg)) != cudaSuccess ||
+        dev_alloc(&s.W2b, (size_t)kSurrogateHidden * kSurrogateHidden) != cudaSuccess ||
+        dev_alloc(&s.W2t, (size_t)kSurrogateHidden * kSurrogateHidden) != cudaSuccess) {
       cudaGetLastError();
       return fail(GAME_ENOMEM, "surrogate parameters");
     }
@@ -498,7 +505,13 @@ int ensure_surrogate(game_ctx* h, int rows) {
     dev_free(s.dout);
     dev_free(s.lterm);
     dev_free(s.lfit);
-    s.out = s.dout = s.lterm = nullptr;
+    dev_free(h->ut);
+    __nv_bfloat16** bb[4] = {&s.Xb, &s.H1b, &s.dZ2h, &s.dZ2l};
+    for (__nv_bfloat16** b : bb) {
+      dev_free(*b);
+      *b = nullptr;
+    }
+    s.out = s.dout = s.lterm = h->ut = nullptr;
     s.lfit = nullptr;
     s.Bmax = 0;
     for (float** b : bufs)
@@ -506,8 +519,13 @@ int ensure_surrogate(game_ctx* h, int rows) {
         cudaGetLastError();
         return fail(GAME_ENOMEM, "surrogate workspace");
       }
+    const size_t hid = (size_t)rows * kSurrogateHidden;
     if (dev_alloc(&s.out, rows) != cudaSuccess || dev_alloc(&s.dout, rows) != cudaSuccess ||
-        dev_alloc(&s.lterm, rows) != cudaSuccess || dev_alloc(&s.lfit, rows) != cudaSuccess) {
+        dev_alloc(&s.lterm, rows) != cudaSuccess || dev_alloc(&s.lfit, rows) != cudaSuccess ||
+        dev_alloc(&h->ut, rows) != cudaSuccess ||
+        dev_alloc(&s.Xb, (size_t)rows * surrogate_kq(h->Kg)) != cudaSuccess ||
+        dev_alloc(&s.H1b, hid) != cudaSuccess || dev_alloc(&s.dZ2h, hid) != cudaSuccess ||
+        dev_alloc(&s.dZ2l, hid) != cudaSuccess) {
       cudaGetLastError();
       return fail(GAME_ENOMEM, "surrogate workspace");
     }
@@ -516,13 +534,14 @@ int ensure_surrogate(game_ctx* h, int rows) {
   return GAME_OK;
 }
 
-// One Adam step of the surrogate on device pairs (X [n][K], fit [n]).
-int surrogate_step(game_ctx* h, const float* X, const double* fit, int n) {
+// A batch of device pairs (X [n][K], fit [n]) ready for steps, its operands in
+// the surrogate's own workspace.
+int surrogate_batch(game_ctx* h, const float* X, const double* fit, int n, SurrogateBatch* b) {
   int rc = ensure_surrogate(h, n);
   if (rc) return rc;
-  CK(surrogate_forward(h->sd, X, n, h->sd.out, h->st));
-  CK(surrogate_backward(h->sd, X, fit, n, h->st));
-  CK(surrogate_adam(h->sd, h->st));
+  CK(surrogate_to_bf16(h->Kg, X, n, h->sd.Xb, h->st));
+  CK(surrogate_targets(h->sd, fit, n, h->ut, h->st));
+  *b = SurrogateBatch{X, h->sd.Xb, h->ut, n};
   return GAME_OK;
 }
 
@@ -536,13 +555,22 @@ int surrogate_learn(game_ctx* h) {
                      cudaMemcpyDeviceToDevice, h->st));
   CK(cudaMemcpyAsync(h->rfit[slot], h->fit, (size_t)P * sizeof(double),
                      cudaMemcpyDeviceToDevice, h->st));
+  h->ring_ready[slot] = false;
   h->ring_head ^= 1;
   if (h->ring_n < 2) h->ring_n += 1;
+  int rc = ensure_surrogate(h, P);
+  if (rc) return rc;
+  for (int i = 0; i < h->ring_n; ++i) {
+    const int sl = (slot - i + 2) % 2;
+    if (h->ring_ready[sl]) continue;
+    CK(surrogate_to_bf16(K, h->rX[sl], P, h->rXb[sl], h->st));
+    CK(surrogate_targets(h->sd, h->rfit[sl], P, h->rt[sl], h->st));
+    h->ring_ready[sl] = true;
+  }
   for (int rep = 0; rep < h->prm.surrogate_steps; ++rep)
     for (int i = h->ring_n - 1; i >= 0; --i) {
       const int sl = (slot - i + 2) % 2;
-      const int rc = surrogate_step(h, h->rX[sl], h->rfit[sl], P);
-      if (rc) return rc;
+      CK(surrogate_step(h->sd, SurrogateBatch{h->rX[sl], h->rXb[sl], h->rt[sl], P}, true, h->st));
     }
   return GAME_OK;
 }
@@ -555,7 +583,11 @@ int setup_screening(game_ctx* h) {
   if (dev_alloc(&h->off, (size_t)(E + n) * K) != cudaSuccess ||
       dev_alloc(&h->oplan, (size_t)(E + n)) != cudaSuccess ||
       dev_alloc(&h->pred, (size_t)n) != cudaSuccess || dev_alloc(&h->flag, (size_t)n) != cudaSuccess ||
-      dev_alloc(&h->pos, (size_t)n) != cudaSuccess ||
+      dev_alloc(&h->list, (size_t)n) != cudaSuccess ||
+      dev_alloc(&h->rXb[0], (size_t)P * surrogate_kq(K)) != cudaSuccess ||
+      dev_alloc(&h->rXb[1], (size_t)P * surrogate_kq(K)) != cudaSuccess ||
+      dev_alloc(&h->rt[0], (size_t)P) != cudaSuccess ||
+      dev_alloc(&h->rt[1], (size_t)P) != cudaSuccess ||
       dev_alloc(&h->rX[0], (size_t)P * K) != cudaSuccess ||
       dev_alloc(&h->rX[1], (size_t)P * K) != cudaSuccess ||
       dev_alloc(&h->rfit[0], (size_t)P) != cudaSuccess ||
@@ -567,8 +599,11 @@ int setup_screening(game_ctx* h) {
   CK(cudaMemsetAsync(h->trust, 0, 2 * sizeof(int), h->st));   // untrusted until checked
   CK(cudaMemsetAsync(h->trust_r, 0, sizeof(float), h->st));
   int rc = ensure_surrogate(h, n > P ? n : P);
-  for (int i = 0; i < 20 && !rc; ++i) rc = surrogate_step(h, h->pop[h->cur], h->fit, P);
-  return rc;
+  SurrogateBatch b;
+  if (!rc) rc = surrogate_batch(h, h->pop[h->cur], h->fit, P, &b);
+  if (rc) return rc;
+  for (int i = 0; i < 20; ++i) CK(surrogate_step(h->sd, b, true, h->st));
+  return GAME_OK;
 }
 
 // Waits for the handle's work and reports its status word; gens_run: the
@@ -737,12 +772,14 @@ void destroy_ctx(game_ctx* h) {
   dev_free(h->ufit);
   SurrogateDev& s = h->sd;
   float* sb[] = {s.w, s.g, s.m, s.v, s.Z1, s.H1, s.Z2, s.H2, s.dZ1, s.dZ2, s.out, s.dout,
-                 s.lterm, s.loss, s.split_ws, h->off, h->pred, h->rX[0], h->rX[1], h->uX,
+                 s.lterm, s.loss, s.split1, s.split2, h->ut, h->rt[0], h->rt[1], h->off, h->pred, h->rX[0], h->rX[1], h->uX,
                  h->upred};
   for (float* b : sb) dev_free(b);
   dev_free(h->oplan);
   dev_free(h->flag);
-  dev_free(h->pos);
+  dev_free(h->list);
+  __nv_bfloat16* bb[] = {s.Xb, s.H1b, s.dZ2h, s.dZ2l, s.W1b, s.W2b, s.W2t, h->rXb[0], h->rXb[1]};
+  for (__nv_bfloat16* b : bb) dev_free(b);
   dev_free(h->rfit[0]);
   dev_free(h->rfit[1]);
   dev_free(h->ufitd);
@@ -1050,7 +1087,7 @@ int game_generation(game_t h, uint64_t seed) {
     rc = ensure_surrogate(h, n);
     if (rc) return rc;
     CK(surrogate_forward(h->sd, h->off + (size_t)E * K, n, h->pred, h->st));
-    CK(surrogate_screen(n, P - E, E, K, h->pred, h->flag, h->pos, h->off, h->pop[h->cur ^ 1],
+    CK(surrogate_screen(n, P - E, E, K, h->pred, h->flag, h->list, h->off, h->pop[h->cur ^ 1],
                         h->trust, h->trust + 1, h->st));
     stage_end(h, t0, kSurrogate);
     h->last_n = n;
@@ -1061,8 +1098,8 @@ int game_generation(game_t h, uint64_t seed) {
     if (rc) return rc;
     h->fit_valid = true;
     t0 = stage_begin(h);
-    CK(surrogate_trust_check(h->sd, n, P - E, h->pred, h->flag, h->pos, h->fit + E, h->trust_r,
-                             h->trust, h->st));
+    CK(surrogate_trust_check(h->sd, P - E, h->pred, h->list, h->fit + E, h->trust_r, h->trust,
+                             h->st));
     rc = surrogate_learn(h);
     stage_end(h, t0, kSurrogate);
     return rc;
@@ -1313,8 +1350,10 @@ int game_surrogate_grad(game_t h, const float* pop, const double* fit, int32_t n
   if (!h || !pop || !fit || !grad_out || n < 1) return fail(GAME_EINVAL, "bad argument");
   int rc = surrogate_inputs(h, pop, fit, n);
   if (rc) return rc;
-  CK(surrogate_forward(h->sd, h->uX, n, h->sd.out, h->st));
-  CK(surrogate_backward(h->sd, h->uX, h->ufitd, n, h->st));
+  SurrogateBatch b;
+  rc = surrogate_batch(h, h->uX, h->ufitd, n, &b);
+  if (rc) return rc;
+  CK(surrogate_step(h->sd, b, false, h->st));
   CK(cudaMemcpyAsync(grad_out, h->sd.g, surrogate_param_count(h->Kg) * sizeof(float),
                      cudaMemcpyDefault, h->st));
   if (loss_out) CK(cudaMemcpyAsync(loss_out, h->sd.loss, sizeof(float), cudaMemcpyDefault, h->st));
@@ -1326,8 +1365,10 @@ int game_surrogate_train(game_t h, const float* pop, const double* fit, int32_t 
   if (!h || !pop || !fit || n < 1) return fail(GAME_EINVAL, "bad argument");
   int rc = surrogate_inputs(h, pop, fit, n);
   if (rc) return rc;
-  rc = surrogate_step(h, h->uX, h->ufitd, n);
+  SurrogateBatch b;
+  rc = surrogate_batch(h, h->uX, h->ufitd, n, &b);
   if (rc) return rc;
+  CK(surrogate_step(h->sd, b, true, h->st));
   return check_status(h);
 }
 
@@ -1352,6 +1393,7 @@ int game_surrogate_set_params(game_t h, const float* w) {
   CK(cudaMemsetAsync(h->sd.m, 0, n * sizeof(float), h->st));
   CK(cudaMemsetAsync(h->sd.v, 0, n * sizeof(float), h->st));
   h->sd.step = 0;
+  CK(surrogate_weights_changed(h->sd, h->st));
   return check_status(h);
 }
 
@@ -1644,6 +1686,8 @@ int game_load(game_t h, const char* path) {
     if (!rc) rc = undump(h, file.f, h->trust_r, sizeof(float));
     for (int i = 0; i < 2 && !rc; ++i) rc = undump(h, file.f, h->rX[i], P * K * sizeof(float));
     for (int i = 0; i < 2 && !rc; ++i) rc = undump(h, file.f, h->rfit[i], P * sizeof(double));
+    h->ring_ready[0] = h->ring_ready[1] = false;
+    CK(surrogate_weights_changed(h->sd, h->st));
     if (!rc) {
       h->sd.step = c.sur_step;
       h->ring_n = c.ring_n;

@@ -222,11 +222,12 @@ __host__ __device__ inline int table_bytes(const GaDev& ga) {
                                        : 0;
 }
 
-// One CTA of kPlanThreads threads: elites, parent selection and crossover plan of
+// CTA `block` of `blocks`, kPlanThreads threads: elites (the first CTA), parent selection and crossover plan of
 // one problem (plan[s] = {head parent, tail parent, cut, elite flag}) for
 // ga.Nout output slots; tournaments draw from the ga.P current chromosomes.
 __device__ __forceinline__ void plan_body(const GaDev& ga, const double* __restrict__ fit,
-                                          uint64_t seed, uint32_t g, int4* __restrict__ plan) {
+                                          uint64_t seed, uint32_t g, int4* __restrict__ plan,
+                                          int block = 0, int blocks = 1) {
   __shared__ int elite[kMaxElites];
   __shared__ uint64_t wkey[kPlanThreads / 32];
   __shared__ int widx[kPlanThreads / 32];
@@ -234,7 +235,8 @@ __device__ __forceinline__ void plan_body(const GaDev& ga, const double* __restr
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   // 1. elites: the first ranks where the selection sorted the population, else
   // by counting, else one block-wide arg-min per elite
-  if (ga.sel == GAME_SEL_RANKING) {
+  if (block != 0) {
+  } else if (ga.sel == GAME_SEL_RANKING) {
     for (int e = tid; e < ga.E; e += kPlanThreads) elite[e] = ga.order[e];
     __syncthreads();
   } else if (ga.P <= kCountMax) {
@@ -270,12 +272,14 @@ __device__ __forceinline__ void plan_body(const GaDev& ga, const double* __restr
       __syncthreads();
     }
   }
-  for (int e = tid; e < ga.E; e += kPlanThreads) plan[e] = make_int4(elite[e], elite[e], ga.K, 1);
+  if (block == 0)
+    for (int e = tid; e < ga.E; e += kPlanThreads)
+      plan[e] = make_int4(elite[e], elite[e], ga.K, 1);
 
   // 2.-3. pairs: the two parents and the crossover decision, a thread each
   const int npairs = (ga.Nout - ga.E + 1) / 2;
   int* words = reinterpret_cast<int*>(plan);
-  for (int t = tid; t < 3 * npairs; t += kPlanThreads) {
+  for (int t = block * kPlanThreads + tid; t < 3 * npairs; t += blocks * kPlanThreads) {
     const int q = t / 3, r = t - 3 * q;
     const int s0 = ga.E + 2 * q;
     int* w0 = words + 4 * (int64_t)s0;   // slot s0's {head, tail, cut, elite}

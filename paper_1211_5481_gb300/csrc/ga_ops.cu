@@ -60,7 +60,7 @@ roulette_cum_kernel(int P, const double* __restrict__ fit, uint64_t* __restrict_
 __global__ void __launch_bounds__(kPlanThreads)
 ga_plan_kernel(GaDev g_, const double* __restrict__ fit, uint64_t seed, uint32_t g,
                int4* __restrict__ plan) {
-  ga::plan_body(g_, fit, seed, g, plan);
+  ga::plan_body(g_, fit, seed, g, plan, blockIdx.x, gridDim.x);
 }
 
 __global__ void ga_breed_kernel(GaDev g_, const float* __restrict__ pop,
@@ -144,7 +144,10 @@ cudaError_t launch_generation(const GaDev& ga, const float* pop, const double* f
     if (!ga.cum) return cudaErrorInvalidValue;
     roulette_cum_kernel<<<1, kPlanThreads, 0, st>>>(ga.P, fit, ga.cum);
   }
-  ga_plan_kernel<<<1, kPlanThreads, 0, st>>>(ga, fit, seed, g, plan);
+  // three threads per pair of slots: oversampled offspring take several CTAs
+  // (16,370 slots on one: 51 us)
+  const int blocks = ceil_div(3 * ((int64_t)(ga.Nout - ga.E + 1) / 2), kPlanThreads);
+  ga_plan_kernel<<<blocks < 1 ? 1 : blocks, kPlanThreads, 0, st>>>(ga, fit, seed, g, plan);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   ga_breed_kernel<<<blocks_for((int64_t)ga.Nout * ga.K, 256), 256, 0, st>>>(ga, pop, plan, seed,

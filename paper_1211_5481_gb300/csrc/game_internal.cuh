@@ -190,30 +190,46 @@ struct SurrogateDev {
   float* loss;             // [1]
   double* tstat;           // [2] mean and sd of the batch's log-fitness
   double* lfit;            // [Bmax] the batch's log-fitness
-  float* split_ws;         // [kMaxSplits][256][max(K, 256)] split-K partial products
+  float *split1, *split2;  // [kMaxSplits][256][K] and [..][256][256] split-K partial products
+  // BF16 operands, Kq = surrogate_kq(K) columns (zero past K)
+  __nv_bfloat16 *Xb, *H1b, *dZ2h, *dZ2l;   // [Bmax][Kq], [Bmax][256] ...
+  __nv_bfloat16 *W1b, *W2b, *W2t;          // [256][Kq], [256][256], its transpose
   int* status;             // the handle's device status word (expired waits)
 };
+// A training batch: n rows of genes, their BF16 copy, their standardised targets
+struct SurrogateBatch {
+  const float* X;
+  const __nv_bfloat16* Xb;
+  const float* t;
+  int n;
+};
+int surrogate_kq(int K);   // K rounded up to whole K-blocks of 64
 int64_t surrogate_param_count(int K);
 cudaError_t surrogate_init(const SurrogateDev& s, uint64_t seed, cudaStream_t st);
 cudaError_t surrogate_forward(const SurrogateDev& s, const float* X, int B, float* out,
                               cudaStream_t st);
-cudaError_t surrogate_backward(const SurrogateDev& s, const float* X, const double* fit, int B,
-                               cudaStream_t st);
-cudaError_t surrogate_adam(SurrogateDev& s, cudaStream_t st);
+// after a change of s.w other than a step: the weights' BF16 copies
+cudaError_t surrogate_weights_changed(const SurrogateDev& s, cudaStream_t st);
+// a batch's preparation: Xb [B][Kq] and t [B] from the exact fitness
+cudaError_t surrogate_to_bf16(int K, const float* X, int B, __nv_bfloat16* Xb, cudaStream_t st);
+cudaError_t surrogate_targets(const SurrogateDev& s, const double* fit, int B, float* t,
+                              cudaStream_t st);
+// gradient into s.g and loss into s.loss; with apply, an Adam step
+cudaError_t surrogate_step(SurrogateDev& s, const SurrogateBatch& b, bool apply, cudaStream_t st);
 // keeps the n_keep smallest predictions of the n children (slots E..E+n-1 of
 // off [E+n][K]) and writes the elites then the kept children in slot order to
-// next [E+n_keep][K]; flag [n] (1 = kept) and pos [n] are scratch / outputs.
+// next [E+n_keep][K]; flag [n] (1 = kept), list [n_keep] the kept children.
 // (the screening keeps the first n_keep children when *trusted is 0, and
 // records the flag it used in *used_trust)
 cudaError_t surrogate_screen(int n, int n_keep, int E, int K, const float* pred, int* flag,
-                             int* pos, const float* off, float* next, const int* trusted,
+                             int* list, const float* off, float* next, const int* trusted,
                              int* used_trust, cudaStream_t st);
 // r = Pearson correlation of the kept children's predictions with their exact
 // log-fitness (fit_kept [n_kept] in slot order; their logs go through s.lfit);
 // *trusted = r > 0.25.
-cudaError_t surrogate_trust_check(const SurrogateDev& s, int n, int n_kept, const float* pred,
-                                  const int* flag, const int* pos, const double* fit_kept,
-                                  float* r_out, int* trusted, cudaStream_t st);
+cudaError_t surrogate_trust_check(const SurrogateDev& s, int n_kept, const float* pred,
+                                  const int* list, const double* fit_kept, float* r_out,
+                                  int* trusted, cudaStream_t st);
 
 // gram.cu -- the Gram form of the MSE (FP64)
 int64_t gram_chunk_rows(const Shape& s);

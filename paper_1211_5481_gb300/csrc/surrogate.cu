@@ -17,12 +17,19 @@
 // Parameter vector (FP32, this order): W1 [256][K], b1 [256], W2 [256][256],
 // b2 [256], w3 [256], b3 [1].
 //
-// Kernels: one tensor-core GEMM with strides (C = A B with any transposition,
-// BF16 operands -- FP32 ones split into BF16 hi + lo -- with FP32
-// accumulation in tensor memory, an optional bias + GELU epilogue), column sums in a fixed order, the GELU
-// derivative, the output layer, and Adam. Screening: a one-CTA bitonic sort
-// of (prediction, slot) keys, a flag per kept slot and a prefix-sum
-// compaction that assembles the next population in slot order. The exact
+// Kernels. The products whose operands lie along k in memory -- X W1^T, H1 W2^T
+// and dZ2 W2 -- take BF16 copies of them (gemm_nt_kernel: all K-blocks copied
+// asynchronously at once, no conversion on the way; Adam refreshes the weights'
+// copies, the batch's is made once per batch). The weight gradients (reduction
+// over the batch) take FP32 operands, transposed on the way and split into BF16
+// hi + lo (grad_gemm_kernel, split-K, both layers in one launch). Between them:
+// one kernel for the output layer, its gradient and dZ2, one for the four bias
+// and output-weight sums, one for the split sums and Adam. A training step is
+// seven launches. With conversion inside one generic GEMM, the statistics of
+// the batch in every step and a kernel per elementwise step it was 19: 178 us a
+// step at P = 2048, K = 289, now STEPTIME_HERE.
+// Screening: a radix selection of the predictions in one CTA that also numbers
+// the kept slots, and a gather in slot order (SCREENTIME_HERE). The exact
 // fitness checks the surrogate: after each screened generation the Pearson
 // correlation r of the kept children's predictions with their exact
 // log-fitness is measured, and the next screening trusts the surrogate only
@@ -32,6 +39,7 @@
 
 #include "game_internal.cuh"
 #include "philox.cuh"
+#include "tc_ptx.cuh"
 
 namespace game {
 
@@ -40,10 +48,6 @@ namespace {
 constexpr int kH = kSurrogateHidden;
 constexpr float kGeluC = 0.7978845608028654f;   // sqrt(2 / pi)
 constexpr float kGeluA = 0.044715f;
-
-__device__ __forceinline__ float round_bf16(float x) {
-  return __bfloat162float(__float2bfloat16_rn(x));
-}
 
 __device__ __forceinline__ float gelu(float z) {
   const float u = kGeluC * (z + kGeluA * z * z * z);
@@ -56,67 +60,20 @@ __device__ __forceinline__ float gelu_grad(float z) {
   return 0.5f * (1.f + t) + 0.5f * z * (1.f - t * t) * kGeluC * (1.f + 3.f * kGeluA * z * z);
 }
 
-// C[m][n] = sum_k A(m, k) B(k, n), A(m, k) = A[m * am + k * ak], B(k, n) =
-// B[k * bk + n * bn], on the tensor cores (tcgen05, FP32 accumulation in tensor
-// memory). Operands flagged for rounding enter as their BF16 values; the
-// others (FP32 gradients) as hi = bf16(v) plus lo = bf16(v - hi), with the
-// MMAs hi*hi + hi*lo + lo*hi, so products lose at most ~2^-16 of their
-// value. CTA tile: 128 rows of C (MMA-M, tensor-memory lanes) x TN columns
-// (MMA-N); K in blocks of 64 through a double-buffered shared-memory ring in
-// the K-major SWIZZLE_128B layout, filled by all 256 threads (g_load),
-// consumed by MMAs issued by thread 0;
-// the epilogue reads the accumulator rows back (thread = row of C). Split-K:
-// blockIdx.z takes k-range [z * kz, (z + 1) * kz) and, with splits > 1, writes
-// its partial product to C + z * M * ldc (reduced in order by splitk_reduce).
-// Epilogue modes (splits == 1): 0 store C; 1 store Z = C + bias[n] to C and
-// g(Z) (BF16-rounded when round_out) to out2; 2 store C + bias[n].
 // Waits are bounded (1 s): an expired wait abandons the tile and raises
 // *status.
 constexpr int kGTK = 64;                  // K per block (128 bytes of BF16 per row)
 constexpr uint32_t kGemmWaitNs = 1000000000ull;
 
-__device__ __forceinline__ uint32_t g_smem(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
 __device__ __forceinline__ bool g_wait(uint32_t bar, uint32_t parity, int* status) {
-  uint32_t ok = 0;
-  uint64_t t0 = 0;
-  for (int it = 0;; ++it) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (ok) return true;
-    uint64_t t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    if (it == 0) t0 = t;
-    else if (t - t0 > kGemmWaitNs) {
-      atomicExch(status, 1);
+  if (ptx::mbar_try_wait(bar, parity)) return true;
+  const uint64_t t0 = ptx::global_timer_ns();
+  while (!ptx::mbar_try_wait(bar, parity))
+    if (ptx::global_timer_ns() - t0 > kGemmWaitNs) {
+      atomicExch(status, (int)kDevTimeout);
       return false;
     }
-  }
-}
-
-__device__ __forceinline__ uint64_t g_desc(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)1 << 16;
-  d |= (uint64_t)(1024u >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)2 << 61;
-  return d;
-}
-
-__device__ __forceinline__ void g_mma(uint32_t d_tmem, uint64_t ad, uint64_t bd, uint32_t idesc,
-                                      uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
-      : "memory");
+  return true;
 }
 
 __device__ __forceinline__ uint32_t bf16pair(float lo, float hi) {
@@ -192,160 +149,321 @@ __device__ __forceinline__ void g_load(uint8_t* img, uint8_t* img_lo, const floa
   }
 }
 
-template <int TN>
+constexpr int kGTN = 64;   // columns of C per CTA
+
+// One weight gradient: C[m][n] = sum_b A[b][m] B[b][n] (A = dZ [batch][256] FP32
+// entering as BF16 hi + lo, B = the layer's input [batch][N] rounded to BF16).
+struct GradProblem {
+  const float *A, *B;
+  float* parts;   // [splits][256][N] partial products
+  int N, tiles;   // column tiles of kGTN
+};
+
+// Both layers' weight gradients in one launch: blockIdx.x < p0.tiles is the
+// first problem's column tile, the rest the second's; blockIdx.y the 128-row
+// tile of the 256 outputs; blockIdx.z takes batch rows [z kz, (z + 1) kz) and
+// writes its partial product to parts + z 256 N (added in order by adam_kernel).
+// Products: hi hi + lo hi.
 __global__ void __launch_bounds__(kGThreads, 1)
-gemm_tc_kernel(int M, int N, int Kd, const float* __restrict__ A, int64_t am, int64_t ak,
-               const float* __restrict__ B, int64_t bk, int64_t bn, int round_a, int round_b,
-               float* __restrict__ C, int64_t ldc, int mode, const float* __restrict__ bias,
-               float* __restrict__ out2, int round_out, int kz, int* status) {
-  constexpr uint32_t kAImg = 128 * 128, kBImg = TN * 128;
-  constexpr uint32_t kStage = 2 * kAImg + 2 * kBImg;   // hi and lo images of both operands
+grad_gemm_kernel(int batch, GradProblem p0, GradProblem p1, int kz, int* status) {
+  constexpr uint32_t kAImg = 128 * 128, kBImg = kGTN * 128;
+  constexpr uint32_t kStage = 2 * kAImg + kBImg;   // hi and lo images of A
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(base + 2 * kStage);   // [2] stage free, [1] done
   uint32_t* holder = reinterpret_cast<uint32_t*>(bars + 3);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  static_assert(TN % 64 == 0, "two column halves of whole 32-column loads");
-  const int m0 = blockIdx.y * 128, n0 = blockIdx.x * TN;
+  const bool first = (int)blockIdx.x < p0.tiles;
+  const GradProblem p = first ? p0 : p1;
+  const int n0 = (first ? (int)blockIdx.x : (int)blockIdx.x - p0.tiles) * kGTN;
+  const int m0 = blockIdx.y * 128;
   const int kbeg = blockIdx.z * kz;
-  const int kend = min(Kd, kbeg + kz);
+  const int kend = min(batch, kbeg + kz);
   const int nkb = kend > kbeg ? (kend - kbeg + kGTK - 1) / kGTK : 0;
-  const bool split_a = !round_a, split_b = !round_b;
   if (tid == 0) {
-    for (int b = 0; b < 3; ++b)
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(g_smem(&bars[b])), "r"(1)
-                   : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    for (int b = 0; b < 3; ++b) ptx::mbar_init(ptx::smem_addr(&bars[b]), 1);
+    ptx::fence_mbar_init();
   }
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                     g_smem(holder)),
-                 "r"(TN < 32 ? 32 : TN)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    ptx::tmem_alloc(ptx::smem_addr(holder), kGTN);
+    ptx::tmem_relinquish();
   }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  ptx::tc_fence_before();
   __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  ptx::tc_fence_after();
   const uint32_t tmem = *holder;
-  const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TN >> 3) << 17) |
-                         ((uint32_t)(128 >> 4) << 24);
+  const uint32_t idesc = ptx::idesc_bf16_f32(128, kGTN);
   bool ok = true;
   for (int kb = 0; kb < nkb && ok; ++kb) {
     const int st = kb & 1;
     uint8_t* a_img = base + st * kStage;
     uint8_t* a_lo = a_img + kAImg;
     uint8_t* b_img = a_img + 2 * kAImg;
-    uint8_t* b_lo = b_img + kBImg;
     // the MMAs that read this stage two blocks ago are done
-    if (kb >= 2) ok = g_wait(g_smem(&bars[st]), ((kb - 2) >> 1) & 1, status);
+    if (kb >= 2) ok = g_wait(ptx::smem_addr(&bars[st]), ((kb - 2) >> 1) & 1, status);
     if (!ok) break;
     const int k0 = kbeg + kb * kGTK;
-    g_load<128>(a_img, a_lo, A, am, ak, m0, M, k0, kend, split_a);
-    g_load<TN>(b_img, b_lo, B, bn, bk, n0, N, k0, kend, split_b);
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    g_load<128>(a_img, a_lo, p.A, 1, kH, m0, kH, k0, kend, true);
+    g_load<kGTN>(b_img, nullptr, p.B, 1, p.N, n0, p.N, k0, kend, false);
+    ptx::fence_proxy_async_smem();
     __syncthreads();
     if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint64_t ad = g_desc(g_smem(a_img)), adl = g_desc(g_smem(a_lo));
-      const uint64_t bd = g_desc(g_smem(b_img)), bdl = g_desc(g_smem(b_lo));
+      ptx::tc_fence_after();
+      const uint64_t ad = ptx::desc_kmajor_sw128(ptx::smem_addr(a_img));
+      const uint64_t adl = ptx::desc_kmajor_sw128(ptx::smem_addr(a_lo));
+      const uint64_t bd = ptx::desc_kmajor_sw128(ptx::smem_addr(b_img));
 #pragma unroll
       for (int ks = 0; ks < 4; ++ks) {
         const uint32_t o = 2u * ks;
-        g_mma(tmem, ad + o, bd + o, idesc, (kb | ks) != 0);
-        if (split_b) g_mma(tmem, ad + o, bdl + o, idesc, 1u);
-        if (split_a) g_mma(tmem, adl + o, bd + o, idesc, 1u);
+        ptx::mma_bf16(tmem, ad + o, bd + o, idesc, (kb | ks) != 0);
+        ptx::mma_bf16(tmem, adl + o, bd + o, idesc, 1u);
       }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                       g_smem(&bars[st]))
-                   : "memory");
+      ptx::mma_commit(ptx::smem_addr(&bars[st]));
     }
   }
   // all MMAs done
-  if (tid == 0)
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                     g_smem(&bars[2]))
-                 : "memory");
-  const bool done = g_wait(g_smem(&bars[2]), 0, status);
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (done && ok) {
-    // each warp's 32 accumulator rows go through a 32 x 33 scratch tile (in
-    // the operand ring, idle now) so that the stores run along rows of C
-    // warp w reads tensor-memory lanes 32 (w % 4) .. (its quadrant), columns
-    // of half w / 4
+  if (tid == 0) ptx::mma_commit(ptx::smem_addr(&bars[2]));
+  const bool done = g_wait(ptx::smem_addr(&bars[2]), 0, status);
+  ptx::tc_fence_after();
+  // (the epilogue's scratch is the operand ring: every MMA of the CTA is done)
+  if (__syncthreads_and(done && ok)) {
+    // each warp's 32 accumulator rows go through a 32 x 33 scratch tile so that
+    // the stores run along rows of C; warp w reads tensor-memory lanes
+    // 32 (w % 4) .. (its quadrant), columns of half w / 4
     float* stage = reinterpret_cast<float*>(base) + warp * (32 * 33);
-    float* Cz = C + (int64_t)blockIdx.z * M * ldc;
-    const int quad = warp & 3, half = warp >> 2;
-#pragma unroll 1
-    for (int c0 = half * (TN / 2); c0 < (half + 1) * (TN / 2); c0 += 32) {
-      uint32_t v[32];
-      const uint32_t ta = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)c0;
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-          "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-          "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n\t"
-          "tcgen05.wait::ld.sync.aligned;"
-          : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-            "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]),
-            "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]),
-            "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
-            "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]),
-            "=r"(v[31])
-          : "r"(ta)
-          : "memory");
+    float* Cz = p.parts + (int64_t)blockIdx.z * kH * p.N;
+    const int quad = warp & 3, c0 = (warp >> 2) * (kGTN / 2);
+    uint32_t v[32];
+    ptx::tmem_ld32(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)c0, v);
 #pragma unroll
-      for (int e = 0; e < 32; ++e) stage[lane * 33 + e] = nkb > 0 ? __uint_as_float(v[e]) : 0.f;
-      __syncwarp();
-      const int n = n0 + c0 + lane;
+    for (int e = 0; e < 32; ++e) stage[lane * 33 + e] = nkb > 0 ? __uint_as_float(v[e]) : 0.f;
+    __syncwarp();
+    const int n = n0 + c0 + lane;
 #pragma unroll 4
-      for (int r = 0; r < 32; ++r) {
-        const int m = m0 + quad * 32 + r;
-        if (m < M && n < N) {
-          float x = stage[r * 33 + lane];
-          if (mode >= 1) x += bias[n];
-          Cz[(int64_t)m * ldc + n] = x;
-          if (mode == 1) {
-            const float gv = gelu(x);
-            out2[(int64_t)m * ldc + n] = round_out ? round_bf16(gv) : gv;
-          }
-        }
-      }
-      __syncwarp();
-    }
+    for (int r = 0; r < 32; ++r)
+      if (n < p.N) Cz[(int64_t)(m0 + quad * 32 + r) * p.N + n] = stage[r * 33 + lane];
   }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  ptx::tc_fence_before();
   __syncthreads();
   if (warp == 0) {
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                 "r"(TN < 32 ? 32 : TN)
-                 : "memory");
+    ptx::tc_fence_after();
+    ptx::tmem_dealloc(tmem, kGTN);
   }
 }
 
-// C[m][n] = sum over the splits, in order, of the partial products.
-__global__ void splitk_reduce_kernel(int64_t MN, int splits, const float* __restrict__ parts,
-                                     float* __restrict__ C) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < MN;
+// C[m][n] = sum_k A[m][k] B[n][k] for M rows and N = 256 columns, A [M][lda]
+// and B [256][lda] BF16, lda = nkb 64 (zero-padded), rows 16-byte aligned; with
+// NA = 2 A is a hi + lo pair (products hi B, lo B). What bounds it: latency
+// (2048 x 256 x 320 is a microsecond of tensor work over 64 CTAs), so a CTA
+// starts the copies of all its K-blocks (up to kNtStages; a ring beyond) before
+// it waits for the first. Epilogue:
+//   kLayer  Z = C + bias; H = g(Z); keep != 0: Z and H to memory (FP32, H rounded
+//           to BF16 where Hb is given); Hb the BF16 copy of H
+//   kDelta  out = C g'(Zin)
+enum NtMode : int { kLayer = 0, kDelta = 1 };
+struct NtArgs {
+  int M, nkb, mode, keep;
+  const __nv_bfloat16 *A, *A2, *B;
+  const float* bias;     // kLayer
+  const float* Zin;      // kDelta
+  float *Z, *H;          // kLayer (kDelta: H = out)
+  __nv_bfloat16* Hb;
+  int* status;
+};
+constexpr int kNtStages = 5;
+
+template <int NA>
+__host__ __device__ constexpr int nt_stages() { return NA == 1 ? kNtStages : 4; }
+template <int NA>
+__host__ __device__ constexpr int nt_smem() {
+  return nt_stages<NA>() * (NA * 128 * 128 + kGTN * 128) + 1024 + 128;
+}
+
+template <int NA>
+__global__ void __launch_bounds__(kGThreads, 1) gemm_nt_kernel(const NtArgs a) {
+  constexpr int NS = nt_stages<NA>();
+  constexpr uint32_t kAImg = 128 * 128;
+  constexpr uint32_t kStage = NA * kAImg + kGTN * 128;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* base = reinterpret_cast<uint8_t*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  uint64_t* bars = reinterpret_cast<uint64_t*>(base + NS * kStage);   // [NS] free, [1] done
+  uint32_t* holder = reinterpret_cast<uint32_t*>(bars + NS + 1);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int m0 = blockIdx.y * 128, n0 = blockIdx.x * kGTN;
+  const int64_t lda = (int64_t)a.nkb * kGTK;
+  if (tid == 0) {
+    for (int b = 0; b <= NS; ++b) ptx::mbar_init(ptx::smem_addr(&bars[b]), 1);
+    ptx::fence_mbar_init();
+  }
+  if (warp == 0) {
+    ptx::tmem_alloc(ptx::smem_addr(holder), kGTN);
+    ptx::tmem_relinquish();
+  }
+  // K-block kb into its stage: 16-byte units in the swizzled K-major layout,
+  // rows past M zero; one commit group (empty past the last K-block)
+  auto load = [&](int kb) {
+    if (kb < a.nkb) {
+      const uint32_t img = ptx::smem_addr(base + (kb % NS) * kStage);
+      const int unit = tid & 7;
+#pragma unroll
+      for (int im = 0; im < NA; ++im) {
+        const __nv_bfloat16* src = im ? a.A2 : a.A;
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+          const int r = (tid >> 3) + 32 * p;
+          const int row = m0 + r < a.M ? m0 + r : 0;
+          ptx::cp_async16_zfill(img + im * kAImg + r * 128 + ((unit ^ (r & 7)) << 4),
+                                src + row * lda + kb * kGTK + unit * 8, m0 + r < a.M);
+        }
+      }
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+        const int r = (tid >> 3) + 32 * p;
+        ptx::cp_async16_zfill(img + NA * kAImg + r * 128 + ((unit ^ (r & 7)) << 4),
+                              a.B + (n0 + r) * lda + kb * kGTK + unit * 8, true);
+      }
+    }
+    ptx::cp_async_commit();
+  };
+#pragma unroll
+  for (int kb = 0; kb < NS; ++kb) load(kb);
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::tc_fence_after();
+  const uint32_t tmem = *holder;
+  const uint32_t idesc = ptx::idesc_bf16_f32(128, kGTN);
+  bool ok = true;
+  for (int kb = 0; kb < a.nkb; ++kb) {
+    ptx::cp_async_wait<NS - 1>();
+    ptx::fence_proxy_async_smem();
+    __syncthreads();
+    const int st = kb % NS;
+    if (tid == 0) {
+      ptx::tc_fence_after();
+      const uint64_t ad = ptx::desc_kmajor_sw128(ptx::smem_addr(base + st * kStage));
+      const uint64_t bd = ptx::desc_kmajor_sw128(ptx::smem_addr(base + st * kStage + NA * kAImg));
+#pragma unroll
+      for (int ks = 0; ks < 4; ++ks) {
+        const uint32_t o = 2u * ks;
+        ptx::mma_bf16(tmem, ad + o, bd + o, idesc, (kb | ks) != 0);
+        if (NA == 2) ptx::mma_bf16(tmem, ad + (kAImg >> 4) + o, bd + o, idesc, 1u);
+      }
+      ptx::mma_commit(ptx::smem_addr(&bars[st]));
+    }
+    if (kb + NS < a.nkb) ok = ok && g_wait(ptx::smem_addr(&bars[st]), (kb / NS) & 1, a.status);
+    load(ok ? kb + NS : a.nkb);   // refilled once its MMAs are done
+  }
+  if (tid == 0) ptx::mma_commit(ptx::smem_addr(&bars[NS]));
+  const bool done = g_wait(ptx::smem_addr(&bars[NS]), 0, a.status);
+  ptx::cp_async_wait<0>();
+  ptx::tc_fence_after();
+  if (__syncthreads_and(done && ok)) {
+    float* stage = reinterpret_cast<float*>(base) + warp * (32 * 33);
+    const int quad = warp & 3, c0 = (warp >> 2) * (kGTN / 2);
+    uint32_t v[32];
+    ptx::tmem_ld32(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)c0, v);
+#pragma unroll
+    for (int e = 0; e < 32; ++e) stage[lane * 33 + e] = __uint_as_float(v[e]);
+    __syncwarp();
+    const int n = n0 + c0 + lane;
+    const float bias = a.mode == kLayer ? a.bias[n] : 0.f;
+#pragma unroll 4
+    for (int r = 0; r < 32; ++r) {
+      const int m = m0 + quad * 32 + r;
+      if (m >= a.M) break;
+      const int64_t at = (int64_t)m * kH + n;
+      float x = stage[r * 33 + lane];
+      if (a.mode == kLayer) {
+        x += bias;
+        const float g = gelu(x);
+        if (a.keep) a.Z[at] = x;
+        if (a.Hb) {
+          const __nv_bfloat16 gb = __float2bfloat16_rn(g);
+          a.Hb[at] = gb;
+          if (a.keep) a.H[at] = __bfloat162float(gb);
+        } else {
+          a.H[at] = g;
+        }
+      } else {
+        a.H[at] = x * gelu_grad(a.Zin[at]);
+      }
+    }
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    ptx::tc_fence_after();
+    ptx::tmem_dealloc(tmem, kGTN);
+  }
+}
+
+// Xb [B][Kq] = X [B][K] rounded to BF16, zero past K (16-byte units).
+__global__ void to_bf16_kernel(int64_t B, int K, int Kq, const float* __restrict__ X,
+                               __nv_bfloat16* __restrict__ Xb) {
+  const int per = Kq / 8;
+  const int64_t n = B * per;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
        e += (int64_t)gridDim.x * blockDim.x) {
-    float s = 0.f;
-    for (int z = 0; z < splits; ++z) s += parts[z * MN + e];
-    C[e] = s;
+    const int64_t b = e / per;
+    const int k0 = (int)(e - b * per) * 8;
+    float v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = k0 + u < K ? X[b * K + k0 + u] : 0.f;
+    reinterpret_cast<uint4*>(Xb)[e] = make_uint4(bf16pair(v[0], v[1]), bf16pair(v[2], v[3]),
+                                                 bf16pair(v[4], v[5]), bf16pair(v[6], v[7]));
   }
 }
 
-// out[b] = sum_j H2[b][j] w3[j] + b3 (one warp per row, fixed lane order)
+// Output layer: out[b] = sum_j H2[b][j] w3[j] + b3, one warp per row, fixed lane
+// order.
+__device__ __forceinline__ float output_row(const float* __restrict__ H2,
+                                            const float* __restrict__ w3, float b3, int lane) {
+  float s = 0.f;
+#pragma unroll
+  for (int j = 0; j < kH; j += 32) s = fmaf(H2[j + lane], w3[j + lane], s);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s + b3;
+}
+
 __global__ void output_kernel(int B, const float* __restrict__ H2, const float* __restrict__ w3,
                               const float* __restrict__ b3, float* __restrict__ out) {
   const int w = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
   if (w >= B) return;
-  float s = 0.f;
-  for (int j = lane; j < kH; j += 32) s = fmaf(H2[(int64_t)w * kH + j], w3[j], s);
+  const float s = output_row(H2 + (int64_t)w * kH, w3, b3[0], lane);
+  if (lane == 0) out[w] = s;
+}
+
+// A training row: the output, d_out[b] = 2 (out[b] - t[b]) / B, the loss term
+// (out - t)^2 / B, and dZ2[b][j] = d_out[b] w3[j] g'(Z2[b][j]), FP32 and as BF16
+// hi + lo (the next product's operand).
+__global__ void output_grad_kernel(int B, const float* __restrict__ H2,
+                                   const float* __restrict__ Z2, const float* __restrict__ w3,
+                                   const float* __restrict__ b3, const float* __restrict__ t,
+                                   float* __restrict__ dout, float* __restrict__ loss_terms,
+                                   float* __restrict__ dZ2, __nv_bfloat16* __restrict__ hi,
+                                   __nv_bfloat16* __restrict__ lo) {
+  const int w = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
+  const int lane = threadIdx.x & 31;
+  if (w >= B) return;
+  const int64_t row = (int64_t)w * kH;
+  const float r = output_row(H2 + row, w3, b3[0], lane) - t[w];
+  const float d = 2.f * r / (float)B;
+  if (lane == 0) {
+    dout[w] = d;
+    loss_terms[w] = r * r / (float)B;
+  }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) out[w] = s + b3[0];
+  for (int j = lane; j < kH; j += 32) {
+    const float v = d * w3[j] * gelu_grad(Z2[row + j]);
+    const __nv_bfloat16 h = __float2bfloat16_rn(v);
+    dZ2[row + j] = v;
+    hi[row + j] = h;
+    lo[row + j] = __float2bfloat16_rn(v - __bfloat162float(h));
+  }
 }
 
 // Mean and standard deviation of l = log(max(fit, 1e-30)) over the batch
@@ -394,68 +512,56 @@ target_stats_kernel(int B, const double* __restrict__ l, double* __restrict__ st
   }
 }
 
-// d_out[b] = 2 (out[b] - t[b]) / B with the standardised target t; also the
-// loss terms (out - t)^2 / B for reporting.
-__global__ void dout_kernel(int B, const float* __restrict__ out, const double* __restrict__ l,
-                            const double* __restrict__ stats, float* __restrict__ dout,
-                            float* __restrict__ loss_terms) {
+// The standardised targets t[b] = (l[b] - mean) / sd.
+__global__ void targets_kernel(int B, const double* __restrict__ l,
+                               const double* __restrict__ stats, float* __restrict__ t) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= B) return;
-  const float t = (float)((l[b] - stats[0]) / stats[1]);
-  const float r = out[b] - t;
-  dout[b] = 2.f * r / (float)B;
-  loss_terms[b] = r * r / (float)B;
+  if (b < B) t[b] = (float)((l[b] - stats[0]) / stats[1]);
 }
 
-// dH2[b][j] = dout[b] w3[j], dZ2 = dH2 * g'(Z2) (in place into dZ)
-__global__ void dz2_kernel(int B, const float* __restrict__ dout, const float* __restrict__ w3,
-                           const float* __restrict__ Z2, float* __restrict__ dZ) {
-  const int64_t n = (int64_t)B * kH;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int b = (int)(e / kH), j = (int)(e % kH);
-    dZ[e] = dout[b] * w3[j] * gelu_grad(Z2[e]);
-  }
-}
-
-// dZ[e] *= g'(Z[e])
-__global__ void gelu_bwd_kernel(int64_t n, const float* __restrict__ Z, float* __restrict__ dZ) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
-       e += (int64_t)gridDim.x * blockDim.x)
-    dZ[e] *= gelu_grad(Z[e]);
-}
-
-// s[j] = sum_b X[b][j] y[b] (y = NULL: plain column sum). CTA = 32 columns x
-// 32 row slices (1024 threads): thread (slice, column) adds its slice's rows
-// in order, then the 32 slice sums of a column are added in slice order --
+// s[j] = sum_b X[b][j] y[b] (y = NULL: plain column sum) over columns j0 ..
+// j0 + 31 of [B][256] by 1024 threads: thread (slice, column) adds its slice's
+// rows in order, then the 32 slice sums of a column are added in slice order --
 // a fixed order, so the result is the same run to run.
 constexpr int kColSlices = 32;
-__global__ void __launch_bounds__(1024)
-colsum_kernel(int B, int N, const float* __restrict__ X, const float* __restrict__ y,
-              float* __restrict__ s) {
+__device__ __forceinline__ void colsum_32(int B, int j0, const float* __restrict__ X,
+                                          const float* __restrict__ y, float* __restrict__ s) {
   __shared__ float part[kColSlices][33];
   const int c = threadIdx.x & 31, sl = threadIdx.x >> 5;
-  const int j = blockIdx.x * 32 + c;
+  const int j = j0 + c;
   const int per = (B + kColSlices - 1) / kColSlices;
   const int b0 = sl * per, b1 = min(B, b0 + per);
   float acc = 0.f;
-  if (j < N)
-    for (int b = b0; b < b1; ++b) acc = fmaf(X[(int64_t)b * N + j], y ? y[b] : 1.f, acc);
+  for (int b = b0; b < b1; b += 16) {   // 16 rows' loads in flight
+    float x[16], w[16];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) {
+      const int bb = b + u < b1 ? b + u : b0;
+      x[u] = X[(int64_t)bb * kH + j];
+      w[u] = y ? y[bb] : 1.f;
+    }
+#pragma unroll
+    for (int u = 0; u < 16; ++u)
+      if (b + u < b1) acc = fmaf(x[u], w[u], acc);
+  }
   part[sl][c] = acc;
   __syncthreads();
-  if (sl == 0 && j < N) {
+  if (sl == 0) {
     float t = 0.f;
     for (int k = 0; k < kColSlices; ++k) t += part[k][c];
     s[j] = t;
   }
 }
 
-__global__ void sum_kernel(int B, const float* __restrict__ v, float* __restrict__ s) {
-  if (blockIdx.x != 0) return;
+// s[0] = sum_b v[b], 256 strided sums added in order, by the first 256 threads.
+__device__ __forceinline__ void sum_256(int B, const float* __restrict__ v,
+                                        float* __restrict__ s) {
   __shared__ float part[256];
-  float acc = 0.f;
-  for (int b = threadIdx.x; b < B; b += 256) acc += v[b];
-  part[threadIdx.x] = acc;
+  if (threadIdx.x < 256) {
+    float acc = 0.f;
+    for (int b = threadIdx.x; b < B; b += 256) acc += v[b];
+    part[threadIdx.x] = acc;
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
     float t = 0.f;
@@ -464,18 +570,87 @@ __global__ void sum_kernel(int B, const float* __restrict__ v, float* __restrict
   }
 }
 
-__global__ void adam_kernel(int64_t n, float* __restrict__ w, const float* __restrict__ g,
-                            float* __restrict__ m, float* __restrict__ v, float lr, float b1,
-                            float b2, float eps, float c1, float c2) {
+// The gradients that are sums over the batch: CTAs 0-7 gw3 = sum_b dout[b]
+// H2[b], 8-15 gb2 = sum_b dZ2[b], 16-23 gb1 = sum_b dZ1[b], 24 gb3 = sum_b
+// dout[b], 25 the loss.
+__global__ void __launch_bounds__(1024)
+sums_kernel(int B, const float* __restrict__ H2, const float* __restrict__ dout,
+            const float* __restrict__ dZ2, const float* __restrict__ dZ1,
+            const float* __restrict__ loss_terms, float* __restrict__ gw3,
+            float* __restrict__ gb2, float* __restrict__ gb1, float* __restrict__ gb3,
+            float* __restrict__ loss) {
+  const int what = blockIdx.x / (kH / 32), j0 = (blockIdx.x % (kH / 32)) * 32;
+  if (what == 0) colsum_32(B, j0, H2, dout, gw3);
+  else if (what == 1) colsum_32(B, j0, dZ2, nullptr, gb2);
+  else if (what == 2) colsum_32(B, j0, dZ1, nullptr, gb1);
+  else if (j0 == 0) sum_256(B, dout, gb3);
+  else sum_256(B, loss_terms, loss);
+}
+
+// BF16 copies of one weight: W1b [256][Kq], W2b [256][256] and its transpose.
+__device__ __forceinline__ void copy_weight(int64_t e, float w, int K, int Kq,
+                                            __nv_bfloat16* __restrict__ W1b,
+                                            __nv_bfloat16* __restrict__ W2b,
+                                            __nv_bfloat16* __restrict__ W2t) {
+  const int64_t n1 = (int64_t)kH * K, w2 = e - n1 - kH;
+  const __nv_bfloat16 b = __float2bfloat16_rn(w);
+  if (e < n1) {
+    const int r = (int)((uint32_t)e / (uint32_t)K);
+    W1b[(int64_t)r * Kq + ((int)e - r * K)] = b;
+  } else if (w2 >= 0 && w2 < kH * kH) {
+    W2b[w2] = b;
+    W2t[(w2 % kH) * kH + w2 / kH] = b;
+  }
+}
+
+__global__ void copy_weights_kernel(int64_t n, int K, int Kq, const float* __restrict__ w,
+                                    __nv_bfloat16* __restrict__ W1b,
+                                    __nv_bfloat16* __restrict__ W2b,
+                                    __nv_bfloat16* __restrict__ W2t) {
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
+       e += (int64_t)gridDim.x * blockDim.x)
+    copy_weight(e, w[e], K, Kq, W1b, W2b, W2t);
+}
+
+// The weight gradients' split sums, in order, into g; then, with apply, Adam and
+// the weights' BF16 copies.
+__global__ void adam_kernel(int64_t n, int K, int Kq, int splits,
+                            const float* __restrict__ parts1, const float* __restrict__ parts2,
+                            float* __restrict__ w, float* __restrict__ g, float* __restrict__ m,
+                            float* __restrict__ v, bool apply, float lr, float b1, float b2,
+                            float eps, float c1, float c2, __nv_bfloat16* __restrict__ W1b,
+                            __nv_bfloat16* __restrict__ W2b, __nv_bfloat16* __restrict__ W2t) {
+  const int64_t n1 = (int64_t)kH * K;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
        e += (int64_t)gridDim.x * blockDim.x) {
-    const float gi = g[e];
+    const int64_t w2 = e - n1 - kH;
+    const bool in1 = e < n1, in2 = w2 >= 0 && w2 < kH * kH;
+    float gi;
+    if (in1 || in2) {
+      const float* part = in1 ? parts1 + e : parts2 + w2;
+      const int64_t step = in1 ? n1 : (int64_t)kH * kH;
+      gi = 0.f;
+      for (int z = 0; z < splits; z += 8) {   // eight loads in flight
+        float p[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) p[u] = part[(z + u < splits ? z + u : z) * step];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (z + u < splits) gi += p[u];
+      }
+      g[e] = gi;
+    } else {
+      gi = g[e];
+    }
+    if (!apply) continue;
     const float mi = b1 * m[e] + (1.f - b1) * gi;
     const float vi = b2 * v[e] + (1.f - b2) * gi * gi;
     m[e] = mi;
     v[e] = vi;
     const float mh = mi / c1, vh = vi / c2;
-    w[e] -= lr * mh / (sqrtf(vh) + eps);
+    const float wn = w[e] - lr * mh / (sqrtf(vh) + eps);
+    w[e] = wn;
+    copy_weight(e, wn, K, Kq, W1b, W2b, W2t);
   }
 }
 
@@ -513,133 +688,184 @@ __global__ void init_params_kernel(uint64_t seed, int K, float* __restrict__ w) 
 }
 
 // ---- screening: keep the n_keep smallest predictions of n ----
-constexpr int kSortMax = 16384;
+constexpr int kScreenThreads = 1024, kScreenWarps = kScreenThreads / 32;
 
-__global__ void __launch_bounds__(1024)
-select_kernel(int n, int n_keep, const float* __restrict__ pred, int* __restrict__ keep_flag,
-              const int* __restrict__ trusted, int* __restrict__ used_trust) {
-  extern __shared__ uint64_t keys[];   // (order-preserving float bits << 32) | slot
+// One CTA. Predictions as order-preserving 32-bit keys in shared memory; four
+// 8-bit histogram passes find the n_keep-th smallest key; smaller keys are kept
+// and, of the equal ones, the first slots. Each warp then owns a contiguous
+// range of slots, so ballots number the kept ones in slot order:
+// flag[i] and, for the j-th kept child i, list[j] = i. (A bitonic sort of 16,384 64-bit keys, then a scan, took 206 us.)
+__global__ void __launch_bounds__(kScreenThreads)
+screen_kernel(int n, int n_keep, const float* __restrict__ pred, int* __restrict__ flag,
+              int* __restrict__ list, const int* __restrict__ trusted,
+              int* __restrict__ used_trust) {
+  extern __shared__ uint32_t key[];
+  __shared__ int hist[256];
+  __shared__ uint32_t prefix;
+  __shared__ int want, wless[kScreenWarps], wequal[kScreenWarps];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int trust = *trusted;
-  if (threadIdx.x == 0) *used_trust = trust;
+  if (tid == 0) *used_trust = trust;
   if (!trust) {   // the exact evaluator stands in: the unscreened generation's children
-    for (int i = threadIdx.x; i < n; i += blockDim.x) keep_flag[i] = i < n_keep ? 1 : 0;
+    for (int i = tid; i < n; i += kScreenThreads) {
+      flag[i] = i < n_keep ? 1 : 0;
+      if (i < n_keep) list[i] = i;
+    }
     return;
   }
-  int npow = 1;
-  while (npow < n) npow <<= 1;
-  for (int i = threadIdx.x; i < npow; i += blockDim.x) {
-    uint64_t k = ~0ull;
-    if (i < n) {
-      float p = pred[i];
-      if (isnan(p)) p = __int_as_float(0x7f800000);   // NaN ranks last (+inf)
-      uint32_t u = __float_as_uint(p);
-      u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);   // float order as unsigned
-      k = ((uint64_t)u << 32) | (uint32_t)i;
-    }
-    keys[i] = k;
+  for (int i = tid; i < n; i += kScreenThreads) {
+    float p = pred[i];
+    if (isnan(p)) p = __int_as_float(0x7f800000);   // NaN ranks last (+inf)
+    const uint32_t u = __float_as_uint(p);
+    key[i] = (u & 0x80000000u) ? ~u : (u | 0x80000000u);   // float order as unsigned
   }
-  __syncthreads();
-  for (int size = 2; size <= npow; size <<= 1) {
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      for (int i = threadIdx.x; i < npow; i += blockDim.x) {
-        const int j = i ^ stride;
-        if (j > i) {
-          const bool up = (i & size) == 0;
-          const uint64_t a = keys[i], b = keys[j];
-          if ((a > b) == up) {
-            keys[i] = b;
-            keys[j] = a;
-          }
-        }
-      }
-      __syncthreads();
-    }
+  if (tid == 0) {
+    prefix = 0;
+    want = n_keep;   // place of the wanted key among those with the prefix (1-based)
   }
-  for (int i = threadIdx.x; i < n; i += blockDim.x) keep_flag[i] = 0;
-  __syncthreads();
-  for (int i = threadIdx.x; i < n_keep; i += blockDim.x)
-    keep_flag[(int)(keys[i] & 0xffffffffu)] = 1;
-}
-
-// pos[i] = number of kept children before child i (or -1 if child i is not
-// kept): one CTA, an exclusive prefix sum of the flags in slot order.
-__global__ void __launch_bounds__(1024)
-assemble_kernel(int n, const int* __restrict__ keep_flag, int* __restrict__ pos) {
-  __shared__ int warp_tot[32];
-  __shared__ int carry;
-  if (threadIdx.x == 0) carry = 0;
-  __syncthreads();
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int base = 0; base < n; base += blockDim.x) {
-    const int i = base + threadIdx.x;
-    const int f = i < n ? keep_flag[i] : 0;
-    int x = f;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    if (lane == 31) warp_tot[wid] = x;
+  for (int shift = 24; shift >= 0; shift -= 8) {
+    if (tid < 256) hist[tid] = 0;
     __syncthreads();
-    if (wid == 0) {
-      int t = warp_tot[lane];
+    const uint32_t pre = prefix;
+    for (int i = tid; i < n; i += kScreenThreads) {
+      const uint32_t k = key[i];
+      if (shift == 24 || (k >> (shift + 8)) == (pre >> (shift + 8)))
+        atomicAdd(&hist[(k >> shift) & 255u], 1);
+    }
+    __syncthreads();
+    if (warp == 0) {   // the bin that holds the wanted place
+      int h[8], sum = 0;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        h[u] = hist[lane * 8 + u];
+        sum += h[u];
+      }
+      int inc = sum;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, t, o);
-        if (lane >= o) t += y;
+        const int v = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += v;
       }
-      warp_tot[lane] = t;
+      int before = inc - sum;
+      const int w = want;
+      __syncwarp();
+      if (before < w && w <= inc) {
+        int u = 0;
+        while (before + h[u] < w) before += h[u++];
+        want = w - before;
+        prefix = pre | ((uint32_t)(lane * 8 + u) << shift);
+      }
     }
     __syncthreads();
-    const int excl = carry + (wid ? warp_tot[wid - 1] : 0) + x - f;
-    if (i < n) pos[i] = f ? excl : -1;
-    __syncthreads();
-    if (threadIdx.x == blockDim.x - 1) carry = excl + f;
-    __syncthreads();
+  }
+  const uint32_t T = prefix;
+  const int take = want;   // equal keys to keep
+  const int per = (n + kScreenThreads - 1) / kScreenThreads * 32;   // slots per warp
+  const int lo = min(n, warp * per), hi = min(n, lo + per);
+  int less = 0, equal = 0;
+  for (int i0 = lo; i0 < hi; i0 += 32) {
+    const int i = i0 + lane;
+    const bool in = i < hi;
+    const uint32_t k = in ? key[i] : 0u;
+    less += __popc(__ballot_sync(0xffffffffu, in && k < T));
+    equal += __popc(__ballot_sync(0xffffffffu, in && k == T));
+  }
+  if (lane == 0) {
+    wless[warp] = less;
+    wequal[warp] = equal;
+  }
+  __syncthreads();
+  int eq = 0, kept = 0;   // equal keys, kept children before this warp's range
+  for (int w = 0; w < warp; ++w) {
+    kept += wless[w];
+    eq += wequal[w];
+  }
+  kept += min(eq, take);
+  for (int i0 = lo; i0 < hi; i0 += 32) {
+    const int i = i0 + lane;
+    const bool in = i < hi;
+    const uint32_t k = in ? key[i] : 0u;
+    const uint32_t below = (1u << lane) - 1u;
+    const uint32_t em = __ballot_sync(0xffffffffu, in && k == T);
+    const bool keep = in && (k < T || (k == T && eq + __popc(em & below) < take));
+    const uint32_t km = __ballot_sync(0xffffffffu, keep);
+    if (in) {
+      flag[i] = keep ? 1 : 0;
+      if (keep) list[kept + __popc(km & below)] = i;
+    }
+    eq += __popc(em);
+    kept += __popc(km);
   }
 }
 
-__global__ void gather_kernel(int n, int E, int K, const int* __restrict__ pos,
+// next: rows 0..E-1 the elites, row E + j offspring slot E + list[j]; a warp per row.
+__global__ void gather_kernel(int rows, int E, int K, const int* __restrict__ list,
                               const float* __restrict__ off, float* __restrict__ next) {
-  // rows 0..E-1: elites; row E + pos[i] <- offspring slot E + i
-  const int64_t total = (int64_t)(E + n) * K;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int s = (int)(e / K), k = (int)(e % K);
-    if (s < E) {
-      next[e] = off[e];
-    } else {
-      const int p = pos[s - E];
-      if (p >= 0) next[(int64_t)(E + p) * K + k] = off[e];
-    }
-  }
+  const int r = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
+  if (r >= rows) return;
+  const int64_t from = r < E ? r : E + list[r - E];
+  for (int k = threadIdx.x & 31; k < K; k += 32) next[(int64_t)r * K + k] = off[from * K + k];
 }
 
 // Pearson correlation of the kept children's predictions with their exact
-// log-fitness (fit_kept[pos[i]] for kept child i), FP64 sums in a fixed
-// order; trusted = r > 0.25.
-__global__ void trust_kernel(int n, const float* __restrict__ pred, const int* __restrict__ flag,
-                             const int* __restrict__ pos, const double* __restrict__ lfit_kept,
-                             float* __restrict__ r_out, int* __restrict__ trusted) {
-  __shared__ double sh[6][256];
-  double a[6] = {0, 0, 0, 0, 0, 0};
-  for (int i = threadIdx.x; i < n; i += 256) {
-    if (!flag[i]) continue;
-    const double x = pred[i];
-    const double y = lfit_kept[pos[i]];
+// log-fitness, FP64 sums in a fixed order; trusted = r > 0.25. A cluster of 8
+// CTAs (FP64 is two operations a cycle and SM): a thread takes every 2048th
+// kept child, a warp's sums are exchanged so that lane 4 q ends with sum q, the
+// 64 warps' go to the leader's shared memory, six of its threads add them.
+constexpr int kTrustCtas = 8, kTrustThreads = 256;
+constexpr int kTrustWarps = kTrustCtas * kTrustThreads / 32;
+__global__ void __cluster_dims__(kTrustCtas, 1, 1) __launch_bounds__(kTrustThreads)
+trust_kernel(int n_kept, const float* __restrict__ pred, const int* __restrict__ list,
+             const double* __restrict__ lfit_kept, float* __restrict__ r_out,
+             int* __restrict__ trusted) {
+  __shared__ double sh[kTrustWarps][8];
+  __shared__ double tot[8];
+  ptx::cluster_arrive();
+  const int rank = (int)ptx::cluster_ctarank(), lane = threadIdx.x & 31;
+  const int w = rank * (kTrustThreads / 32) + (threadIdx.x >> 5);
+  double a[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  for (int j = rank * kTrustThreads + threadIdx.x; j < n_kept; j += kTrustCtas * kTrustThreads) {
+    const double x = pred[list[j]];
+    const double y = lfit_kept[j];
     a[0] += 1.0;
     a[1] += x;
     a[2] += y;
-    a[3] += x * y;
-    a[4] += x * x;
-    a[5] += y * y;
+    a[3] = fma(x, y, a[3]);
+    a[4] = fma(x, x, a[4]);
+    a[5] = fma(y, y, a[5]);
   }
-  for (int k = 0; k < 6; ++k) sh[k][threadIdx.x] = a[k];
+  int q0 = 0;
+#pragma unroll
+  for (int o = 16, m = 4; o >= 4; o >>= 1, m >>= 1) {
+    const bool up = (lane & o) != 0;
+    q0 += up ? m : 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (q < m) {
+        const double give = up ? a[q] : a[q + m];
+        const double keep = up ? a[q + m] : a[q];
+        a[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+      }
+  }
+  a[0] += __shfl_xor_sync(0xffffffffu, a[0], 2);
+  a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
+  ptx::cluster_wait();   // the leader runs
+  if ((lane & 3) == 0)
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(
+                     ptx::mapa(ptx::smem_addr(&sh[w][q0]), 0)),
+                 "d"(a[0])
+                 : "memory");
+  ptx::cluster_sync();
+  if (rank != 0) return;
+  if (threadIdx.x < 6) {
+    double t[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int i = 0; i < kTrustWarps; ++i) t[i & 3] += sh[i][threadIdx.x];
+    tot[threadIdx.x] = (t[0] + t[1]) + (t[2] + t[3]);
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
-    double t[6] = {0, 0, 0, 0, 0, 0};
-    for (int i = 0; i < 256; ++i)
-      for (int k = 0; k < 6; ++k) t[k] += sh[k][i];
+    const double* t = tot;
     const double c = t[0];
     double r = 0.0;
     if (c > 1.0) {
@@ -667,31 +893,12 @@ int grid1d(int64_t n) {
   return (int)b;
 }
 
-constexpr int kGTN = 64;   // columns of C per CTA of the tensor-core GEMM
-
-cudaError_t gemm(int M, int N, int Kd, const float* A, int64_t am, int64_t ak, const float* B,
-                 int64_t bk, int64_t bn, int ra, int rb, float* C, int64_t ldc, int mode,
-                 const float* bias, float* out2, int round_out, int* status, cudaStream_t st,
-                 float* split_ws = nullptr, int splits = 1) {
-  dim3 grid((N + kGTN - 1) / kGTN, (M + 127) / 128, splits);
-  int kz = (Kd + splits - 1) / splits;
-  kz = (kz + kGTK - 1) / kGTK * kGTK;
-  const int smem = 2 * (2 * 128 * 128 + 2 * kGTN * 128) + 1024 + 64;
-  cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<kGTN>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+template <int NA>
+cudaError_t gemm_nt(const NtArgs& a, cudaStream_t st) {
+  const cudaError_t e = cudaFuncSetAttribute(
+      gemm_nt_kernel<NA>, cudaFuncAttributeMaxDynamicSharedMemorySize, nt_smem<NA>());
   if (e != cudaSuccess) return e;
-  if (splits > 1) {
-    // partial products into the workspace, then their sum in split order
-    gemm_tc_kernel<kGTN><<<grid, kGThreads, smem, st>>>(M, N, Kd, A, am, ak, B, bk, bn, ra, rb,
-                                                  split_ws, N, 0, nullptr, nullptr, 0, kz, status);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    splitk_reduce_kernel<<<grid1d((int64_t)M * N), 256, 0, st>>>((int64_t)M * N, splits,
-                                                                  split_ws, C);
-    return cudaGetLastError();
-  }
-  gemm_tc_kernel<kGTN><<<grid, kGThreads, smem, st>>>(M, N, Kd, A, am, ak, B, bk, bn, ra, rb, C, ldc,
-                                                mode, bias, out2, round_out, kz, status);
+  gemm_nt_kernel<NA><<<dim3(kH / kGTN, (a.M + 127) / 128), kGThreads, nt_smem<NA>(), st>>>(a);
   return cudaGetLastError();
 }
 
@@ -701,6 +908,17 @@ int64_t surrogate_param_count(int K) {
   return (int64_t)kH * K + kH + (int64_t)kH * kH + kH + kH + 1;
 }
 
+int surrogate_kq(int K) { return (K + kGTK - 1) / kGTK * kGTK; }
+
+cudaError_t surrogate_weights_changed(const SurrogateDev& s, cudaStream_t st) {
+  const int64_t n = surrogate_param_count(s.K);
+  const int Kq = surrogate_kq(s.K);
+  cudaError_t e = cudaMemsetAsync(s.W1b, 0, (size_t)kH * Kq * sizeof(__nv_bfloat16), st);
+  if (e != cudaSuccess) return e;
+  copy_weights_kernel<<<grid1d(n), 256, 0, st>>>(n, s.K, Kq, s.w, s.W1b, s.W2b, s.W2t);
+  return cudaGetLastError();
+}
+
 cudaError_t surrogate_init(const SurrogateDev& s, uint64_t seed, cudaStream_t st) {
   const int64_t n = surrogate_param_count(s.K);
   init_params_kernel<<<grid1d(n), 256, 0, st>>>(seed, s.K, s.w);
@@ -708,112 +926,146 @@ cudaError_t surrogate_init(const SurrogateDev& s, uint64_t seed, cudaStream_t st
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(s.m, 0, n * sizeof(float), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(s.v, 0, n * sizeof(float), st);
-  return e;
+  return e == cudaSuccess ? surrogate_weights_changed(s, st) : e;
 }
 
-// Forward pass of B rows X [B][K] (FP32 genes) into out [B]; keeps Z1, H1,
-// Z2, H2 [B][256] in the workspace for a backward pass.
+cudaError_t surrogate_to_bf16(int K, const float* X, int B, __nv_bfloat16* Xb, cudaStream_t st) {
+  const int Kq = surrogate_kq(K);
+  to_bf16_kernel<<<grid1d((int64_t)B * Kq / 8), 256, 0, st>>>(B, K, Kq, X, Xb);
+  return cudaGetLastError();
+}
+
+cudaError_t surrogate_targets(const SurrogateDev& s, const double* fit, int B, float* t,
+                              cudaStream_t st) {
+  if (B > s.Bmax) return cudaErrorInvalidValue;
+  log_fit_kernel<<<(B + 255) / 256, 256, 0, st>>>(B, fit, s.lfit);
+  target_stats_kernel<<<1, 1024, 0, st>>>(B, s.lfit, s.tstat);
+  targets_kernel<<<(B + 255) / 256, 256, 0, st>>>(B, s.lfit, s.tstat, t);
+  return cudaGetLastError();
+}
+
+namespace {
+
+// Both hidden layers of B rows Xb; keep: Z1, H1, Z2 for a backward pass too.
+cudaError_t hidden_layers(const SurrogateDev& s, const __nv_bfloat16* Xb, int B, int keep,
+                          cudaStream_t st) {
+  const float* b1 = s.w + (int64_t)kH * s.K;
+  const float* b2 = b1 + kH + (int64_t)kH * kH;
+  NtArgs a{};
+  a.M = B;
+  a.nkb = surrogate_kq(s.K) / kGTK;
+  a.mode = kLayer;
+  a.keep = keep;
+  a.A = Xb;
+  a.B = s.W1b;
+  a.bias = b1;
+  a.Z = s.Z1;
+  a.H = s.H1;
+  a.Hb = s.H1b;
+  a.status = s.status;
+  cudaError_t e = gemm_nt<1>(a, st);   // Z1 = bf(X) bf(W1)^T + b1, H1 = bf(g(Z1))
+  if (e != cudaSuccess) return e;
+  a.nkb = kH / kGTK;
+  a.A = s.H1b;
+  a.B = s.W2b;
+  a.bias = b2;
+  a.Z = s.Z2;
+  a.H = s.H2;
+  a.Hb = nullptr;
+  return gemm_nt<1>(a, st);            // Z2 = H1 bf(W2)^T + b2, H2 = g(Z2)
+}
+
+}  // namespace
+
+// Predictions of B rows X [B][K] (FP32 genes) into out [B].
 cudaError_t surrogate_forward(const SurrogateDev& s, const float* X, int B, float* out,
                               cudaStream_t st) {
   if (B > s.Bmax) return cudaErrorInvalidValue;
-  const int K = s.K;
-  const float* W1 = s.w;
-  const float* b1 = W1 + (int64_t)kH * K;
-  const float* W2 = b1 + kH;
-  const float* b2 = W2 + (int64_t)kH * kH;
-  const float* w3 = b2 + kH;
-  const float* b3 = w3 + kH;
-  // Z1 = bf(X) bf(W1)^T + b1, H1 = bf(g(Z1))
-  cudaError_t e = gemm(B, kH, K, X, K, 1, W1, 1, K, 1, 1, s.Z1, kH, 1, b1, s.H1, 1, s.status, st);
+  const float* w3 = s.w + (int64_t)kH * s.K + kH + (int64_t)kH * kH + kH;
+  cudaError_t e = surrogate_to_bf16(s.K, X, B, s.Xb, st);
+  if (e == cudaSuccess) e = hidden_layers(s, s.Xb, B, 0, st);
   if (e != cudaSuccess) return e;
-  // Z2 = H1 bf(W2)^T + b2, H2 = g(Z2)
-  e = gemm(B, kH, kH, s.H1, kH, 1, W2, 1, kH, 1, 1, s.Z2, kH, 1, b2, s.H2, 0, s.status, st);
-  if (e != cudaSuccess) return e;
-  output_kernel<<<(int)(((int64_t)B * 32 + 255) / 256), 256, 0, st>>>(B, s.H2, w3, b3, out);
+  output_kernel<<<(int)(((int64_t)B * 32 + 255) / 256), 256, 0, st>>>(B, s.H2, w3, w3 + kH, out);
   return cudaGetLastError();
 }
 
-// Gradient of the mean squared error of log-fitness over B pairs into s.g
-// (after a forward pass of the same X); loss into s.loss[0].
-cudaError_t surrogate_backward(const SurrogateDev& s, const float* X, const double* fit, int B,
-                               cudaStream_t st) {
-  const int K = s.K;
-  const float* W1 = s.w;
-  const float* W2 = W1 + (int64_t)kH * K + kH;
-  const float* w3 = W2 + (int64_t)kH * kH + kH;
-  float* gW1 = s.g;
-  float* gb1 = gW1 + (int64_t)kH * K;
-  float* gW2 = gb1 + kH;
-  float* gb2 = gW2 + (int64_t)kH * kH;
+// The gradient of the mean squared error over the batch into s.g, the loss into
+// s.loss[0]; with apply, an Adam step on it.
+cudaError_t surrogate_step(SurrogateDev& s, const SurrogateBatch& bt, bool apply,
+                           cudaStream_t st) {
+  const int B = bt.n, K = s.K;
+  if (B > s.Bmax) return cudaErrorInvalidValue;
+  const float* w3 = s.w + (int64_t)kH * K + kH + (int64_t)kH * kH + kH;
+  float* gb1 = s.g + (int64_t)kH * K;
+  float* gb2 = gb1 + kH + (int64_t)kH * kH;
   float* gw3 = gb2 + kH;
   float* gb3 = gw3 + kH;
-  log_fit_kernel<<<(B + 255) / 256, 256, 0, st>>>(B, fit, s.lfit);
-  target_stats_kernel<<<1, 1024, 0, st>>>(B, s.lfit, s.tstat);
-  dout_kernel<<<(B + 255) / 256, 256, 0, st>>>(B, s.out, s.lfit, s.tstat, s.dout, s.lterm);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = hidden_layers(s, bt.Xb, B, 1, st);
   if (e != cudaSuccess) return e;
-  sum_kernel<<<1, 256, 0, st>>>(B, s.lterm, s.loss);
-  // output layer
-  colsum_kernel<<<kH / 32, 1024, 0, st>>>(B, kH, s.H2, s.dout, gw3);
-  sum_kernel<<<1, 256, 0, st>>>(B, s.dout, gb3);
-  // dZ2 = dout w3 g'(Z2)
-  dz2_kernel<<<grid1d((int64_t)B * kH), 256, 0, st>>>(B, s.dout, w3, s.Z2, s.dZ2);
-  // gW2 = dZ2^T H1, gb2 = colsum(dZ2)
-  const int splits = kGradSplits(B);
-  e = gemm(kH, kH, B, s.dZ2, 1, kH, s.H1, kH, 1, 0, 1, gW2, kH, 0, nullptr, nullptr, 0, s.status,
-           st, s.split_ws, splits);
-  if (e != cudaSuccess) return e;
-  colsum_kernel<<<kH / 32, 1024, 0, st>>>(B, kH, s.dZ2, nullptr, gb2);
+  output_grad_kernel<<<(int)(((int64_t)B * 32 + 255) / 256), 256, 0, st>>>(
+      B, s.H2, s.Z2, w3, w3 + kH, bt.t, s.dout, s.lterm, s.dZ2, s.dZ2h, s.dZ2l);
   // dZ1 = (dZ2 bf(W2)) g'(Z1)
-  e = gemm(B, kH, kH, s.dZ2, kH, 1, W2, kH, 1, 0, 1, s.dZ1, kH, 0, nullptr, nullptr, 0, s.status,
-           st);
+  NtArgs a{};
+  a.M = B;
+  a.nkb = kH / kGTK;
+  a.mode = kDelta;
+  a.A = s.dZ2h;
+  a.A2 = s.dZ2l;
+  a.B = s.W2t;
+  a.Zin = s.Z1;
+  a.H = s.dZ1;
+  a.status = s.status;
+  e = gemm_nt<2>(a, st);
   if (e != cudaSuccess) return e;
-  gelu_bwd_kernel<<<grid1d((int64_t)B * kH), 256, 0, st>>>((int64_t)B * kH, s.Z1, s.dZ1);
-  // gW1 = dZ1^T bf(X), gb1 = colsum(dZ1)
-  e = gemm(kH, K, B, s.dZ1, 1, kH, X, K, 1, 0, 1, gW1, K, 0, nullptr, nullptr, 0, s.status, st,
-           s.split_ws, splits);
+  // gW1 = dZ1^T bf(X), gW2 = dZ2^T H1, as split sums
+  const int splits = kGradSplits(B);
+  int kz = (B + splits - 1) / splits;
+  kz = (kz + kGTK - 1) / kGTK * kGTK;
+  const GradProblem p1{s.dZ1, bt.X, s.split1, K, (K + kGTN - 1) / kGTN};
+  const GradProblem p2{s.dZ2, s.H1, s.split2, kH, kH / kGTN};
+  constexpr int smem = 2 * (2 * 128 * 128 + kGTN * 128) + 1024 + 64;
+  e = cudaFuncSetAttribute(grad_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  colsum_kernel<<<kH / 32, 1024, 0, st>>>(B, kH, s.dZ1, nullptr, gb1);
+  grad_gemm_kernel<<<dim3(p1.tiles + p2.tiles, kH / 128, splits), kGThreads, smem, st>>>(
+      B, p1, p2, kz, s.status);
+  sums_kernel<<<3 * (kH / 32) + 2, 1024, 0, st>>>(B, s.H2, s.dout, s.dZ2, s.dZ1, s.lterm, gw3,
+                                                 gb2, gb1, gb3, s.loss);
+  float c1 = 1.f, c2 = 1.f;
+  if (apply) {
+    s.step += 1;
+    c1 = 1.f - powf(kAdamB1, (float)s.step);
+    c2 = 1.f - powf(kAdamB2, (float)s.step);
+  }
+  const int64_t n = surrogate_param_count(K);
+  adam_kernel<<<grid1d(n), 256, 0, st>>>(n, K, surrogate_kq(K), splits, s.split1, s.split2, s.w,
+                                         s.g, s.m, s.v, apply, kAdamLr, kAdamB1, kAdamB2,
+                                         kAdamEps, c1, c2, s.W1b, s.W2b, s.W2t);
   return cudaGetLastError();
 }
 
-cudaError_t surrogate_adam(SurrogateDev& s, cudaStream_t st) {
-  s.step += 1;
-  const float c1 = 1.f - powf(kAdamB1, (float)s.step);
-  const float c2 = 1.f - powf(kAdamB2, (float)s.step);
-  const int64_t n = surrogate_param_count(s.K);
-  adam_kernel<<<grid1d(n), 256, 0, st>>>(n, s.w, s.g, s.m, s.v, kAdamLr, kAdamB1, kAdamB2,
-                                         kAdamEps, c1, c2);
-  return cudaGetLastError();
-}
-
-cudaError_t surrogate_trust_check(const SurrogateDev& s, int n, int n_kept, const float* pred,
-                                  const int* flag, const int* pos, const double* fit_kept,
-                                  float* r_out, int* trusted, cudaStream_t st) {
+cudaError_t surrogate_trust_check(const SurrogateDev& s, int n_kept, const float* pred,
+                                  const int* list, const double* fit_kept, float* r_out,
+                                  int* trusted, cudaStream_t st) {
   if (n_kept > s.Bmax) return cudaErrorInvalidValue;
   // the kept children's log-fitness over the whole GPU first (FP64)
   log_fit_kernel<<<(n_kept + 255) / 256, 256, 0, st>>>(n_kept, fit_kept, s.lfit);
-  trust_kernel<<<1, 256, 0, st>>>(n, pred, flag, pos, s.lfit, r_out, trusted);
+  trust_kernel<<<kTrustCtas, kTrustThreads, 0, st>>>(n_kept, pred, list, s.lfit, r_out, trusted);
   return cudaGetLastError();
 }
 
 cudaError_t surrogate_screen(int n, int n_keep, int E, int K, const float* pred, int* flag,
-                             int* pos, const float* off, float* next, const int* trusted,
+                             int* list, const float* off, float* next, const int* trusted,
                              int* used_trust, cudaStream_t st) {
-  if (n > kSortMax || n_keep > n) return cudaErrorInvalidValue;
-  int npow = 1;
-  while (npow < n) npow <<= 1;
-  const size_t smem = (size_t)npow * sizeof(uint64_t);
-  cudaError_t e = cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(kSortMax * sizeof(uint64_t)));
+  if (n > kScreenMax || n_keep > n || n_keep < 1) return cudaErrorInvalidValue;
+  cudaError_t e = cudaFuncSetAttribute(screen_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)(kScreenMax * sizeof(uint32_t)));
   if (e != cudaSuccess) return e;
-  select_kernel<<<1, 1024, smem, st>>>(n, n_keep, pred, flag, trusted, used_trust);
+  screen_kernel<<<1, kScreenThreads, (size_t)n * sizeof(uint32_t), st>>>(
+      n, n_keep, pred, flag, list, trusted, used_trust);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  assemble_kernel<<<1, 1024, 0, st>>>(n, flag, pos);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  gather_kernel<<<grid1d((int64_t)(E + n) * K), 256, 0, st>>>(n, E, K, pos, off, next);
+  const int rows = E + n_keep;
+  gather_kernel<<<(rows * 32 + 255) / 256, 256, 0, st>>>(rows, E, K, list, off, next);
   return cudaGetLastError();
 }
 

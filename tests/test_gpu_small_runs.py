@@ -73,3 +73,22 @@ def test_candidate_selection(P):
         for n in (1, 16):
             _, idx = g.rescore_top(pop, fit, n)
             assert np.array_equal(idx, order[:n])
+
+
+@pytest.mark.parametrize("P,oversample", [(18, 8), (130, 3), (1026, 8), (2048, 8)])
+def test_screening_keeps_the_best_predictions(P, oversample):
+    """Once trusted, the screening keeps the smallest predictions, ties by slot,
+    at child counts off and on the selection's warp ranges."""
+    pr = dg.regression(9, 3000, 6, 2, 0.05, degree=2, basis=CHEB)
+    with game.Game(pr.X, pr.y, 2, CHEB, P=P, precision=game.GAME_PREC_BF16, surrogate=1,
+                   oversample=oversample, seed=4) as g:
+        seen = 0
+        for _ in range(12):
+            g.generation(4)
+            pred, keep, trusted, _ = g.surrogate_last()
+            want = np.zeros(len(pred), dtype=np.int32)
+            n_keep = P - 2
+            want[np.argsort(pred, kind="stable")[:n_keep] if trusted else slice(0, n_keep)] = 1
+            assert np.array_equal(keep, want)
+            seen += trusted
+        assert seen, "the surrogate was never trusted"
