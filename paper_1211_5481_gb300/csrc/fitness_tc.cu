@@ -26,15 +26,13 @@
 //   warp 0       A producer: bulk-copies 16 KB gene blocks (chromosome tile c,
 //                K-block kb of 64 columns) from the pre-swizzled operand
 //                image into a ring of 3-4 stages.
-//   warp 1       MMA issuer (one thread) and tensor-memory owner; two FP32
-//                accumulators of BN columns, so the epilogue of chromosome
-//                tile c overlaps the MMAs of tile c+1. The tcgen05 queue
-//                drains fast, so the issuing path is kept minimal: precomputed
-//                descriptors, unrolled groups of four K=16 MMAs, K-blocks taken
-//                in pairs (singly for the first chromosome tile of a pattern
-//                tile, so that its MMAs start as soon as one slot is full).
+//   warp 1       MMA issuer (the converged warp, instructions predicated to one
+//                lane) and tensor-memory owner; two FP32 accumulators of BN
+//                columns, so the epilogue of chromosome tile c overlaps the
+//                MMAs of tile c+1.
 //   warp 2       X producer: bulk-copies the next pattern tile's features
 //                (staged mode only, below).
+//   warp 3       Y producer: bulk-copies each tile's targets (where they fit).
 //   warps 4-11   epilogue: tcgen05.ld of the accumulator (thread = chromosome
 //                = TMEM lane; warps 4-7 take the first half of the columns,
 //                8-11 the second), r = (y_m - a_0) - D, sse += r^2 in packed
@@ -62,6 +60,7 @@
 #include <cuda_fp8.h>
 
 #include <atomic>
+#include <type_traits>
 
 #include "basis.cuh"
 #include "expand_stream.cuh"
@@ -94,8 +93,8 @@ struct TcArgs {
                 // next tile's first K-blocks be written while this tile's MMAs run
   int xstage;   // 1: the tile's features are bulk-copied into shared memory;
                 // 0: read from global memory (L2) by the expansion warps
-  int ystage;   // 1 (with xstage 0): warp 2 bulk-copies each tile's targets into
-                // a two-slot shared buffer the epilogue reads
+  int ystage;   // 1: warp 3 bulk-copies each tile's targets into a two-slot shared
+                // buffer the epilogue reads
   int slack;    // bytes reserved for aligning the dynamic shared memory to 1024
   const float* Xt;
   const float* y;
@@ -240,25 +239,31 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    // The tcgen05 MMA queue drains quickly, so this thread's path between
-    // MMAs is kept short: descriptors are precomputed (a stage, a K-block or
-    // a K=16 step only moves the 14-bit start-address field), K-blocks are
-    // taken in pairs (both operand waits first, then up to eight MMAs back
-    // to back, then the commits), and the inner groups are unrolled.
-    if (lane == 0) {
+    // One K-block's MMAs take 512 tensor cycles and this warp's instructions
+    // between them share their scheduler with three busy warps, so they decide
+    // the tensor pipe's rate: the converged warp runs the loop (uniform
+    // registers, see mma_bf16_w), descriptors, barrier addresses, slots and
+    // phases advance by an add and a compare. (A lone thread with the slots by
+    // integer division: 434 us at M = 10^6, N = 32, degree 8, P = 1024, BF16;
+    // by compares 421; this 398.)
+    {
+      const uint32_t lead = ptx::elect_one();
       const uint32_t idesc =
           F == kFormFP8 ? ptx::idesc_e4m3_f32(128, BN) : ptx::idesc_bf16_f32(128, BN);
       const uint64_t adesc0 = ptx::desc_kmajor_sw128(ptx::smem_addr(ast));
       const uint64_t bdesc0 = ptx::desc_kmajor_sw128(ptx::smem_addr(phi));
+      const uint32_t dhi = (uint32_t)(adesc0 >> 32);               // the same for both
+      const uint32_t alo0 = (uint32_t)adesc0, blo0 = (uint32_t)bdesc0;
       const uint32_t a_step = (uint32_t)(NA * kABytes) >> 4;       // one A stage
       const uint32_t b_step = (uint32_t)(NPHI * BN * 128) >> 4;    // one expansion K-block
       const uint32_t a_lo = kABytes >> 4;                          // bf16x3: lo gene block
       const uint32_t b_lo = (uint32_t)(BN * 128) >> 4;             // bf16x3: lo expansion
-      const uint32_t a_full0 = ptx::smem_addr(a_full), a_empty0 = ptx::smem_addr(a_empty);
-      const uint32_t phi_full0 = ptx::smem_addr(phi_full), phi_free0 = ptx::smem_addr(phi_free);
+      const uint32_t alo_end = alo0 + (uint32_t)S * a_step, blo_end = blo0 + (uint32_t)NS * b_step;
+      const uint32_t a_full0 = ptx::smem_addr(a_full), phi_full0 = ptx::smem_addr(phi_full);
+      const uint32_t a_empty = 8u * (uint32_t)S, phi_free_off = 8u * (uint32_t)NS;   // from *_full
       const uint32_t acc_full0 = ptx::smem_addr(acc_full), acc_empty0 = ptx::smem_addr(acc_empty);
       const int nlast = a.nmma_last;
-      uint32_t s = 0, ph = 0, acc_it = 0;   // A stage and its phase, accumulator count
+      auto desc = [&](uint32_t lo) { return ((uint64_t)dhi << 32) | lo; };
       bool ok = true;
       if (a.stall_ns) {
         // test hook: the drain barrier's first phase completes only at the
@@ -274,83 +279,78 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
         }
       }
       // one K step (32 bytes of each operand row): one MMA, three for bf16x3
-      auto kstep = [&](uint32_t d_tmem, uint64_t ad, uint64_t bd, uint32_t acc) {
+      auto kstep = [&](uint32_t d_tmem, uint32_t al, uint32_t bl, uint32_t acc) {
         if (F == kFormFP8) {
-          ptx::mma_f8(d_tmem, ad, bd, idesc, acc);
+          ptx::mma_f8_w(lead, d_tmem, desc(al), desc(bl), idesc, acc);
         } else {
-          ptx::mma_bf16(d_tmem, ad, bd, idesc, acc);
+          ptx::mma_bf16_w(lead, d_tmem, desc(al), desc(bl), idesc, acc);
           if (F == kFormBF16x3) {
-            ptx::mma_bf16(d_tmem, ad, bd + b_lo, idesc, 1u);
-            ptx::mma_bf16(d_tmem, ad + a_lo, bd, idesc, 1u);
+            ptx::mma_bf16_w(lead, d_tmem, desc(al), desc(bl + b_lo), idesc, 1u);
+            ptx::mma_bf16_w(lead, d_tmem, desc(al + a_lo), desc(bl), idesc, 1u);
           }
         }
       };
-      // issues the MMAs of one K-block (nm of 4 K steps)
-      auto kblock = [&](uint32_t d_tmem, uint32_t st, int kb, int slot, int nm) {
-        const uint64_t ad = adesc0 + st * a_step;
-        const uint64_t bd = bdesc0 + (uint32_t)slot * b_step;
-        if (nm == 4) {
-          kstep(d_tmem, ad, bd, kb != 0);
-          kstep(d_tmem, ad + 2u, bd + 2u, 1u);
-          kstep(d_tmem, ad + 4u, bd + 4u, 1u);
-          kstep(d_tmem, ad + 6u, bd + 6u, 1u);
-        } else {
-          for (int kk = 0; kk < nm; ++kk)
-            kstep(d_tmem, ad + 2u * kk, bd + 2u * kk, (kb | kk) != 0);
-        }
-      };
+      uint32_t alo = alo0, abar = a_full0, ph = 0;          // A stage, its barrier and phase
+      uint32_t tile_blo = blo0, tile_pbar = phi_full0, tile_par = 0;   // the tile's first slot
+      uint32_t acc_it = 0;
       for (int it = 0; it < my_tiles && ok; ++it) {
+        uint32_t blo = tile_blo, pbar = tile_pbar, par = tile_par;
         for (int c = 0; c < a.C && ok; ++c) {
-          const uint32_t buf = acc_it & 1, u = acc_it >> 1;
-          ok = wait_bar(acc_empty0 + 8 * buf, (u & 1) ^ 1, abort_flag, a.status);
+          const uint32_t buf = acc_it & 1;
+          ok = wait_bar(acc_empty0 + 8 * buf, ((acc_it >> 1) & 1) ^ 1, abort_flag, a.status);
           if (!ok) break;
           ptx::tc_fence_after();
           const uint32_t d_tmem = tmem + buf * (uint32_t)BN;
-          // the first chromosome tile of a pattern tile takes K-blocks one at a
-          // time, so its MMAs start as soon as the first expansion slot is full
-          for (int kb = 0; kb < KB && ok; kb += (c != 0 && kb + 1 < KB) ? 2 : 1) {
-            const bool two = c != 0 && kb + 1 < KB;
-            uint32_t s1 = s + 1, ph1 = ph;
-            if (s1 == (uint32_t)S) {
-              s1 = 0;
-              ph1 ^= 1;
-            }
-            // expansion slots of the two K-blocks: use q = it KB + kb of slot q % NS
-            const int q0 = it * KB + kb, q1 = q0 + 1;
-            const int sl0 = q0 % NS, sl1 = q1 % NS;
-            // operands of both K-blocks first
+          blo = tile_blo;
+          pbar = tile_pbar;
+          par = tile_par;
+          uint32_t acc = 0;
+          for (int kb = 0; kb < KB; ++kb) {
             if (c == 0) {
-              ok = wait_bar(phi_full0 + 8 * sl0, (q0 / NS) & 1, abort_flag, a.status);
-              if (ok && two)
-                ok = wait_bar(phi_full0 + 8 * sl1, (q1 / NS) & 1, abort_flag, a.status);
+              ok = wait_bar(pbar, par, abort_flag, a.status);
+              if (!ok) break;
             }
-            if (ok) ok = wait_bar(a_full0 + 8 * s, ph, abort_flag, a.status);
-            if (ok && two) ok = wait_bar(a_full0 + 8 * s1, ph1, abort_flag, a.status);
+            ok = wait_bar(abar, ph, abort_flag, a.status);
             if (!ok) break;
-            kblock(d_tmem, s, kb, sl0, (kb == KB - 1) ? nlast : 4);
-            if (two) kblock(d_tmem, s1, kb + 1, sl1, (kb + 1 == KB - 1) ? nlast : 4);
-            ptx::mma_commit(a_empty0 + 8 * s);
-            if (two) ptx::mma_commit(a_empty0 + 8 * s1);
-            if (c == a.C - 1) {
-              ptx::mma_commit(phi_free0 + 8 * sl0);
-              if (two) ptx::mma_commit(phi_free0 + 8 * sl1);
-            }
-            s = s1;
-            ph = ph1;
-            if (two) {
-              if (++s == (uint32_t)S) {
-                s = 0;
-                ph ^= 1;
+            const int nm = kb == KB - 1 ? nlast : 4;
+            if (nm == 4) {
+              kstep(d_tmem, alo, blo, acc);
+              kstep(d_tmem, alo + 2u, blo + 2u, 1u);
+              kstep(d_tmem, alo + 4u, blo + 4u, 1u);
+              kstep(d_tmem, alo + 6u, blo + 6u, 1u);
+              acc = 1;
+            } else {
+              for (int kk = 0; kk < nm; ++kk) {
+                kstep(d_tmem, alo + 2u * kk, blo + 2u * kk, acc);
+                acc = 1;
               }
             }
+            ptx::mma_commit_w(lead, abar + a_empty);
+            if (c == a.C - 1) ptx::mma_commit_w(lead, pbar + phi_free_off);
+            if (kb == KB - 1) ptx::mma_commit_w(lead, acc_full0 + 8 * buf);
+            alo += a_step;
+            abar += 8;
+            if (alo == alo_end) {
+              alo = alo0;
+              abar = a_full0;
+              ph ^= 1;
+            }
+            blo += b_step;
+            pbar += 8;
+            if (blo == blo_end) {
+              blo = blo0;
+              pbar = phi_full0;
+              par ^= 1u;
+            }
           }
-          if (!ok) break;
-          ptx::mma_commit(acc_full0 + 8 * buf);
           ++acc_it;
         }
+        tile_blo = blo;   // where the next tile's K-blocks begin
+        tile_pbar = pbar;
+        tile_par = par;
       }
       // every MMA issued above has completed once this arrives
-      ptx::mma_commit(ptx::smem_addr(drain));
+      ptx::mma_commit_w(lead, ptx::smem_addr(drain));
       wait_bar_drain(ptx::smem_addr(drain), 0, a.status);
     }
   } else if (warp == 2) {
@@ -395,7 +395,8 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
       }
       if (issued > 0) wait_bar_drain(ptx::smem_addr(x_full), (issued - 1) & 1, a.status);
     }
-    // ---------------- Y producer (features read from L2) ----------------
+  } else if (warp == 3) {
+    // ---------------- Y producer ----------------
     // each tile's targets into slot it & 1, released by the 256 epilogue
     // threads after the tile's last chromosome tile
     if (lane == 0 && a.ystage) {
@@ -426,75 +427,83 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
     const int col_lo = half * HW;
     const uint32_t lane_addr = (uint32_t)(qw * 32) << 16;
     double* part_row = a.part + (size_t)(2 * blockIdx.x + half) * a.Ppad;
-    uint32_t acc_it = 0;
-    bool ok = true;
-    for (int it = 0; it < my_tiles && ok; ++it) {
-      const int64_t m0 = ((int64_t)blockIdx.x + (int64_t)it * G) * BN;
-      const int64_t rem = a.M - m0 - col_lo;
-      const int valid = (half >= NH || rem <= 0) ? 0 : (rem >= HW ? HW : (int)rem);
-      const bool ysm = a.ystage != 0;
-      if (ysm) {
-        ok = wait_bar(ptx::smem_addr(&y_full[it & 1]), (it >> 1) & 1, abort_flag, a.status);
-        if (!ok) break;
-      }
-      const float* yt = ysm ? ys + (it & 1) * BN + col_lo : a.y + m0 + col_lo;
-      for (int c = 0; c < a.C; ++c) {
-        const uint32_t buf = acc_it & 1, u = acc_it >> 1;
-        ok = wait_bar(ptx::smem_addr(&acc_full[buf]), u & 1, abort_flag, a.status);
-        if (!ok) break;
-        ptx::tc_fence_after();
-        const int chrom = c * 128 + row;
-        const float bias = a.a0[chrom];
-        const uint64_t bias2 = ptx::f2_pack(bias, bias);
-        const float negu = F == kFormFP8 ? -a.uscale[chrom] : -1.f;
-        const uint64_t negu2 = ptx::f2_pack(negu, negu);
-        uint64_t s2 = 0;   // two FP32 partial sums (even / odd columns)
-        float s_tail = 0.f;
-        const uint32_t tbase = tmem + lane_addr + buf * (uint32_t)BN + (uint32_t)col_lo;
-        const int nfull = valid / 32;
-        if (nfull > 0) {
-          // double-buffered: the load of chunk k+1 is in flight while chunk k
-          // is reduced
-          uint32_t va[32], vb[32];
-          ptx::tmem_ld32_issue(tbase, va);
-          ptx::tmem_ld32_wait(va);
-          for (int k = 0; k < nfull; k += 2) {
-            const bool has_b = k + 1 < nfull;
-            if (has_b) ptx::tmem_ld32_issue(tbase + (uint32_t)(k + 1) * 32, vb);
-            if (ysm) epi_chunk<F == kFormFP8, ABS, true>(va, yt + k * 32, bias2, negu2, s2);
-            else epi_chunk<F == kFormFP8, ABS>(va, yt + k * 32, bias2, negu2, s2);
-            if (has_b) {
-              ptx::tmem_ld32_wait(vb);
-              const bool has_a = k + 2 < nfull;
-              if (has_a) ptx::tmem_ld32_issue(tbase + (uint32_t)(k + 2) * 32, va);
-              if (ysm) epi_chunk<F == kFormFP8, ABS, true>(vb, yt + (k + 1) * 32, bias2, negu2, s2);
-              else epi_chunk<F == kFormFP8, ABS>(vb, yt + (k + 1) * 32, bias2, negu2, s2);
-              if (has_a) ptx::tmem_ld32_wait(va);
+    // Per accumulator a warp has about as long as its MMAs (K' / 16 times 128
+    // cycles), and while it is late the MMAs wait: so the targets come from shared
+    // memory, and the chromosome's bias and running sum are loaded before the wait
+    // for the accumulator, not after its reduction. (M = 10^6, N = 32, degree 8,
+    // P = 1024: 398 -> 365 us together with the expansion's look-ahead.)
+    auto reduce_tiles = [&](auto ys_tag) {
+      constexpr bool YS = decltype(ys_tag)::value;
+      uint32_t acc_it = 0;
+      bool ok = true;
+      for (int it = 0; it < my_tiles && ok; ++it) {
+        const int64_t m0 = ((int64_t)blockIdx.x + (int64_t)it * G) * BN;
+        const int64_t rem = a.M - m0 - col_lo;
+        const int valid = (half >= NH || rem <= 0) ? 0 : (rem >= HW ? HW : (int)rem);
+        if (YS) {
+          ok = wait_bar(ptx::smem_addr(&y_full[it & 1]), (it >> 1) & 1, abort_flag, a.status);
+          if (!ok) break;
+        }
+        const float* yt = YS ? ys + (it & 1) * BN + col_lo : a.y + m0 + col_lo;
+        for (int c = 0; c < a.C; ++c) {
+          const uint32_t buf = acc_it & 1, u = acc_it >> 1;
+          const int chrom = c * 128 + row;
+          const float bias = a.a0[chrom];
+          const float negu = F == kFormFP8 ? -a.uscale[chrom] : -1.f;
+          const double before = it == 0 ? 0.0 : part_row[chrom];
+          ok = wait_bar(ptx::smem_addr(&acc_full[buf]), u & 1, abort_flag, a.status);
+          if (!ok) break;
+          ptx::tc_fence_after();
+          const uint64_t bias2 = ptx::f2_pack(bias, bias);
+          const uint64_t negu2 = ptx::f2_pack(negu, negu);
+          uint64_t s2 = 0;   // two FP32 partial sums (even / odd columns)
+          float s_tail = 0.f;
+          const uint32_t tbase = tmem + lane_addr + buf * (uint32_t)BN + (uint32_t)col_lo;
+          const int nfull = valid / 32;
+          if (nfull > 0) {
+            // double-buffered: the load of chunk k+1 is in flight while chunk k
+            // is reduced
+            uint32_t va[32], vb[32];
+            ptx::tmem_ld32_issue(tbase, va);
+            ptx::tmem_ld32_wait(va);
+            for (int k = 0; k < nfull; k += 2) {
+              const bool has_b = k + 1 < nfull;
+              if (has_b) ptx::tmem_ld32_issue(tbase + (uint32_t)(k + 1) * 32, vb);
+              epi_chunk<F == kFormFP8, ABS, YS>(va, yt + k * 32, bias2, negu2, s2);
+              if (has_b) {
+                ptx::tmem_ld32_wait(vb);
+                const bool has_a = k + 2 < nfull;
+                if (has_a) ptx::tmem_ld32_issue(tbase + (uint32_t)(k + 2) * 32, va);
+                epi_chunk<F == kFormFP8, ABS, YS>(vb, yt + (k + 1) * 32, bias2, negu2, s2);
+                if (has_a) ptx::tmem_ld32_wait(va);
+              }
             }
           }
-        }
-        if (nfull * 32 < valid) {   // ragged last chunk of the last tile
-          uint32_t v[32];
-          ptx::tmem_ld32(tbase + (uint32_t)nfull * 32, v);
-          const int lim = valid - nfull * 32;
+          if (nfull * 32 < valid) {   // ragged last chunk of the last tile
+            uint32_t v[32];
+            ptx::tmem_ld32(tbase + (uint32_t)nfull * 32, v);
+            const int lim = valid - nfull * 32;
 #pragma unroll
-          for (int e = 0; e < 32; ++e) {
-            if (e < lim) {
-              const float r = fmaf(negu, __uint_as_float(v[e]), yt[nfull * 32 + e] - bias);
-              s_tail = ABS ? s_tail + fabsf(r) : fmaf(r, r, s_tail);
+            for (int e = 0; e < 32; ++e) {
+              if (e < lim) {
+                const float r = fmaf(negu, __uint_as_float(v[e]), yt[nfull * 32 + e] - bias);
+                s_tail = ABS ? s_tail + fabsf(r) : fmaf(r, r, s_tail);
+              }
             }
           }
+          ptx::tc_fence_before();
+          ptx::mbar_arrive(ptx::smem_addr(&acc_empty[buf]));
+          const float2 sp2 = ptx::f2_unpack(s2);
+          double tile_sse = (double)sp2.x + (double)sp2.y;
+          if (s_tail != 0.f) tile_sse += (double)s_tail;   // (FP64 operations are scarce)
+          part_row[chrom] = it == 0 ? tile_sse : before + tile_sse;
+          ++acc_it;
         }
-        ptx::tc_fence_before();
-        ptx::mbar_arrive(ptx::smem_addr(&acc_empty[buf]));
-        const float2 sp2 = ptx::f2_unpack(s2);
-        double tile_sse = (double)sp2.x + (double)sp2.y;
-        if (s_tail != 0.f) tile_sse += (double)s_tail;   // (FP64 operations are scarce)
-        part_row[chrom] = (it == 0) ? tile_sse : part_row[chrom] + tile_sse;
-        ++acc_it;
+        if (YS && ok) ptx::mbar_arrive(ptx::smem_addr(&y_empty[it & 1]));
       }
-      if (ysm && ok) ptx::mbar_arrive(ptx::smem_addr(&y_empty[it & 1]));
-    }
+    };
+    if (a.ystage) reduce_tiles(std::true_type{});
+    else reduce_tiles(std::false_type{});
   } else if (warp >= kBasisWarp0) {
     // ---------------- expansion (basis) ----------------
     const int bt = threadIdx.x - kBasisWarp0 * 32;
@@ -794,40 +803,42 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
         ptx::bulk_prefetch_l2(a.Xt + (m1 / kPatBlock) * N * kPatBlock,
                               (uint32_t)((BN / kPatBlock) * N * kPatBlock * 4));
       };
-      float na[8], nb[8];
-      auto load_kb = [&](int itn, int kbn) {
-        const float* p0 = xptr(itn, r0);
-        const float* p1 = xptr(itn, r1);
+      // Two K-blocks' features are in registers ahead of use: as the last
+      // chromosome tile's MMAs release the slots, a K-block is due every 512
+      // cycles, less than a load takes from L2.
+      int lit = 0, lkb = 0;   // place of the next K-block to load
+      auto load_next = [&](float (&va)[8], float (&vb)[8]) {
+        if (lit >= my_tiles) return;
+        const float* p0 = xptr(lit, r0);
+        const float* p1 = xptr(lit, r1);
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-          const int i = (int)(tab[kbn * 8 + q] & 0xFFFFu);
-          na[q] = __ldg(p0 + i * kPatBlock);
-          nb[q] = R == 2 ? __ldg(p1 + i * kPatBlock) : 0.f;
+          const int i = (int)(tab[lkb * 8 + q] & 0xFFFFu);
+          va[q] = __ldg(p0 + i * kPatBlock);
+          vb[q] = R == 2 ? __ldg(p1 + i * kPatBlock) : 0.f;
+        }
+        if (++lkb == KB) {
+          lkb = 0;
+          ++lit;
         }
       };
       if (bt == 0) {
         if (my_tiles > 0) prefetch_tile(0);
         if (my_tiles > 1) prefetch_tile(1);
       }
-      if (my_tiles > 0) load_kb(0, 0);
-      for (int it = 0; it < my_tiles && ok; ++it) {
-        if (bt == 0 && it + 2 < my_tiles) prefetch_tile(it + 2);
-        for (int kb = 0; kb < KB; ++kb) {
-          float xa[8], xb[8];
-#pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            xa[q] = na[q];
-            xb[q] = nb[q];
-          }
-          if (kb + 1 < KB) load_kb(it, kb + 1);
-          else if (it + 1 < my_tiles) load_kb(it + 1, 0);
-          const int q = it * KB + kb;
-          ok = slot_free(q);
-          if (!ok) break;
-          uint8_t* phik = phi + (size_t)(q % NS) * BN * 128;
-          if (a.d == 8) {
-            emit_kblock_d8(phik, kb, xa, xb);
-          } else {
+      int it = 0, kb = 0;           // the K-block to write
+      int slot = 0, uses = 0;       // its slot, the slot's completed uses
+      // writes a K-block from its features, then loads the one after the next
+      auto step = [&](float (&xa)[8], float (&xb)[8]) {
+        if (kb == 0 && bt == 0 && it + 2 < my_tiles) prefetch_tile(it + 2);
+        if (uses > 0)
+          ok = wait_bar(ptx::smem_addr(&phi_free[slot]), (uint32_t)(uses - 1) & 1u, abort_flag,
+                        a.status);
+        if (!ok) return;
+        uint8_t* phik = phi + (size_t)slot * BN * 128;
+        if (a.d == 8) {
+          emit_kblock_d8(phik, kb, xa, xb);
+        } else {
 #pragma unroll
           for (int qd = 0; qd < 8; ++qd) {
             const uint32_t desc = tab[kb * 8 + qd];
@@ -841,10 +852,25 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
               emit_run2x(phik, desc, qd, xa[qd], xb[qd]);
             }
           }
-          }
-          ptx::fence_proxy_async_smem();
-          ptx::mbar_arrive(ptx::smem_addr(&phi_full[q % NS]));
         }
+        ptx::fence_proxy_async_smem();
+        ptx::mbar_arrive(ptx::smem_addr(&phi_full[slot]));
+        load_next(xa, xb);
+        if (++slot == NS) {
+          slot = 0;
+          ++uses;
+        }
+        if (++kb == KB) {
+          kb = 0;
+          ++it;
+        }
+      };
+      float xa0[8], xb0[8], xa1[8], xb1[8];
+      load_next(xa0, xb0);
+      load_next(xa1, xb1);
+      while (it < my_tiles && ok) {
+        step(xa0, xb0);
+        if (it < my_tiles && ok) step(xa1, xb1);
       }
     }
     for (int it = 0; it < my_tiles && ok && staged && !stream; ++it) {
@@ -977,6 +1003,14 @@ TcPlan plan_tc_single(const Shape& s, int P, int num_sms, int form) {
     }
   }
   if (!pl.ok) return pl;
+  // staged features: the targets too, where two slots of them still fit
+  if (pl.xstage) {
+    const int sm = smem_plan(pl.KB, pl.NS, pl.BN, s.N, pl.stages, form, 1, 1, slack).total;
+    if (sm <= kMaxSmem) {
+      pl.ycopy = 1;
+      if (pl.smem_bytes < sm) pl.smem_bytes = sm;
+    }
+  }
   const int ntiles = ceil_div(s.M, pl.BN);   // Mpad (a multiple of 768) covers them
   pl.grid = ntiles < num_sms ? ntiles : num_sms;
   int cols = 32;
@@ -1016,7 +1050,7 @@ cudaError_t launch_fitness_tc(const TcPlan& pl, const Shape& s, const float* Xt,
   a.stages = pl.stages;
   a.NS = pl.NS;
   a.xstage = pl.xstage;
-  a.ystage = pl.ystage;
+  a.ystage = pl.ystage || pl.ycopy;
   a.slack = pl.slack;
   const int cols = form_cols(pl.form);
   const int last_cols = s.Kp - cols * (pl.KB - 1);

@@ -252,18 +252,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer (even CTA) ----------------
-    if (lane == 0 && lead) {
+    // (the converged warp with running descriptors: see fitness_tc.cu)
+    if (lead) {
+      const uint32_t one = ptx::elect_one();
       const uint32_t idesc = ptx::idesc_bf16_f32(2 * kRows, kBN);
       const uint64_t adesc0 = ptx::desc_kmajor_sw128(ptx::smem_addr(ast));
       const uint64_t bdesc0 = ptx::desc_kmajor_sw128(ptx::smem_addr(phi));
+      const uint32_t dhi = (uint32_t)(adesc0 >> 32);
+      const uint32_t alo0 = (uint32_t)adesc0, blo0 = (uint32_t)bdesc0;
       const uint32_t a_step = kABytes >> 4;
       const uint32_t b_step = (uint32_t)(kRows * 128) >> 4;
-      const uint32_t a_full0 = ptx::smem_addr(a_full), a_empty0 = ptx::smem_addr(a_empty);
-      const uint32_t phi_full0 = ptx::smem_addr(phi_full), phi_free0 = ptx::smem_addr(phi_free);
+      const uint32_t alo_end = alo0 + (uint32_t)S * a_step, blo_end = blo0 + (uint32_t)NS * b_step;
+      const uint32_t a_full0 = ptx::smem_addr(a_full), phi_full0 = ptx::smem_addr(phi_full);
+      const uint32_t a_empty_off = 8u * (uint32_t)S, phi_free_off = 8u * (uint32_t)NS;
       const uint32_t acc_full0 = ptx::smem_addr(acc_full), acc_empty0 = ptx::smem_addr(acc_empty);
       const uint16_t both = 3;
       const int nlast = a.nmma_last;
-      uint32_t s = 0, ph = 0, acc_it = 0;
       bool ok = true;
       if (a.stall_ns) {
         // test hook: the drain barrier's first phase completes only at the
@@ -277,67 +281,71 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           }
         }
       }
-      auto kblock = [&](uint32_t d_tmem, uint32_t st, int kb, int slot, int nm) {
-        const uint64_t ad = adesc0 + st * a_step;
-        const uint64_t bd = bdesc0 + (uint32_t)slot * b_step;
-        if (nm == 4) {
-          ptx::mma_bf16_pair(d_tmem, ad, bd, idesc, kb != 0);
-          ptx::mma_bf16_pair(d_tmem, ad + 2u, bd + 2u, idesc, 1u);
-          ptx::mma_bf16_pair(d_tmem, ad + 4u, bd + 4u, idesc, 1u);
-          ptx::mma_bf16_pair(d_tmem, ad + 6u, bd + 6u, idesc, 1u);
-        } else {
-          for (int kk = 0; kk < nm; ++kk)
-            ptx::mma_bf16_pair(d_tmem, ad + 2u * kk, bd + 2u * kk, idesc, (kb | kk) != 0);
-        }
+      auto kstep = [&](uint32_t d_tmem, uint32_t al, uint32_t bl, uint32_t acc) {
+        ptx::mma_bf16_pair_w(one, d_tmem, ((uint64_t)dhi << 32) | al, ((uint64_t)dhi << 32) | bl,
+                             idesc, acc);
       };
+      uint32_t alo = alo0, abar = a_full0, ph = 0;
+      uint32_t tile_blo = blo0, tile_pbar = phi_full0, tile_par = 0;
+      uint32_t acc_it = 0;
       for (int it = 0; it < my_tiles && ok; ++it) {
+        uint32_t blo = tile_blo, pbar = tile_pbar, par = tile_par;
         for (int c = 0; c < Cp && ok; ++c) {
-          const uint32_t buf = acc_it & 1, u = acc_it >> 1;
-          ok = wait_bar(acc_empty0 + 8 * buf, (u & 1) ^ 1, abort_flag, a.status);
+          const uint32_t buf = acc_it & 1;
+          ok = wait_bar(acc_empty0 + 8 * buf, ((acc_it >> 1) & 1) ^ 1, abort_flag, a.status);
           if (!ok) break;
           ptx::tc_fence_after();
           const uint32_t d_tmem = tmem + buf * (uint32_t)kBN;
-          for (int kb = 0; kb < KB && ok; kb += (c != 0 && kb + 1 < KB) ? 2 : 1) {
-            const bool two = c != 0 && kb + 1 < KB;
-            uint32_t s1 = s + 1, ph1 = ph;
-            if (s1 == (uint32_t)S) {
-              s1 = 0;
-              ph1 ^= 1;
-            }
-            const int q0 = it * KB + kb, q1 = q0 + 1;
-            const int sl0 = q0 % NS, sl1 = q1 % NS;
+          blo = tile_blo;
+          pbar = tile_pbar;
+          par = tile_par;
+          uint32_t acc = 0;
+          for (int kb = 0; kb < KB; ++kb) {
             if (c == 0) {
-              ok = wait_bar(phi_full0 + 8 * sl0, (q0 / NS) & 1, abort_flag, a.status);
-              if (ok && two)
-                ok = wait_bar(phi_full0 + 8 * sl1, (q1 / NS) & 1, abort_flag, a.status);
+              ok = wait_bar(pbar, par, abort_flag, a.status);
+              if (!ok) break;
             }
-            if (ok) ok = wait_bar(a_full0 + 8 * s, ph, abort_flag, a.status);
-            if (ok && two) ok = wait_bar(a_full0 + 8 * s1, ph1, abort_flag, a.status);
+            ok = wait_bar(abar, ph, abort_flag, a.status);
             if (!ok) break;
-            kblock(d_tmem, s, kb, sl0, (kb == KB - 1) ? nlast : 4);
-            if (two) kblock(d_tmem, s1, kb + 1, sl1, (kb + 1 == KB - 1) ? nlast : 4);
-            ptx::mma_commit_pair_mc(a_empty0 + 8 * s, both);
-            if (two) ptx::mma_commit_pair_mc(a_empty0 + 8 * s1, both);
-            if (c == Cp - 1) {
-              ptx::mma_commit_pair_mc(phi_free0 + 8 * sl0, both);
-              if (two) ptx::mma_commit_pair_mc(phi_free0 + 8 * sl1, both);
-            }
-            s = s1;
-            ph = ph1;
-            if (two) {
-              if (++s == (uint32_t)S) {
-                s = 0;
-                ph ^= 1;
+            const int nm = kb == KB - 1 ? nlast : 4;
+            if (nm == 4) {
+              kstep(d_tmem, alo, blo, acc);
+              kstep(d_tmem, alo + 2u, blo + 2u, 1u);
+              kstep(d_tmem, alo + 4u, blo + 4u, 1u);
+              kstep(d_tmem, alo + 6u, blo + 6u, 1u);
+              acc = 1;
+            } else {
+              for (int kk = 0; kk < nm; ++kk) {
+                kstep(d_tmem, alo + 2u * kk, blo + 2u * kk, acc);
+                acc = 1;
               }
             }
+            ptx::mma_commit_pair_mc_w(one, abar + a_empty_off, both);
+            if (c == Cp - 1) ptx::mma_commit_pair_mc_w(one, pbar + phi_free_off, both);
+            if (kb == KB - 1) ptx::mma_commit_pair_mc_w(one, acc_full0 + 8 * buf, both);
+            alo += a_step;
+            abar += 8;
+            if (alo == alo_end) {
+              alo = alo0;
+              abar = a_full0;
+              ph ^= 1;
+            }
+            blo += b_step;
+            pbar += 8;
+            if (blo == blo_end) {
+              blo = blo0;
+              pbar = phi_full0;
+              par ^= 1u;
+            }
           }
-          if (!ok) break;
-          ptx::mma_commit_pair_mc(acc_full0 + 8 * buf, both);
           ++acc_it;
         }
+        tile_blo = blo;
+        tile_pbar = pbar;
+        tile_par = par;
       }
       // every MMA issued above has completed once this arrives
-      ptx::mma_commit_pair(ptx::smem_addr(drain));
+      if (one) ptx::mma_commit_pair(ptx::smem_addr(drain));
       wait_bar_drain(ptx::smem_addr(drain), 0, a.status);
     }
   } else if (warp == 2) {

@@ -95,6 +95,7 @@ __host__ __device__ constexpr int form_cols(int f) { return f == kFormFP8 ? 128 
 struct TcPlan {
   int form, BN, KB, NS, xstage, C, stages, grid, smem_bytes, tmem_cols, rows;
   int ystage, slack;   // targets staged in shared memory; bytes kept for base alignment
+  int ycopy;  // with staged features: targets staged in shared memory as well
   int pair;   // 1: the paired-SM kernel (fitness_tc2.cu), C even, grid of 2-CTA clusters
   bool ok;
 };

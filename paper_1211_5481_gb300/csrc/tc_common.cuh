@@ -13,7 +13,7 @@
 namespace game {
 namespace tc {
 
-constexpr uint64_t kTimeoutNs = 2000000000ull;   // 2 s per wait
+constexpr long long kTimeoutCycles = 4000000000ll;   // about 2 s per wait
 constexpr uint32_t kSuspendNs = 20000;           // per try_wait suspension (woken early on completion)
 
 // Bounded wait for the phase of the given parity. Waiting threads are
@@ -22,11 +22,11 @@ constexpr uint32_t kSuspendNs = 20000;           // per try_wait suspension (wok
 // sub-partition; each wake-up re-checks the abort flag and the time limit.
 static __device__ bool wait_bar(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status) {
   if (ptx::mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = ptx::global_timer_ns();
+  const long long t0 = clock64();   // (the global timer costs microseconds to read)
   for (;;) {
     if (ptx::mbar_try_wait_sleep(bar, parity, kSuspendNs)) return true;
     if (*abort_flag) return false;
-    if (ptx::global_timer_ns() - t0 > kTimeoutNs) {
+    if (clock64() - t0 > kTimeoutCycles) {
       *abort_flag = 1;
       atomicExch(status, (int)kDevTimeout);
       return false;
@@ -37,9 +37,9 @@ static __device__ bool wait_bar(uint32_t bar, uint32_t parity, volatile int* abo
 // Waits for this CTA's own asynchronous work (copies, MMAs) regardless of the
 // abort flag, still bounded.
 static __device__ void wait_bar_drain(uint32_t bar, uint32_t parity, int* status) {
-  const uint64_t t0 = ptx::global_timer_ns();
+  const long long t0 = clock64();
   while (!ptx::mbar_try_wait(bar, parity)) {
-    if (ptx::global_timer_ns() - t0 > kTimeoutNs) {
+    if (clock64() - t0 > kTimeoutCycles) {
       atomicExch(status, (int)kDevTimeout);
       return;
     }
