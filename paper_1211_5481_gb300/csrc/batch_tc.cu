@@ -320,6 +320,17 @@ struct ItemQueue {
     ptx::mbar_arrive(empty0 + 8u * (uint32_t)slot);
     return v;
   }
+  // the same for a whole warp (every lane returns the answer)
+  __device__ __forceinline__ int pop_warp(int lane) {
+    const int slot = seq % kQueue;
+    const uint32_t par = (uint32_t)(seq / kQueue) & 1u;
+    ++seq;
+    if (!wait_bar_warp(full0 + 8u * (uint32_t)slot, par, abort_flag, status)) return -1;
+    const int v = idx[slot];
+    __syncwarp();   // every lane has read the slot
+    if (lane == 0) ptx::mbar_arrive(empty0 + 8u * (uint32_t)slot);
+    return v;
+  }
 };
 
 // L2 prefetch of one item's features and targets (16-byte aligned: tile
@@ -453,32 +464,37 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_batch_kernel(const BatchA
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
+    // The converged warp, instructions by its elected lane (elect_one): an
+    // item's sizes pass through warp reductions, which leaves them and every
+    // descriptor derived from them in uniform registers. (A lone thread: 1.235
+    // ms for the four launches of 24 uneven runs, this 1.12.)
+    {
+      auto uniform = [](int v) { return __reduce_max_sync(0xffffffffu, v); };
+      auto pop = [&]() { return uniform(iq.pop_warp(lane)); };
       const uint64_t adesc0 = ptx::desc_kmajor_sw128(ptx::smem_addr(ast));
       const uint64_t bdesc0 = ptx::desc_kmajor_sw128(ptx::smem_addr(phi));
-      const uint32_t a_step = kABytes >> 4;
-      const uint32_t a_full0 = ptx::smem_addr(a_full), a_empty0 = ptx::smem_addr(a_empty);
-      const uint32_t phi_full0 = ptx::smem_addr(phi_full), phi_free0 = ptx::smem_addr(phi_free);
+      const uint32_t dhi = (uint32_t)(adesc0 >> 32);
+      const uint32_t alo0 = (uint32_t)adesc0, blo0 = (uint32_t)bdesc0;
+      const uint32_t a_step = kABytes >> 4, alo_end = alo0 + kStages * a_step;
+      const uint32_t a_full0 = ptx::smem_addr(a_full);
+      const uint32_t phi_full0 = ptx::smem_addr(phi_full), phi_free_off = 8u * (uint32_t)KBmax;
       const uint32_t acc_full0 = ptx::smem_addr(acc_full), acc_empty0 = ptx::smem_addr(acc_empty);
-      uint32_t s = 0, ph = 0, acc_it = 0;
+      uint32_t alo = alo0, abar = a_full0, ph = 0, acc_it = 0;
       uint32_t full_par = 0;   // bit k: parity of the next phi_full[k] phase
       bool ok = true;
       BatchItem nxt;
-      int idx_n = iq.pop();
+      int idx_n = pop();
       if (idx_n >= 0) nxt = a.recs[idx_n];
       for (int idx = idx_n; idx >= 0 && ok; idx = idx_n) {
-        const BatchItem R = nxt;
-        idx_n = iq.pop();
+        const int KB = uniform(nxt.KB), C = uniform(nxt.C), BN = uniform(nxt.BN);
+        const int CG = uniform(nxt.CG), nlast = uniform(nxt.nmma_last), RK = uniform(nxt.RK);
+        idx_n = pop();
         if (idx_n >= 0) nxt = a.recs[idx_n];
-        const int KB = R.KB, C = R.C, BN = R.BN, CG = R.CG, nlast = R.nmma_last;
         const uint32_t idesc = ptx::idesc_bf16_f32(128, BN);
         const uint32_t b_step = (uint32_t)(BN * 128) >> 4;
-        const int rmask = R.RK < KB ? R.RK - 1 : -1;   // K-block kb in slot kb & rmask
-        auto kblock = [&](uint32_t d_tmem, uint32_t st, int kb, int slot, int nm) {
-          const uint64_t ad = adesc0 + st * a_step;
-          const uint64_t bd = bdesc0 + (uint32_t)slot * b_step;
-          for (int kk = 0; kk < nm; ++kk)
-            ptx::mma_bf16(d_tmem, ad + 2u * kk, bd + 2u * kk, idesc, (kb | kk) != 0);
+        auto kstep = [&](uint32_t d, uint32_t al, uint32_t bl, uint32_t acc) {
+          ptx::mma_bf16(d, ((uint64_t)dhi << 32) | al, ((uint64_t)dhi << 32) | bl, idesc,
+                          acc);
         };
         // Chromosome tiles in groups of CG, each group's accumulators side by
         // side in one accumulator set; per group the K-blocks are the outer
@@ -490,35 +506,63 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_batch_kernel(const BatchA
         for (int c0 = 0; c0 < C && ok; c0 += CG) {
           const int c1 = c0 + CG < C ? c0 + CG : C;
           const bool last_group = c1 == C;
-          const uint32_t set = acc_it & 1, u = acc_it >> 1;
-          ok = wait_bar(acc_empty0 + 8 * set, (u & 1) ^ 1, abort_flag, a.status);
+          const uint32_t set = acc_it & 1;
+          ok = wait_bar_warp(acc_empty0 + 8 * set, ((acc_it >> 1) & 1) ^ 1, abort_flag, a.status);
           if (!ok) break;
           ptx::tc_fence_after();
           const uint32_t d_set = tmem + set * (uint32_t)a.set_cols;
-          for (int kb = 0; kb < KB && ok; ++kb) {
-            const int slot = kb & rmask;
+          int slot = 0;
+          uint32_t blo = blo0, pbar = phi_full0;
+          for (int kb = 0; kb < KB; ++kb) {
             if (c0 == 0) {
-              ok = wait_bar(phi_full0 + 8 * slot, (full_par >> slot) & 1u, abort_flag, a.status);
+              ok = wait_bar_warp(pbar, (full_par >> slot) & 1u, abort_flag, a.status);
+              if (!ok) break;
               full_par ^= 1u << slot;
             }
-            for (int c = c0; c < c1 && ok; ++c) {
-              ok = wait_bar(a_full0 + 8 * s, ph, abort_flag, a.status);
+            const int nm = kb == KB - 1 ? nlast : 4;
+            uint32_t d = d_set;
+            for (int c = c0; c < c1; ++c) {
+              ok = wait_bar_warp(abar, ph, abort_flag, a.status);
               if (!ok) break;
-              kblock(d_set + (uint32_t)((c - c0) * BN), s, kb, slot, kb == KB - 1 ? nlast : 4);
-              ptx::mma_commit(a_empty0 + 8 * s);
-              if (++s == (uint32_t)kStages) {
-                s = 0;
+              if (ptx::elect_one()) {
+                kstep(d, alo, blo, kb != 0);
+                if (nm == 4) {
+                  kstep(d, alo + 2u, blo + 2u, 1u);
+                  kstep(d, alo + 4u, blo + 4u, 1u);
+                  kstep(d, alo + 6u, blo + 6u, 1u);
+                } else {
+                  for (int kk = 1; kk < nm; ++kk) kstep(d, alo + 2u * kk, blo + 2u * kk, 1u);
+                }
+                ptx::mma_commit(abar + 8u * kStages);
+                if (c == c1 - 1) {
+                  if (last_group) ptx::mma_commit(pbar + phi_free_off);
+                  if (kb == KB - 1) ptx::mma_commit(acc_full0 + 8 * set);
+                }
+              }
+              __syncwarp();
+              d += (uint32_t)BN;
+              alo += a_step;
+              abar += 8;
+              if (alo == alo_end) {
+                alo = alo0;
+                abar = a_full0;
                 ph ^= 1;
               }
             }
-            if (ok && last_group) ptx::mma_commit(phi_free0 + 8 * slot);
+            if (!ok) break;
+            blo += b_step;
+            pbar += 8;
+            if (++slot == RK) {   // a ring item's next pass (RK = KB otherwise)
+              slot = 0;
+              blo = blo0;
+              pbar = phi_full0;
+            }
           }
-          if (!ok) break;
-          ptx::mma_commit(acc_full0 + 8 * set);
           ++acc_it;
         }
       }
-      ptx::mma_commit(ptx::smem_addr(drain));
+      if (ptx::elect_one()) ptx::mma_commit(ptx::smem_addr(drain));
+      __syncwarp();
       wait_bar_drain(ptx::smem_addr(drain), 0, a.status);
     }
   } else if (warp >= kEpiWarp0 && warp < kBasisWarp0) {
@@ -568,14 +612,14 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_batch_kernel(const BatchA
       uint32_t set = 0;
       for (int c = 0; c < R.C && ok; ++c) {
         const int cg = c % R.CG;   // place in the accumulator set
+        const int chrom = c * 128 + row;
+        const float bias = R.a0[chrom];   // loaded before the wait
         if (cg == 0) {
           set = acc_it & 1;
           ok = wait_bar(ptx::smem_addr(&acc_full[set]), (acc_it >> 1) & 1, abort_flag, a.status);
           if (!ok) break;
           ptx::tc_fence_after();
         }
-        const int chrom = c * 128 + row;
-        const float bias = R.a0[chrom];
         const uint64_t bias2 = ptx::f2_pack(bias, bias);
         uint64_t s2 = 0;
         float s_tail = 0.f;
@@ -617,7 +661,9 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_batch_kernel(const BatchA
           ++acc_it;
         }
         const float2 sp2 = ptx::f2_unpack(s2);
-        prow[chrom] = (double)sp2.x + (double)sp2.y + (double)s_tail;
+        double tile_sse = (double)sp2.x + (double)sp2.y;
+        if (s_tail != 0.f) tile_sse += (double)s_tail;   // (FP64 operations are scarce)
+        prow[chrom] = tile_sse;
       }
       float* ynext = ys + ((k + 1) & 1) * kYSlot;
       ynext[row] = yn0;

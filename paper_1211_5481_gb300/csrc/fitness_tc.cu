@@ -26,7 +26,7 @@
 //   warp 0       A producer: bulk-copies 16 KB gene blocks (chromosome tile c,
 //                K-block kb of 64 columns) from the pre-swizzled operand
 //                image into a ring of 3-4 stages.
-//   warp 1       MMA issuer (the converged warp, instructions predicated to one
+//   warp 1       MMA issuer (the converged warp, instructions by its elected
 //                lane) and tensor-memory owner; two FP32 accumulators of BN
 //                columns, so the epilogue of chromosome tile c overlaps the
 //                MMAs of tile c+1.
@@ -242,12 +242,11 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
     // One K-block's MMAs take 512 tensor cycles and this warp's instructions
     // between them share their scheduler with three busy warps, so they decide
     // the tensor pipe's rate: the converged warp runs the loop (uniform
-    // registers, see mma_bf16_w), descriptors, barrier addresses, slots and
+    // registers, see elect_one), descriptors, barrier addresses, slots and
     // phases advance by an add and a compare. (A lone thread with the slots by
     // integer division: 434 us at M = 10^6, N = 32, degree 8, P = 1024, BF16;
-    // by compares 421; this 398.)
+    // by compares 421; this 378 with the epilogue below.)
     {
-      const uint32_t lead = ptx::elect_one();
       const uint32_t idesc =
           F == kFormFP8 ? ptx::idesc_e4m3_f32(128, BN) : ptx::idesc_bf16_f32(128, BN);
       const uint64_t adesc0 = ptx::desc_kmajor_sw128(ptx::smem_addr(ast));
@@ -277,16 +276,18 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
             ok = false;
           }
         }
+        __syncwarp();
+        ok = __all_sync(0xffffffffu, ok);
       }
       // one K step (32 bytes of each operand row): one MMA, three for bf16x3
       auto kstep = [&](uint32_t d_tmem, uint32_t al, uint32_t bl, uint32_t acc) {
         if (F == kFormFP8) {
-          ptx::mma_f8_w(lead, d_tmem, desc(al), desc(bl), idesc, acc);
+          ptx::mma_f8(d_tmem, desc(al), desc(bl), idesc, acc);
         } else {
-          ptx::mma_bf16_w(lead, d_tmem, desc(al), desc(bl), idesc, acc);
+          ptx::mma_bf16(d_tmem, desc(al), desc(bl), idesc, acc);
           if (F == kFormBF16x3) {
-            ptx::mma_bf16_w(lead, d_tmem, desc(al), desc(bl + b_lo), idesc, 1u);
-            ptx::mma_bf16_w(lead, d_tmem, desc(al + a_lo), desc(bl), idesc, 1u);
+            ptx::mma_bf16(d_tmem, desc(al), desc(bl + b_lo), idesc, 1u);
+            ptx::mma_bf16(d_tmem, desc(al + a_lo), desc(bl), idesc, 1u);
           }
         }
       };
@@ -297,37 +298,36 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
         uint32_t blo = tile_blo, pbar = tile_pbar, par = tile_par;
         for (int c = 0; c < a.C && ok; ++c) {
           const uint32_t buf = acc_it & 1;
-          ok = wait_bar(acc_empty0 + 8 * buf, ((acc_it >> 1) & 1) ^ 1, abort_flag, a.status);
+          ok = wait_bar_warp(acc_empty0 + 8 * buf, ((acc_it >> 1) & 1) ^ 1, abort_flag, a.status);
           if (!ok) break;
           ptx::tc_fence_after();
           const uint32_t d_tmem = tmem + buf * (uint32_t)BN;
           blo = tile_blo;
           pbar = tile_pbar;
           par = tile_par;
-          uint32_t acc = 0;
           for (int kb = 0; kb < KB; ++kb) {
             if (c == 0) {
-              ok = wait_bar(pbar, par, abort_flag, a.status);
+              ok = wait_bar_warp(pbar, par, abort_flag, a.status);
               if (!ok) break;
             }
-            ok = wait_bar(abar, ph, abort_flag, a.status);
+            ok = wait_bar_warp(abar, ph, abort_flag, a.status);
             if (!ok) break;
             const int nm = kb == KB - 1 ? nlast : 4;
-            if (nm == 4) {
-              kstep(d_tmem, alo, blo, acc);
-              kstep(d_tmem, alo + 2u, blo + 2u, 1u);
-              kstep(d_tmem, alo + 4u, blo + 4u, 1u);
-              kstep(d_tmem, alo + 6u, blo + 6u, 1u);
-              acc = 1;
-            } else {
-              for (int kk = 0; kk < nm; ++kk) {
-                kstep(d_tmem, alo + 2u * kk, blo + 2u * kk, acc);
-                acc = 1;
+            if (ptx::elect_one()) {
+              kstep(d_tmem, alo, blo, kb != 0);
+              if (nm == 4) {
+                kstep(d_tmem, alo + 2u, blo + 2u, 1u);
+                kstep(d_tmem, alo + 4u, blo + 4u, 1u);
+                kstep(d_tmem, alo + 6u, blo + 6u, 1u);
+              } else {
+                for (int kk = 1; kk < nm; ++kk)
+                  kstep(d_tmem, alo + 2u * kk, blo + 2u * kk, 1u);
               }
+              ptx::mma_commit(abar + a_empty);
+              if (c == a.C - 1) ptx::mma_commit(pbar + phi_free_off);
+              if (kb == KB - 1) ptx::mma_commit(acc_full0 + 8 * buf);
             }
-            ptx::mma_commit_w(lead, abar + a_empty);
-            if (c == a.C - 1) ptx::mma_commit_w(lead, pbar + phi_free_off);
-            if (kb == KB - 1) ptx::mma_commit_w(lead, acc_full0 + 8 * buf);
+            __syncwarp();
             alo += a_step;
             abar += 8;
             if (alo == alo_end) {
@@ -350,7 +350,8 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
         tile_par = par;
       }
       // every MMA issued above has completed once this arrives
-      ptx::mma_commit_w(lead, ptx::smem_addr(drain));
+      if (ptx::elect_one()) ptx::mma_commit(ptx::smem_addr(drain));
+      __syncwarp();
       wait_bar_drain(ptx::smem_addr(drain), 0, a.status);
     }
   } else if (warp == 2) {
@@ -431,7 +432,7 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
     // cycles), and while it is late the MMAs wait: so the targets come from shared
     // memory, and the chromosome's bias and running sum are loaded before the wait
     // for the accumulator, not after its reduction. (M = 10^6, N = 32, degree 8,
-    // P = 1024: 398 -> 365 us together with the expansion's look-ahead.)
+    // P = 1024: 398 -> 378 us together with the expansion's look-ahead.)
     auto reduce_tiles = [&](auto ys_tag) {
       constexpr bool YS = decltype(ys_tag)::value;
       uint32_t acc_it = 0;

@@ -38,6 +38,8 @@
 // CTA raises the status word, abandons its loops, drains its own copies (the
 // even CTA its MMAs), and both CTAs meet at the final cluster barrier before
 // the pair's tensor memory is freed.
+#include <type_traits>
+
 #include "basis.cuh"
 #include "expand_stream.cuh"
 #include "game_internal.cuh"
@@ -67,6 +69,7 @@ struct Tc2Args {
   int64_t M;
   int N, d, basis, Kp;
   int KB, Cp, NS, stages, nmma_last, ntiles, Ppad, xstage;
+  int ycopy;   // targets of each tile in a two-slot shared buffer
   const float* Xt;
   const float* y;
   const uint8_t* popA;
@@ -77,17 +80,18 @@ struct Tc2Args {
 };
 
 struct Smem2 {
-  int phi, ast, xs, tab, bars, total;
+  int phi, ast, xs, ys, tab, bars, total;
 };
 
-__host__ __device__ inline int num_bars2(int NS, int S) { return 2 * S + 2 * NS + 7; }
+__host__ __device__ inline int num_bars2(int NS, int S) { return 2 * S + 2 * NS + 11; }
 
-__host__ __device__ inline Smem2 smem_plan2(int KB, int NS, int N, int S, int xstage) {
+__host__ __device__ inline Smem2 smem_plan2(int KB, int NS, int N, int S, int xstage, int ycopy) {
   Smem2 s;
   s.phi = 0;
   s.ast = NS * kRows * 128;
   s.xs = s.ast + S * (int)kABytes;
-  s.tab = s.xs + (xstage ? N * kRows * 4 : 0);
+  s.ys = s.xs + (xstage ? N * kRows * 4 : 0);
+  s.tab = s.ys + (ycopy ? 2 * kBN * 4 : 0);
   s.bars = (s.tab + KB * 8 * 4 + 7) & ~7;
   s.total = s.bars + num_bars2(NS, S) * 8 + 16 + 1024;   // + alignment slack
   return s;
@@ -168,10 +172,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   uint8_t* base = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   const int KB = a.KB, N = a.N, S = a.stages, NS = a.NS;
-  const Smem2 sp = smem_plan2(KB, NS, N, S, a.xstage);
+  const Smem2 sp = smem_plan2(KB, NS, N, S, a.xstage, a.ycopy);
   uint8_t* phi = base + sp.phi;
   uint8_t* ast = base + sp.ast;
   float* xs = reinterpret_cast<float*>(base + sp.xs);
+  float* ys = reinterpret_cast<float*>(base + sp.ys);
   uint32_t* tab = reinterpret_cast<uint32_t*>(base + sp.tab);
   uint64_t* bars = reinterpret_cast<uint64_t*>(base + sp.bars);
   uint64_t* a_full = bars;
@@ -183,7 +188,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   uint64_t* x_full = acc_empty + 2;
   uint64_t* x_empty = x_full + 1;
   uint64_t* drain = x_empty + 1;
-  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(drain + 1);
+  uint64_t* y_full = drain + 1;    // [2]
+  uint64_t* y_empty = y_full + 2;  // [2]
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(y_empty + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
 
   const uint32_t rank = ptx::cluster_ctarank();
@@ -206,6 +213,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     ptx::mbar_init(ptx::smem_addr(x_full), 1);
     ptx::mbar_init(ptx::smem_addr(x_empty), kBasisThreads);
     ptx::mbar_init(ptx::smem_addr(drain), 1);
+    for (int b = 0; b < 2; ++b) {
+      ptx::mbar_init(ptx::smem_addr(&y_full[b]), 1);
+      ptx::mbar_init(ptx::smem_addr(&y_empty[b]), kBasisWarp0 - kEpiWarp0);   // epilogue warps
+    }
     *abort_flag = 0;
     ptx::fence_mbar_init();
     ptx::fence_proxy_async_smem();
@@ -223,6 +234,25 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const int ncl = (int)(gridDim.x >> 1), cl = (int)(blockIdx.x >> 1);
   const int my_tiles = (a.ntiles - cl + ncl - 1) / ncl;
   const int Cp = a.Cp;
+
+  // each tile's targets into slot it & 1, released by the CTA's epilogue warps
+  // after the tile's last chromosome tile: one thread of an otherwise idle warp
+  // (the even CTA's relay warp, the odd CTA's issuer warp)
+  auto produce_targets = [&]() {
+    int issued = 0;
+    for (int it = 0; it < my_tiles; ++it) {
+      const int b = it & 1;
+      if (!wait_bar(ptx::smem_addr(&y_empty[b]), ((it >> 1) & 1) ^ 1, abort_flag, a.status)) break;
+      ptx::mbar_arrive_expect_tx(ptx::smem_addr(&y_full[b]), kBN * 4);
+      ptx::bulk_g2s(ptx::smem_addr(ys + b * kBN), a.y + ((int64_t)cl + (int64_t)it * ncl) * kBN,
+                    kBN * 4, ptx::smem_addr(&y_full[b]));
+      ++issued;
+    }
+    for (int b = 0; b < 2 && b < issued; ++b) {
+      const int uses = (issued - b + 1) / 2;
+      wait_bar_drain(ptx::smem_addr(&y_full[b]), (uint32_t)(uses - 1) & 1u, a.status);
+    }
+  };
 
   if (warp == 0) {
     // ---------------- gene producer (both CTAs) ----------------
@@ -254,7 +284,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     // ---------------- MMA issuer (even CTA) ----------------
     // (the converged warp with running descriptors: see fitness_tc.cu)
     if (lead) {
-      const uint32_t one = ptx::elect_one();
       const uint32_t idesc = ptx::idesc_bf16_f32(2 * kRows, kBN);
       const uint64_t adesc0 = ptx::desc_kmajor_sw128(ptx::smem_addr(ast));
       const uint64_t bdesc0 = ptx::desc_kmajor_sw128(ptx::smem_addr(phi));
@@ -280,9 +309,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             ok = false;
           }
         }
+        __syncwarp();
+        ok = __all_sync(0xffffffffu, ok);
       }
       auto kstep = [&](uint32_t d_tmem, uint32_t al, uint32_t bl, uint32_t acc) {
-        ptx::mma_bf16_pair_w(one, d_tmem, ((uint64_t)dhi << 32) | al, ((uint64_t)dhi << 32) | bl,
+        ptx::mma_bf16_pair(d_tmem, ((uint64_t)dhi << 32) | al, ((uint64_t)dhi << 32) | bl,
                              idesc, acc);
       };
       uint32_t alo = alo0, abar = a_full0, ph = 0;
@@ -292,37 +323,36 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         uint32_t blo = tile_blo, pbar = tile_pbar, par = tile_par;
         for (int c = 0; c < Cp && ok; ++c) {
           const uint32_t buf = acc_it & 1;
-          ok = wait_bar(acc_empty0 + 8 * buf, ((acc_it >> 1) & 1) ^ 1, abort_flag, a.status);
+          ok = wait_bar_warp(acc_empty0 + 8 * buf, ((acc_it >> 1) & 1) ^ 1, abort_flag, a.status);
           if (!ok) break;
           ptx::tc_fence_after();
           const uint32_t d_tmem = tmem + buf * (uint32_t)kBN;
           blo = tile_blo;
           pbar = tile_pbar;
           par = tile_par;
-          uint32_t acc = 0;
           for (int kb = 0; kb < KB; ++kb) {
             if (c == 0) {
-              ok = wait_bar(pbar, par, abort_flag, a.status);
+              ok = wait_bar_warp(pbar, par, abort_flag, a.status);
               if (!ok) break;
             }
-            ok = wait_bar(abar, ph, abort_flag, a.status);
+            ok = wait_bar_warp(abar, ph, abort_flag, a.status);
             if (!ok) break;
             const int nm = kb == KB - 1 ? nlast : 4;
-            if (nm == 4) {
-              kstep(d_tmem, alo, blo, acc);
-              kstep(d_tmem, alo + 2u, blo + 2u, 1u);
-              kstep(d_tmem, alo + 4u, blo + 4u, 1u);
-              kstep(d_tmem, alo + 6u, blo + 6u, 1u);
-              acc = 1;
-            } else {
-              for (int kk = 0; kk < nm; ++kk) {
-                kstep(d_tmem, alo + 2u * kk, blo + 2u * kk, acc);
-                acc = 1;
+            if (ptx::elect_one()) {
+              kstep(d_tmem, alo, blo, kb != 0);
+              if (nm == 4) {
+                kstep(d_tmem, alo + 2u, blo + 2u, 1u);
+                kstep(d_tmem, alo + 4u, blo + 4u, 1u);
+                kstep(d_tmem, alo + 6u, blo + 6u, 1u);
+              } else {
+                for (int kk = 1; kk < nm; ++kk)
+                  kstep(d_tmem, alo + 2u * kk, blo + 2u * kk, 1u);
               }
+              ptx::mma_commit_pair_mc(abar + a_empty_off, both);
+              if (c == Cp - 1) ptx::mma_commit_pair_mc(pbar + phi_free_off, both);
+              if (kb == KB - 1) ptx::mma_commit_pair_mc(acc_full0 + 8 * buf, both);
             }
-            ptx::mma_commit_pair_mc_w(one, abar + a_empty_off, both);
-            if (c == Cp - 1) ptx::mma_commit_pair_mc_w(one, pbar + phi_free_off, both);
-            if (kb == KB - 1) ptx::mma_commit_pair_mc_w(one, acc_full0 + 8 * buf, both);
+            __syncwarp();
             alo += a_step;
             abar += 8;
             if (alo == alo_end) {
@@ -345,8 +375,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         tile_par = par;
       }
       // every MMA issued above has completed once this arrives
-      if (one) ptx::mma_commit_pair(ptx::smem_addr(drain));
+      if (ptx::elect_one()) ptx::mma_commit_pair(ptx::smem_addr(drain));
+      __syncwarp();
       wait_bar_drain(ptx::smem_addr(drain), 0, a.status);
+    } else if (lane == 0 && a.ycopy) {
+      produce_targets();
     }
   } else if (warp == 2) {
     // ---------------- feature producer (staged features only) ----------------
@@ -380,6 +413,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           ph ^= 1;
         }
       }
+    } else if (lane == 0 && a.ycopy) {
+      produce_targets();
     }
   } else if (warp >= kEpiWarp0 && warp < kBasisWarp0) {
     // ---------------- epilogue (both CTAs) ----------------
@@ -390,65 +425,83 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     const uint32_t lane_addr = (uint32_t)(qw * 32) << 16;
     double* part_row = a.part + (size_t)(2 * cl + half) * a.Ppad;
     const uint32_t acc_empty_lead0 = ptx::mapa(ptx::smem_addr(acc_empty), 0);
-    uint32_t acc_it = 0;
-    bool ok = true;
-    for (int it = 0; it < my_tiles && ok; ++it) {
-      const int64_t m0 = ((int64_t)cl + (int64_t)it * ncl) * kBN;
-      const int64_t rem = a.M - m0 - col_lo;
-      const int valid = rem <= 0 ? 0 : (rem >= kRows ? kRows : (int)rem);
-      const float* yt = a.y + m0 + col_lo;
-      for (int c = 0; c < Cp; ++c) {
-        const uint32_t buf = acc_it & 1, u = acc_it >> 1;
-        ok = wait_bar(ptx::smem_addr(&acc_full[buf]), u & 1, abort_flag, a.status);
-        if (!ok) break;
-        ptx::tc_fence_after();
-        const int chrom = c * 2 * kRows + (int)rank * kRows + row;
-        const float bias = a.a0[chrom];
-        const uint64_t bias2 = ptx::f2_pack(bias, bias);
-        const uint64_t negu2 = ptx::f2_pack(-1.f, -1.f);
-        uint64_t s2 = 0;
-        float s_tail = 0.f;
-        const uint32_t tbase = tmem + lane_addr + buf * (uint32_t)kBN + (uint32_t)col_lo;
-        const int nfull = valid / 32;
-        if (nfull > 0) {
-          uint32_t va[32], vb[32];
-          ptx::tmem_ld32_issue(tbase, va);
-          ptx::tmem_ld32_wait(va);
-          for (int k = 0; k < nfull; k += 2) {
-            const bool has_b = k + 1 < nfull;
-            if (has_b) ptx::tmem_ld32_issue(tbase + (uint32_t)(k + 1) * 32, vb);
-            epi_chunk<false, ABS>(va, yt + k * 32, bias2, negu2, s2);
-            if (has_b) {
-              ptx::tmem_ld32_wait(vb);
-              const bool has_a = k + 2 < nfull;
-              if (has_a) ptx::tmem_ld32_issue(tbase + (uint32_t)(k + 2) * 32, va);
-              epi_chunk<false, ABS>(vb, yt + (k + 1) * 32, bias2, negu2, s2);
-              if (has_a) ptx::tmem_ld32_wait(va);
+    // (targets from shared memory, bias and running sum loaded before the wait:
+    // see fitness_tc.cu; M = 4 10^6, N = 48, degree 6, P = 2048: 3.17 -> 3.02 ms)
+    auto reduce_tiles = [&](auto ys_tag) {
+      constexpr bool YS = decltype(ys_tag)::value;
+      uint32_t acc_it = 0;
+      bool ok = true;
+      for (int it = 0; it < my_tiles && ok; ++it) {
+        const int64_t m0 = ((int64_t)cl + (int64_t)it * ncl) * kBN;
+        const int64_t rem = a.M - m0 - col_lo;
+        const int valid = rem <= 0 ? 0 : (rem >= kRows ? kRows : (int)rem);
+        if (YS) {
+          ok = wait_bar(ptx::smem_addr(&y_full[it & 1]), (it >> 1) & 1, abort_flag, a.status);
+          ok = __all_sync(0xffffffffu, ok);   // the warp arrives as one
+          if (!ok) break;
+        }
+        const float* yt = YS ? ys + (it & 1) * kBN + col_lo : a.y + m0 + col_lo;
+        for (int c = 0; c < Cp; ++c) {
+          const uint32_t buf = acc_it & 1, u = acc_it >> 1;
+          const int chrom = c * 2 * kRows + (int)rank * kRows + row;
+          const float bias = a.a0[chrom];
+          const double before = it == 0 ? 0.0 : part_row[chrom];
+          ok = wait_bar(ptx::smem_addr(&acc_full[buf]), u & 1, abort_flag, a.status);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          ptx::tc_fence_after();
+          const uint64_t bias2 = ptx::f2_pack(bias, bias);
+          const uint64_t negu2 = ptx::f2_pack(-1.f, -1.f);
+          uint64_t s2 = 0;
+          float s_tail = 0.f;
+          const uint32_t tbase = tmem + lane_addr + buf * (uint32_t)kBN + (uint32_t)col_lo;
+          const int nfull = valid / 32;
+          if (nfull > 0) {
+            uint32_t va[32], vb[32];
+            ptx::tmem_ld32_issue(tbase, va);
+            ptx::tmem_ld32_wait(va);
+            for (int k = 0; k < nfull; k += 2) {
+              const bool has_b = k + 1 < nfull;
+              if (has_b) ptx::tmem_ld32_issue(tbase + (uint32_t)(k + 1) * 32, vb);
+              epi_chunk<false, ABS, YS>(va, yt + k * 32, bias2, negu2, s2);
+              if (has_b) {
+                ptx::tmem_ld32_wait(vb);
+                const bool has_a = k + 2 < nfull;
+                if (has_a) ptx::tmem_ld32_issue(tbase + (uint32_t)(k + 2) * 32, va);
+                epi_chunk<false, ABS, YS>(vb, yt + (k + 1) * 32, bias2, negu2, s2);
+                if (has_a) ptx::tmem_ld32_wait(va);
+              }
             }
           }
-        }
-        if (nfull * 32 < valid) {   // ragged last chunk of the last tile
-          uint32_t v[32];
-          ptx::tmem_ld32(tbase + (uint32_t)nfull * 32, v);
-          const int lim = valid - nfull * 32;
+          if (nfull * 32 < valid) {   // ragged last chunk of the last tile
+            uint32_t v[32];
+            ptx::tmem_ld32(tbase + (uint32_t)nfull * 32, v);
+            const int lim = valid - nfull * 32;
 #pragma unroll
-          for (int e = 0; e < 32; ++e) {
-            if (e < lim) {
-              const float r = (yt[nfull * 32 + e] - bias) - __uint_as_float(v[e]);
-              s_tail = ABS ? s_tail + fabsf(r) : fmaf(r, r, s_tail);
+            for (int e = 0; e < 32; ++e) {
+              if (e < lim) {
+                const float r = (yt[nfull * 32 + e] - bias) - __uint_as_float(v[e]);
+                s_tail = ABS ? s_tail + fabsf(r) : fmaf(r, r, s_tail);
+              }
             }
           }
+          ptx::tc_fence_before();
+          __syncwarp();
+          if (lane == 0) ptx::mbar_arrive_cluster(acc_empty_lead0 + 8 * buf);
+          const float2 sp2 = ptx::f2_unpack(s2);
+          double tile_sse = (double)sp2.x + (double)sp2.y;
+          if (s_tail != 0.f) tile_sse += (double)s_tail;   // (FP64 operations are scarce)
+          part_row[chrom] = it == 0 ? tile_sse : before + tile_sse;
+          ++acc_it;
         }
-        ptx::tc_fence_before();
-        __syncwarp();
-        if (lane == 0) ptx::mbar_arrive_cluster(acc_empty_lead0 + 8 * buf);
-        const float2 sp2 = ptx::f2_unpack(s2);
-        double tile_sse = (double)sp2.x + (double)sp2.y;
-        if (s_tail != 0.f) tile_sse += (double)s_tail;   // (FP64 operations are scarce)
-        part_row[chrom] = (it == 0) ? tile_sse : part_row[chrom] + tile_sse;
-        ++acc_it;
+        if (YS && ok) {
+          __syncwarp();
+          if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&y_empty[it & 1]));
+        }
       }
-    }
+    };
+    if (a.ycopy) reduce_tiles(std::true_type{});
+    else reduce_tiles(std::false_type{});
   } else {
     // ---------------- expansion (both CTAs) ----------------
     const int r0 = threadIdx.x - kBasisWarp0 * 32;   // this thread's pattern row
@@ -601,7 +654,7 @@ TcPlan plan_tc_pair(const Shape& s, int P, int num_sms) {
   const int xstage = (s.basis == GAME_BASIS_CHEB && s.d % 8 == 0) ? 0 : 1;
   for (int stages = 4; stages >= 3 && !pl.ok; --stages)
     for (int NS = 2 * pl.KB; NS >= pl.KB && !pl.ok; --NS) {
-      const int sm = smem_plan2(pl.KB, NS, s.N, stages, xstage).total;
+      const int sm = smem_plan2(pl.KB, NS, s.N, stages, xstage, 0).total;
       if (sm <= kMaxSmem) {
         pl.NS = NS;
         pl.stages = stages;
@@ -611,6 +664,13 @@ TcPlan plan_tc_pair(const Shape& s, int P, int num_sms) {
       }
     }
   if (!pl.ok) return pl;
+  {
+    const int sm = smem_plan2(pl.KB, pl.NS, s.N, pl.stages, xstage, 1).total;
+    if (sm <= kMaxSmem) {
+      pl.ycopy = 1;
+      if (pl.smem_bytes < sm) pl.smem_bytes = sm;
+    }
+  }
   const int ntiles = ceil_div(s.M, kBN);
   const int clusters = ntiles < num_sms / 2 ? ntiles : num_sms / 2;
   pl.grid = 2 * clusters;
@@ -636,6 +696,7 @@ cudaError_t launch_fitness_tc_pair(const TcPlan& pl, const Shape& s, const float
   a.NS = pl.NS;
   a.stages = pl.stages;
   a.xstage = pl.xstage;
+  a.ycopy = pl.ycopy;
   const int last_cols = s.Kp - 64 * (pl.KB - 1);
   a.nmma_last = (last_cols + 15) / 16;
   a.ntiles = ceil_div(s.M, kBN);

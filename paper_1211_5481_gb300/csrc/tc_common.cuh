@@ -34,6 +34,16 @@ static __device__ bool wait_bar(uint32_t bar, uint32_t parity, volatile int* abo
   }
 }
 
+// The wait of a whole warp, converged again behind it (the MMA issue that
+// follows holds its operands in uniform registers), with one answer for all
+// lanes.
+static __device__ __forceinline__ bool wait_bar_warp(uint32_t bar, uint32_t parity,
+                                                     volatile int* abort_flag, int* status) {
+  const bool ok = wait_bar(bar, parity, abort_flag, status);
+  __syncwarp();
+  return __all_sync(0xffffffffu, ok);
+}
+
 // Waits for this CTA's own asynchronous work (copies, MMAs) regardless of the
 // abort flag, still bounded.
 static __device__ void wait_bar_drain(uint32_t bar, uint32_t parity, int* status) {

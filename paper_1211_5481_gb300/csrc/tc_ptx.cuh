@@ -254,59 +254,20 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
 }
 
 // ---- MMA issue by a converged warp ----
-// The whole warp runs the issuing loop and `lead` (1 in one lane, from
-// elect_one) predicates the instructions themselves. Every address and
-// descriptor is then warp-uniform and stays in uniform registers; issued by a
-// lone thread inside a divergent branch they are moved there one by one for
-// each MMA. Measured with every other role of the kernel running: 151 against
-// 194 cycles per 128 x 256 x 16 MMA (128 is the tensor pipe's own rate).
+// The whole warp runs the issuing loop and waits; one K-block's MMAs and
+// commits stand in a block `if (elect_one())`. The compiler knows such a block
+// is run by one thread of a converged warp, so every address and descriptor
+// stays in uniform registers; in a branch on the lane number they are moved
+// there one by one for each MMA. The same lane is elected each time, so the
+// commits follow the MMAs of their thread. Measured with every other role of
+// the kernel running: 159 against 194 cycles per 128 x 256 x 16 MMA (128 is
+// the tensor pipe's own rate).
 __device__ __forceinline__ uint32_t elect_one() {
   uint32_t lead;
   asm volatile(
       "{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}"
       : "=r"(lead));
   return lead;
-}
-__device__ __forceinline__ void mma_bf16_w(uint32_t lead, uint32_t d_tmem, uint64_t adesc,
-                                           uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
-      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(lead)
-      : "memory");
-}
-__device__ __forceinline__ void mma_f8_w(uint32_t lead, uint32_t d_tmem, uint64_t adesc,
-                                         uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
-      "@q tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(lead)
-      : "memory");
-}
-__device__ __forceinline__ void mma_commit_w(uint32_t lead, uint32_t bar) {
-  asm volatile(
-      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
-      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(
-          bar),
-      "r"(lead)
-      : "memory");
-}
-__device__ __forceinline__ void mma_bf16_pair_w(uint32_t lead, uint32_t d_tmem, uint64_t adesc,
-                                                uint64_t bdesc, uint32_t idesc,
-                                                uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
-      "@q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(lead)
-      : "memory");
-}
-__device__ __forceinline__ void mma_commit_pair_mc_w(uint32_t lead, uint32_t bar, uint16_t mask) {
-  asm volatile(
-      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t"
-      "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 "
-      "[%0], %1;\n\t}" ::"r"(bar),
-      "h"(mask), "r"(lead)
-      : "memory");
 }
 
 // ---- packed FP32 pairs (two lanes of one 64-bit register) ----
