@@ -320,17 +320,6 @@ struct ItemQueue {
     ptx::mbar_arrive(empty0 + 8u * (uint32_t)slot);
     return v;
   }
-  // the same for a whole warp (every lane returns the answer)
-  __device__ __forceinline__ int pop_warp(int lane) {
-    const int slot = seq % kQueue;
-    const uint32_t par = (uint32_t)(seq / kQueue) & 1u;
-    ++seq;
-    if (!wait_bar_warp(full0 + 8u * (uint32_t)slot, par, abort_flag, status)) return -1;
-    const int v = idx[slot];
-    __syncwarp();   // every lane has read the slot
-    if (lane == 0) ptx::mbar_arrive(empty0 + 8u * (uint32_t)slot);
-    return v;
-  }
 };
 
 // L2 prefetch of one item's features and targets (16-byte aligned: tile
@@ -464,13 +453,10 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_batch_kernel(const BatchA
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    // The converged warp, instructions by its elected lane (elect_one): an
-    // item's sizes pass through warp reductions, which leaves them and every
-    // descriptor derived from them in uniform registers. (A lone thread: 1.235
-    // ms for the four launches of 24 uneven runs, this 1.12.)
+    // One elected thread (elect_one), descriptors and barrier addresses advance by
+    // an add and a compare. (Lane 0: 1.235 ms for the four launches of 24 uneven
+    // runs, this 1.10.)
     {
-      auto uniform = [](int v) { return __reduce_max_sync(0xffffffffu, v); };
-      auto pop = [&]() { return uniform(iq.pop_warp(lane)); };
       const uint64_t adesc0 = ptx::desc_kmajor_sw128(ptx::smem_addr(ast));
       const uint64_t bdesc0 = ptx::desc_kmajor_sw128(ptx::smem_addr(phi));
       const uint32_t dhi = (uint32_t)(adesc0 >> 32);
@@ -482,49 +468,49 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_batch_kernel(const BatchA
       uint32_t alo = alo0, abar = a_full0, ph = 0, acc_it = 0;
       uint32_t full_par = 0;   // bit k: parity of the next phi_full[k] phase
       bool ok = true;
-      BatchItem nxt;
-      int idx_n = pop();
-      if (idx_n >= 0) nxt = a.recs[idx_n];
-      for (int idx = idx_n; idx >= 0 && ok; idx = idx_n) {
-        const int KB = uniform(nxt.KB), C = uniform(nxt.C), BN = uniform(nxt.BN);
-        const int CG = uniform(nxt.CG), nlast = uniform(nxt.nmma_last), RK = uniform(nxt.RK);
-        idx_n = pop();
+      if (ptx::elect_one()) {
+        BatchItem nxt;
+        int idx_n = iq.pop();
         if (idx_n >= 0) nxt = a.recs[idx_n];
-        const uint32_t idesc = ptx::idesc_bf16_f32(128, BN);
-        const uint32_t b_step = (uint32_t)(BN * 128) >> 4;
-        auto kstep = [&](uint32_t d, uint32_t al, uint32_t bl, uint32_t acc) {
-          ptx::mma_bf16(d, ((uint64_t)dhi << 32) | al, ((uint64_t)dhi << 32) | bl, idesc,
-                          acc);
-        };
-        // Chromosome tiles in groups of CG, each group's accumulators side by
-        // side in one accumulator set; per group the K-blocks are the outer
-        // loop, so with one group (C <= 256 / BN) a K-block is released as
-        // soon as every tile has used it and the next item's expansion
-        // follows this item's MMAs K-block by K-block. K-block kb sits in
-        // slot kb (ring items, one group by construction: kb mod RK, the
-        // expansion refilling slots within the item).
-        for (int c0 = 0; c0 < C && ok; c0 += CG) {
-          const int c1 = c0 + CG < C ? c0 + CG : C;
-          const bool last_group = c1 == C;
-          const uint32_t set = acc_it & 1;
-          ok = wait_bar_warp(acc_empty0 + 8 * set, ((acc_it >> 1) & 1) ^ 1, abort_flag, a.status);
-          if (!ok) break;
-          ptx::tc_fence_after();
-          const uint32_t d_set = tmem + set * (uint32_t)a.set_cols;
-          int slot = 0;
-          uint32_t blo = blo0, pbar = phi_full0;
-          for (int kb = 0; kb < KB; ++kb) {
-            if (c0 == 0) {
-              ok = wait_bar_warp(pbar, (full_par >> slot) & 1u, abort_flag, a.status);
-              if (!ok) break;
-              full_par ^= 1u << slot;
-            }
-            const int nm = kb == KB - 1 ? nlast : 4;
-            uint32_t d = d_set;
-            for (int c = c0; c < c1; ++c) {
-              ok = wait_bar_warp(abar, ph, abort_flag, a.status);
-              if (!ok) break;
-              if (ptx::elect_one()) {
+        for (int idx = idx_n; idx >= 0 && ok; idx = idx_n) {
+          const int KB = nxt.KB, C = nxt.C, BN = nxt.BN;
+          const int CG = nxt.CG, nlast = nxt.nmma_last, RK = nxt.RK;
+          idx_n = iq.pop();
+          if (idx_n >= 0) nxt = a.recs[idx_n];
+          const uint32_t idesc = ptx::idesc_bf16_f32(128, BN);
+          const uint32_t b_step = (uint32_t)(BN * 128) >> 4;
+          auto kstep = [&](uint32_t d, uint32_t al, uint32_t bl, uint32_t acc) {
+            ptx::mma_bf16(d, ((uint64_t)dhi << 32) | al, ((uint64_t)dhi << 32) | bl, idesc,
+                            acc);
+          };
+          // Chromosome tiles in groups of CG, each group's accumulators side by
+          // side in one accumulator set; per group the K-blocks are the outer
+          // loop, so with one group (C <= 256 / BN) a K-block is released as
+          // soon as every tile has used it and the next item's expansion
+          // follows this item's MMAs K-block by K-block. K-block kb sits in
+          // slot kb (ring items, one group by construction: kb mod RK, the
+          // expansion refilling slots within the item).
+          for (int c0 = 0; c0 < C && ok; c0 += CG) {
+            const int c1 = c0 + CG < C ? c0 + CG : C;
+            const bool last_group = c1 == C;
+            const uint32_t set = acc_it & 1;
+            ok = wait_bar(acc_empty0 + 8 * set, ((acc_it >> 1) & 1) ^ 1, abort_flag, a.status);
+            if (!ok) break;
+            ptx::tc_fence_after();
+            const uint32_t d_set = tmem + set * (uint32_t)a.set_cols;
+            int slot = 0;
+            uint32_t blo = blo0, pbar = phi_full0;
+            for (int kb = 0; kb < KB; ++kb) {
+              if (c0 == 0) {
+                ok = wait_bar(pbar, (full_par >> slot) & 1u, abort_flag, a.status);
+                if (!ok) break;
+                full_par ^= 1u << slot;
+              }
+              const int nm = kb == KB - 1 ? nlast : 4;
+              uint32_t d = d_set;
+              for (int c = c0; c < c1; ++c) {
+                ok = wait_bar(abar, ph, abort_flag, a.status);
+                if (!ok) break;
                 kstep(d, alo, blo, kb != 0);
                 if (nm == 4) {
                   kstep(d, alo + 2u, blo + 2u, 1u);
@@ -538,30 +524,29 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_batch_kernel(const BatchA
                   if (last_group) ptx::mma_commit(pbar + phi_free_off);
                   if (kb == KB - 1) ptx::mma_commit(acc_full0 + 8 * set);
                 }
+                d += (uint32_t)BN;
+                alo += a_step;
+                abar += 8;
+                if (alo == alo_end) {
+                  alo = alo0;
+                  abar = a_full0;
+                  ph ^= 1;
+                }
               }
-              __syncwarp();
-              d += (uint32_t)BN;
-              alo += a_step;
-              abar += 8;
-              if (alo == alo_end) {
-                alo = alo0;
-                abar = a_full0;
-                ph ^= 1;
+              if (!ok) break;
+              blo += b_step;
+              pbar += 8;
+              if (++slot == RK) {   // a ring item's next pass (RK = KB otherwise)
+                slot = 0;
+                blo = blo0;
+                pbar = phi_full0;
               }
             }
-            if (!ok) break;
-            blo += b_step;
-            pbar += 8;
-            if (++slot == RK) {   // a ring item's next pass (RK = KB otherwise)
-              slot = 0;
-              blo = blo0;
-              pbar = phi_full0;
-            }
+            ++acc_it;
           }
-          ++acc_it;
         }
+        ptx::mma_commit(ptx::smem_addr(drain));
       }
-      if (ptx::elect_one()) ptx::mma_commit(ptx::smem_addr(drain));
       __syncwarp();
       wait_bar_drain(ptx::smem_addr(drain), 0, a.status);
     }

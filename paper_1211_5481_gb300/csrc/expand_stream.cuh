@@ -1,7 +1,7 @@
 // expand_stream.cuh -- the expansion role of the tensor-core fitness kernels
 // with the basis and the degree compile-time constants (degrees 1..10).
 //
-// What bounds it: four warps, one per scheduler, produce every expansion value
+// What bounds it: eight warps, two per scheduler, produce every expansion value
 // of the SM, so the instructions per value decide. The chunk generator it
 // replaces for these degrees decoded a descriptor per 8 columns, restarted the
 // feature's recurrence there (for the trigonometric basis with another sincosf
@@ -41,7 +41,7 @@ struct StreamArgs {
   int xstride, xblocks; // xblocks: rows in 128-row blocks of N features
   int N, KB, NS;
   int RW, R, QS;        // rows per pass, passes, threads per row
-  int bt;               // thread of the role, 0..127
+  int bt;               // thread of the role, 0..255
   int my_tiles;
   volatile int* abort_flag;
   int* status;

@@ -26,8 +26,7 @@
 //   warp 0       A producer: bulk-copies 16 KB gene blocks (chromosome tile c,
 //                K-block kb of 64 columns) from the pre-swizzled operand
 //                image into a ring of 3-4 stages.
-//   warp 1       MMA issuer (the converged warp, instructions by its elected
-//                lane) and tensor-memory owner; two FP32 accumulators of BN
+//   warp 1       MMA issuer (one elected thread) and tensor-memory owner; two FP32 accumulators of BN
 //                columns, so the epilogue of chromosome tile c overlaps the
 //                MMAs of tile c+1.
 //   warp 2       X producer: bulk-copies the next pattern tile's features
@@ -37,7 +36,7 @@
 //                = TMEM lane; warps 4-7 take the first half of the columns,
 //                8-11 the second), r = (y_m - a_0) - D, sse += r^2 in packed
 //                FP32 pairs, then added to an FP64 partial per (CTA, half).
-//   warps 12-15  expansion: each thread owns fixed pattern rows; the basis
+//   warps 12-19  expansion: each thread owns fixed pattern rows; the basis
 //                recurrences run in registers, are rounded to the operand form
 //                and stored in the K-major SWIZZLE_128B operand layout: whole
 //                features at a time for degrees 1..10 (expand_stream.cuh),
@@ -76,12 +75,16 @@ namespace {
 using namespace tc;
 
 constexpr uint32_t kABytes = 128 * 128;   // one (chromosome tile, K-block) gene block
-constexpr int kWarps = 16;
-constexpr int kThreads = kWarps * 32;
 constexpr int kEpiWarp0 = 4;
 constexpr int kEpiThreads = 256;          // warps 4..11
 constexpr int kBasisWarp0 = 12;
-constexpr int kBasisThreads = 128;        // warps 12..15
+// Eight expansion warps: with few chromosome tiles the expansion's own latencies
+// decide, and four warps, one per scheduler, leave them open. us per evaluation
+// with 4 -> 8: BF16, M = 10^6, N = 32, degree 8, P = 128: 139 -> 112; FP8, P =
+// 1024: 365 -> 328; bf16x3, M = 150,001, N = 17, trigonometric degree 5, P = 300:
+// 90 -> 72.
+constexpr int kBasisThreads = 256;        // warps 12..19
+constexpr int kThreads = kBasisWarp0 * 32 + kBasisThreads;
 constexpr int kMaxSmem = 232448;          // 227 KB opt-in per CTA
 constexpr int kMinSmem = 120 * 1024;
 
@@ -177,7 +180,9 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
       ptx::mbar_init(ptx::smem_addr(&a_empty[s]), 1);
     }
     for (int sl = 0; sl < NS; ++sl) {
-      ptx::mbar_init(ptx::smem_addr(&phi_full[sl]), kBasisThreads);
+      // (features from L2: a K-block is one warpgroup's)
+      ptx::mbar_init(ptx::smem_addr(&phi_full[sl]),
+                     F == kFormBF16 && !TRI && !a.xstage ? 128 : kBasisThreads);
       ptx::mbar_init(ptx::smem_addr(&phi_free[sl]), 1);
     }
     for (int b = 0; b < 2; ++b) {
@@ -211,6 +216,10 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
   const bool xblocks = BN % 128 == 0;
   const int XW = xblocks ? 128 : BN;    // patterns per feature row in xs
 
+  // 5 warpgroups x 96 registers a thread: 80 for the first, 104 for the two of the
+  // epilogue, 96 for the expansion's two (without: 399 us for 340 at M = 10^6,
+  // N = 32, degree 8, P = 1024, BF16, from spills)
+  if (warp < kEpiWarp0) ptx::regs_dec<80>();
   if (warp == 0) {
     // ---------------- A producer ----------------
     if (lane == 0) {
@@ -239,13 +248,12 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    // One K-block's MMAs take 512 tensor cycles and this warp's instructions
-    // between them share their scheduler with three busy warps, so they decide
-    // the tensor pipe's rate: the converged warp runs the loop (uniform
-    // registers, see elect_one), descriptors, barrier addresses, slots and
-    // phases advance by an add and a compare. (A lone thread with the slots by
-    // integer division: 434 us at M = 10^6, N = 32, degree 8, P = 1024, BF16;
-    // by compares 421; this 378 with the epilogue below.)
+    // One K-block's MMAs take 512 tensor cycles, and the latency of this warp's
+    // instructions between them is of that order, so it decides the tensor pipe's
+    // rate: one elected thread runs the loop (see elect_one); descriptors, barrier
+    // addresses, slots and phases advance by an add and a compare. M = 10^6, N =
+    // 32, degree 8, P = 1024, BF16, us: 434 by lane 0 and slots by division, 372
+    // the converged warp with an election per K-block, 354 this.
     {
       const uint32_t idesc =
           F == kFormFP8 ? ptx::idesc_e4m3_f32(128, BN) : ptx::idesc_bf16_f32(128, BN);
@@ -291,29 +299,29 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
           }
         }
       };
-      uint32_t alo = alo0, abar = a_full0, ph = 0;          // A stage, its barrier and phase
-      uint32_t tile_blo = blo0, tile_pbar = phi_full0, tile_par = 0;   // the tile's first slot
-      uint32_t acc_it = 0;
-      for (int it = 0; it < my_tiles && ok; ++it) {
-        uint32_t blo = tile_blo, pbar = tile_pbar, par = tile_par;
-        for (int c = 0; c < a.C && ok; ++c) {
-          const uint32_t buf = acc_it & 1;
-          ok = wait_bar_warp(acc_empty0 + 8 * buf, ((acc_it >> 1) & 1) ^ 1, abort_flag, a.status);
-          if (!ok) break;
-          ptx::tc_fence_after();
-          const uint32_t d_tmem = tmem + buf * (uint32_t)BN;
-          blo = tile_blo;
-          pbar = tile_pbar;
-          par = tile_par;
-          for (int kb = 0; kb < KB; ++kb) {
-            if (c == 0) {
-              ok = wait_bar_warp(pbar, par, abort_flag, a.status);
-              if (!ok) break;
-            }
-            ok = wait_bar_warp(abar, ph, abort_flag, a.status);
+      if (ptx::elect_one()) {
+        uint32_t alo = alo0, abar = a_full0, ph = 0;          // A stage, its barrier and phase
+        uint32_t tile_blo = blo0, tile_pbar = phi_full0, tile_par = 0;   // the tile's first slot
+        uint32_t acc_it = 0;
+        for (int it = 0; it < my_tiles && ok; ++it) {
+          uint32_t blo = tile_blo, pbar = tile_pbar, par = tile_par;
+          for (int c = 0; c < a.C && ok; ++c) {
+            const uint32_t buf = acc_it & 1;
+            ok = wait_bar(acc_empty0 + 8 * buf, ((acc_it >> 1) & 1) ^ 1, abort_flag, a.status);
             if (!ok) break;
-            const int nm = kb == KB - 1 ? nlast : 4;
-            if (ptx::elect_one()) {
+            ptx::tc_fence_after();
+            const uint32_t d_tmem = tmem + buf * (uint32_t)BN;
+            blo = tile_blo;
+            pbar = tile_pbar;
+            par = tile_par;
+            for (int kb = 0; kb < KB; ++kb) {
+              if (c == 0) {
+                ok = wait_bar(pbar, par, abort_flag, a.status);
+                if (!ok) break;
+              }
+              ok = wait_bar(abar, ph, abort_flag, a.status);
+              if (!ok) break;
+              const int nm = kb == KB - 1 ? nlast : 4;
               kstep(d_tmem, alo, blo, kb != 0);
               if (nm == 4) {
                 kstep(d_tmem, alo + 2u, blo + 2u, 1u);
@@ -326,31 +334,30 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
               ptx::mma_commit(abar + a_empty);
               if (c == a.C - 1) ptx::mma_commit(pbar + phi_free_off);
               if (kb == KB - 1) ptx::mma_commit(acc_full0 + 8 * buf);
+              alo += a_step;
+              abar += 8;
+              if (alo == alo_end) {
+                alo = alo0;
+                abar = a_full0;
+                ph ^= 1;
+              }
+              blo += b_step;
+              pbar += 8;
+              if (blo == blo_end) {
+                blo = blo0;
+                pbar = phi_full0;
+                par ^= 1u;
+              }
             }
-            __syncwarp();
-            alo += a_step;
-            abar += 8;
-            if (alo == alo_end) {
-              alo = alo0;
-              abar = a_full0;
-              ph ^= 1;
-            }
-            blo += b_step;
-            pbar += 8;
-            if (blo == blo_end) {
-              blo = blo0;
-              pbar = phi_full0;
-              par ^= 1u;
-            }
+            ++acc_it;
           }
-          ++acc_it;
+          tile_blo = blo;   // where the next tile's K-blocks begin
+          tile_pbar = pbar;
+          tile_par = par;
         }
-        tile_blo = blo;   // where the next tile's K-blocks begin
-        tile_pbar = pbar;
-        tile_par = par;
+        // every MMA issued above has completed once this arrives
+        ptx::mma_commit(ptx::smem_addr(drain));
       }
-      // every MMA issued above has completed once this arrives
-      if (ptx::elect_one()) ptx::mma_commit(ptx::smem_addr(drain));
       __syncwarp();
       wait_bar_drain(ptx::smem_addr(drain), 0, a.status);
     }
@@ -421,6 +428,7 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
   } else if (warp >= kEpiWarp0 && warp < kBasisWarp0) {
     // ---------------- epilogue ----------------
     const int qw = warp & 3;
+    ptx::regs_inc<104>();
     const int half = (warp - kEpiWarp0) >> 2;
     const int row = qw * 32 + lane;
     const int NH = BN >= 64 ? 2 : 1;          // column halves in use
@@ -428,15 +436,13 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
     const int col_lo = half * HW;
     const uint32_t lane_addr = (uint32_t)(qw * 32) << 16;
     double* part_row = a.part + (size_t)(2 * blockIdx.x + half) * a.Ppad;
-    // Per accumulator a warp has about as long as its MMAs (K' / 16 times 128
-    // cycles), and while it is late the MMAs wait: so the targets come from shared
-    // memory, and the chromosome's bias and running sum are loaded before the wait
-    // for the accumulator, not after its reduction. (M = 10^6, N = 32, degree 8,
-    // P = 1024: 398 -> 378 us together with the expansion's look-ahead.)
+    // (what bounds it: see epi_reduce's header)
     auto reduce_tiles = [&](auto ys_tag) {
       constexpr bool YS = decltype(ys_tag)::value;
       uint32_t acc_it = 0;
       bool ok = true;
+      LastSum last;
+      float bias_n = a.a0[row], negu_n = F == kFormFP8 ? -a.uscale[row] : -1.f;   // the next's
       for (int it = 0; it < my_tiles && ok; ++it) {
         const int64_t m0 = ((int64_t)blockIdx.x + (int64_t)it * G) * BN;
         const int64_t rem = a.M - m0 - col_lo;
@@ -448,59 +454,34 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
         const float* yt = YS ? ys + (it & 1) * BN + col_lo : a.y + m0 + col_lo;
         for (int c = 0; c < a.C; ++c) {
           const uint32_t buf = acc_it & 1, u = acc_it >> 1;
-          const int chrom = c * 128 + row;
-          const float bias = a.a0[chrom];
-          const float negu = F == kFormFP8 ? -a.uscale[chrom] : -1.f;
-          const double before = it == 0 ? 0.0 : part_row[chrom];
+          const int chrom = c * 128 + row, next = (c + 1 == a.C ? 0 : c + 1) * 128 + row;
+          const float bias = bias_n, negu = negu_n;
+          bias_n = a.a0[next];
+          if (F == kFormFP8) negu_n = -a.uscale[next];
+          last.begin();
+          float4 ya[4];
+          if (valid >= 32) epi_targets<YS>(yt, ya);
           ok = wait_bar(ptx::smem_addr(&acc_full[buf]), u & 1, abort_flag, a.status);
           if (!ok) break;
           ptx::tc_fence_after();
-          const uint64_t bias2 = ptx::f2_pack(bias, bias);
-          const uint64_t negu2 = ptx::f2_pack(negu, negu);
-          uint64_t s2 = 0;   // two FP32 partial sums (even / odd columns)
-          float s_tail = 0.f;
-          const uint32_t tbase = tmem + lane_addr + buf * (uint32_t)BN + (uint32_t)col_lo;
-          const int nfull = valid / 32;
-          if (nfull > 0) {
-            // double-buffered: the load of chunk k+1 is in flight while chunk k
-            // is reduced
-            uint32_t va[32], vb[32];
-            ptx::tmem_ld32_issue(tbase, va);
-            ptx::tmem_ld32_wait(va);
-            for (int k = 0; k < nfull; k += 2) {
-              const bool has_b = k + 1 < nfull;
-              if (has_b) ptx::tmem_ld32_issue(tbase + (uint32_t)(k + 1) * 32, vb);
-              epi_chunk<F == kFormFP8, ABS, YS>(va, yt + k * 32, bias2, negu2, s2);
-              if (has_b) {
-                ptx::tmem_ld32_wait(vb);
-                const bool has_a = k + 2 < nfull;
-                if (has_a) ptx::tmem_ld32_issue(tbase + (uint32_t)(k + 2) * 32, va);
-                epi_chunk<F == kFormFP8, ABS, YS>(vb, yt + (k + 1) * 32, bias2, negu2, s2);
-                if (has_a) ptx::tmem_ld32_wait(va);
-              }
-            }
-          }
-          if (nfull * 32 < valid) {   // ragged last chunk of the last tile
-            uint32_t v[32];
-            ptx::tmem_ld32(tbase + (uint32_t)nfull * 32, v);
-            const int lim = valid - nfull * 32;
-#pragma unroll
-            for (int e = 0; e < 32; ++e) {
-              if (e < lim) {
-                const float r = fmaf(negu, __uint_as_float(v[e]), yt[nfull * 32 + e] - bias);
-                s_tail = ABS ? s_tail + fabsf(r) : fmaf(r, r, s_tail);
-              }
-            }
-          }
+          float2 sum;
+          float tail;
+          epi_reduce<F == kFormFP8, ABS, YS>(
+              tmem + lane_addr + buf * (uint32_t)BN + (uint32_t)col_lo, yt, valid, ya, bias, negu,
+              last, sum, tail);
           ptx::tc_fence_before();
           ptx::mbar_arrive(ptx::smem_addr(&acc_empty[buf]));
-          const float2 sp2 = ptx::f2_unpack(s2);
-          double tile_sse = (double)sp2.x + (double)sp2.y;
-          if (s_tail != 0.f) tile_sse += (double)s_tail;   // (FP64 operations are scarce)
-          part_row[chrom] = it == 0 ? tile_sse : before + tile_sse;
+          last.sum = sum;
+          last.tail = tail;
+          last.row = part_row + chrom;
+          last.first = it == 0;
           ++acc_it;
         }
         if (YS && ok) ptx::mbar_arrive(ptx::smem_addr(&y_empty[it & 1]));
+      }
+      if (ok) {
+        last.begin();
+        last.end();
       }
     };
     if (a.ystage) reduce_tiles(std::true_type{});
@@ -550,7 +531,7 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
     // pass, R = 3, two unit groups; BN < 128: BN rows, R = 1, 128 / BN groups
     const int RW = TRI ? 64 : (BN < 128 ? BN : 128);
     const int R = TRI ? 3 : BN / RW;
-    const int QS = 128 / RW;
+    const int QS = kBasisThreads / RW;
     const int r0 = bt % RW, q0 = bt / RW;
     auto xrow_of = [&](int r) -> const float* {
       return xblocks ? xs + (r >> 7) * N * 128 + (r & 127) : xs + r;
@@ -804,12 +785,20 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
         ptx::bulk_prefetch_l2(a.Xt + (m1 / kPatBlock) * N * kPatBlock,
                               (uint32_t)((BN / kPatBlock) * N * kPatBlock * 4));
       };
-      // Two K-blocks' features are in registers ahead of use: as the last
-      // chromosome tile's MMAs release the slots, a K-block is due every 512
-      // cycles, less than a load takes from L2.
-      int lit = 0, lkb = 0;   // place of the next K-block to load
+      // The two warpgroups take the K-blocks in turn. (Not with one slot: a
+      // group would await the second release ahead, which a parity cannot tell.)
+      const int ngr = NS > 1 ? 2 : 1, grp = bt >> 7;
+      const int run_tiles = grp < ngr ? my_tiles : 0;
+      int lit = grp / KB, lkb = grp % KB;   // place of the next K-block to load
+      auto advance = [&](int& t, int& b) {
+        b += ngr;
+        while (b >= KB) {
+          b -= KB;
+          ++t;
+        }
+      };
       auto load_next = [&](float (&va)[8], float (&vb)[8]) {
-        if (lit >= my_tiles) return;
+        if (lit >= run_tiles) return;
         const float* p0 = xptr(lit, r0);
         const float* p1 = xptr(lit, r1);
 #pragma unroll
@@ -818,20 +807,20 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
           va[q] = __ldg(p0 + i * kPatBlock);
           vb[q] = R == 2 ? __ldg(p1 + i * kPatBlock) : 0.f;
         }
-        if (++lkb == KB) {
-          lkb = 0;
-          ++lit;
-        }
+        advance(lit, lkb);
       };
       if (bt == 0) {
         if (my_tiles > 0) prefetch_tile(0);
         if (my_tiles > 1) prefetch_tile(1);
       }
-      int it = 0, kb = 0;           // the K-block to write
-      int slot = 0, uses = 0;       // its slot, the slot's completed uses
+      int it = grp / KB, kb = grp % KB;        // the K-block to write
+      int slot = grp % NS, uses = grp / NS;    // its slot, the slot's completed uses
+      int fetched = 0;                         // tiles whose successor but one is prefetched
       // writes a K-block from its features, then loads the one after the next
       auto step = [&](float (&xa)[8], float (&xb)[8]) {
-        if (kb == 0 && bt == 0 && it + 2 < my_tiles) prefetch_tile(it + 2);
+        if (bt == 0)
+          for (; fetched <= it; ++fetched)
+            if (fetched + 2 < my_tiles) prefetch_tile(fetched + 2);
         if (uses > 0)
           ok = wait_bar(ptx::smem_addr(&phi_free[slot]), (uint32_t)(uses - 1) & 1u, abort_flag,
                         a.status);
@@ -857,22 +846,16 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
         ptx::fence_proxy_async_smem();
         ptx::mbar_arrive(ptx::smem_addr(&phi_full[slot]));
         load_next(xa, xb);
-        if (++slot == NS) {
-          slot = 0;
+        slot += ngr;
+        if (slot >= NS) {
+          slot -= NS;
           ++uses;
         }
-        if (++kb == KB) {
-          kb = 0;
-          ++it;
-        }
+        advance(it, kb);
       };
-      float xa0[8], xb0[8], xa1[8], xb1[8];
+      float xa0[8], xb0[8];
       load_next(xa0, xb0);
-      load_next(xa1, xb1);
-      while (it < my_tiles && ok) {
-        step(xa0, xb0);
-        if (it < my_tiles && ok) step(xa1, xb1);
-      }
+      while (it < run_tiles && ok) step(xa0, xb0);
     }
     for (int it = 0; it < my_tiles && ok && staged && !stream; ++it) {
       ok = wait_bar(ptx::smem_addr(x_full), it & 1, abort_flag, a.status);

@@ -27,8 +27,9 @@
 //                (warps 4-7 the first 128 pattern columns, 8-11 the second),
 //                r = (y_m - a_0) - D, sse += r^2 in packed FP32 pairs, FP64
 //                partials per (cluster, column half).
-//   warps 12-15  expansion: thread = one of this CTA's 128 patterns; per 8-column
-//                chunk the basis recurrence in registers, BF16, stored in the
+//   warps 12-19  expansion of this CTA's 128 patterns (degrees 1..10 whole
+//                features at a time, expand_stream.cuh; beyond, per 8-column
+//                chunk): the basis recurrence in registers, BF16, stored in the
 //                K-major SWIZZLE_128B layout, into a ring of K-block slots.
 // Barriers: the MMA issuer waits on the even CTA's barriers only; the odd
 // CTA's producers reach them by cluster-scope arrivals (one per warp for the
@@ -53,16 +54,18 @@ namespace {
 using namespace tc;
 
 constexpr uint32_t kABytes = 128 * 128;   // one CTA's gene block: 128 chromosomes x 64 genes
-constexpr int kWarps = 16;
-constexpr int kThreads = kWarps * 32;
 constexpr int kEpiWarp0 = 4;
 constexpr int kBasisWarp0 = 12;
-constexpr int kBasisThreads = 128;
+// (eight expansion warps, one elected issuing thread, epilogue one step ahead: M =
+// 4 10^6, N = 48, degree 6, P = 2048: 3.02 -> 2.69 ms; M = 94,601, N = 26,
+// trigonometric degree 11, P = 1092, the chunk generator: 360 -> 232 us)
+constexpr int kBasisThreads = 256;        // warps 12..19
+constexpr int kThreads = kBasisWarp0 * 32 + kBasisThreads;
 constexpr int kRows = 128;                // patterns of a tile held by one CTA
 constexpr int kBN = 2 * kRows;            // patterns per tile (MMA N)
 constexpr int kMaxSmem = 232448;          // 227 KB opt-in per CTA
 constexpr int kMinSmem = 120 * 1024;      // one CTA per SM
-constexpr uint32_t kPhiArrivals = 8;      // expansion warps of both CTAs
+constexpr uint32_t kPhiArrivals = 16;     // expansion warps of both CTAs
 constexpr uint32_t kAccArrivals = 16;     // epilogue warps of both CTAs
 
 struct Tc2Args {
@@ -203,7 +206,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       ptx::mbar_init(ptx::smem_addr(&a_empty[s]), 1);
     }
     for (int sl = 0; sl < NS; ++sl) {
-      ptx::mbar_init(ptx::smem_addr(&phi_full[sl]), kPhiArrivals);
+      // (features from L2: a K-block is one warpgroup's in each CTA)
+      ptx::mbar_init(ptx::smem_addr(&phi_full[sl]), a.xstage ? kPhiArrivals : kPhiArrivals / 2);
       ptx::mbar_init(ptx::smem_addr(&phi_free[sl]), 1);
     }
     for (int b = 0; b < 2; ++b) {
@@ -254,6 +258,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     }
   };
 
+  // (registers: see fitness_tc.cu)
+  if (warp < kEpiWarp0) ptx::regs_dec<80>();
   if (warp == 0) {
     // ---------------- gene producer (both CTAs) ----------------
     if (lane == 0) {
@@ -282,7 +288,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer (even CTA) ----------------
-    // (the converged warp with running descriptors: see fitness_tc.cu)
+    // (one elected thread, running descriptors: see fitness_tc.cu)
     if (lead) {
       const uint32_t idesc = ptx::idesc_bf16_f32(2 * kRows, kBN);
       const uint64_t adesc0 = ptx::desc_kmajor_sw128(ptx::smem_addr(ast));
@@ -316,29 +322,29 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         ptx::mma_bf16_pair(d_tmem, ((uint64_t)dhi << 32) | al, ((uint64_t)dhi << 32) | bl,
                              idesc, acc);
       };
-      uint32_t alo = alo0, abar = a_full0, ph = 0;
-      uint32_t tile_blo = blo0, tile_pbar = phi_full0, tile_par = 0;
-      uint32_t acc_it = 0;
-      for (int it = 0; it < my_tiles && ok; ++it) {
-        uint32_t blo = tile_blo, pbar = tile_pbar, par = tile_par;
-        for (int c = 0; c < Cp && ok; ++c) {
-          const uint32_t buf = acc_it & 1;
-          ok = wait_bar_warp(acc_empty0 + 8 * buf, ((acc_it >> 1) & 1) ^ 1, abort_flag, a.status);
-          if (!ok) break;
-          ptx::tc_fence_after();
-          const uint32_t d_tmem = tmem + buf * (uint32_t)kBN;
-          blo = tile_blo;
-          pbar = tile_pbar;
-          par = tile_par;
-          for (int kb = 0; kb < KB; ++kb) {
-            if (c == 0) {
-              ok = wait_bar_warp(pbar, par, abort_flag, a.status);
-              if (!ok) break;
-            }
-            ok = wait_bar_warp(abar, ph, abort_flag, a.status);
+      if (ptx::elect_one()) {
+        uint32_t alo = alo0, abar = a_full0, ph = 0;
+        uint32_t tile_blo = blo0, tile_pbar = phi_full0, tile_par = 0;
+        uint32_t acc_it = 0;
+        for (int it = 0; it < my_tiles && ok; ++it) {
+          uint32_t blo = tile_blo, pbar = tile_pbar, par = tile_par;
+          for (int c = 0; c < Cp && ok; ++c) {
+            const uint32_t buf = acc_it & 1;
+            ok = wait_bar(acc_empty0 + 8 * buf, ((acc_it >> 1) & 1) ^ 1, abort_flag, a.status);
             if (!ok) break;
-            const int nm = kb == KB - 1 ? nlast : 4;
-            if (ptx::elect_one()) {
+            ptx::tc_fence_after();
+            const uint32_t d_tmem = tmem + buf * (uint32_t)kBN;
+            blo = tile_blo;
+            pbar = tile_pbar;
+            par = tile_par;
+            for (int kb = 0; kb < KB; ++kb) {
+              if (c == 0) {
+                ok = wait_bar(pbar, par, abort_flag, a.status);
+                if (!ok) break;
+              }
+              ok = wait_bar(abar, ph, abort_flag, a.status);
+              if (!ok) break;
+              const int nm = kb == KB - 1 ? nlast : 4;
               kstep(d_tmem, alo, blo, kb != 0);
               if (nm == 4) {
                 kstep(d_tmem, alo + 2u, blo + 2u, 1u);
@@ -351,31 +357,30 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
               ptx::mma_commit_pair_mc(abar + a_empty_off, both);
               if (c == Cp - 1) ptx::mma_commit_pair_mc(pbar + phi_free_off, both);
               if (kb == KB - 1) ptx::mma_commit_pair_mc(acc_full0 + 8 * buf, both);
+              alo += a_step;
+              abar += 8;
+              if (alo == alo_end) {
+                alo = alo0;
+                abar = a_full0;
+                ph ^= 1;
+              }
+              blo += b_step;
+              pbar += 8;
+              if (blo == blo_end) {
+                blo = blo0;
+                pbar = phi_full0;
+                par ^= 1u;
+              }
             }
-            __syncwarp();
-            alo += a_step;
-            abar += 8;
-            if (alo == alo_end) {
-              alo = alo0;
-              abar = a_full0;
-              ph ^= 1;
-            }
-            blo += b_step;
-            pbar += 8;
-            if (blo == blo_end) {
-              blo = blo0;
-              pbar = phi_full0;
-              par ^= 1u;
-            }
+            ++acc_it;
           }
-          ++acc_it;
+          tile_blo = blo;
+          tile_pbar = pbar;
+          tile_par = par;
         }
-        tile_blo = blo;
-        tile_pbar = pbar;
-        tile_par = par;
+        // every MMA issued above has completed once this arrives
+        ptx::mma_commit_pair(ptx::smem_addr(drain));
       }
-      // every MMA issued above has completed once this arrives
-      if (ptx::elect_one()) ptx::mma_commit_pair(ptx::smem_addr(drain));
       __syncwarp();
       wait_bar_drain(ptx::smem_addr(drain), 0, a.status);
     } else if (lane == 0 && a.ycopy) {
@@ -419,18 +424,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   } else if (warp >= kEpiWarp0 && warp < kBasisWarp0) {
     // ---------------- epilogue (both CTAs) ----------------
     const int qw = warp & 3;
+    ptx::regs_inc<104>();
     const int half = (warp - kEpiWarp0) >> 2;
     const int row = qw * 32 + lane;
     const int col_lo = half * kRows;
     const uint32_t lane_addr = (uint32_t)(qw * 32) << 16;
     double* part_row = a.part + (size_t)(2 * cl + half) * a.Ppad;
     const uint32_t acc_empty_lead0 = ptx::mapa(ptx::smem_addr(acc_empty), 0);
-    // (targets from shared memory, bias and running sum loaded before the wait:
-    // see fitness_tc.cu; M = 4 10^6, N = 48, degree 6, P = 2048: 3.17 -> 3.02 ms)
+    // (what bounds it: see epi_reduce's header)
     auto reduce_tiles = [&](auto ys_tag) {
       constexpr bool YS = decltype(ys_tag)::value;
       uint32_t acc_it = 0;
       bool ok = true;
+      LastSum last;
+      float bias_n = a.a0[(int)rank * kRows + row];   // the next accumulator's
       for (int it = 0; it < my_tiles && ok; ++it) {
         const int64_t m0 = ((int64_t)cl + (int64_t)it * ncl) * kBN;
         const int64_t rem = a.M - m0 - col_lo;
@@ -444,54 +451,26 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         for (int c = 0; c < Cp; ++c) {
           const uint32_t buf = acc_it & 1, u = acc_it >> 1;
           const int chrom = c * 2 * kRows + (int)rank * kRows + row;
-          const float bias = a.a0[chrom];
-          const double before = it == 0 ? 0.0 : part_row[chrom];
+          const float bias = bias_n;
+          bias_n = a.a0[(c + 1 == Cp ? 0 : c + 1) * 2 * kRows + (int)rank * kRows + row];
+          last.begin();
+          float4 ya[4];
+          if (valid >= 32) epi_targets<YS>(yt, ya);
           ok = wait_bar(ptx::smem_addr(&acc_full[buf]), u & 1, abort_flag, a.status);
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
           ptx::tc_fence_after();
-          const uint64_t bias2 = ptx::f2_pack(bias, bias);
-          const uint64_t negu2 = ptx::f2_pack(-1.f, -1.f);
-          uint64_t s2 = 0;
-          float s_tail = 0.f;
-          const uint32_t tbase = tmem + lane_addr + buf * (uint32_t)kBN + (uint32_t)col_lo;
-          const int nfull = valid / 32;
-          if (nfull > 0) {
-            uint32_t va[32], vb[32];
-            ptx::tmem_ld32_issue(tbase, va);
-            ptx::tmem_ld32_wait(va);
-            for (int k = 0; k < nfull; k += 2) {
-              const bool has_b = k + 1 < nfull;
-              if (has_b) ptx::tmem_ld32_issue(tbase + (uint32_t)(k + 1) * 32, vb);
-              epi_chunk<false, ABS, YS>(va, yt + k * 32, bias2, negu2, s2);
-              if (has_b) {
-                ptx::tmem_ld32_wait(vb);
-                const bool has_a = k + 2 < nfull;
-                if (has_a) ptx::tmem_ld32_issue(tbase + (uint32_t)(k + 2) * 32, va);
-                epi_chunk<false, ABS, YS>(vb, yt + (k + 1) * 32, bias2, negu2, s2);
-                if (has_a) ptx::tmem_ld32_wait(va);
-              }
-            }
-          }
-          if (nfull * 32 < valid) {   // ragged last chunk of the last tile
-            uint32_t v[32];
-            ptx::tmem_ld32(tbase + (uint32_t)nfull * 32, v);
-            const int lim = valid - nfull * 32;
-#pragma unroll
-            for (int e = 0; e < 32; ++e) {
-              if (e < lim) {
-                const float r = (yt[nfull * 32 + e] - bias) - __uint_as_float(v[e]);
-                s_tail = ABS ? s_tail + fabsf(r) : fmaf(r, r, s_tail);
-              }
-            }
-          }
+          float2 sum;
+          float tail;
+          epi_reduce<false, ABS, YS>(tmem + lane_addr + buf * (uint32_t)kBN + (uint32_t)col_lo, yt,
+                                     valid, ya, bias, -1.f, last, sum, tail);
           ptx::tc_fence_before();
           __syncwarp();
           if (lane == 0) ptx::mbar_arrive_cluster(acc_empty_lead0 + 8 * buf);
-          const float2 sp2 = ptx::f2_unpack(s2);
-          double tile_sse = (double)sp2.x + (double)sp2.y;
-          if (s_tail != 0.f) tile_sse += (double)s_tail;   // (FP64 operations are scarce)
-          part_row[chrom] = it == 0 ? tile_sse : before + tile_sse;
+          last.sum = sum;
+          last.tail = tail;
+          last.row = part_row + chrom;
+          last.first = it == 0;
           ++acc_it;
         }
         if (YS && ok) {
@@ -499,13 +478,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&y_empty[it & 1]));
         }
       }
+      if (ok) {
+        last.begin();
+        last.end();
+      }
     };
     if (a.ycopy) reduce_tiles(std::true_type{});
     else reduce_tiles(std::false_type{});
   } else {
     // ---------------- expansion (both CTAs) ----------------
-    const int r0 = threadIdx.x - kBasisWarp0 * 32;   // this thread's pattern row
-    for (int cid = r0; cid < KB * 8; cid += kBasisThreads)
+    const int bt = threadIdx.x - kBasisWarp0 * 32;
+    const int r0 = bt & (kRows - 1), grp = bt >> 7;   // this thread's pattern row, warpgroup
+    for (int cid = bt; cid < KB * 8; cid += kBasisThreads)
       tab[cid] = chunk_desc(cid, a.basis, a.d, a.Kp);
     ptx::named_bar(1, kBasisThreads);
     const uint32_t phi_full_lead0 = ptx::mapa(ptx::smem_addr(phi_full), 0);
@@ -530,8 +514,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       sa.NS = NS;
       sa.RW = kRows / 2;
       sa.R = 2;
-      sa.QS = 2;
-      sa.bt = r0;
+      sa.QS = 2 * kBasisThreads / kRows;
+      sa.bt = bt;
       sa.my_tiles = my_tiles;
       sa.abort_flag = abort_flag;
       sa.status = a.status;
@@ -560,48 +544,52 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         const int64_t blk = ((int64_t)cl + (int64_t)itn * ncl) * 2 + rank;
         ptx::bulk_prefetch_l2(a.Xt + blk * N * kPatBlock, (uint32_t)(N * kPatBlock * 4));
       };
+      // The two warpgroups take the K-blocks in turn. (Not with one slot: a
+      // group would await the second release ahead, which a parity cannot tell.)
+      const int ngr = NS > 1 ? 2 : 1;
+      const int nq = grp < ngr ? my_tiles * KB : 0;
       float nx[8];
       auto load_kb = [&](int itn, int kbn) {
         const float* p = xptr(itn);
 #pragma unroll
         for (int q = 0; q < 8; ++q) nx[q] = __ldg(p + (int)(tab[kbn * 8 + q] & 0xFFFFu) * kPatBlock);
       };
-      if (r0 == 0) {
+      if (bt == 0) {
         if (my_tiles > 0) prefetch_tile(0);
         if (my_tiles > 1) prefetch_tile(1);
       }
-      if (my_tiles > 0) load_kb(0, 0);
-      for (int it = 0; it < my_tiles && ok; ++it) {
-        if (r0 == 0 && it + 2 < my_tiles) prefetch_tile(it + 2);
-        for (int kb = 0; kb < KB; ++kb) {
-          float x[8];
+      if (grp < nq) load_kb(grp / KB, grp % KB);
+      int fetched = 0;   // tiles whose successor but one is prefetched
+      for (int q = grp; q < nq; q += ngr) {
+        const int it = q / KB, kb = q - it * KB;
+        if (bt == 0)
+          for (; fetched <= it; ++fetched)
+            if (fetched + 2 < my_tiles) prefetch_tile(fetched + 2);
+        float x[8];
 #pragma unroll
-          for (int q = 0; q < 8; ++q) x[q] = nx[q];
-          if (kb + 1 < KB) load_kb(it, kb + 1);
-          else if (it + 1 < my_tiles) load_kb(it + 1, 0);
-          const int q = it * KB + kb;
-          ok = slot_free(q);
-          if (!ok) break;
-          uint8_t* phik = phi + (size_t)(q % NS) * kRows * 128;
+        for (int e = 0; e < 8; ++e) x[e] = nx[e];
+        if (q + ngr < nq) load_kb((q + ngr) / KB, (q + ngr) % KB);
+        ok = slot_free(q);
+        if (!ok) break;
+        uint8_t* phik = phi + (size_t)(q % NS) * kRows * 128;
 #pragma unroll
-          for (int qd = 0; qd < 8; qd += 2) {
-            const uint32_t da = tab[kb * 8 + qd], db = tab[kb * 8 + qd + 1];
-            float va[8], vb[8];
-            cheb_run_pair(x[qd], (int)((da >> 16) & 31u), x[qd + 1], (int)((db >> 16) & 31u),
-                          va, vb);
-            if (da & kChunkZero) {
+        for (int qd = 0; qd < 8; qd += 2) {
+          const uint32_t da = tab[kb * 8 + qd], db = tab[kb * 8 + qd + 1];
+          float va[8], vb[8];
+          cheb_run_pair(x[qd], (int)((da >> 16) & 31u), x[qd + 1], (int)((db >> 16) & 31u),
+                        va, vb);
+          if (da & kChunkZero) {
 #pragma unroll
-              for (int e = 0; e < 8; ++e) va[e] = 0.f;
-            }
-            if (db & kChunkZero) {
-#pragma unroll
-              for (int e = 0; e < 8; ++e) vb[e] = 0.f;
-            }
-            store_bf16x8(phik, r0, qd, va);
-            store_bf16x8(phik, r0, qd + 1, vb);
+            for (int e = 0; e < 8; ++e) va[e] = 0.f;
           }
-          publish(q);
+          if (db & kChunkZero) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) vb[e] = 0.f;
+          }
+          store_bf16x8(phik, r0, qd, va);
+          store_bf16x8(phik, r0, qd + 1, vb);
         }
+        publish(q);
       }
     } else if (!stream) {
       const float* xrow = xs + r0;   // block layout [N][128]
@@ -614,7 +602,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           if (!ok) break;
           uint8_t* phik = phi + (size_t)(q % NS) * kRows * 128;
 #pragma unroll 1
-          for (int qd = 0; qd < 8; qd += 2) {
+          for (int qd = 4 * grp; qd < 4 * grp + 4; qd += 2) {
             float va[8], vb[8];
             gen8(tab[kb * 8 + qd], a.basis, a.d, N, xrow, kRows, va);
             gen8(tab[kb * 8 + qd + 1], a.basis, a.d, N, xrow, kRows, vb);

@@ -187,6 +187,24 @@ __device__ __forceinline__ void tmem_ld32_wait(uint32_t (&v)[32]) {
                : "memory");
 }
 
+__device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t (&v)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
+        "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]),
+        "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+      : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld16_wait(uint32_t (&v)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]),
+                 "+r"(v[6]), "+r"(v[7]), "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]),
+                 "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15])
+               :
+               : "memory");
+}
+
 // ---- MMA ----
 // Shared-memory matrix descriptor, K-major operand in the 128-byte swizzle:
 // rows of 128 bytes, 8-row groups 1024 bytes apart (stride byte offset),
@@ -253,15 +271,24 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
                : "memory");
 }
 
-// ---- MMA issue by a converged warp ----
-// The whole warp runs the issuing loop and waits; one K-block's MMAs and
-// commits stand in a block `if (elect_one())`. The compiler knows such a block
-// is run by one thread of a converged warp, so every address and descriptor
-// stays in uniform registers; in a branch on the lane number they are moved
-// there one by one for each MMA. The same lane is elected each time, so the
-// commits follow the MMAs of their thread. Measured with every other role of
-// the kernel running: 159 against 194 cycles per 128 x 256 x 16 MMA (128 is
-// the tensor pipe's own rate).
+// ---- registers of a warpgroup (all its warps; the launch's total is fixed) ----
+template <int N>
+__device__ __forceinline__ void regs_inc() {
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
+}
+template <int N>
+__device__ __forceinline__ void regs_dec() {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
+}
+
+// ---- MMA issue by an elected thread ----
+// The issuing loop, waits included, stands in a block `if (elect_one())`. The
+// compiler knows that such a block is run by one thread, so addresses and
+// descriptors stay in uniform registers; in a branch on the lane number they
+// are moved there one by one for each MMA. What decides the rate is the
+// latency of this one warp's instructions: per K-block of four MMAs (512 tensor
+// cycles) the warp needed 720 cycles with a converged loop and an election per
+// K-block.
 __device__ __forceinline__ uint32_t elect_one() {
   uint32_t lead;
   asm volatile(
