@@ -173,25 +173,6 @@ struct RowCursor {
   }
 };
 
-// sse += ((y - bias) - acc)^2 over 32 columns with the targets in shared
-// memory (the arithmetic of epi_chunk<false>: one packed subtraction and one
-// packed FMA per two columns)
-__device__ __forceinline__ void epi_chunk_smem(const uint32_t (&v)[32], const float* yc,
-                                               uint64_t bias2, uint64_t& s2) {
-#pragma unroll
-  for (int e4 = 0; e4 < 8; ++e4) {
-    const float4 yv = reinterpret_cast<const float4*>(yc)[e4];
-    const uint64_t ya = ptx::f2_sub(ptx::f2_pack(yv.x, yv.y), bias2);
-    const uint64_t yb = ptx::f2_sub(ptx::f2_pack(yv.z, yv.w), bias2);
-    const uint64_t da = ptx::f2_pack(__uint_as_float(v[4 * e4 + 0]), __uint_as_float(v[4 * e4 + 1]));
-    const uint64_t db = ptx::f2_pack(__uint_as_float(v[4 * e4 + 2]), __uint_as_float(v[4 * e4 + 3]));
-    const uint64_t ra = ptx::f2_sub(ya, da);
-    const uint64_t rb = ptx::f2_sub(yb, db);
-    s2 = ptx::f2_fma(ra, ra, s2);
-    s2 = ptx::f2_fma(rb, rb, s2);
-  }
-}
-
 __device__ __forceinline__ uint4 pack8(const float* v) {
   return make_uint4(bf16x2_bits(v[0], v[1]), bf16x2_bits(v[2], v[3]), bf16x2_bits(v[4], v[5]),
                     bf16x2_bits(v[6], v[7]));
@@ -455,7 +436,7 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_batch_kernel(const BatchA
     // ---------------- MMA issuer ----------------
     // One elected thread (elect_one), descriptors and barrier addresses advance by
     // an add and a compare. (Lane 0: 1.235 ms for the four launches of 24 uneven
-    // runs, this 1.10.)
+    // runs, this 1.10, 1.05 with the epilogue one step ahead.)
     {
       const uint64_t adesc0 = ptx::desc_kmajor_sw128(ptx::smem_addr(ast));
       const uint64_t bdesc0 = ptx::desc_kmajor_sw128(ptx::smem_addr(phi));
@@ -583,6 +564,10 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_batch_kernel(const BatchA
     ptx::named_bar(1, kEpiThreads);
     uint32_t acc_it = 0;
     bool ok = true;
+    // (one step ahead of use: see epi_reduce's header)
+    LastSum last;
+    last.first = true;   // each sum has its own place
+    float bias_n = idx >= 0 ? nxt.a0[row] : 0.f;
     for (int k = 0; idx >= 0; ++k) {
       const BatchItem R = nxt;
       const int idx_n = ebc[(k + 1) & 1];
@@ -598,57 +583,31 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_batch_kernel(const BatchA
       for (int c = 0; c < R.C && ok; ++c) {
         const int cg = c % R.CG;   // place in the accumulator set
         const int chrom = c * 128 + row;
-        const float bias = R.a0[chrom];   // loaded before the wait
+        const float bias = bias_n;
+        if (c + 1 < R.C) bias_n = R.a0[chrom + 128];
+        else if (idx_n >= 0) bias_n = nxt.a0[row];
+        last.begin();
+        float4 ya[4];
+        if (valid >= 32) epi_targets<true>(yt, ya);
         if (cg == 0) {
           set = acc_it & 1;
           ok = wait_bar(ptx::smem_addr(&acc_full[set]), (acc_it >> 1) & 1, abort_flag, a.status);
           if (!ok) break;
           ptx::tc_fence_after();
         }
-        const uint64_t bias2 = ptx::f2_pack(bias, bias);
-        uint64_t s2 = 0;
-        float s_tail = 0.f;
-        const uint32_t tbase =
-            tmem + lane_addr + set * (uint32_t)a.set_cols + (uint32_t)(cg * R.BN);
-        const int nfull = valid / 32;
-        if (nfull > 0) {
-          uint32_t va[32], vb[32];
-          ptx::tmem_ld32_issue(tbase, va);
-          ptx::tmem_ld32_wait(va);
-          for (int k = 0; k < nfull; k += 2) {
-            const bool has_b = k + 1 < nfull;
-            if (has_b) ptx::tmem_ld32_issue(tbase + (uint32_t)(k + 1) * 32, vb);
-            epi_chunk_smem(va, yt + k * 32, bias2, s2);
-            if (has_b) {
-              ptx::tmem_ld32_wait(vb);
-              const bool has_a = k + 2 < nfull;
-              if (has_a) ptx::tmem_ld32_issue(tbase + (uint32_t)(k + 2) * 32, va);
-              epi_chunk_smem(vb, yt + (k + 1) * 32, bias2, s2);
-              if (has_a) ptx::tmem_ld32_wait(va);
-            }
-          }
-        }
-        if (nfull * 32 < valid) {
-          uint32_t v[32];
-          ptx::tmem_ld32(tbase + (uint32_t)nfull * 32, v);
-          const int lim = valid - nfull * 32;
-#pragma unroll
-          for (int e = 0; e < 32; ++e) {
-            if (e < lim) {
-              const float r = (yt[nfull * 32 + e] - bias) - __uint_as_float(v[e]);
-              s_tail = fmaf(r, r, s_tail);
-            }
-          }
-        }
+        float2 sum;
+        float tail;
+        epi_reduce<false, false, true>(
+            tmem + lane_addr + set * (uint32_t)a.set_cols + (uint32_t)(cg * R.BN), yt, valid, ya,
+            bias, -1.f, last, sum, tail);
         if (cg == R.CG - 1 || c == R.C - 1) {   // the set's last tile: release it
           ptx::tc_fence_before();
           ptx::mbar_arrive(ptx::smem_addr(&acc_empty[set]));
           ++acc_it;
         }
-        const float2 sp2 = ptx::f2_unpack(s2);
-        double tile_sse = (double)sp2.x + (double)sp2.y;
-        if (s_tail != 0.f) tile_sse += (double)s_tail;   // (FP64 operations are scarce)
-        prow[chrom] = tile_sse;
+        last.sum = sum;
+        last.tail = tail;
+        last.row = prow + chrom;
       }
       float* ynext = ys + ((k + 1) & 1) * kYSlot;
       ynext[row] = yn0;
@@ -656,6 +615,10 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_batch_kernel(const BatchA
       if (row == 0) ebc[k & 1] = idx_n >= 0 ? iq.pop() : -1;   // item k + 2
       ptx::named_bar(1, kEpiThreads);
       idx = idx_n;
+    }
+    if (ok) {
+      last.begin();
+      last.end();
     }
   } else if (warp >= kBasisWarp0) {
     // ---------------- expansion (basis) ----------------

@@ -110,7 +110,7 @@ struct LastSum {
   }
 };
 
-// The sums of `valid` columns (<= 128, a multiple of 32 but in the last tile)
+// The sums of `valid` columns (a multiple of 32 but in the last tile)
 // of this thread's row at tensor-memory address tbase. ya: the first 16
 // columns' targets (epi_targets), where valid >= 32. 16 columns at a time, the
 // next load in flight (by 32 the registers spill).
