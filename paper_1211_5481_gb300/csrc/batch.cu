@@ -58,6 +58,7 @@ __global__ void init_batch_kernel(const BatchGaRun* __restrict__ g) {
 // Genes 1..K-1 of pop[src] to the BF16 operand image (as pack_bf16 in layout.cu).
 __global__ void pack_batch_kernel(const BatchRun* __restrict__ runs,
                                   const BatchGaRun* __restrict__ g, int src) {
+  wait_previous();
   const BatchRun& R = runs[blockIdx.y];
   const float* pop = g[blockIdx.y].pop[src];
   const int K = R.K, P = R.P, KB = R.KB;
@@ -90,12 +91,14 @@ __global__ void pack_batch_kernel(const BatchRun* __restrict__ runs,
 
 __global__ void __launch_bounds__(ga::kPlanThreads)
 plan_batch_kernel(const BatchGaRun* __restrict__ g, const uint32_t* __restrict__ gens) {
+  wait_previous();
   const BatchGaRun& R = g[blockIdx.x];
   ga::plan_body(R.ga, R.fit, R.seed, gens[blockIdx.x], R.plan);
 }
 
 __global__ void breed_batch_kernel(const BatchGaRun* __restrict__ g,
                                    const uint32_t* __restrict__ gens, int src) {
+  wait_previous();
   const BatchGaRun& R = g[blockIdx.y];
   const uint32_t gen = gens[blockIdx.y];
   const float* pop = R.pop[src];
@@ -115,6 +118,7 @@ __global__ void reduce_batch_kernel(const BatchRun* __restrict__ runs,
                                     const int* __restrict__ chrom_begin, int R, int total,
                                     const double* __restrict__ part, uint32_t* __restrict__ gens,
                                     int inc) {
+  wait_previous();
   const int w = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
   if (w >= total) return;
@@ -407,29 +411,25 @@ int enqueue_pack(game_batch* b, int src) {
     maxg = std::max(maxg, b->P[r] * b->shape[r].K);
   }
   (void)maxg;
-  pack_batch_kernel<<<dim3(blocks_for(maxu, 256, 4096), b->R), 256, 0, b->st>>>(b->runs_d,
-                                                                                b->ga_d, src);
-  BCK(cudaGetLastError());
+  BCK(launch_behind(pack_batch_kernel, dim3(blocks_for(maxu, 256, 4096), b->R), 256, 0, b->st,
+                    b->runs_d, b->ga_d, src));
   return GAME_OK;
 }
 
 int enqueue_reduce(game_batch* b, int inc) {
   const int threads = 256;
   const int blocks = (int)(((int64_t)b->total_chrom * 32 + threads - 1) / threads);
-  reduce_batch_kernel<<<blocks, threads, 0, b->st>>>(b->runs_d, b->ga_d, b->chrom_begin, b->R,
-                                                     b->total_chrom, b->part, b->gens, inc);
-  BCK(cudaGetLastError());
+  BCK(launch_behind(reduce_batch_kernel, blocks, threads, 0, b->st, b->runs_d, b->ga_d,
+                    b->chrom_begin, b->R, b->total_chrom, b->part, b->gens, inc));
   return GAME_OK;
 }
 
 int enqueue_operators(game_batch* b, int src) {
   int maxg = 1;
   for (int r = 0; r < b->R; ++r) maxg = std::max(maxg, b->P[r] * b->shape[r].K);
-  plan_batch_kernel<<<b->R, ga::kPlanThreads, 0, b->st>>>(b->ga_d, b->gens);
-  BCK(cudaGetLastError());
-  breed_batch_kernel<<<dim3(blocks_for(maxg, 256, 4096), b->R), 256, 0, b->st>>>(b->ga_d,
-                                                                                 b->gens, src);
-  BCK(cudaGetLastError());
+  BCK(launch_behind(plan_batch_kernel, b->R, ga::kPlanThreads, 0, b->st, b->ga_d, b->gens));
+  BCK(launch_behind(breed_batch_kernel, dim3(blocks_for(maxg, 256, 4096), b->R), 256, 0, b->st,
+                    b->ga_d, b->gens, src));
   return GAME_OK;
 }
 

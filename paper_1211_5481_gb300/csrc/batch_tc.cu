@@ -376,6 +376,7 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_batch_kernel(const BatchA
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = *tmem_holder;
+  wait_previous();   // (only shared and tensor memory so far)
 
   ItemQueue iq{ptx::smem_addr(q_full), ptx::smem_addr(q_empty), qidx, abort_flag, a.status, 0};
 
@@ -674,8 +675,7 @@ cudaError_t prepare_fitness_batch(int smem_bytes) {
 
 cudaError_t launch_fitness_batch(const BatchArgs& a, int grid, int smem_bytes, cudaStream_t st) {
   if (a.KBmax > 32 || smem_bytes > 232448) return cudaErrorInvalidValue;
-  fitness_batch_kernel<<<grid, kThreads, smem_bytes, st>>>(a);
-  return cudaGetLastError();
+  return launch_behind(fitness_batch_kernel, grid, kThreads, smem_bytes, st, a);
 }
 
 }  // namespace game

@@ -256,6 +256,7 @@ fitness_fp32_kernel(int64_t M, int N, int d, int basis, int Kc,
   constexpr int BP = 16 * U;              // chromosomes per CTA
   constexpr int NG = U / 4;               // a thread's groups of 4 chromosomes, 64 apart
   extern __shared__ __align__(16) uint8_t smem[];
+  wait_previous();
   Fp32Smem<U>& sm = *reinterpret_cast<Fp32Smem<U>*>(smem);
   volatile int* abort_flag = &sm.abort_flag;
 
@@ -434,9 +435,8 @@ cudaError_t launch_fitness_fp32(const Fp32Plan& pl, const Shape& s, const float*
     const cudaError_t e =
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    kern<<<grid, kThreads, smem, st>>>(s.M, s.N, s.d, s.basis, pl.Kc, Xt, y, popT, a0, Ppad,
-                                       ntiles, part, status);
-    return cudaGetLastError();
+    return launch_behind(kern, grid, kThreads, smem, st, s.M, s.N, s.d, s.basis, pl.Kc, Xt, y, popT,
+                         a0, Ppad, ntiles, part, status);
   };
   const bool abs = err == GAME_ERR_MAE;
   switch (pl.U) {

@@ -148,6 +148,7 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
   // ends the launch before any shared memory is touched
   const uint32_t pad = (1024u - (ptx::smem_addr(smem_raw) & 1023u)) & 1023u;
   if (pad > (uint32_t)a.slack) {
+    wait_previous();
     if (threadIdx.x == 0) atomicExch(a.status, (int)kDevSmemBase);
     return;
   }
@@ -208,6 +209,7 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = *tmem_holder;
+  wait_previous();   // (only shared and tensor memory so far)
 
   const int G = gridDim.x;
   const int my_tiles = (a.ntiles - (int)blockIdx.x + G - 1) / G;
@@ -1061,8 +1063,7 @@ cudaError_t launch_fitness_tc(const TcPlan& pl, const Shape& s, const float* Xt,
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        pl.smem_bytes);
   if (e != cudaSuccess) return e;
-  kern<<<pl.grid, kThreads, pl.smem_bytes, st>>>(a);
-  return cudaGetLastError();
+  return launch_behind(kern, pl.grid, kThreads, pl.smem_bytes, st, a);
 }
 
 }  // namespace game

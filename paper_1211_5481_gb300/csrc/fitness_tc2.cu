@@ -234,6 +234,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   ptx::cluster_sync();   // the peer's barriers exist before any arrival on them
   ptx::tc_fence_after();
   const uint32_t tmem = *tmem_holder;
+  wait_previous();   // (only shared and tensor memory so far)
 
   const int ncl = (int)(gridDim.x >> 1), cl = (int)(blockIdx.x >> 1);
   const int my_tiles = (a.ntiles - cl + ncl - 1) / ncl;
@@ -701,8 +702,7 @@ cudaError_t launch_fitness_tc_pair(const TcPlan& pl, const Shape& s, const float
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        pl.smem_bytes);
   if (e != cudaSuccess) return e;
-  kern<<<pl.grid, kThreads, pl.smem_bytes, st>>>(a);
-  return cudaGetLastError();
+  return launch_behind(kern, pl.grid, kThreads, pl.smem_bytes, st, a);
 }
 
 }  // namespace game

@@ -49,23 +49,27 @@ __global__ void init_population_kernel(uint64_t seed, int P, int K, float* __res
 __global__ void __launch_bounds__(kPlanThreads)
 ranking_order_kernel(int P, const double* __restrict__ fit, int* __restrict__ order) {
   extern __shared__ __align__(16) uint64_t skey[];
+  wait_previous();
   ga::ranking_sort_body(P, fit, skey, reinterpret_cast<int*>(skey + ga::pow2_at_least(P)), order);
 }
 
 __global__ void __launch_bounds__(kPlanThreads)
 roulette_cum_kernel(int P, const double* __restrict__ fit, uint64_t* __restrict__ cum) {
+  wait_previous();
   ga::roulette_cum_body(P, fit, cum);
 }
 
 __global__ void __launch_bounds__(kPlanThreads)
 ga_plan_kernel(GaDev g_, const double* __restrict__ fit, uint64_t seed, uint32_t g,
                int4* __restrict__ plan) {
+  wait_previous();
   ga::plan_body(g_, fit, seed, g, plan, blockIdx.x, gridDim.x);
 }
 
 __global__ void ga_breed_kernel(GaDev g_, const float* __restrict__ pop,
                                 const int4* __restrict__ plan, uint64_t seed, uint32_t g,
                                 float* __restrict__ next) {
+  wait_previous();
   const int64_t n = (int64_t)g_.Nout * g_.K;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
        e += (int64_t)gridDim.x * blockDim.x)
@@ -83,6 +87,7 @@ __global__ void __launch_bounds__(kPlanThreads)
 ga_fused_kernel(GaDev g_, const float* __restrict__ pop, const double* __restrict__ fit,
                 uint64_t seed, uint32_t g, float* __restrict__ next) {
   extern __shared__ __align__(16) uint64_t fsm[];
+  wait_previous();
   GaDev ga = g_;
   const int tb = (ga::table_bytes(g_) + 15) & ~15;
   int4* plan = reinterpret_cast<int4*>(reinterpret_cast<char*>(fsm) + tb);
@@ -128,31 +133,30 @@ cudaError_t launch_generation(const GaDev& ga, const float* pop, const double* f
   if (ga.E > kMaxElites) return cudaErrorInvalidValue;
   if (ga.P <= kFusedMax && ga.Nout <= kFusedMax && (int64_t)ga.Nout * ga.K <= kFusedGenes) {
     const int smem = ((ga::table_bytes(ga) + 15) & ~15) + ga.Nout * (int)sizeof(int4);
-    ga_fused_kernel<<<1, kPlanThreads, smem, st>>>(ga, pop, fit, seed, g, next);
-    return cudaGetLastError();
+    return launch_behind(ga_fused_kernel, 1, kPlanThreads, smem, st, ga, pop, fit, seed, g, next);
   }
+  cudaError_t e = cudaSuccess;
   if (ga.sel == GAME_SEL_RANKING) {
     if (ga.P > kMaxRankingP || !ga.order) return cudaErrorInvalidValue;
     const int smem = ranking_smem_bytes(ga.P);
     if (smem > 48 * 1024) {
-      const cudaError_t e =
-          cudaFuncSetAttribute(ranking_order_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      e = cudaFuncSetAttribute(ranking_order_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
       if (e != cudaSuccess) return e;
     }
-    ranking_order_kernel<<<1, kPlanThreads, smem, st>>>(ga.P, fit, ga.order);
+    e = launch_behind(ranking_order_kernel, 1, kPlanThreads, smem, st, ga.P, fit, ga.order);
   } else if (ga.sel == GAME_SEL_ROULETTE) {
     if (!ga.cum) return cudaErrorInvalidValue;
-    roulette_cum_kernel<<<1, kPlanThreads, 0, st>>>(ga.P, fit, ga.cum);
+    e = launch_behind(roulette_cum_kernel, 1, kPlanThreads, 0, st, ga.P, fit, ga.cum);
   }
   // three threads per pair of slots: oversampled offspring take several CTAs
   // (16,370 slots on one: 51 us)
   const int blocks = ceil_div(3 * ((int64_t)(ga.Nout - ga.E + 1) / 2), kPlanThreads);
-  ga_plan_kernel<<<blocks < 1 ? 1 : blocks, kPlanThreads, 0, st>>>(ga, fit, seed, g, plan);
-  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess)
+    e = launch_behind(ga_plan_kernel, blocks < 1 ? 1 : blocks, kPlanThreads, 0, st, ga, fit, seed, g,
+                      plan);
   if (e != cudaSuccess) return e;
-  ga_breed_kernel<<<blocks_for((int64_t)ga.Nout * ga.K, 256), 256, 0, st>>>(ga, pop, plan, seed,
-                                                                        g, next);
-  return cudaGetLastError();
+  return launch_behind(ga_breed_kernel, blocks_for((int64_t)ga.Nout * ga.K, 256), 256, 0, st, ga, pop,
+                       plan, seed, g, next);
 }
 
 }  // namespace game

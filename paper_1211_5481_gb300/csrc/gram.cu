@@ -240,12 +240,13 @@ quad_pairs_kernel(int P, int K, double m, double rm, int err, const float* __res
                   const int* __restrict__ idx, const double* __restrict__ Gp,
                   const uint16_t* __restrict__ kk, const double* __restrict__ b,
                   const double* __restrict__ yy, double* __restrict__ fit) {
+  wait_previous();
   __shared__ double as[kPairWarps][kPairK];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q = blockIdx.x * kPairWarps + warp;
   if (q >= P) return;
   const int p = idx ? idx[q] : q;
-  for (int k = lane; k < K; k += 32) as[warp][k] = (double)pop[(int64_t)p * K + k];
+  for (int k = lane; k < K; k += 32) as[warp][k] = (double)__ldcg(pop + (int64_t)p * K + k);
   __syncwarp();
   const double v = quad_pairs(K, as[warp], Gp, kk, b, lane);
   if (lane == 0) fit[p] = finish_error(divide_by(*yy + v, m, rm), err);
@@ -288,6 +289,7 @@ quad_rows_kernel(int P, int K, double m, double rm, int err, int S, const float*
                  const int* __restrict__ idx, const double* __restrict__ T,
                  const double* __restrict__ b, const double* __restrict__ yy,
                  double* __restrict__ fit) {
+  wait_previous();
   constexpr int kAhead = GRP >= 4 ? 8 : kAheadMax;   // loads in flight
   extern __shared__ double as[];   // [K + kAheadMax][GRP] genes of the group (zero past the last)
   __shared__ double red[kQuadRanges][GRP];   // the leader's: every range's sums
@@ -301,7 +303,7 @@ quad_rows_kernel(int P, int K, double m, double rm, int err, int S, const float*
     const float* genes = q < ng ? pop + (int64_t)(idx ? idx[p0 + q] : p0 + q) * K : nullptr;
 #pragma unroll 4
     for (int k = threadIdx.x / GRP; k < K; k += 32 * kQuadWarps / GRP)
-      as[k * GRP + q] = genes ? (double)genes[k] : 0.0;
+      as[k * GRP + q] = genes ? (double)__ldcg(genes + k) : 0.0;
   }
   __syncthreads();
   if (S > 1) ptx::cluster_wait();
@@ -503,12 +505,14 @@ cudaError_t launch_rows(const Shape& s, const float* pop, int P, const int* idx,
   cfg.blockDim = dim3(32 * kQuadWarps);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = (unsigned)S;
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // (see launch_behind)
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, quad_rows_kernel<GRP>, P, s.K, (double)s.M,
                             1.0 / (double)s.M, err, S, pop, idx, (const double*)g.list,
                             (const double*)g.b, (const double*)g.yy, fit);
@@ -518,9 +522,8 @@ cudaError_t launch_rows(const Shape& s, const float* pop, int P, const int* idx,
 cudaError_t launch_gram_fitness(const Shape& s, const float* pop, int P, const int* idx,
                                 const GramDev& g, double* fit, int err, cudaStream_t st) {
   if (s.K <= kPairK) {
-    quad_pairs_kernel<<<ceil_div(P, kPairWarps), 32 * kPairWarps, 0, st>>>(
-        P, s.K, (double)s.M, 1.0 / (double)s.M, err, pop, idx, g.list, g.kk, g.b, g.yy, fit);
-    return cudaGetLastError();
+    return launch_behind(quad_pairs_kernel, ceil_div(P, kPairWarps), 32 * kPairWarps, 0, st, P, s.K,
+                         (double)s.M, 1.0 / (double)s.M, err, pop, idx, g.list, g.kk, g.b, g.yy, fit);
   }
   // Four chromosomes share each entry where that still makes two CTAs per SM
   // (152 SMs); else one each, every load of a range in flight. Cluster size: about six

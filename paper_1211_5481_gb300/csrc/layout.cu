@@ -71,17 +71,19 @@ __global__ void relayout_X_kernel(const float* __restrict__ X, const float* __re
 
 __global__ void pack_fp32_kernel(const float* __restrict__ pop, int P, int Ppad, int K,
                                  int Kc, float* __restrict__ popT, float* __restrict__ a0) {
+  wait_previous();
   const int64_t n = (int64_t)Kc * Ppad;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
        e += (int64_t)gridDim.x * blockDim.x) {
     const int k = (int)(e / Ppad), p = (int)(e % Ppad);
-    popT[e] = (p < P && k + 1 < K) ? pop[(int64_t)p * K + 1 + k] : 0.f;
-    if (k == 0) a0[p] = p < P ? pop[(int64_t)p * K] : 0.f;
+    popT[e] = (p < P && k + 1 < K) ? __ldcg(pop + (int64_t)p * K + 1 + k) : 0.f;
+    if (k == 0) a0[p] = p < P ? __ldcg(pop + (int64_t)p * K) : 0.f;
   }
 }
 
 __global__ void pack_bf16_kernel(const float* __restrict__ pop, int P, int C, int K, int KB,
                                  uint8_t* __restrict__ popA, float* __restrict__ a0) {
+  wait_previous();
   // one thread per (chromosome row, K-block, 16-byte chunk)
   const int64_t n = (int64_t)C * 128 * KB * 8;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
@@ -97,19 +99,20 @@ __global__ void pack_bf16_kernel(const float* __restrict__ pop, int P, int C, in
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         const int kc = kb * 64 + q * 8 + 2 * h + u;   // contraction column
-        v[u] = (p < P && kc + 1 < K) ? pop[(int64_t)p * K + 1 + kc] : 0.f;
+        v[u] = (p < P && kc + 1 < K) ? __ldcg(pop + (int64_t)p * K + 1 + kc) : 0.f;
       }
       const __nv_bfloat162 b2 = __floats2bfloat162_rn(v[0], v[1]);
       w[h] = *reinterpret_cast<const uint32_t*>(&b2);
     }
     uint8_t* dst = popA + ((int64_t)(c * KB + kb) * 128 + r) * 128 + ((q ^ (r & 7)) << 4);
     *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
-    if (kb == 0 && q == 0) a0[p] = p < P ? pop[(int64_t)p * K] : 0.f;
+    if (kb == 0 && q == 0) a0[p] = p < P ? __ldcg(pop + (int64_t)p * K) : 0.f;
   }
 }
 
 __global__ void pack_bf16x3_kernel(const float* __restrict__ pop, int P, int C, int K, int KB,
                                    uint8_t* __restrict__ popA, float* __restrict__ a0) {
+  wait_previous();
   const int64_t n = (int64_t)C * 128 * KB * 8;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -124,7 +127,7 @@ __global__ void pack_bf16x3_kernel(const float* __restrict__ pop, int P, int C, 
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         const int kc = kb * 64 + q * 8 + 2 * h + u;
-        v[u] = (p < P && kc + 1 < K) ? pop[(int64_t)p * K + 1 + kc] : 0.f;
+        v[u] = (p < P && kc + 1 < K) ? __ldcg(pop + (int64_t)p * K + 1 + kc) : 0.f;
       }
       const __nv_bfloat162 hi = __floats2bfloat162_rn(v[0], v[1]);
       const float2 hf = __bfloat1622float2(hi);
@@ -135,7 +138,7 @@ __global__ void pack_bf16x3_kernel(const float* __restrict__ pop, int P, int C, 
     uint8_t* dst = popA + ((int64_t)(c * KB + kb) * 2 * 128 + r) * 128 + ((q ^ (r & 7)) << 4);
     *reinterpret_cast<uint4*>(dst) = make_uint4(wh[0], wh[1], wh[2], wh[3]);
     *reinterpret_cast<uint4*>(dst + 128 * 128) = make_uint4(wl[0], wl[1], wl[2], wl[3]);
-    if (kb == 0 && q == 0) a0[p] = p < P ? pop[(int64_t)p * K] : 0.f;
+    if (kb == 0 && q == 0) a0[p] = p < P ? __ldcg(pop + (int64_t)p * K) : 0.f;
   }
 }
 
@@ -143,6 +146,7 @@ __global__ void pack_bf16x3_kernel(const float* __restrict__ pop, int P, int C, 
 __global__ void pack_fp8_kernel(const float* __restrict__ pop, int P, int C, int K, int KB,
                                 const float* __restrict__ colscale, uint8_t* __restrict__ popA,
                                 float* __restrict__ a0, float* __restrict__ uscale) {
+  wait_previous();
   const int lane = threadIdx.x & 31;
   const int64_t nrows = (int64_t)C * 128;
   for (int64_t p = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; p < nrows;
@@ -151,7 +155,7 @@ __global__ void pack_fp8_kernel(const float* __restrict__ pop, int P, int C, int
     const float* gene = pop + p * K + 1;   // genes 1..K-1 (read only when real)
     float mx = 0.f;
     if (real)
-      for (int k = lane; k < K - 1; k += 32) mx = fmaxf(mx, fabsf(gene[k] * colscale[k]));
+      for (int k = lane; k < K - 1; k += 32) mx = fmaxf(mx, fabsf(__ldcg(gene + k) * colscale[k]));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     const float u = mx > 0.f ? mx / 448.f : 1.f;
@@ -165,7 +169,7 @@ __global__ void pack_fp8_kernel(const float* __restrict__ pop, int P, int C, int
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
           const int k = kb * 128 + q * 16 + 4 * h + t;
-          v[t] = (real && k < K - 1) ? gene[k] * colscale[k] / u : 0.f;
+          v[t] = (real && k < K - 1) ? __ldcg(gene + k) * colscale[k] / u : 0.f;
         }
         const uint32_t lo =
             __nv_cvt_float2_to_fp8x2(make_float2(v[0], v[1]), __NV_SATFINITE, __NV_E4M3);
@@ -177,7 +181,7 @@ __global__ void pack_fp8_kernel(const float* __restrict__ pop, int P, int C, int
       *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
     }
     if (lane == 0) {
-      a0[p] = real ? pop[p * K] : 0.f;
+      a0[p] = real ? __ldcg(pop + p * K) : 0.f;
       uscale[p] = u;
     }
   }
@@ -227,6 +231,7 @@ __global__ void colscales_kernel(const unsigned int* __restrict__ colmax, int nc
 // 1 + b d + (j - 1).
 __global__ void replicate_tied_kernel(const float* __restrict__ pop, int P, int K, int Bd,
                                       float* __restrict__ full) {
+  wait_previous();
   const int64_t n = (int64_t)P * K;
   const int Kg = Bd + 1;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
@@ -254,33 +259,29 @@ cudaError_t launch_relayout_X(const float* X, const float* y, const Shape& s, fl
 cudaError_t launch_pack_fp32(const float* pop, int P, int Ppad, const Shape& s, int Kc,
                              float* popT, float* a0, cudaStream_t st) {
   const int64_t n = (int64_t)Kc * Ppad;
-  pack_fp32_kernel<<<grid_for(n, 256), 256, 0, st>>>(pop, P, Ppad, s.K, Kc, popT, a0);
-  return cudaGetLastError();
+  return launch_behind(pack_fp32_kernel, grid_for(n, 256), 256, 0, st, pop, P, Ppad, s.K, Kc, popT,
+                       a0);
 }
 
 cudaError_t launch_replicate_tied(const float* pop, int P, const Shape& s, float* full,
                                   cudaStream_t st) {
   const int64_t n = (int64_t)P * s.K;
-  replicate_tied_kernel<<<grid_for(n, 256), 256, 0, st>>>(pop, P, s.K, s.B * s.d, full);
-  return cudaGetLastError();
+  return launch_behind(replicate_tied_kernel, grid_for(n, 256), 256, 0, st, pop, P, s.K, s.B * s.d,
+                       full);
 }
 
 cudaError_t launch_pack_tc(int form, const float* pop, int P, int C, const Shape& s, int KB,
                            const float* colscale, uint8_t* popA, float* a0, float* uscale,
                            cudaStream_t st) {
   const int64_t n = (int64_t)C * 128 * KB * 8;
-  if (form == kFormBF16) {
-    pack_bf16_kernel<<<grid_for(n, 256), 256, 0, st>>>(pop, P, C, s.K, KB, popA, a0);
-  } else if (form == kFormBF16x3) {
-    pack_bf16x3_kernel<<<grid_for(n, 256), 256, 0, st>>>(pop, P, C, s.K, KB, popA, a0);
-  } else if (form == kFormFP8) {
-    if (!colscale || !uscale) return cudaErrorInvalidValue;
-    pack_fp8_kernel<<<grid_for((int64_t)C * 128 * 32, 256), 256, 0, st>>>(
-        pop, P, C, s.K, KB, colscale, popA, a0, uscale);
-  } else {
-    return cudaErrorInvalidValue;
-  }
-  return cudaGetLastError();
+  if (form == kFormBF16)
+    return launch_behind(pack_bf16_kernel, grid_for(n, 256), 256, 0, st, pop, P, C, s.K, KB, popA, a0);
+  if (form == kFormBF16x3)
+    return launch_behind(pack_bf16x3_kernel, grid_for(n, 256), 256, 0, st, pop, P, C, s.K, KB, popA,
+                         a0);
+  if (form != kFormFP8 || !colscale || !uscale) return cudaErrorInvalidValue;
+  return launch_behind(pack_fp8_kernel, grid_for((int64_t)C * 128 * 32, 256), 256, 0, st, pop, P, C,
+                       s.K, KB, colscale, popA, a0, uscale);
 }
 
 cudaError_t launch_colmax(const Shape& s, const float* Xt, unsigned int* colmax, int ncols,

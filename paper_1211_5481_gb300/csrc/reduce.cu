@@ -23,6 +23,7 @@ __global__ void __launch_bounds__(kChroms * kGroups)
 reduce_rows_kernel(const double* __restrict__ part, int rows, int P, int Ppad, int err, double m,
                    double rm, double* __restrict__ fit) {
   __shared__ double sum[kGroups][kChroms];
+  wait_previous();
   const int c = threadIdx.x % kChroms, grp = threadIdx.x / kChroms;
   const int p = blockIdx.x * kChroms + c;   // Ppad is a multiple of 128: in bounds past P
   double s = 0.0;
@@ -55,9 +56,8 @@ reduce_rows_kernel(const double* __restrict__ part, int rows, int P, int Ppad, i
 
 cudaError_t launch_reduce(const double* part, int rows, int P, int Ppad, int64_t M, int err,
                           double* fit, cudaStream_t st) {
-  reduce_rows_kernel<<<ceil_div(P, kChroms), kChroms * kGroups, 0, st>>>(
-      part, rows, P, Ppad, err, (double)M, 1.0 / (double)M, fit);
-  return cudaGetLastError();
+  return launch_behind(reduce_rows_kernel, ceil_div(P, kChroms), kChroms * kGroups, 0, st, part,
+                       rows, P, Ppad, err, (double)M, 1.0 / (double)M, fit);
 }
 
 }  // namespace game

@@ -69,6 +69,7 @@ struct TopList {
 
 __global__ void __launch_bounds__(kSelThreads)
 select_top_kernel(const double* __restrict__ fit, int P, int n, int* __restrict__ cand) {
+  wait_previous();
   __shared__ uint64_t wk[kSelThreads / 32][kMaxRescore];
   __shared__ int wi[kSelThreads / 32][kMaxRescore];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -109,6 +110,7 @@ constexpr int kRankWarps = 8;
 constexpr int kRankChunk = 2048;   // keys staged in shared memory at a time
 __global__ void __launch_bounds__(32 * kRankWarps)
 select_rank_kernel(const double* __restrict__ fit, int P, int n, int* __restrict__ cand) {
+  wait_previous();
   __shared__ uint64_t key[kRankChunk];
   const int lane = threadIdx.x & 31;
   const int i = blockIdx.x * kRankWarps + (threadIdx.x >> 5);
@@ -135,10 +137,9 @@ cudaError_t launch_select_top(const double* fit, int P, int n, int* cand, cudaSt
   if (n < 1) return cudaSuccess;
   if (n > kMaxRescore || n > P) return cudaErrorInvalidValue;
   if (P <= kRankMax)
-    select_rank_kernel<<<ceil_div(P, kRankWarps), 32 * kRankWarps, 0, st>>>(fit, P, n, cand);
-  else
-    select_top_kernel<<<1, kSelThreads, 0, st>>>(fit, P, n, cand);
-  return cudaGetLastError();
+    return launch_behind(select_rank_kernel, ceil_div(P, kRankWarps), 32 * kRankWarps, 0, st, fit, P,
+                         n, cand);
+  return launch_behind(select_top_kernel, 1, kSelThreads, 0, st, fit, P, n, cand);
 }
 
 }  // namespace game

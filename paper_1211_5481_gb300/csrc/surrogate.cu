@@ -166,6 +166,7 @@ struct GradProblem {
 // Products: hi hi + lo hi.
 __global__ void __launch_bounds__(kGThreads, 1)
 grad_gemm_kernel(int batch, GradProblem p0, GradProblem p1, int kz, int* status) {
+  wait_previous();
   constexpr uint32_t kAImg = 128 * 128, kBImg = kGTN * 128;
   constexpr uint32_t kStage = 2 * kAImg + kBImg;   // hi and lo images of A
   extern __shared__ uint8_t smem_raw[];
@@ -282,6 +283,7 @@ __host__ __device__ constexpr int nt_smem() {
 
 template <int NA>
 __global__ void __launch_bounds__(kGThreads, 1) gemm_nt_kernel(const NtArgs a) {
+  wait_previous();
   constexpr int NS = nt_stages<NA>();
   constexpr uint32_t kAImg = 128 * 128;
   constexpr uint32_t kStage = NA * kAImg + kGTN * 128;
@@ -402,6 +404,7 @@ __global__ void __launch_bounds__(kGThreads, 1) gemm_nt_kernel(const NtArgs a) {
 // Xb [B][Kq] = X [B][K] rounded to BF16, zero past K (16-byte units).
 __global__ void to_bf16_kernel(int64_t B, int K, int Kq, const float* __restrict__ X,
                                __nv_bfloat16* __restrict__ Xb) {
+  wait_previous();
   const int per = Kq / 8;
   const int64_t n = B * per;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
@@ -410,7 +413,7 @@ __global__ void to_bf16_kernel(int64_t B, int K, int Kq, const float* __restrict
     const int k0 = (int)(e - b * per) * 8;
     float v[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) v[u] = k0 + u < K ? X[b * K + k0 + u] : 0.f;
+    for (int u = 0; u < 8; ++u) v[u] = k0 + u < K ? __ldcg(X + b * K + k0 + u) : 0.f;
     reinterpret_cast<uint4*>(Xb)[e] = make_uint4(bf16pair(v[0], v[1]), bf16pair(v[2], v[3]),
                                                  bf16pair(v[4], v[5]), bf16pair(v[6], v[7]));
   }
@@ -430,6 +433,7 @@ __device__ __forceinline__ float output_row(const float* __restrict__ H2,
 
 __global__ void output_kernel(int B, const float* __restrict__ H2, const float* __restrict__ w3,
                               const float* __restrict__ b3, float* __restrict__ out) {
+  wait_previous();
   const int w = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
   if (w >= B) return;
@@ -446,6 +450,7 @@ __global__ void output_grad_kernel(int B, const float* __restrict__ H2,
                                    float* __restrict__ dout, float* __restrict__ loss_terms,
                                    float* __restrict__ dZ2, __nv_bfloat16* __restrict__ hi,
                                    __nv_bfloat16* __restrict__ lo) {
+  wait_previous();
   const int w = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
   if (w >= B) return;
@@ -487,14 +492,16 @@ __device__ __forceinline__ double tree_sum_1024(double v, double* sh) {
 // l[b] = log(max(fit[b], 1e-30)) in FP64, over the whole GPU (FP64 is slow
 // on one SM)
 __global__ void log_fit_kernel(int B, const double* __restrict__ fit, double* __restrict__ l) {
+  wait_previous();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B) return;
-  const double f = fit[b];
+  const double f = __ldcg(fit + b);
   l[b] = log(f > 1e-30 ? f : 1e-30);
 }
 
 __global__ void __launch_bounds__(1024)
 target_stats_kernel(int B, const double* __restrict__ l, double* __restrict__ stats) {
+  wait_previous();
   __shared__ double sh[1024];
   double a = 0.0;
   for (int b = threadIdx.x; b < B; b += 1024) a += l[b];
@@ -515,6 +522,7 @@ target_stats_kernel(int B, const double* __restrict__ l, double* __restrict__ st
 // The standardised targets t[b] = (l[b] - mean) / sd.
 __global__ void targets_kernel(int B, const double* __restrict__ l,
                                const double* __restrict__ stats, float* __restrict__ t) {
+  wait_previous();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b < B) t[b] = (float)((l[b] - stats[0]) / stats[1]);
 }
@@ -579,6 +587,7 @@ sums_kernel(int B, const float* __restrict__ H2, const float* __restrict__ dout,
             const float* __restrict__ loss_terms, float* __restrict__ gw3,
             float* __restrict__ gb2, float* __restrict__ gb1, float* __restrict__ gb3,
             float* __restrict__ loss) {
+  wait_previous();
   const int what = blockIdx.x / (kH / 32), j0 = (blockIdx.x % (kH / 32)) * 32;
   if (what == 0) colsum_32(B, j0, H2, dout, gw3);
   else if (what == 1) colsum_32(B, j0, dZ2, nullptr, gb2);
@@ -620,6 +629,7 @@ __global__ void adam_kernel(int64_t n, int K, int Kq, int splits,
                             float* __restrict__ v, bool apply, float lr, float b1, float b2,
                             float eps, float c1, float c2, __nv_bfloat16* __restrict__ W1b,
                             __nv_bfloat16* __restrict__ W2b, __nv_bfloat16* __restrict__ W2t) {
+  wait_previous();
   const int64_t n1 = (int64_t)kH * K;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -699,6 +709,7 @@ __global__ void __launch_bounds__(kScreenThreads)
 screen_kernel(int n, int n_keep, const float* __restrict__ pred, int* __restrict__ flag,
               int* __restrict__ list, const int* __restrict__ trusted,
               int* __restrict__ used_trust) {
+  wait_previous();
   extern __shared__ uint32_t key[];
   __shared__ int hist[256];
   __shared__ uint32_t prefix;
@@ -801,6 +812,7 @@ screen_kernel(int n, int n_keep, const float* __restrict__ pred, int* __restrict
 // next: rows 0..E-1 the elites, row E + j offspring slot E + list[j]; a warp per row.
 __global__ void gather_kernel(int rows, int E, int K, const int* __restrict__ list,
                               const float* __restrict__ off, float* __restrict__ next) {
+  wait_previous();
   const int r = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
   if (r >= rows) return;
   const int64_t from = r < E ? r : E + list[r - E];
@@ -818,6 +830,7 @@ __global__ void __cluster_dims__(kTrustCtas, 1, 1) __launch_bounds__(kTrustThrea
 trust_kernel(int n_kept, const float* __restrict__ pred, const int* __restrict__ list,
              const double* __restrict__ lfit_kept, float* __restrict__ r_out,
              int* __restrict__ trusted) {
+  wait_previous();
   __shared__ double sh[kTrustWarps][8];
   __shared__ double tot[8];
   ptx::cluster_arrive();
@@ -898,8 +911,8 @@ cudaError_t gemm_nt(const NtArgs& a, cudaStream_t st) {
   const cudaError_t e = cudaFuncSetAttribute(
       gemm_nt_kernel<NA>, cudaFuncAttributeMaxDynamicSharedMemorySize, nt_smem<NA>());
   if (e != cudaSuccess) return e;
-  gemm_nt_kernel<NA><<<dim3(kH / kGTN, (a.M + 127) / 128), kGThreads, nt_smem<NA>(), st>>>(a);
-  return cudaGetLastError();
+  return launch_behind(gemm_nt_kernel<NA>, dim3(kH / kGTN, (a.M + 127) / 128), kGThreads,
+                       nt_smem<NA>(), st, a);
 }
 
 }  // namespace
@@ -931,17 +944,17 @@ cudaError_t surrogate_init(const SurrogateDev& s, uint64_t seed, cudaStream_t st
 
 cudaError_t surrogate_to_bf16(int K, const float* X, int B, __nv_bfloat16* Xb, cudaStream_t st) {
   const int Kq = surrogate_kq(K);
-  to_bf16_kernel<<<grid1d((int64_t)B * Kq / 8), 256, 0, st>>>(B, K, Kq, X, Xb);
-  return cudaGetLastError();
+  return launch_behind(to_bf16_kernel, grid1d((int64_t)B * Kq / 8), 256, 0, st, B, K, Kq, X, Xb);
 }
 
 cudaError_t surrogate_targets(const SurrogateDev& s, const double* fit, int B, float* t,
                               cudaStream_t st) {
   if (B > s.Bmax) return cudaErrorInvalidValue;
-  log_fit_kernel<<<(B + 255) / 256, 256, 0, st>>>(B, fit, s.lfit);
-  target_stats_kernel<<<1, 1024, 0, st>>>(B, s.lfit, s.tstat);
-  targets_kernel<<<(B + 255) / 256, 256, 0, st>>>(B, s.lfit, s.tstat, t);
-  return cudaGetLastError();
+  cudaError_t e = launch_behind(log_fit_kernel, (B + 255) / 256, 256, 0, st, B, fit, s.lfit);
+  if (e == cudaSuccess)
+    e = launch_behind(target_stats_kernel, 1, 1024, 0, st, B, s.lfit, s.tstat);
+  if (e != cudaSuccess) return e;
+  return launch_behind(targets_kernel, (B + 255) / 256, 256, 0, st, B, s.lfit, s.tstat, t);
 }
 
 namespace {
@@ -985,8 +998,8 @@ cudaError_t surrogate_forward(const SurrogateDev& s, const float* X, int B, floa
   cudaError_t e = surrogate_to_bf16(s.K, X, B, s.Xb, st);
   if (e == cudaSuccess) e = hidden_layers(s, s.Xb, B, 0, st);
   if (e != cudaSuccess) return e;
-  output_kernel<<<(int)(((int64_t)B * 32 + 255) / 256), 256, 0, st>>>(B, s.H2, w3, w3 + kH, out);
-  return cudaGetLastError();
+  return launch_behind(output_kernel, (int)(((int64_t)B * 32 + 255) / 256), 256, 0, st, B, s.H2, w3,
+                       w3 + kH, out);
 }
 
 // The gradient of the mean squared error over the batch into s.g, the loss into
@@ -1002,8 +1015,9 @@ cudaError_t surrogate_step(SurrogateDev& s, const SurrogateBatch& bt, bool apply
   float* gb3 = gw3 + kH;
   cudaError_t e = hidden_layers(s, bt.Xb, B, 1, st);
   if (e != cudaSuccess) return e;
-  output_grad_kernel<<<(int)(((int64_t)B * 32 + 255) / 256), 256, 0, st>>>(
-      B, s.H2, s.Z2, w3, w3 + kH, bt.t, s.dout, s.lterm, s.dZ2, s.dZ2h, s.dZ2l);
+  e = launch_behind(output_grad_kernel, (int)(((int64_t)B * 32 + 255) / 256), 256, 0, st, B, s.H2,
+                    s.Z2, w3, w3 + kH, bt.t, s.dout, s.lterm, s.dZ2, s.dZ2h, s.dZ2l);
+  if (e != cudaSuccess) return e;
   // dZ1 = (dZ2 bf(W2)) g'(Z1)
   NtArgs a{};
   a.M = B;
@@ -1026,10 +1040,12 @@ cudaError_t surrogate_step(SurrogateDev& s, const SurrogateBatch& bt, bool apply
   constexpr int smem = 2 * (2 * 128 * 128 + kGTN * 128) + 1024 + 64;
   e = cudaFuncSetAttribute(grad_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  grad_gemm_kernel<<<dim3(p1.tiles + p2.tiles, kH / 128, splits), kGThreads, smem, st>>>(
-      B, p1, p2, kz, s.status);
-  sums_kernel<<<3 * (kH / 32) + 2, 1024, 0, st>>>(B, s.H2, s.dout, s.dZ2, s.dZ1, s.lterm, gw3,
-                                                 gb2, gb1, gb3, s.loss);
+  e = launch_behind(grad_gemm_kernel, dim3(p1.tiles + p2.tiles, kH / 128, splits), kGThreads, smem,
+                    st, B, p1, p2, kz, s.status);
+  if (e == cudaSuccess)
+    e = launch_behind(sums_kernel, 3 * (kH / 32) + 2, 1024, 0, st, B, s.H2, s.dout, s.dZ2, s.dZ1,
+                      s.lterm, gw3, gb2, gb1, gb3, s.loss);
+  if (e != cudaSuccess) return e;
   float c1 = 1.f, c2 = 1.f;
   if (apply) {
     s.step += 1;
@@ -1037,10 +1053,9 @@ cudaError_t surrogate_step(SurrogateDev& s, const SurrogateBatch& bt, bool apply
     c2 = 1.f - powf(kAdamB2, (float)s.step);
   }
   const int64_t n = surrogate_param_count(K);
-  adam_kernel<<<grid1d(n), 256, 0, st>>>(n, K, surrogate_kq(K), splits, s.split1, s.split2, s.w,
-                                         s.g, s.m, s.v, apply, kAdamLr, kAdamB1, kAdamB2,
-                                         kAdamEps, c1, c2, s.W1b, s.W2b, s.W2t);
-  return cudaGetLastError();
+  return launch_behind(adam_kernel, grid1d(n), 256, 0, st, n, K, surrogate_kq(K), splits, s.split1,
+                       s.split2, s.w, s.g, s.m, s.v, apply, kAdamLr, kAdamB1, kAdamB2, kAdamEps, c1,
+                       c2, s.W1b, s.W2b, s.W2t);
 }
 
 cudaError_t surrogate_trust_check(const SurrogateDev& s, int n_kept, const float* pred,
@@ -1048,9 +1063,11 @@ cudaError_t surrogate_trust_check(const SurrogateDev& s, int n_kept, const float
                                   int* trusted, cudaStream_t st) {
   if (n_kept > s.Bmax) return cudaErrorInvalidValue;
   // the kept children's log-fitness over the whole GPU first (FP64)
-  log_fit_kernel<<<(n_kept + 255) / 256, 256, 0, st>>>(n_kept, fit_kept, s.lfit);
-  trust_kernel<<<kTrustCtas, kTrustThreads, 0, st>>>(n_kept, pred, list, s.lfit, r_out, trusted);
-  return cudaGetLastError();
+  const cudaError_t e = launch_behind(log_fit_kernel, (n_kept + 255) / 256, 256, 0, st, n_kept,
+                                      fit_kept, s.lfit);
+  if (e != cudaSuccess) return e;
+  return launch_behind(trust_kernel, kTrustCtas, kTrustThreads, 0, st, n_kept, pred, list, s.lfit,
+                       r_out, trusted);
 }
 
 cudaError_t surrogate_screen(int n, int n_keep, int E, int K, const float* pred, int* flag,
@@ -1060,13 +1077,12 @@ cudaError_t surrogate_screen(int n, int n_keep, int E, int K, const float* pred,
   cudaError_t e = cudaFuncSetAttribute(screen_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)(kScreenMax * sizeof(uint32_t)));
   if (e != cudaSuccess) return e;
-  screen_kernel<<<1, kScreenThreads, (size_t)n * sizeof(uint32_t), st>>>(
-      n, n_keep, pred, flag, list, trusted, used_trust);
-  e = cudaGetLastError();
+  e = launch_behind(screen_kernel, 1, kScreenThreads, (size_t)n * sizeof(uint32_t), st, n, n_keep,
+                    pred, flag, list, trusted, used_trust);
   if (e != cudaSuccess) return e;
   const int rows = E + n_keep;
-  gather_kernel<<<(rows * 32 + 255) / 256, 256, 0, st>>>(rows, E, K, list, off, next);
-  return cudaGetLastError();
+  return launch_behind(gather_kernel, (rows * 32 + 255) / 256, 256, 0, st, rows, E, K, list, off,
+                       next);
 }
 
 }  // namespace game
