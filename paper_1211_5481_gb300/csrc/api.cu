@@ -98,6 +98,7 @@ struct game_ctx {
   int64_t gen = 0;
   int4* plan = nullptr;
   int* status = nullptr;   // device status word written by kernels
+  int* status_h = nullptr; // its page-locked copy on the host
   // elite re-scoring
   int* cand = nullptr;
   // selection tables (ranking order, roulette weight sums)
@@ -606,12 +607,25 @@ int setup_screening(game_ctx* h) {
   return GAME_OK;
 }
 
+// Enqueues the status word's copy to the host. Ahead of a result's copy into
+// pageable memory, which waits for the stream, it costs no wait of its own: one
+// evaluation from numpy (bf16, M = 30,011, N = 11, trigonometric degree 7, P =
+// 100) 56 -> 48 us.
+int enqueue_status(game_ctx* h) {
+  CK(cudaMemcpyAsync(h->status_h, h->status, 2 * sizeof(int), cudaMemcpyDeviceToHost, h->st));
+  return GAME_OK;
+}
+
 // Waits for the handle's work and reports its status word; gens_run: the
 // generations the last whole-generation launch ran (its second word).
-int check_status(game_ctx* h, int* gens_run = nullptr) {
-  int word[2] = {0, 0};
-  CK(cudaMemcpyAsync(word, h->status, sizeof(word), cudaMemcpyDeviceToHost, h->st));
+// enqueued: enqueue_status was called behind the last kernel.
+int check_status(game_ctx* h, int* gens_run = nullptr, bool enqueued = false) {
+  if (!enqueued) {
+    const int rc = enqueue_status(h);
+    if (rc) return rc;
+  }
   CK(cudaStreamSynchronize(h->st));
+  const volatile int* word = h->status_h;
   const int st = word[0];
   if (gens_run) *gens_run = word[1];
   if (st != kDevOk) {
@@ -751,6 +765,7 @@ void destroy_ctx(game_ctx* h) {
   dev_free(h->fit);
   dev_free(h->plan);
   dev_free(h->status);
+  if (h->status_h) cudaFreeHost(h->status_h);
   dev_free(h->cand);
   dev_free(h->sel_order);
   dev_free(h->sel_cum);
@@ -913,6 +928,7 @@ int game_create(const float* X, const float* y, int64_t M, int32_t N, int32_t de
       dev_alloc(&h->fit, (size_t)p.P) != cudaSuccess ||
       dev_alloc(&h->plan, (size_t)p.P) != cudaSuccess ||
       dev_alloc(&h->status, 4) != cudaSuccess ||
+      cudaMallocHost(reinterpret_cast<void**>(&h->status_h), 2 * sizeof(int)) != cudaSuccess ||
       dev_alloc(&h->cand, kMaxRescore) != cudaSuccess ||
       (p.selection == GAME_SEL_RANKING && dev_alloc(&h->sel_order, (size_t)p.P) != cudaSuccess) ||
       (p.selection == GAME_SEL_ROULETTE &&
@@ -1025,9 +1041,10 @@ int game_eval_fitness_prec(game_t h, const float* pop, int32_t P, int32_t precis
   CK(cudaMemcpyAsync(h->upop, pop, (size_t)P * h->Kg * sizeof(float), cudaMemcpyHostToDevice,
                      h->st));
   rc = eval_device(h, h->upop, P, precision, h->ufit);
+  if (!rc) rc = enqueue_status(h);
   if (rc) return rc;
   CK(cudaMemcpyAsync(fit_out, h->ufit, (size_t)P * sizeof(double), cudaMemcpyDeviceToHost, h->st));
-  return check_status(h);
+  return check_status(h, nullptr, true);
 }
 
 int game_eval_fitness(game_t h, const float* pop, int32_t P, double* fit_out) {
@@ -1186,23 +1203,23 @@ int game_get_population(game_t h, float* pop_out, double* fit_out, int64_t* gene
   g_last_error.clear();
   if (!h) return fail(GAME_EINVAL, "NULL handle");
   if (generation) *generation = h->gen;
-  bool host = false;
-  if (pop_out) {
-    host |= !is_device_ptr(pop_out);
+  if (fit_out && !h->fit_valid) {
+    int rc = eval_state(h);
+    if (rc) return rc;
+    h->fit_valid = true;
+  }
+  const bool host = (pop_out && !is_device_ptr(pop_out)) || (fit_out && !is_device_ptr(fit_out));
+  if (host) {
+    int rc = enqueue_status(h);
+    if (rc) return rc;
+  }
+  if (pop_out)
     CK(cudaMemcpyAsync(pop_out, h->pop[h->cur], (size_t)h->prm.P * h->Kg * sizeof(float),
                        cudaMemcpyDefault, h->st));
-  }
-  if (fit_out) {
-    if (!h->fit_valid) {
-      int rc = eval_state(h);
-      if (rc) return rc;
-      h->fit_valid = true;
-    }
-    host |= !is_device_ptr(fit_out);
+  if (fit_out)
     CK(cudaMemcpyAsync(fit_out, h->fit, (size_t)h->prm.P * sizeof(double), cudaMemcpyDefault,
                        h->st));
-  }
-  if (host) return check_status(h);
+  if (host) return check_status(h, nullptr, true);
   return GAME_OK;
 }
 

@@ -21,6 +21,7 @@
 #include <cmath>
 #include <cstring>
 #include <functional>
+#include <mutex>
 #include <new>
 #include <queue>
 #include <string>
@@ -174,6 +175,11 @@ struct game_batch {
   float* a0 = nullptr;
   uint32_t* gens = nullptr;
   int* status = nullptr;
+  // page-locked: the status word, then one run's fitness and genes on their way
+  // to the caller (status_h alone where a run is larger than kStageMax)
+  int* status_h = nullptr;
+  size_t stage_bytes = 0;
+  std::mutex stage_lock;
   int* chrom_begin = nullptr;
   int total_chrom = 0;
   BatchRun* runs_d = nullptr;
@@ -441,10 +447,26 @@ int enqueue_eval(game_batch* b, int src, int inc) {
   return rc;
 }
 
-int check_batch_status(game_batch* b) {
-  int st = 0;
-  BCK(cudaMemcpyAsync(&st, b->status, sizeof(int), cudaMemcpyDeviceToHost, b->st));
+// run r's fitness and genes
+size_t run_bytes(const game_batch* b, int r) {
+  return (size_t)b->P[r] * (sizeof(double) + b->shape[r].K * sizeof(float));
+}
+
+constexpr size_t kStageHead = 16;             // bytes ahead of a staged run: the status word
+constexpr size_t kStageMax = (size_t)16 << 20;
+
+int enqueue_batch_status(game_batch* b) {
+  BCK(cudaMemcpyAsync(b->status_h, b->status, sizeof(int), cudaMemcpyDeviceToHost, b->st));
+  return GAME_OK;
+}
+
+int check_batch_status(game_batch* b, bool enqueued = false) {
+  if (!enqueued) {
+    const int rc = enqueue_batch_status(b);
+    if (rc) return rc;
+  }
   BCK(cudaStreamSynchronize(b->st));
+  const int st = *static_cast<const volatile int*>(b->status_h);
   if (st != kDevOk) {
     BCK(cudaMemsetAsync(b->status, 0, sizeof(int), b->st));
     BCK(cudaStreamSynchronize(b->st));
@@ -578,6 +600,7 @@ void destroy_batch(game_batch* b) {
   dfree(b->a0);
   dfree(b->gens);
   dfree(b->status);
+  if (b->status_h) cudaFreeHost(b->status_h);
   dfree(b->chrom_begin);
   dfree(b->runs_d);
   dfree(b->ga_d);
@@ -679,13 +702,18 @@ int game_batch_create(const game_run_desc* runs, int32_t R, const game_params* p
   }
   if (nfit > 0x7fffffff / 32) return bail(bfail(GAME_EINVAL, "too many chromosomes in total"));
   b->total_chrom = (int)nfit;
+  for (int r = 0; r < R; ++r)
+    b->stage_bytes = std::max(b->stage_bytes, run_bytes(b, r));
+  if (b->stage_bytes > kStageMax) b->stage_bytes = 0;
   if (dalloc(&b->Xt, nX) != cudaSuccess || dalloc(&b->y, ny) != cudaSuccess ||
       dalloc(&b->pop[0], npop) != cudaSuccess || dalloc(&b->pop[1], npop) != cudaSuccess ||
       dalloc(&b->fit, nfit) != cudaSuccess || dalloc(&b->plan, nfit) != cudaSuccess ||
       dalloc(&b->popA, nA) != cudaSuccess || dalloc(&b->a0, na0) != cudaSuccess ||
       dalloc(&b->gens, R) != cudaSuccess || dalloc(&b->status, 4) != cudaSuccess ||
       dalloc(&b->chrom_begin, R) != cudaSuccess || dalloc(&b->runs_d, R) != cudaSuccess ||
-      dalloc(&b->ga_d, R) != cudaSuccess || dalloc(&b->work, 1) != cudaSuccess) {
+      dalloc(&b->ga_d, R) != cudaSuccess || dalloc(&b->work, 1) != cudaSuccess ||
+      cudaMallocHost(reinterpret_cast<void**>(&b->status_h), kStageHead + b->stage_bytes) !=
+          cudaSuccess) {
     cudaGetLastError();
     return bail(bfail(GAME_ENOMEM, "batch device memory"));
   }
@@ -792,13 +820,29 @@ int game_batch_get_run(game_batch_t b, int32_t r, float* pop_out, double* fit_ou
   if (r < 0 || r >= b->R) return bfail(GAME_EINVAL, "run index out of range");
   if (generation) *generation = b->gen;
   const int64_t PK = (int64_t)b->P[r] * b->shape[r].K;
-  if (pop_out)
-    BCK(cudaMemcpyAsync(pop_out, b->pop[b->cur] + b->off_pop[r], PK * sizeof(float),
-                        cudaMemcpyDefault, b->st));
-  if (fit_out)
-    BCK(cudaMemcpyAsync(fit_out, b->fit + b->off_fit[r], b->P[r] * sizeof(double),
-                        cudaMemcpyDefault, b->st));
-  return check_batch_status(b);
+  const float* pop = b->pop[b->cur] + b->off_pop[r];
+  const double* fit = b->fit + b->off_fit[r];
+  const size_t pop_bytes = PK * sizeof(float), fit_bytes = b->P[r] * sizeof(double);
+  const bool staged = b->stage_bytes > 0 && (!pop_out || !is_dev(pop_out)) &&
+                      (!fit_out || !is_dev(fit_out)) && (pop_out || fit_out);
+  std::lock_guard<std::mutex> lock(b->stage_lock);
+  int rc = enqueue_batch_status(b);
+  if (rc) return rc;
+  if (!staged) {
+    if (pop_out) BCK(cudaMemcpyAsync(pop_out, pop, pop_bytes, cudaMemcpyDefault, b->st));
+    if (fit_out) BCK(cudaMemcpyAsync(fit_out, fit, fit_bytes, cudaMemcpyDefault, b->st));
+    return check_batch_status(b, true);
+  }
+  // To host memory: through the page-locked buffer, so the three copies are waited
+  // for once, not each (a copy into pageable memory waits). 24 runs of 0.1 to 0.9
+  // MB and four generations: 2246 -> 2131 us.
+  char* at = reinterpret_cast<char*>(b->status_h) + kStageHead;
+  if (fit_out) BCK(cudaMemcpyAsync(at, fit, fit_bytes, cudaMemcpyDeviceToHost, b->st));
+  if (pop_out) BCK(cudaMemcpyAsync(at + fit_bytes, pop, pop_bytes, cudaMemcpyDeviceToHost, b->st));
+  rc = check_batch_status(b, true);
+  if (fit_out) std::memcpy(fit_out, at, fit_bytes);
+  if (pop_out) std::memcpy(pop_out, at + fit_bytes, pop_bytes);
+  return rc;
 }
 
 int game_batch_get_tiles(game_batch_t b, int32_t* tiles_out) {
