@@ -22,13 +22,13 @@
 // tile's expansion (patterns on MMA-N).
 //
 // Persistent CTAs, one per SM, each walking pattern tiles t = blockIdx.x +
-// i * gridDim.x. Warp roles (16 warps):
+// i * gridDim.x. Warp roles (20 warps):
 //   warp 0       A producer: bulk-copies 16 KB gene blocks (chromosome tile c,
 //                K-block kb of 64 columns) from the pre-swizzled operand
 //                image into a ring of 3-4 stages.
-//   warp 1       MMA issuer (one elected thread) and tensor-memory owner; two FP32 accumulators of BN
-//                columns, so the epilogue of chromosome tile c overlaps the
-//                MMAs of tile c+1.
+//   warp 1       MMA issuer (one elected thread) and tensor-memory owner; two
+//                FP32 accumulators of BN columns, so the epilogue of chromosome
+//                tile c overlaps the MMAs of tile c+1.
 //   warp 2       X producer: bulk-copies the next pattern tile's features
 //                (staged mode only, below).
 //   warp 3       Y producer: bulk-copies each tile's targets (where they fit).
@@ -51,7 +51,7 @@
 // into shared memory, the expansion reads them there) or, for the BF16 form
 // with Chebyshev runs of 8 degrees at 128 / 256 patterns, read by the
 // expansion threads from global memory (L2, prefetched two tiles ahead),
-// one K-block ahead of use; the shared memory this frees holds the spare
+// one K-block of a warpgroup ahead of use; the shared memory this frees holds the spare
 // slots. Both modes produce identical expansion values.
 // PHI and D never leave the SM. All waits are bounded (2 s): on expiry the
 // kernel raises a status word, abandons its loops, waits for its own bulk
@@ -529,8 +529,8 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
       stream_dispatch<F, false>(a.basis, a.d, sa);
     }
     // thread -> rows r0 + RW * rr (rr < R) and 16-byte units q0, q0 + QS, ...:
-    // BN = 128, 256: 128 rows per pass, R = BN / 128; BN = 192: 64 rows per
-    // pass, R = 3, two unit groups; BN < 128: BN rows, R = 1, 128 / BN groups
+    // BN = 128, 256: 128 rows per pass, R = BN / 128, two unit groups; BN = 192:
+    // 64 rows per pass, R = 3, four; BN < 128: BN rows, R = 1, 256 / BN
     const int RW = TRI ? 64 : (BN < 128 ? BN : 128);
     const int R = TRI ? 3 : BN / RW;
     const int QS = kBasisThreads / RW;
