@@ -1151,15 +1151,21 @@ int game_train(game_t h, int32_t generations, int32_t* generations_run) {
   if (h->fit_valid && whole_generations(h) && h->gen + generations < 0xFFFFFFFFll) {
     // at most kGensPerLaunch at a time: a launch stays in the milliseconds
     constexpr int kGensPerLaunch = 1000;
-    int done = 0;
+    int done = 0, late = GAME_OK;
     while (done < generations) {
       const int n = generations - done < kGensPerLaunch ? generations - done : kGensPerLaunch;
       int rc = enqueue_generations(h, h->prm.seed, n, done, use_stop);
       if (rc) return rc;
       int ran = n;
       if (use_stop) {
+        // The launch has left its population in the other buffer and its fitness
+        // in place, so what ran is taken over also where the status word reports a
+        // wait that an earlier call only enqueued; the call then ends as without
+        // it, and returns that.
+        ran = -1;
         rc = check_status(h, &ran);
-        if (rc) return rc;
+        if (ran < 0) return rc;   // the stream itself failed
+        if (rc) late = rc;
       }
       if (ran > 0) h->cur ^= 1;
       h->gen += ran;
@@ -1167,7 +1173,7 @@ int game_train(game_t h, int32_t generations, int32_t* generations_run) {
       if (generations_run) *generations_run = done;
       if (ran < n) break;
     }
-    return use_stop ? GAME_OK : check_status(h);
+    return use_stop ? late : check_status(h);
   }
   double* fit_h = nullptr;
   if (use_stop) {

@@ -112,3 +112,34 @@ def test_every_allocation_failure_of_a_batch_is_clean():
     with game.Batch(args, autotune=False) as b:
         b.generation()
         b.sync()
+
+
+# a threshold no run reaches, and one that the first check meets (no generation runs)
+@pytest.mark.parametrize("threshold", [1e-12, 1e12])
+def test_a_pending_timeout_leaves_genes_and_fitness_together(threshold):
+    """An evaluation on device arrays only enqueues; its expired wait shows in the
+    next call that waits. A training call that reports it leaves a population with
+    its own fitness, and the state of the same call without the timeout."""
+    pr = dg.regression(19, 3000, 6, 3, 0.05, degree=4)
+    pop = torch.from_numpy(dg.random_population(5, 300, pr.K)).cuda()
+    states = []
+    for stall in (False, True):
+        with game.Game(pr.X, pr.y, 4, CHEB, P=24, precision=game.GAME_PREC_GRAM,
+                       mse_threshold=threshold, check_every=3) as g:
+            before = g.population()
+            if stall:
+                game.game_test_hook(game.GAME_HOOK_STALL_NS, 20_000_000)
+                g.eval_fitness(pop, game.GAME_PREC_BF16)
+                with pytest.raises(game.GameError) as ei:
+                    g.train(7)
+                assert ei.value.code == game.GAME_ETIMEOUT
+            else:
+                g.train(7)
+            genes, fit, gen = g.population()
+            assert gen == (7 if threshold < 1 else 0)
+            assert np.array_equal(genes, before[0]) == (gen == 0)
+            assert np.array_equal(fit, g.eval_fitness(genes))
+            g.generation(5)
+            states.append((genes, fit) + g.population())
+    for a, b in zip(*states):
+        assert np.array_equal(a, b)
