@@ -237,7 +237,7 @@ __global__ void replicate_tied_kernel(const float* __restrict__ pop, int P, int 
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
        e += (int64_t)gridDim.x * blockDim.x) {
     const int p = (int)(e / K), k = (int)(e % K);
-    full[e] = pop[(int64_t)p * Kg + (k == 0 ? 0 : 1 + (k - 1) % Bd)];
+    full[e] = __ldcg(pop + (int64_t)p * Kg + (k == 0 ? 0 : 1 + (k - 1) % Bd));
   }
 }
 

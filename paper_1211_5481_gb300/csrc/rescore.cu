@@ -75,7 +75,7 @@ select_top_kernel(const double* __restrict__ fit, int P, int n, int* __restrict_
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   TopList L;
   L.clear();
-  for (int p = tid; p < P; p += kSelThreads) L.insert(ga::rank_key(fit[p]), p);
+  for (int p = tid; p < P; p += kSelThreads) L.insert(ga::rank_key(__ldcg(fit + p)), p);
   // each warp: n rounds of arg-min over its lanes' list heads
   for (int r = 0; r < n; ++r) {
     uint64_t k = L.k[0];
@@ -114,12 +114,12 @@ select_rank_kernel(const double* __restrict__ fit, int P, int n, int* __restrict
   __shared__ uint64_t key[kRankChunk];
   const int lane = threadIdx.x & 31;
   const int i = blockIdx.x * kRankWarps + (threadIdx.x >> 5);
-  const uint64_t mine = i < P ? ga::rank_key(fit[i]) : kNoKey;
+  const uint64_t mine = i < P ? ga::rank_key(__ldcg(fit + i)) : kNoKey;
   int before = i < P ? 0 : n;
   for (int c0 = 0; c0 < P; c0 += kRankChunk) {
     const int len = min(kRankChunk, P - c0);
 #pragma unroll 8
-    for (int k = threadIdx.x; k < len; k += 32 * kRankWarps) key[k] = ga::rank_key(fit[c0 + k]);
+    for (int k = threadIdx.x; k < len; k += 32 * kRankWarps) key[k] = ga::rank_key(__ldcg(fit + c0 + k));
     __syncthreads();
     for (int k0 = 0; k0 < len && before < n; k0 += 32) {
       const int k = k0 + lane;
