@@ -229,7 +229,7 @@ int ensure_gram(game_ctx* h) {
   double* phi = nullptr;
   double* part = nullptr;
   GramDev g{};
-  const size_t list = (size_t)gram_list(gs);
+  const size_t list = (size_t)gram_list(gs), parts = (size_t)gram_rescore_parts(gs, h->num_sms);
   auto drop = [&]() {
     dev_free(phi);
     dev_free(part);
@@ -238,10 +238,12 @@ int ensure_gram(game_ctx* h) {
     dev_free(g.yy);
     dev_free(g.list);
     dev_free(g.kk);
+    dev_free(g.part);
   };
   if (dev_alloc(&g.G, (size_t)K * K) != cudaSuccess || dev_alloc(&g.b, (size_t)K) != cudaSuccess ||
       dev_alloc(&g.yy, 1) != cudaSuccess || dev_alloc(&g.list, list) != cudaSuccess ||
       dev_alloc(&g.kk, gs.K <= 64 ? list : 1) != cudaSuccess ||
+      (parts > 0 && dev_alloc(&g.part, parts) != cudaSuccess) ||
       dev_alloc(&phi, (size_t)rows * K) != cudaSuccess ||
       dev_alloc(&part, (size_t)gram_part_doubles(gs, h->num_sms)) != cudaSuccess) {
     cudaGetLastError();
@@ -456,7 +458,8 @@ int rescore_device(game_ctx* h, const float* dpop, int P, int n, double* dfit) {
   if (rc) return rc;
   cudaEvent_t t0 = stage_begin(h);
   CK(launch_select_top(dfit, P, n, h->cand, h->st));
-  CK(launch_gram_fitness(gram_shape(h), dpop, n, h->cand, h->gram, dfit, h->prm.error, h->st));
+  CK(launch_gram_rescore(gram_shape(h), dpop, n, h->cand, h->gram, dfit, h->prm.error, h->num_sms,
+                         h->st));
   stage_end(h, t0, kRescore);
   return GAME_OK;
 }
@@ -779,6 +782,7 @@ void destroy_ctx(game_ctx* h) {
   dev_free(h->gram.yy);
   dev_free(h->gram.list);
   dev_free(h->gram.kk);
+  dev_free(h->gram.part);
   dev_free(h->colmax);
   dev_free(h->colscale);
   dev_free(h->colinv);

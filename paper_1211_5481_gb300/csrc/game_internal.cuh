@@ -282,14 +282,19 @@ struct GramDev {
   double *G, *b, *yy;
   double* list;    // [gram_list(s)]: K <= 64 pairs k1 <= k2, else 32-row steps
   uint16_t* kk;    // K <= 64: [gram_list(s)] k1 | k2 << 8
+  double* part;    // [gram_rescore_parts(s)] the re-scoring's partial sums
 };
 int64_t gram_list(const Shape& s);
 cudaError_t launch_gram_list(const Shape& s, const GramDev& g, cudaStream_t st);
 // fit of the P chromosomes pop [P][K] (idx NULL), or of rows idx[0..P-1]
-// written to fit[idx[p]] (the elite re-scoring); err GAME_ERR_MSE or
-// GAME_ERR_RMSE
+// written to fit[idx[p]]; err GAME_ERR_MSE or GAME_ERR_RMSE
 cudaError_t launch_gram_fitness(const Shape& s, const float* pop, int P, const int* idx,
                                 const GramDev& g, double* fit, int err, cudaStream_t st);
+// the elite re-scoring: n <= kMaxRescore rows idx[q] into fit[idx[q]]
+int64_t gram_rescore_parts(const Shape& s, int num_sms);
+cudaError_t launch_gram_rescore(const Shape& s, const float* pop, int n, const int* idx,
+                                const GramDev& g, double* fit, int err, int num_sms,
+                                cudaStream_t st);
 
 // predict.cu: Out(m) of chrom [Kg] in FP64 for M patterns of X (tiled: the
 // handle's [Mpad/128][N][128] layout, else row-major [M][N]) into out (may be

@@ -407,6 +407,77 @@ quad_rows_kernel(int P, int K, double m, double rm, int err, int S, const float*
   }
 }
 
+// The elite re-scoring where the evaluation's kernels leave the GPU idle (see
+// spread_serves; n <= kMaxRescore chromosomes): their products are spread over the
+// whole GPU and share each entry of G. CTA (bx, by) owns rows
+// k1 in [128 bx, 128 bx + 128) (one per thread) and the columns
+// [by ks, (by + 1) ks) of the full square; each thread forms a_q[k1] h_q (and,
+// in split 0, -2 a_q[k1] b[k1]); the CTA's sum per candidate (lanes by
+// xor-butterfly, warps in order) goes to part[by][bx][q]. quad_spread_finish
+// adds the parts in order.
+constexpr int kSpreadRows = 128;
+__global__ void __launch_bounds__(kSpreadRows)
+quad_spread_kernel(int n, int K, int ks, const float* __restrict__ pop,
+                   const int* __restrict__ idx, const double* __restrict__ G,
+                   const double* __restrict__ b, double* __restrict__ part) {
+  wait_previous();
+  extern __shared__ double av[];   // [n][ks] genes of the column range
+  __shared__ double red[kMaxRescore][kSpreadRows / 32];
+  const int k1 = blockIdx.x * kSpreadRows + threadIdx.x;
+  const int k2lo = blockIdx.y * ks, len = min(K - k2lo, ks);
+  for (int e = threadIdx.x; e < n * ks; e += kSpreadRows) {
+    const int q = e / ks, c = e % ks;
+    av[e] = c < len ? (double)__ldcg(pop + (int64_t)idx[q] * K + k2lo + c) : 0.0;
+  }
+  __syncthreads();
+  double h[kMaxRescore];
+#pragma unroll
+  for (int q = 0; q < kMaxRescore; ++q) h[q] = 0.0;
+  if (k1 < K) {
+    for (int c = 0; c < len; ++c) {
+      const double g = G[(int64_t)(k2lo + c) * K + k1];
+#pragma unroll
+      for (int q = 0; q < kMaxRescore; ++q)
+        if (q < n) h[q] = fma(g, av[q * ks + c], h[q]);
+    }
+  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int q = 0; q < kMaxRescore; ++q) {
+    if (q >= n) break;
+    double v = 0.0;
+    if (k1 < K) {
+      const double ak = __ldcg(pop + (int64_t)idx[q] * K + k1);
+      v = ak * h[q];
+      if (blockIdx.y == 0) v -= 2.0 * ak * b[k1];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) red[q][warp] = v;
+  }
+  __syncthreads();
+  if (threadIdx.x < n) {
+    double sum = 0.0;
+    for (int w = 0; w < kSpreadRows / 32; ++w) sum += red[threadIdx.x][w];
+    part[((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * n + threadIdx.x] = sum;
+  }
+}
+
+// One warp per candidate q: lane l adds parts l, l + 32, ... in order, then
+// a fixed xor-butterfly.
+__global__ void quad_spread_finish(int n, int nparts, double m, double rm, int err,
+                                   const int* __restrict__ idx, const double* __restrict__ part,
+                                   const double* __restrict__ yy, double* __restrict__ fit) {
+  wait_previous();
+  const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (q >= n) return;
+  double s = 0.0;
+  for (int j = lane; j < nparts; j += 32) s += part[(int64_t)j * n + q];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) fit[idx[q]] = finish_error(divide_by(*yy + s, m, rm), err);
+}
+
 int blocks_for(int64_t n) {
   int64_t b = (n + 255) / 256;
   if (b < 1) b = 1;
@@ -536,6 +607,53 @@ cudaError_t launch_gram_fitness(const Shape& s, const float* pop, int P, const i
   while (S < 8 && (int64_t)ceil_div(P, grp) * S < 6 * kSms) S <<= 1;
   return grp == 4 ? launch_rows<4>(s, pop, P, idx, g, fit, err, S, st)
                   : launch_rows<1>(s, pop, P, idx, g, fit, err, S, st);
+}
+
+// The re-scoring is spread over the GPU where the kernels of the evaluation leave
+// it idle: at K = 49 to 64 for up to 8 candidates (the pair list gives each one
+// warp) and from K = 1200 on (a candidate has at most one cluster, and each reads
+// the whole list). us per call with the selection, P = 16, evaluation's kernels /
+// spread: K = 37: 11.8 / 10.1 (n = 2), 11.7 / 14.2 (n = 8); K = 49: 16.1 / 10.0,
+// 16.2 / 14.3 (n = 8), 16.1 / 20.5 (n = 16); K = 64: 22.1 / 9.9, 22.6 / 14.4, 22.5 /
+// 20.7; with n = 16, K = 257: 14.4 / 26.4; 801: 38 / 44; 1025: 54 / 58; 1281: 76 /
+// 74; 2001: 163 / 135; 3073: 360 / 291; 4097: 992 / 524. CTAs of 128 rows; no more
+// than two per SM, a third on some SMs costs half the time again (the FP64 pipes):
+// K = 3073, n = 16: 389 with 325 CTAs on 152 SMs, 291 with 300.
+constexpr int kSpreadK = 1200;
+static bool spread_serves(int K, int n) { return K >= kSpreadK || (K >= 49 && K <= kPairK && n <= 8); }
+struct Spread { int bx, by, ks; };
+static Spread spread(int K, int num_sms) {
+  Spread p;
+  p.bx = ceil_div(K, kSpreadRows);
+  p.by = 2 * num_sms / p.bx;
+  if (p.by < ceil_div(K, 1600)) p.by = ceil_div(K, 1600);   // genes of a range: 200 KB
+  if (p.by > K) p.by = K;
+  p.ks = ceil_div(K, p.by);
+  p.by = ceil_div(K, p.ks);
+  return p;
+}
+
+int64_t gram_rescore_parts(const Shape& s, int num_sms) {
+  if (!spread_serves(s.K, 1)) return 0;
+  const Spread p = spread(s.K, num_sms);
+  return (int64_t)p.bx * p.by * kMaxRescore;
+}
+
+cudaError_t launch_gram_rescore(const Shape& s, const float* pop, int n, const int* idx,
+                                const GramDev& g, double* fit, int err, int num_sms,
+                                cudaStream_t st) {
+  if (n < 1 || n > kMaxRescore) return cudaErrorInvalidValue;
+  if (!spread_serves(s.K, n)) return launch_gram_fitness(s, pop, n, idx, g, fit, err, st);
+  const Spread p = spread(s.K, num_sms);
+  const size_t smem = (size_t)n * p.ks * sizeof(double);
+  cudaError_t e = cudaFuncSetAttribute(quad_spread_kernel,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  if (e != cudaSuccess) return e;
+  e = launch_behind(quad_spread_kernel, dim3(p.bx, p.by), kSpreadRows, smem, st, n, s.K, p.ks, pop,
+                    idx, g.G, g.b, g.part);
+  if (e != cudaSuccess) return e;
+  return launch_behind(quad_spread_finish, 1, 32 * n, 0, st, n, p.bx * p.by, (double)s.M,
+                       1.0 / (double)s.M, err, idx, g.part, g.yy, fit);
 }
 
 }  // namespace game
