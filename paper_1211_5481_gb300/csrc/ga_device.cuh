@@ -233,13 +233,17 @@ __device__ __forceinline__ void plan_body(const GaDev& ga, const double* __restr
   __shared__ int widx[kPlanThreads / 32];
   __shared__ uint64_t key[kCountMax];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  // 1. elites: the first ranks where the selection sorted the population, else
-  // by counting, else one block-wide arg-min per elite
+  // 1. elites: the first ranks where the selection sorted the population, else by
+  // counting (P^2 compares, whatever the number of elites) or by one block-wide
+  // arg-min per elite. us per generation of a tiny run (M = 100, K = 3), counting /
+  // arg-min: P = 72: 12.2 / 12.0 (1 elite), 12.0 / 12.3 (2); 128: 13.1 / 12.9 (2);
+  // 200: 15.7 / 15.1 (4); 256: 16.9 / 17.3 (8); 300: 18.7 / 17.8 (8); 400: 23.0 /
+  // 23.7 (16); 512: 27.5 / 15.8 (2), 27.4 / 36.6 (32).
   if (block != 0) {
   } else if (ga.sel == GAME_SEL_RANKING) {
     for (int e = tid; e < ga.E; e += kPlanThreads) elite[e] = ga.order[e];
     __syncthreads();
-  } else if (ga.P <= kCountMax) {
+  } else if (ga.P <= kCountMax && ga.P * ga.P <= 8000 * ga.E) {
     count_ranks(ga.P, fit, key, [&](int r, int i) {
       if (r < ga.E) elite[r] = i;
     });
