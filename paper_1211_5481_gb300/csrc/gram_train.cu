@@ -25,7 +25,13 @@ namespace {
 
 constexpr int kCluster = 8;
 constexpr int kWarps = ga::kPlanThreads / 32;
-constexpr int kMaxP = 1024;
+// Every CTA plans and breeds the whole population, so beyond 96 chromosomes the
+// separate kernels are faster. us for 20 generations, separate kernels / one
+// launch, tournament, K = 5: P = 19: 147 / 108; 64: 159 / 134; 96: 168 / 167; 128:
+// 181 / 194; 300: 279 / 443; 1000: 329 / 896; K = 17, P = 96: 209 / 215, ranking
+// 220 / 216. (One generation alone pays the set-up: 16.3 / 18.9 at P = 19, 17.2 /
+// 22.1 at P = 96.)
+constexpr int kMaxP = 96;
 constexpr int kMaxSmem = 200 * 1024;
 // FP64 operations of one CTA's chromosomes per generation above which the
 // separate kernels, with the whole GPU's FP64 pipes, are faster: one SM does
