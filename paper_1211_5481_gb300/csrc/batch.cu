@@ -17,6 +17,8 @@
 // (the autotuner), or is the largest feasible width. Fitness values depend on BN
 // in their last bits (the FP32 sums inside a tile), so a run is reproducible
 // for a given tile choice; game_batch_get_tiles returns the choice.
+#include <unistd.h>
+
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -175,11 +177,11 @@ struct game_batch {
   float* a0 = nullptr;
   uint32_t* gens = nullptr;
   int* status = nullptr;
-  // page-locked: the status word, then one run's fitness and genes on their way
-  // to the caller (status_h alone where a run is larger than kStageMax)
+  // page-locked: the status word, then a run's fitness on its way to the caller.
+  // Whoever uses it holds host_lock, so runs may be read from several threads.
   int* status_h = nullptr;
   size_t stage_bytes = 0;
-  std::mutex stage_lock;
+  std::mutex host_lock;
   int* chrom_begin = nullptr;
   int total_chrom = 0;
   BatchRun* runs_d = nullptr;
@@ -225,14 +227,19 @@ void dfree(void* p) {
   if (p) cudaFree(p);
 }
 
-bool is_dev(const void* p) {
+cudaMemoryType memory_type(const void* p) {
   cudaPointerAttributes at{};
   if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
     cudaGetLastError();
-    return false;
+    return cudaMemoryTypeUnregistered;
   }
-  return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
+  return at.type;
 }
+bool is_dev(const void* p) {
+  const cudaMemoryType t = memory_type(p);
+  return t == cudaMemoryTypeDevice || t == cudaMemoryTypeManaged;
+}
+bool is_pageable(const void* p) { return memory_type(p) == cudaMemoryTypeUnregistered; }
 
 // Expansion K-block slots of an item with KB K-blocks, C chromosome tiles
 // and tile width bn: one per K-block when they fit the budget; else a ring
@@ -447,24 +454,16 @@ int enqueue_eval(game_batch* b, int src, int inc) {
   return rc;
 }
 
-// run r's fitness and genes
-size_t run_bytes(const game_batch* b, int r) {
-  return (size_t)b->P[r] * (sizeof(double) + b->shape[r].K * sizeof(float));
-}
+constexpr size_t kStageHead = 16;             // bytes ahead of a staged fitness: the status word
+constexpr size_t kStageMax = (size_t)64 << 10;
 
-constexpr size_t kStageHead = 16;             // bytes ahead of a staged run: the status word
-constexpr size_t kStageMax = (size_t)16 << 20;
-
+// The status word on its way to the host, and (behind it) the wait for it; the
+// caller holds host_lock.
 int enqueue_batch_status(game_batch* b) {
   BCK(cudaMemcpyAsync(b->status_h, b->status, sizeof(int), cudaMemcpyDeviceToHost, b->st));
   return GAME_OK;
 }
-
-int check_batch_status(game_batch* b, bool enqueued = false) {
-  if (!enqueued) {
-    const int rc = enqueue_batch_status(b);
-    if (rc) return rc;
-  }
+int read_batch_status(game_batch* b) {
   BCK(cudaStreamSynchronize(b->st));
   const int st = *static_cast<const volatile int*>(b->status_h);
   if (st != kDevOk) {
@@ -473,6 +472,22 @@ int check_batch_status(game_batch* b, bool enqueued = false) {
     return bfail(GAME_ETIMEOUT, "a kernel wait timed out; results are void");
   }
   return GAME_OK;
+}
+
+int check_batch_status(game_batch* b) {
+  std::lock_guard<std::mutex> lock(b->host_lock);
+  const int rc = enqueue_batch_status(b);
+  return rc ? rc : read_batch_status(b);
+}
+
+// Makes a result's pages present: a copy of the device's that has to fault them in
+// one by one is several times slower (518 KB of fresh memory: 232 -> 71 us with its
+// status). What is there stays.
+void touch_pages(void* p, size_t bytes) {
+  static const size_t page = (size_t)sysconf(_SC_PAGESIZE);
+  volatile char* c = static_cast<volatile char*>(p);
+  for (size_t at = 0; at < bytes; at += page) c[at] = c[at];
+  if (bytes) c[bytes - 1] = c[bytes - 1];
 }
 
 // Mean time of the fitness launch over reps launches (after one warm-up).
@@ -703,8 +718,7 @@ int game_batch_create(const game_run_desc* runs, int32_t R, const game_params* p
   if (nfit > 0x7fffffff / 32) return bail(bfail(GAME_EINVAL, "too many chromosomes in total"));
   b->total_chrom = (int)nfit;
   for (int r = 0; r < R; ++r)
-    b->stage_bytes = std::max(b->stage_bytes, run_bytes(b, r));
-  if (b->stage_bytes > kStageMax) b->stage_bytes = 0;
+    b->stage_bytes = std::max(b->stage_bytes, std::min(kStageMax, b->P[r] * sizeof(double)));
   if (dalloc(&b->Xt, nX) != cudaSuccess || dalloc(&b->y, ny) != cudaSuccess ||
       dalloc(&b->pop[0], npop) != cudaSuccess || dalloc(&b->pop[1], npop) != cudaSuccess ||
       dalloc(&b->fit, nfit) != cudaSuccess || dalloc(&b->plan, nfit) != cudaSuccess ||
@@ -823,25 +837,30 @@ int game_batch_get_run(game_batch_t b, int32_t r, float* pop_out, double* fit_ou
   const float* pop = b->pop[b->cur] + b->off_pop[r];
   const double* fit = b->fit + b->off_fit[r];
   const size_t pop_bytes = PK * sizeof(float), fit_bytes = b->P[r] * sizeof(double);
-  const bool staged = b->stage_bytes > 0 && (!pop_out || !is_dev(pop_out)) &&
-                      (!fit_out || !is_dev(fit_out)) && (pop_out || fit_out);
-  std::lock_guard<std::mutex> lock(b->stage_lock);
+  std::lock_guard<std::mutex> lock(b->host_lock);
   int rc = enqueue_batch_status(b);
   if (rc) return rc;
-  if (!staged) {
-    if (pop_out) BCK(cudaMemcpyAsync(pop_out, pop, pop_bytes, cudaMemcpyDefault, b->st));
-    if (fit_out) BCK(cudaMemcpyAsync(fit_out, fit, fit_bytes, cudaMemcpyDefault, b->st));
-    return check_batch_status(b, true);
+  // A copy into pageable memory waits for the stream, so only the last one is
+  // such a copy: the status word and, up to kStageMax, the fitness go through
+  // page-locked memory ahead of it. The genes go to their place (through
+  // page-locked memory as well, a run of 1.3 MB took 124 us for 48, one of 33 KB 20
+  // for 19). Three copies into pageable memory, one after the other: 63, 35.
+  char* stage = nullptr;
+  if (fit_out) {
+    const bool pageable = is_pageable(fit_out);
+    if (pageable && fit_bytes <= b->stage_bytes)
+      stage = reinterpret_cast<char*>(b->status_h) + kStageHead;
+    else if (pageable)
+      touch_pages(fit_out, fit_bytes);
+    BCK(cudaMemcpyAsync(stage ? (void*)stage : (void*)fit_out, fit, fit_bytes, cudaMemcpyDefault,
+                        b->st));
   }
-  // To host memory: through the page-locked buffer, so the three copies are waited
-  // for once, not each (a copy into pageable memory waits). 24 runs of 0.1 to 0.9
-  // MB and four generations: 2246 -> 2131 us.
-  char* at = reinterpret_cast<char*>(b->status_h) + kStageHead;
-  if (fit_out) BCK(cudaMemcpyAsync(at, fit, fit_bytes, cudaMemcpyDeviceToHost, b->st));
-  if (pop_out) BCK(cudaMemcpyAsync(at + fit_bytes, pop, pop_bytes, cudaMemcpyDeviceToHost, b->st));
-  rc = check_batch_status(b, true);
-  if (fit_out) std::memcpy(fit_out, at, fit_bytes);
-  if (pop_out) std::memcpy(pop_out, at + fit_bytes, pop_bytes);
+  if (pop_out) {
+    if (is_pageable(pop_out)) touch_pages(pop_out, pop_bytes);
+    BCK(cudaMemcpyAsync(pop_out, pop, pop_bytes, cudaMemcpyDefault, b->st));
+  }
+  rc = read_batch_status(b);
+  if (stage) std::memcpy(fit_out, stage, fit_bytes);
   return rc;
 }
 
