@@ -768,7 +768,6 @@ void destroy_ctx(game_ctx* h) {
   dev_free(h->fit);
   dev_free(h->plan);
   dev_free(h->status);
-  if (h->status_h) cudaFreeHost(h->status_h);
   dev_free(h->cand);
   dev_free(h->sel_order);
   dev_free(h->sel_cum);
@@ -806,6 +805,7 @@ void destroy_ctx(game_ctx* h) {
   dev_free(h->trust_r);
   dev_free(h->sd.tstat);
   dev_free(h->sd.lfit);
+  host_give(h->status_h, 2 * sizeof(int));   // (the frees have waited for the device)
   delete h;
 }
 
@@ -932,7 +932,7 @@ int game_create(const float* X, const float* y, int64_t M, int32_t N, int32_t de
       dev_alloc(&h->fit, (size_t)p.P) != cudaSuccess ||
       dev_alloc(&h->plan, (size_t)p.P) != cudaSuccess ||
       dev_alloc(&h->status, 4) != cudaSuccess ||
-      cudaMallocHost(reinterpret_cast<void**>(&h->status_h), 2 * sizeof(int)) != cudaSuccess ||
+      (h->status_h = static_cast<int*>(host_take(2 * sizeof(int)))) == nullptr ||
       dev_alloc(&h->cand, kMaxRescore) != cudaSuccess ||
       (p.selection == GAME_SEL_RANKING && dev_alloc(&h->sel_order, (size_t)p.P) != cudaSuccess) ||
       (p.selection == GAME_SEL_ROULETTE &&

@@ -615,7 +615,7 @@ void destroy_batch(game_batch* b) {
   dfree(b->a0);
   dfree(b->gens);
   dfree(b->status);
-  if (b->status_h) cudaFreeHost(b->status_h);
+  host_give(b->status_h, kStageHead + b->stage_bytes);
   dfree(b->chrom_begin);
   dfree(b->runs_d);
   dfree(b->ga_d);
@@ -726,8 +726,7 @@ int game_batch_create(const game_run_desc* runs, int32_t R, const game_params* p
       dalloc(&b->gens, R) != cudaSuccess || dalloc(&b->status, 4) != cudaSuccess ||
       dalloc(&b->chrom_begin, R) != cudaSuccess || dalloc(&b->runs_d, R) != cudaSuccess ||
       dalloc(&b->ga_d, R) != cudaSuccess || dalloc(&b->work, 1) != cudaSuccess ||
-      cudaMallocHost(reinterpret_cast<void**>(&b->status_h), kStageHead + b->stage_bytes) !=
-          cudaSuccess) {
+      (b->status_h = static_cast<int*>(host_take(kStageHead + b->stage_bytes))) == nullptr) {
     cudaGetLastError();
     return bail(bfail(GAME_ENOMEM, "batch device memory"));
   }

@@ -98,6 +98,12 @@ bool hook_alloc_fails();
 uint64_t hook_take_stall_ns();
 
 // ---- kernels and launchers (defined in the .cu files) ----
+// hostmem.cu: host memory for read-backs, page-locked where the process's block has
+// room (NULL: none at all); back by host_give with the same size, once no copy into
+// it is in flight
+void* host_take(size_t bytes);
+void host_give(void* p, size_t bytes);
+
 // layout.cu
 cudaError_t launch_relayout_X(const float* X, const float* y, const Shape& s, float* Xt,
                               float* yp, int* bad_counts, cudaStream_t st);
