@@ -274,12 +274,14 @@ __global__ void steps_kernel(int K, const double* __restrict__ G, double* __rest
 // The list is cut into kQuadRanges contiguous ranges; a warp takes a range at a
 // time for GRP chromosomes and leaves the range's sum per chromosome; the sums
 // are added in a fixed order. A cluster of S CTAs shares a group's ranges and
-// adds them in the leader's shared memory, so the result does not depend on S. With idx, entry q is chromosome idx[q].
+// adds them in the leader's shared memory, so the result does not depend on S; nor on
+// GRP (one chain of steps per segment): a chromosome's value is the same bit for
+// bit in any population. With idx, entry q is chromosome idx[q].
 // Before, one CTA held 8 chromosomes and thread t the rows t, t + 256, ... of
 // the full square: at K = 257 the second pass served a single row, and 128
 // CTAs left 24 SMs idle. P = 1024, K = 257: 231 -> 85 us per
 // evaluation (the FP64 pipes, 1.0 TFLOP/s measured, need 68 us for half the
-// square); the 16 re-scored candidates with their selection: 45 -> 18.5 us.
+// square); the 16 re-scored candidates with their selection: 46 -> 16.9 us.
 constexpr int kQuadWarps = 4;     // per CTA
 constexpr int kQuadRanges = 32;   // kQuadRanges / (S kQuadWarps) ranges per warp
 
@@ -327,12 +329,9 @@ quad_rows_kernel(int P, int K, double m, double rm, int err, int S, const float*
       const int end = base + K - 32 * I;   // the block's steps end
       const int stop = end < s1 ? end : s1;
       const double lin = s == base && k1 < K ? -2.0 * b[k1] : 0.0;
-      double h[GRP], h2[GRP];
+      double h[GRP];
 #pragma unroll
-      for (int q = 0; q < GRP; ++q) {
-        h[q] = lin;
-        h2[q] = 0.0;
-      }
+      for (int q = 0; q < GRP; ++q) h[q] = lin;
       int k2 = 32 * I + (s - base);
       const double* t = T + (int64_t)s * 32 + lane;
       for (; s < stop; s += kAhead, k2 += kAhead, t += kAhead * 32) {
@@ -344,12 +343,7 @@ quad_rows_kernel(int P, int K, double m, double rm, int err, int S, const float*
           if (GRP == 1) {
             // few warps: straight-line code keeps all loads in flight; a step
             // past the segment multiplies by zero (the list's entries are finite)
-#pragma unroll
-            for (int q = 0; q < GRP; ++q) {
-              const double av = s + u < stop ? as[(k2 + u) * GRP + q] : 0.0;
-              if (u & 1) h2[q] = fma(gv[u], av, h2[q]);
-              else h[q] = fma(gv[u], av, h[q]);
-            }
+            h[0] = fma(gv[u], s + u < stop ? as[k2 + u] : 0.0, h[0]);
           } else {
             if (s + u >= stop) break;
 #pragma unroll
@@ -361,7 +355,7 @@ quad_rows_kernel(int P, int K, double m, double rm, int err, int S, const float*
       if (k1 < K) {
 #pragma unroll
         for (int q = 0; q < GRP; ++q)
-          v[q] = fma(as[k1 * GRP + q], GRP == 1 ? h[q] + h2[q] : h[q], v[q]);
+          v[q] = fma(as[k1 * GRP + q], h[q], v[q]);
       }
       base = end;
       ++I;
@@ -610,17 +604,20 @@ cudaError_t launch_gram_fitness(const Shape& s, const float* pop, int P, const i
 }
 
 // The re-scoring is spread over the GPU where the kernels of the evaluation leave
-// it idle: at K = 49 to 64 for up to 8 candidates (the pair list gives each one
-// warp) and from K = 1200 on (a candidate has at most one cluster, and each reads
-// the whole list). us per call with the selection, P = 16, evaluation's kernels /
-// spread: K = 37: 11.8 / 10.1 (n = 2), 11.7 / 14.2 (n = 8); K = 49: 16.1 / 10.0,
-// 16.2 / 14.3 (n = 8), 16.1 / 20.5 (n = 16); K = 64: 22.1 / 9.9, 22.6 / 14.4, 22.5 /
-// 20.7; with n = 16, K = 257: 14.4 / 26.4; 801: 38 / 44; 1025: 54 / 58; 1281: 76 /
-// 74; 2001: 163 / 135; 3073: 360 / 291; 4097: 992 / 524. CTAs of 128 rows; no more
-// than two per SM, a third on some SMs costs half the time again (the FP64 pipes):
-// K = 3073, n = 16: 389 with 325 CTAs on 152 SMs, 291 with 300.
-constexpr int kSpreadK = 1200;
-static bool spread_serves(int K, int n) { return K >= kSpreadK || (K >= 49 && K <= kPairK && n <= 8); }
+// it idle or read too much: at K = 49 to 64 for up to 8 candidates (the pair list
+// gives each one warp), and at long K, where each candidate's cluster reads the
+// whole list: from K = 1900 on for more than 8 candidates, from K = 3900 on, where
+// the list no longer fits one die's half of L2, for any. us per call with the
+// selection, P = 16, evaluation's kernels / spread: K = 37: 11.8 / 10.1 (n = 2), 11.7 /
+// 14.2 (n = 8); K = 49: 16.1 / 10.0, 16.2 / 14.3, 16.1 / 20.5 (n = 16); K = 64:
+// 22.1 / 9.9, 22.6 / 14.4, 22.5 / 20.7; n = 8: K = 1201: 55.6 / 61.4; 2001: 132 / 138;
+// 3841: 457 / 516; 4097: 809 / 552; n = 16: K = 257: 13.7 / 26.4; 1201: 59 / 67;
+// 1801: 118 / 120; 1901: 131 / 124; 3073: 322 / 292; 4097: 815 / 523. CTAs of 128
+// rows; no more than two per SM, a third on some SMs costs half the time again (the
+// FP64 pipes): K = 3073, n = 16: 389 with 325 CTAs on 152 SMs, 291 with 300.
+static bool spread_serves(int K, int n) {
+  return K >= (n > 8 ? 1900 : 3900) || (K >= 49 && K <= kPairK && n <= 8);
+}
 struct Spread { int bx, by, ks; };
 static Spread spread(int K, int num_sms) {
   Spread p;
@@ -634,7 +631,7 @@ static Spread spread(int K, int num_sms) {
 }
 
 int64_t gram_rescore_parts(const Shape& s, int num_sms) {
-  if (!spread_serves(s.K, 1)) return 0;
+  if (!spread_serves(s.K, 1) && !spread_serves(s.K, kMaxRescore)) return 0;
   const Spread p = spread(s.K, num_sms);
   return (int64_t)p.bx * p.by * kMaxRescore;
 }

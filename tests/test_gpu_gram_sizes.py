@@ -27,10 +27,10 @@ def problem(N, d):
     return dg.regression(N + d, M, N, min(d, 4), 0.05, degree=d, basis=CHEB)
 
 
-# K = 49 and 64 (pair list, spread up to 8 candidates), 48 and 65 beside them;
-# 1199 and 1201 on both sides of the long rule; several row blocks, the longest
-@pytest.mark.parametrize("N,d", [(47, 1), (12, 4), (63, 1), (8, 8), (599, 2), (120, 10),
-                                 (100, 20), (128, 32)])
+# K = 49 and 64 (pair list, spread up to 8 candidates), 48 and 65 beside them; 1899
+# and 1901, 3897 and 3901 on both sides of the long rules; the longest
+@pytest.mark.parametrize("N,d", [(47, 1), (12, 4), (63, 1), (8, 8), (146, 13), (100, 19),
+                                 (487, 8), (130, 30), (128, 32)])
 @pytest.mark.parametrize("n", [1, 8, 9, 16])
 def test_rescoring(N, d, n):
     pr = problem(N, d)
@@ -67,3 +67,15 @@ def test_long_forms(N, d, P):
         got = g.eval_fitness(pop)
     want, bound = quad(G, b, yy, pop)
     assert np.all(np.abs(got - want) <= bound)
+
+
+# 4 chromosomes share the entries of G from 153 on, one each below
+@pytest.mark.parametrize("N,d", [(8, 8), (13, 5), (32, 8), (61, 10)])
+def test_a_value_does_not_depend_on_its_population(N, d):
+    pr = problem(N, d)
+    pop = dg.random_population(3, 700, pr.K)
+    with game.Game(pr.X, pr.y, d, CHEB, P=8, precision=game.GAME_PREC_GRAM) as g:
+        whole = g.eval_fitness(pop)
+        for lo, hi in ((0, 1), (5, 12), (100, 700), (301, 605), (699, 700)):
+            part = g.eval_fitness(pop[lo:hi])
+            assert np.array_equal(part, whole[lo:hi])
