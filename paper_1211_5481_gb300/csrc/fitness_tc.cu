@@ -911,10 +911,6 @@ TcPlan plan_tc_single(const Shape& s, int P, int num_sms, int form);
 // 6.57 ms, pairs 5.33 ms.
 namespace {
 int g_base_pad = 1024;
-__global__ void smem_base_probe_kernel(int* out) {
-  extern __shared__ uint8_t probe_smem[];
-  if (threadIdx.x == 0) *out = (int)((1024u - (ptx::smem_addr(probe_smem) & 1023u)) & 1023u);
-}
 }  // namespace
 
 static std::atomic<int> g_slack_override{0};
@@ -930,10 +926,6 @@ void note_smem_base_pad(int pad) {
   while (pad > cur && !seen.compare_exchange_weak(cur, pad)) {
   }
   set_smem_base_pad(seen.load());
-}
-cudaError_t launch_smem_base_probe(int* out, cudaStream_t st) {
-  smem_base_probe_kernel<<<1, 32, 16, st>>>(out);
-  return cudaGetLastError();
 }
 
 TcPlan plan_tc(const Shape& s, int P, int num_sms, int form) {

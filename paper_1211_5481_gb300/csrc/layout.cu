@@ -241,6 +241,15 @@ __global__ void replicate_tied_kernel(const float* __restrict__ pop, int P, int 
   }
 }
 
+// How far the dynamic shared memory starts below the next multiple of 1024. (Here,
+// not beside the tensor-core kernels that plan with it: a handle that does not use
+// them then does not load their 15 MB of code.)
+__global__ void smem_base_probe_kernel(int* out) {
+  extern __shared__ uint8_t probe_smem[];
+  if (threadIdx.x == 0)
+    *out = (int)((1024u - ((uint32_t)__cvta_generic_to_shared(probe_smem) & 1023u)) & 1023u);
+}
+
 int grid_for(int64_t n, int threads) {
   const int64_t b = (n + threads - 1) / threads;
   return (int)(b < 65535 * 16 ? (b < 1 ? 1 : b) : 65535 * 16);
@@ -253,6 +262,11 @@ cudaError_t launch_relayout_X(const float* X, const float* y, const Shape& s, fl
   const int blocks = (int)(s.Mpad / kPatBlock);
   relayout_X_kernel<<<blocks, 256, 0, st>>>(X, y, s.M, s.N, s.basis == GAME_BASIS_CHEB, Xt,
                                            yp, bad_counts);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_smem_base_probe(int* out, cudaStream_t st) {
+  smem_base_probe_kernel<<<1, 32, 16, st>>>(out);
   return cudaGetLastError();
 }
 
