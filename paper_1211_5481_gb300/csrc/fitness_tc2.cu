@@ -101,9 +101,9 @@ __host__ __device__ inline Smem2 smem_plan2(int KB, int NS, int N, int S, int xs
 }
 
 // The 8 expansion values of chunk `desc` for one pattern whose features are
-// xrow[i * xstride]: the same values as gen_chunk, with the Chebyshev run of
-// one feature's degrees and the crossing chunks of d >= 4 on their
-// branch-free generators.
+// xrow[i * xstride] (staged features, degrees above 10): the same values as
+// gen_chunk, with the Chebyshev run of one feature's degrees and the crossing
+// chunks of d >= 4 on their branch-free generators.
 __device__ __forceinline__ void gen8(uint32_t desc, int basis, int d, int N, const float* xrow,
                                      int xstride, float (&v)[8]) {
   if (basis == GAME_BASIS_CHEB && (desc & kChunkRun) && ((desc >> 24) & 15u) == 8u) {
@@ -494,8 +494,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       tab[cid] = chunk_desc(cid, a.basis, a.d, a.Kp);
     ptx::named_bar(1, kBasisThreads);
     const uint32_t phi_full_lead0 = ptx::mapa(ptx::smem_addr(phi_full), 0);
-    // (whole features at a time: see expand_stream.cuh; M = 10^6, N = 32,
-    // trigonometric degree 8, P = 1024: 2.58 -> 0.84 ms per evaluation)
+    // (whole features at a time: see expand_stream.cuh)
     const bool stream = a.xstage && stream_degree(a.d);
     if (stream) {
       StreamArgs sa;

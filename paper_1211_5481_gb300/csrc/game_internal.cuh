@@ -115,7 +115,7 @@ cudaError_t launch_pack_fp32(const float* pop, int P, int Ppad, const Shape& s, 
 cudaError_t launch_replicate_tied(const float* pop, int P, const Shape& s, float* full,
                                   cudaStream_t st);
 // fitness_fp32.cu
-// grid_x: groups of 128 chromosomes; U: chromosomes per thread (16 U per CTA,
+// grid_x: groups of 128 chromosomes, whatever the width; U: chromosomes per thread (16 U per CTA,
 // cta_x CTAs across the population); Ppad: columns popT, a0 and part need
 struct Fp32Plan { int BM, Kc, grid_x, grid_y, U, cta_x, Ppad; };
 Fp32Plan plan_fp32(const Shape& s, int P, int num_sms);

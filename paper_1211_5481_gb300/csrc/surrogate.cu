@@ -99,54 +99,30 @@ __device__ __forceinline__ void g_store8(uint8_t* img, uint8_t* img_lo, int r, i
   if (split) *reinterpret_cast<uint4*>(img_lo + off) = make_uint4(l[0], l[1], l[2], l[3]);
 }
 
-// Rows [0, R) x k in [k0, k0 + 64) of an operand X(r, k) = X[(r0 + r) rs + k ks]
-// (zero where r0 + r >= rlim or k >= kend) into the swizzled image, by the
-// CTA's kGThreads threads. Every thread issues all of its loads before it
-// converts and stores anything, so each waits one memory latency per
-// K-block. With k contiguous (ks == 1) eight threads share a row, each
-// converting one 16-byte unit, so a warp reads four rows' 256 contiguous
-// bytes; otherwise consecutive threads take consecutive rows (a warp's loads
-// span 32 rows) and the row's eight units are split among kGThreads / R
-// threads.
+// Rows [0, R) x k in [k0, k0 + 64) of an operand X(r, k) = X[(r0 + r) + k ks] (zero
+// where r0 + r >= rlim or k >= kend) into the swizzled image, by the CTA's
+// kGThreads threads: consecutive threads take consecutive rows (a warp's loads
+// span 32 rows), the row's eight 16-byte units split among kGThreads / R threads.
+// Every thread issues all of its loads before it converts and stores anything, so
+// each waits one memory latency per K-block.
 constexpr int kGThreads = 256;
 template <int R>
 __device__ __forceinline__ void g_load(uint8_t* img, uint8_t* img_lo, const float* __restrict__ X,
-                                       int64_t rs, int64_t ks, int r0, int rlim, int k0,
-                                       int kend, bool split) {
-  const int tid = threadIdx.x;
-  if (ks == 1) {
-    constexpr int RPP = kGThreads / 8;              // rows per pass
-    constexpr int NP = (R + RPP - 1) / RPP;
-    const int unit = tid & 7, rr = tid >> 3;
-    float v[NP][8];
+                                       int64_t ks, int r0, int rlim, int k0, int kend,
+                                       bool split) {
+  constexpr int TPR = kGThreads / R;              // threads per row
+  constexpr int UPT = 8 / TPR;                    // units per thread
+  const int tid = threadIdx.x, r = tid % R, ug = tid / R, row = r0 + r;
+  float v[UPT][8];
 #pragma unroll
-    for (int p = 0; p < NP; ++p) {
-      const int r = rr + p * RPP, row = r0 + r;
-      const float* src = X + (int64_t)row * rs;
+  for (int u = 0; u < UPT; ++u)
 #pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const int k = k0 + unit * 8 + e;
-        v[p][e] = (r < R && row < rlim && k < kend) ? src[k] : 0.f;
-      }
+    for (int e = 0; e < 8; ++e) {
+      const int k = k0 + (ug * UPT + u) * 8 + e;
+      v[u][e] = (row < rlim && k < kend) ? X[(int64_t)row + (int64_t)k * ks] : 0.f;
     }
 #pragma unroll
-    for (int p = 0; p < NP; ++p)
-      if (rr + p * RPP < R) g_store8(img, img_lo, rr + p * RPP, unit, v[p], split);
-  } else {
-    constexpr int TPR = kGThreads / R;              // threads per row
-    constexpr int UPT = 8 / TPR;                    // units per thread
-    const int r = tid % R, ug = tid / R, row = r0 + r;
-    float v[UPT][8];
-#pragma unroll
-    for (int u = 0; u < UPT; ++u)
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const int k = k0 + (ug * UPT + u) * 8 + e;
-        v[u][e] = (row < rlim && k < kend) ? X[(int64_t)row * rs + (int64_t)k * ks] : 0.f;
-      }
-#pragma unroll
-    for (int u = 0; u < UPT; ++u) g_store8(img, img_lo, r, ug * UPT + u, v[u], split);
-  }
+  for (int u = 0; u < UPT; ++u) g_store8(img, img_lo, r, ug * UPT + u, v[u], split);
 }
 
 constexpr int kGTN = 64;   // columns of C per CTA
@@ -205,8 +181,8 @@ grad_gemm_kernel(int batch, GradProblem p0, GradProblem p1, int kz, int* status)
     if (kb >= 2) ok = g_wait(ptx::smem_addr(&bars[st]), ((kb - 2) >> 1) & 1, status);
     if (!ok) break;
     const int k0 = kbeg + kb * kGTK;
-    g_load<128>(a_img, a_lo, p.A, 1, kH, m0, kH, k0, kend, true);
-    g_load<kGTN>(b_img, nullptr, p.B, 1, p.N, n0, p.N, k0, kend, false);
+    g_load<128>(a_img, a_lo, p.A, kH, m0, kH, k0, kend, true);
+    g_load<kGTN>(b_img, nullptr, p.B, p.N, n0, p.N, k0, kend, false);
     ptx::fence_proxy_async_smem();
     __syncthreads();
     if (tid == 0) {
