@@ -116,14 +116,21 @@ namespace game {
 // A chunk is 8 consecutive contraction columns [8*cid, 8*cid + 8). Its
 // descriptor records where the chunk starts in the feature / group / degree
 // sequence, so the generator needs no division in its inner loop:
-//   bits  0-15  feature i of the first column
-//   bits 16-20  degree j of the first column (1..d)
-//   bit  21     group b of the first column (trigonometric: 0 cos, 1 sin)
-//   bit  22     all 8 columns lie in one (feature, group) run of degrees
+//   bits  0-11  feature i of the first column
+//   bits 12-23  degree j of the first column (1..d), less one
 //   bits 24-27  number of columns below Kp (8 except in the last chunk)
+//   bit  28     group b of the first column (trigonometric: 0 cos, 1 sin)
+//   bit  29     all 8 columns lie in one (feature, group) run of degrees
 //   bit  31     no column below Kp (all-zero chunk)
+// (N d <= 4096: features and degrees less one fit 12 bits each)
 constexpr uint32_t kChunkZero = 1u << 31;
-constexpr uint32_t kChunkRun = 1u << 22;
+constexpr uint32_t kChunkRun = 1u << 29;
+__host__ __device__ constexpr int chunk_feature(uint32_t desc) { return (int)(desc & 0xFFFu); }
+__host__ __device__ constexpr int chunk_degree(uint32_t desc) {
+  return (int)((desc >> 12) & 0xFFFu) + 1;
+}
+__host__ __device__ constexpr int chunk_columns(uint32_t desc) { return (int)((desc >> 24) & 15u); }
+__host__ __device__ constexpr int chunk_group(uint32_t desc) { return (int)((desc >> 28) & 1u); }
 
 __host__ __device__ inline uint32_t chunk_desc(int cid, int basis, int d, int Kp) {
   const int c0 = 8 * cid;
@@ -132,8 +139,8 @@ __host__ __device__ inline uint32_t chunk_desc(int cid, int basis, int d, int Kp
   const int i = c0 / W, off = c0 % W;
   const int b = off / d, j = off % d + 1;
   const int nvalid = (Kp - c0) < 8 ? (Kp - c0) : 8;
-  uint32_t desc = (uint32_t)i | ((uint32_t)j << 16) | ((uint32_t)b << 21) |
-                  ((uint32_t)nvalid << 24);
+  uint32_t desc = (uint32_t)i | ((uint32_t)(j - 1) << 12) | ((uint32_t)nvalid << 24) |
+                  ((uint32_t)b << 28);
   if (j + 7 <= d) desc |= kChunkRun;
   return desc;
 }
@@ -146,9 +153,9 @@ __host__ __device__ inline uint32_t chunk_desc(int cid, int basis, int d, int Kp
 __device__ __forceinline__ void cheb_cross2(uint32_t desc, int d, int N, const float* xrow0,
                                             const float* xrow1, int xstride, bool hasB,
                                             float (&va)[8], float (&vb)[8]) {
-  const int i = (int)(desc & 0xFFFFu);
-  const int j0 = (int)((desc >> 16) & 31u);
-  const int nvalid = (int)((desc >> 24) & 15u);
+  const int i = chunk_feature(desc);
+  const int j0 = chunk_degree(desc);
+  const int nvalid = chunk_columns(desc);
   const int i1 = i + 1 < N ? i + 1 : N - 1, i2 = i + 2 < N ? i + 2 : N - 1;
   const float xa0 = xrow0[i * xstride], xa1 = xrow0[i1 * xstride], xa2 = xrow0[i2 * xstride];
   const float xb0 = hasB ? xrow1[i * xstride] : 0.f;
@@ -201,9 +208,9 @@ __device__ __forceinline__ void cheb_cross2(uint32_t desc, int d, int N, const f
 // One-pattern form of cheb_cross2 (same values as gen_chunk).
 __device__ __forceinline__ void cheb_cross1(uint32_t desc, int d, int N, const float* xrow,
                                             int xstride, float (&v)[8]) {
-  const int i = (int)(desc & 0xFFFFu);
-  const int j0 = (int)((desc >> 16) & 31u);
-  const int nvalid = (int)((desc >> 24) & 15u);
+  const int i = chunk_feature(desc);
+  const int j0 = chunk_degree(desc);
+  const int nvalid = chunk_columns(desc);
   const int i1 = i + 1 < N ? i + 1 : N - 1, i2 = i + 2 < N ? i + 2 : N - 1;
   const float x0 = xrow[i * xstride], x1 = xrow[i1 * xstride], x2 = xrow[i2 * xstride];
   float a2 = x0 + x0, t = x0, tm = 1.f;
@@ -319,10 +326,10 @@ __device__ __forceinline__ void gen_chunk(uint32_t desc, int basis, int d, int N
     for (int e = 0; e < 8; ++e) v[e] = 0.f;
     return;
   }
-  int i = (int)(desc & 0xFFFFu);
-  int j = (int)((desc >> 16) & 31u);
-  int b = (int)((desc >> 21) & 1u);
-  const int nvalid = (int)((desc >> 24) & 15u);
+  int i = chunk_feature(desc);
+  int j = chunk_degree(desc);
+  int b = chunk_group(desc);
+  const int nvalid = chunk_columns(desc);
   float x = xrow[i * xstride];
   if (basis == GAME_BASIS_CHEB) {
     float x2 = x + x, tm1 = 1.f, t = x;

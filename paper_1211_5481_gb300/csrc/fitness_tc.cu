@@ -74,6 +74,8 @@ namespace {
 
 using namespace tc;
 
+static_assert(kMaxK <= 4097, "a chunk descriptor holds features and degrees below 4096");
+
 constexpr uint32_t kABytes = 128 * 128;   // one (chromosome tile, K-block) gene block
 constexpr int kEpiWarp0 = 4;
 constexpr int kEpiThreads = 256;          // warps 4..11
@@ -551,9 +553,9 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
     // tests the end per value.
     auto gen_rows = [&](uint32_t desc, const float* xrow0, const float* xrow1, bool hasB,
                         float (&va)[8], float (&vb)[8]) {
-      if (cheb && (desc & kChunkRun) && ((desc >> 24) & 15u) == 8u) {
-        const int i = (int)(desc & 0xFFFFu);
-        const int j0 = (int)((desc >> 16) & 31u);
+      if (cheb && (desc & kChunkRun) && chunk_columns(desc) == 8) {
+        const int i = chunk_feature(desc);
+        const int j0 = chunk_degree(desc);
         const float xa = xrow0[i * XW];
         const float xb = hasB ? xrow1[i * XW] : 0.f;
         const float a2 = xa + xa, b2 = xb + xb;
@@ -663,7 +665,7 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
     // both rows of a Chebyshev chunk that stays in one feature's run of degrees:
     // two interleaved recurrences, one descriptor decode, no per-value branches
     auto emit_run2x = [&](uint8_t* phik, uint32_t desc, int qd, float xa, float xb) {
-      const int j0 = (int)((desc >> 16) & 31u);
+      const int j0 = chunk_degree(desc);
       const float a2 = xa + xa, b2 = xb + xb;
       float ta = xa, tam = 1.f, tb = xb, tbm = 1.f;
       for (int st = 1; st < j0; ++st) {
@@ -764,7 +766,7 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
             make_uint4(wb[0], wb[1], wb[2], wb[3]);
     };
     auto emit_cheb_run2 = [&](uint8_t* phik, uint32_t desc, int qd) {
-      const int i = (int)(desc & 0xFFFFu);
+      const int i = chunk_feature(desc);
       emit_run2x(phik, desc, qd, xr0[i * XW], R == 2 ? xr1[i * XW] : 0.f);
     };
     // waits until expansion slot q % NS may be written (use q / NS)
@@ -808,7 +810,7 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
         const float* p1 = xptr(lit, r1);
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-          const int i = (int)(tab[lkb * 8 + q] & 0xFFFFu);
+          const int i = chunk_feature(tab[lkb * 8 + q]);
           va[q] = __ldg(p0 + i * kPatBlock);
           vb[q] = R == 2 ? __ldg(p1 + i * kPatBlock) : 0.f;
         }
@@ -873,7 +875,7 @@ __global__ void __launch_bounds__(kThreads, 1) fitness_tc_kernel(const TcArgs a)
         if (F == kFormBF16 && !TRI) {
           for (int qd = q0; qd < 8; qd += QS) {
             const uint32_t desc = tab[kb * 8 + qd];
-            if (cheb && (desc & kChunkRun) && ((desc >> 24) & 15u) == 8u) {
+            if (cheb && (desc & kChunkRun) && chunk_columns(desc) == 8) {
               emit_cheb_run2(phik, desc, qd);
             } else if (cheb && a.d >= 4 && !(desc & kChunkZero)) {
               emit_cheb_cross2(phik, desc, qd);

@@ -106,9 +106,9 @@ __host__ __device__ inline Smem2 smem_plan2(int KB, int NS, int N, int S, int xs
 // chunks of d >= 4 on their branch-free generators.
 __device__ __forceinline__ void gen8(uint32_t desc, int basis, int d, int N, const float* xrow,
                                      int xstride, float (&v)[8]) {
-  if (basis == GAME_BASIS_CHEB && (desc & kChunkRun) && ((desc >> 24) & 15u) == 8u) {
-    const int i = (int)(desc & 0xFFFFu);
-    const int j0 = (int)((desc >> 16) & 31u);
+  if (basis == GAME_BASIS_CHEB && (desc & kChunkRun) && chunk_columns(desc) == 8) {
+    const int i = chunk_feature(desc);
+    const int j0 = chunk_degree(desc);
     const float x = xrow[i * xstride];
     const float x2 = x + x;
     float t = x, tm = 1.f;
@@ -552,7 +552,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       auto load_kb = [&](int itn, int kbn) {
         const float* p = xptr(itn);
 #pragma unroll
-        for (int q = 0; q < 8; ++q) nx[q] = __ldg(p + (int)(tab[kbn * 8 + q] & 0xFFFFu) * kPatBlock);
+        for (int q = 0; q < 8; ++q) nx[q] = __ldg(p + chunk_feature(tab[kbn * 8 + q]) * kPatBlock);
       };
       if (bt == 0) {
         if (my_tiles > 0) prefetch_tile(0);
@@ -576,7 +576,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         for (int qd = 0; qd < 8; qd += 2) {
           const uint32_t da = tab[kb * 8 + qd], db = tab[kb * 8 + qd + 1];
           float va[8], vb[8];
-          cheb_run_pair(x[qd], (int)((da >> 16) & 31u), x[qd + 1], (int)((db >> 16) & 31u),
+          cheb_run_pair(x[qd], chunk_degree(da), x[qd + 1], chunk_degree(db),
                         va, vb);
           if (da & kChunkZero) {
 #pragma unroll
