@@ -410,7 +410,7 @@ int eval_device(game_ctx* h, const float* dpop, int P, int prec, double* dfit,
   cudaEvent_t t0;
   if (prec == GAME_PREC_GRAM) {
     t0 = stage_begin(h);
-    CK(launch_gram_fitness(gram_shape(h), dpop, P, nullptr, h->gram, dfit, err, h->st));
+    CK(launch_gram_fitness(gram_shape(h), dpop, P, nullptr, h->gram, dfit, err, h->num_sms, h->st));
     stage_end(h, t0, kFitness);
     return GAME_OK;
   }

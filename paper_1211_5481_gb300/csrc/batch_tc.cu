@@ -29,7 +29,7 @@
 // through a per-thread ring of asynchronous copies. Each item writes its FP64
 // partial sums to its own row, part[part_base_r + t Ppad_r + p], so the
 // result does not depend on which CTA took the item; the batched reduce adds
-// a problem's rows in tile order. All waits are bounded (2 s) as in
+// a problem's rows in tile order. All waits are bounded (4e9 cycles) as in
 // fitness_tc.cu.
 #include "basis.cuh"
 #include "game_internal.cuh"

@@ -53,7 +53,7 @@
 // expansion threads from global memory (L2, prefetched two tiles ahead),
 // one K-block of a warpgroup ahead of use; the shared memory this frees holds the spare
 // slots. Both modes produce identical expansion values.
-// PHI and D never leave the SM. All waits are bounded (2 s): on expiry the
+// PHI and D never leave the SM. All waits are bounded (4e9 cycles): on expiry the
 // kernel raises a status word, abandons its loops, waits for its own bulk
 // copies and MMAs in flight, frees tensor memory and returns.
 #include <cuda_fp8.h>

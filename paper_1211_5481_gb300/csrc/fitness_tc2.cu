@@ -35,7 +35,7 @@
 // CTA's producers reach them by cluster-scope arrivals (one per warp for the
 // expansion and the epilogue, one relay per gene stage); every MMA commit is
 // multicast to the same barrier in both CTAs, so each CTA's producers and
-// epilogue wait on their own copies. All waits are bounded (2 s): on expiry a
+// epilogue wait on their own copies. All waits are bounded (4e9 cycles): on expiry a
 // CTA raises the status word, abandons its loops, drains its own copies (the
 // even CTA its MMAs), and both CTAs meet at the final cluster barrier before
 // the pair's tensor memory is freed.

@@ -295,7 +295,8 @@ cudaError_t launch_gram_list(const Shape& s, const GramDev& g, cudaStream_t st);
 // fit of the P chromosomes pop [P][K] (idx NULL), or of rows idx[0..P-1]
 // written to fit[idx[p]]; err GAME_ERR_MSE or GAME_ERR_RMSE
 cudaError_t launch_gram_fitness(const Shape& s, const float* pop, int P, const int* idx,
-                                const GramDev& g, double* fit, int err, cudaStream_t st);
+                                const GramDev& g, double* fit, int err, int num_sms,
+                                cudaStream_t st);
 // the elite re-scoring: n <= kMaxRescore rows idx[q] into fit[idx[q]]
 int64_t gram_rescore_parts(const Shape& s, int num_sms);
 cudaError_t launch_gram_rescore(const Shape& s, const float* pop, int n, const int* idx,

@@ -585,20 +585,21 @@ cudaError_t launch_rows(const Shape& s, const float* pop, int P, const int* idx,
 }  // namespace
 
 cudaError_t launch_gram_fitness(const Shape& s, const float* pop, int P, const int* idx,
-                                const GramDev& g, double* fit, int err, cudaStream_t st) {
+                                const GramDev& g, double* fit, int err, int num_sms,
+                                cudaStream_t st) {
   if (s.K <= kPairK) {
     return launch_behind(quad_pairs_kernel, ceil_div(P, kPairWarps), 32 * kPairWarps, 0, st, P, s.K,
                          (double)s.M, 1.0 / (double)s.M, err, pop, idx, g.list, g.kk, g.b, g.yy, fit);
   }
-  // Four chromosomes share each entry where that still makes two CTAs per SM
-  // (152 SMs); else one each, every load of a range in flight. Cluster size: about six
-  // CTAs per SM, so the last SMs to finish are few. P = 1024, K = 257: 85 us
+  // Four chromosomes share each entry where that still makes two CTAs per SM; else
+  // one each, every load of a range in flight. Cluster size: about six CTAs per SM,
+  // so the last SMs to finish are few. On 152 SMs, P = 1024, K = 257: 82 us
   // with four chromosomes and S = 4, 90 with S = 8 or 2, 91 with eight
-  // chromosomes, 113 with one; P = 16: 12.4 us with one and S = 8, 18.5 with four.
-  constexpr int kSms = 152;
-  const int grp = (int64_t)ceil_div(P, 4) * 8 >= 2 * kSms ? 4 : 1;
+  // chromosomes, 113 with one. (P = 16 with one and S = 8, candidate selection included:
+  // 13.7 us.)
+  const int grp = (int64_t)ceil_div(P, 4) * 8 >= 2 * num_sms ? 4 : 1;
   int S = 1;
-  while (S < 8 && (int64_t)ceil_div(P, grp) * S < 6 * kSms) S <<= 1;
+  while (S < 8 && (int64_t)ceil_div(P, grp) * S < 6 * num_sms) S <<= 1;
   return grp == 4 ? launch_rows<4>(s, pop, P, idx, g, fit, err, S, st)
                   : launch_rows<1>(s, pop, P, idx, g, fit, err, S, st);
 }
@@ -640,7 +641,7 @@ cudaError_t launch_gram_rescore(const Shape& s, const float* pop, int n, const i
                                 const GramDev& g, double* fit, int err, int num_sms,
                                 cudaStream_t st) {
   if (n < 1 || n > kMaxRescore) return cudaErrorInvalidValue;
-  if (!spread_serves(s.K, n)) return launch_gram_fitness(s, pop, n, idx, g, fit, err, st);
+  if (!spread_serves(s.K, n)) return launch_gram_fitness(s, pop, n, idx, g, fit, err, num_sms, st);
   const Spread p = spread(s.K, num_sms);
   const size_t smem = (size_t)n * p.ks * sizeof(double);
   cudaError_t e = cudaFuncSetAttribute(quad_spread_kernel,
