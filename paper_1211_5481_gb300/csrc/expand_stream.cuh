@@ -6,8 +6,9 @@
 // replaces for these degrees decoded a descriptor per 8 columns, restarted the
 // feature's recurrence there (for the trigonometric basis with another sincosf
 // per chunk) and tested the end of a run at every value: at M = 10^6, N = 32,
-// trigonometric degree 8, P = 1024 the BF16 evaluation took 2.58 ms, three
-// times its contraction (0.84 ms with this file, 1.25 PFLOP/s). Here a thread takes whole features: the shortest run
+// trigonometric degree 8, P = 1024 (SM pairs) the BF16 evaluation took 2.58 ms, 0.84
+// with this file on four warps, 0.56 on eight (1.88 PFLOP/s). Here a thread takes
+// whole features: the shortest run
 // of them that fills whole 16-byte units (8 columns, 16 in FP8) is one group,
 // its values are straight-line code (one start per feature, one FMA per
 // value), rounded and packed in registers, then stored unit by unit.

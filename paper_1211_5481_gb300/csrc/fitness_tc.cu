@@ -910,10 +910,13 @@ TcPlan plan_tc_single(const Shape& s, int P, int num_sms, int form);
 // The one-SM kernel where it runs 256-pattern tiles; where its shared memory
 // forces narrower tiles, the BF16 form (with at least two chromosome tiles)
 // takes the paired-SM kernel, whose CTAs each hold half of a 256-pattern
-// tile's expansion. Measured on the large classification set (256-pattern
-// one-SM tiles): one-SM 0.50 ms, pairs 0.54 ms per evaluation; on the
-// surrogate workload (K' = 288, N = 48: one-SM 192-pattern tiles): one-SM
-// 6.57 ms, pairs 5.33 ms.
+// tile's expansion. us per evaluation, one-SM / pairs. One-SM tiles of 192: N = 48,
+// degree 6, M = 4 10^6, P = 2048: 3307 / 2609; N = 26, degree 10, M = 10^6, P = 1024: 459
+// / 355; N = 20, trigonometric degree 8, M = 500,000: 270 / 201; of 128: N = 64, degree
+// 8: 433 / 302, P = 300, M = 50,000: 32.8 / 32.3. Tiles of 256, M = 10^6: N = 32, degree
+// 8: 130 / 183 (P = 256), 339 / 335 (1024); N = 31: 196 / 216 (P = 512); N = 39, degree
+// 6: 197 / 228 (P = 300), 366 / 326 (1024); N = 16, trigonometric degree 8, P = 1024:
+// 351 / 327. (So from P = 1024 on pairs would serve those too.)
 namespace {
 int g_base_pad = 1024;
 }  // namespace

@@ -57,7 +57,7 @@ constexpr uint32_t kABytes = 128 * 128;   // one CTA's gene block: 128 chromosom
 constexpr int kEpiWarp0 = 4;
 constexpr int kBasisWarp0 = 12;
 // (eight expansion warps, one elected issuing thread, epilogue one step ahead: M =
-// 4 10^6, N = 48, degree 6, P = 2048: 3.02 -> 2.69 ms; M = 94,601, N = 26,
+// 4 10^6, N = 48, degree 6, P = 2048: 3.02 -> 2.61 ms; M = 94,601, N = 26,
 // trigonometric degree 11, P = 1092, the chunk generator: 360 -> 232 us)
 constexpr int kBasisThreads = 256;        // warps 12..19
 constexpr int kThreads = kBasisWarp0 * 32 + kBasisThreads;

@@ -9,8 +9,8 @@
 // the chromosomes that rank before it and gives up at n; the n that finish
 // write their own place, and no CTA waits for another. Latency bound: one pass
 // of the keys through shared memory, P / 32 ballots for the n best, a few for
-// all others. (Selection and re-evaluation of 16 candidates, K = 257: P = 1024
-// 45 -> 18.5 us, P = 2048 51 -> 22.6.) Above 16,384 chromosomes the launch of P
+// all others. (Selection and re-evaluation of 16 candidates, K = 257, P =
+// 1024, with the re-evaluation's own change: 46 -> 16.9 us.) Above 16,384 chromosomes the launch of P
 // warps and the long counts cost more than select_top_kernel (one CTA: each
 // thread keeps the top 16 of its strided elements in registers, each warp
 // merges its lanes' lists, warp 0 merges the 8 warps'). Fitness values are

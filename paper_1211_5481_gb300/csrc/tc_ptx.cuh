@@ -257,13 +257,12 @@ __device__ __forceinline__ void regs_dec() {
 }
 
 // ---- MMA issue by an elected thread ----
-// The issuing loop, waits included, stands in a block `if (elect_one())`. The
-// compiler knows that such a block is run by one thread, so addresses and
-// descriptors stay in uniform registers; in a branch on the lane number they
-// are moved there one by one for each MMA. What decides the rate is the
-// latency of this one warp's instructions: per K-block of four MMAs (512 tensor
-// cycles) the warp needed 720 cycles with a converged loop and an election per
-// K-block.
+// The issuing loop, waits included, stands in a block `if (elect_one())`. What
+// decides the MMA rate is the latency of this one warp's instructions between
+// MMAs: per K-block of four (512 tensor cycles) a converged loop with an election
+// per K-block needed 720 cycles. Measured, BF16, M = 10^6, N = 32, degree 8, P =
+// 1024, four expansion warps: 434 us in a branch on the lane number, 372 with the
+// converged loop, 354 in one elected block.
 __device__ __forceinline__ uint32_t elect_one() {
   uint32_t lead;
   asm volatile(
