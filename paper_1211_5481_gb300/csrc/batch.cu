@@ -177,7 +177,8 @@ struct game_batch {
   float* a0 = nullptr;
   uint32_t* gens = nullptr;
   int* status = nullptr;
-  // page-locked: the status word, then a run's fitness on its way to the caller.
+  // page-locked: the status word, then a run's fitness (a small run's genes as well)
+  // on its way to the caller.
   // Whoever uses it holds host_lock, so runs may be read from several threads.
   int* status_h = nullptr;
   size_t stage_bytes = 0;
@@ -454,8 +455,15 @@ int enqueue_eval(game_batch* b, int src, int inc) {
   return rc;
 }
 
-constexpr size_t kStageHead = 16;             // bytes ahead of a staged fitness: the status word
-constexpr size_t kStageMax = (size_t)64 << 10;
+constexpr size_t kStageHead = 16;             // bytes ahead of what is staged: the status word
+constexpr size_t kStageMax = (size_t)64 << 10;    // the largest fitness staged
+constexpr size_t kStageRun = (size_t)16 << 10;    // the largest run staged whole
+
+// Bytes of run r that take the page-locked way.
+size_t staged_bytes(const game_batch* b, int r) {
+  const size_t fit = b->P[r] * sizeof(double), pop = (size_t)b->P[r] * b->shape[r].K * sizeof(float);
+  return fit + pop <= kStageRun ? fit + pop : std::min(kStageMax, fit);
+}
 
 // The status word on its way to the host, and (behind it) the wait for it; the
 // caller holds host_lock.
@@ -718,7 +726,7 @@ int game_batch_create(const game_run_desc* runs, int32_t R, const game_params* p
   if (nfit > 0x7fffffff / 32) return bail(bfail(GAME_EINVAL, "too many chromosomes in total"));
   b->total_chrom = (int)nfit;
   for (int r = 0; r < R; ++r)
-    b->stage_bytes = std::max(b->stage_bytes, std::min(kStageMax, b->P[r] * sizeof(double)));
+    b->stage_bytes = std::max(b->stage_bytes, staged_bytes(b, r));
   if (dalloc(&b->Xt, nX) != cudaSuccess || dalloc(&b->y, ny) != cudaSuccess ||
       dalloc(&b->pop[0], npop) != cudaSuccess || dalloc(&b->pop[1], npop) != cudaSuccess ||
       dalloc(&b->fit, nfit) != cudaSuccess || dalloc(&b->plan, nfit) != cudaSuccess ||
@@ -841,25 +849,26 @@ int game_batch_get_run(game_batch_t b, int32_t r, float* pop_out, double* fit_ou
   if (rc) return rc;
   // A copy into pageable memory waits for the stream, so only the last one is
   // such a copy: the status word and, up to kStageMax, the fitness go through
-  // page-locked memory ahead of it. The genes go to their place (through
-  // page-locked memory as well, a run of 1.3 MB took 124 us for 48, one of 33 KB 20
-  // for 19). Three copies into pageable memory, one after the other: 63, 35.
-  char* stage = nullptr;
-  if (fit_out) {
-    const bool pageable = is_pageable(fit_out);
-    if (pageable && fit_bytes <= b->stage_bytes)
-      stage = reinterpret_cast<char*>(b->status_h) + kStageHead;
-    else if (pageable)
-      touch_pages(fit_out, fit_bytes);
-    BCK(cudaMemcpyAsync(stage ? (void*)stage : (void*)fit_out, fit, fit_bytes, cudaMemcpyDefault,
-                        b->st));
-  }
-  if (pop_out) {
-    if (is_pageable(pop_out)) touch_pages(pop_out, pop_bytes);
-    BCK(cudaMemcpyAsync(pop_out, pop, pop_bytes, cudaMemcpyDefault, b->st));
-  }
+  // page-locked memory ahead of it. So do the genes of a run up to kStageRun
+  // (a copy of page-locked memory and the host's cost 17 us for 18 at 1 KB); larger
+  // ones go to their place (through page-locked memory a run of 33 KB took 20 us for
+  // 19, one of 1.3 MB 124 for 48). Three copies into pageable memory, one after the
+  // other: 33 KB 35 us, 1.3 MB 63.
+  char* const stage = reinterpret_cast<char*>(b->status_h) + kStageHead;
+  const bool fit_host = fit_out && is_pageable(fit_out), pop_host = pop_out && is_pageable(pop_out);
+  const bool fit_staged = fit_host && fit_bytes <= b->stage_bytes;
+  const bool pop_staged = pop_host && fit_bytes + pop_bytes <= std::min(kStageRun, b->stage_bytes);
+  if (fit_host && !fit_staged) touch_pages(fit_out, fit_bytes);
+  if (pop_host && !pop_staged) touch_pages(pop_out, pop_bytes);
+  if (fit_out)
+    BCK(cudaMemcpyAsync(fit_staged ? (void*)stage : (void*)fit_out, fit, fit_bytes,
+                        cudaMemcpyDefault, b->st));
+  if (pop_out)
+    BCK(cudaMemcpyAsync(pop_staged ? (void*)(stage + fit_bytes) : (void*)pop_out, pop, pop_bytes,
+                        cudaMemcpyDefault, b->st));
   rc = read_batch_status(b);
-  if (stage) std::memcpy(fit_out, stage, fit_bytes);
+  if (fit_staged) std::memcpy(fit_out, stage, fit_bytes);
+  if (pop_staged) std::memcpy(pop_out, stage + fit_bytes, pop_bytes);
   return rc;
 }
 
