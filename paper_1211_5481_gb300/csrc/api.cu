@@ -450,14 +450,15 @@ int eval_device(game_ctx* h, const float* dpop, int P, int prec, double* dfit,
 
 int ensure_gram(game_ctx* h);
 
-// Enqueues the re-scoring of the n best entries of dfit (device arrays):
+// Enqueues the re-scoring of the n best entries of dfit (device arrays; callers: the
+// caller's):
 // the candidates' FP64 fitness by the Gram form.
-int rescore_device(game_ctx* h, const float* dpop, int P, int n, double* dfit) {
+int rescore_device(game_ctx* h, const float* dpop, int P, int n, double* dfit, bool callers) {
   if (h->prm.error == GAME_ERR_MAE) return fail(GAME_EINVAL, "the MAE has no Gram form to re-score with");
   int rc = ensure_gram(h);
   if (rc) return rc;
   cudaEvent_t t0 = stage_begin(h);
-  CK(launch_select_top(dfit, P, n, h->cand, h->st));
+  CK(launch_select_top(dfit, P, n, h->cand, callers, h->st));
   CK(launch_gram_rescore(gram_shape(h), dpop, n, h->cand, h->gram, dfit, h->prm.error, h->num_sms,
                          h->st));
   stage_end(h, t0, kRescore);
@@ -472,7 +473,7 @@ int eval_state(game_ctx* h) {
   if (rc) return rc;
   const int n = h->prm.rescore_top < h->prm.P ? h->prm.rescore_top : h->prm.P;
   if (h->prm.precision != GAME_PREC_FP32 && h->prm.precision != GAME_PREC_GRAM && n > 0)
-    return rescore_device(h, h->pop[h->cur], h->prm.P, n, h->fit);
+    return rescore_device(h, h->pop[h->cur], h->prm.P, n, h->fit, false);
   return GAME_OK;
 }
 
@@ -1066,14 +1067,14 @@ int game_rescore_top(game_t h, const float* pop, int32_t P, double* fit, int32_t
   if (dev_in != dev_fit) return fail(GAME_EINVAL, "pop and fit must be in the same memory");
   int rc;
   if (dev_in) {
-    rc = rescore_device(h, pop, P, n, fit);
+    rc = rescore_device(h, pop, P, n, fit, true);
   } else {
     rc = ensure_upload(h, P);
     if (rc) return rc;
     CK(cudaMemcpyAsync(h->upop, pop, (size_t)P * h->Kg * sizeof(float),
                        cudaMemcpyHostToDevice, h->st));
     CK(cudaMemcpyAsync(h->ufit, fit, (size_t)P * sizeof(double), cudaMemcpyHostToDevice, h->st));
-    rc = rescore_device(h, h->upop, P, n, h->ufit);
+    rc = rescore_device(h, h->upop, P, n, h->ufit, false);
     if (rc) return rc;
     CK(cudaMemcpyAsync(fit, h->ufit, (size_t)P * sizeof(double), cudaMemcpyDeviceToHost, h->st));
   }

@@ -40,7 +40,8 @@ namespace game {
 // stream ends (programmatic stream serialization; behind anything else than a
 // kernel the launch is an ordinary one). No kernel releases its successor
 // early, so nothing of a successor's runs beside a CTA of its predecessor; a
-// caller's kernel may, so what a caller wrote is read past L1 (__ldcg). A
+// caller's kernel may, so what a caller wrote is read past L1 (__ldcg) or by an
+// ordinary launch. A
 // generation's or evaluation's kernels are 3 to 20 us each with about 1.5 us
 // between two ordinary launches. Ten generations of M = 2000, N = 8, degree 4,
 // P = 64, FP32 (40 launches): 299 -> 217 us; one evaluation of three launches
@@ -214,7 +215,9 @@ cudaError_t prepare_fitness_batch(int smem_bytes);
 cudaError_t launch_fitness_batch(const BatchArgs& a, int grid, int smem_bytes, cudaStream_t st);
 
 // rescore.cu: the n best of fit (by (fit, index), NaN last) into cand [n]
-cudaError_t launch_select_top(const double* fit, int P, int n, int* cand, cudaStream_t st);
+// (callers: fit is the caller's memory, the kernel perhaps the first behind one of the caller's)
+cudaError_t launch_select_top(const double* fit, int P, int n, int* cand, bool callers,
+                              cudaStream_t st);
 // surrogate.cu -- the MLP fitness surrogate (K -> 256 -> 256 -> 1)
 constexpr int kSurrogateHidden = 256;
 constexpr float kAdamLr = 1e-3f, kAdamB1 = 0.9f, kAdamB2 = 0.999f, kAdamEps = 1e-8f;

@@ -75,7 +75,7 @@ select_top_kernel(const double* __restrict__ fit, int P, int n, int* __restrict_
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   TopList L;
   L.clear();
-  for (int p = tid; p < P; p += kSelThreads) L.insert(ga::rank_key(__ldcg(fit + p)), p);
+  for (int p = tid; p < P; p += kSelThreads) L.insert(ga::rank_key(fit[p]), p);
   // each warp: n rounds of arg-min over its lanes' list heads
   for (int r = 0; r < n; ++r) {
     uint64_t k = L.k[0];
@@ -114,12 +114,12 @@ select_rank_kernel(const double* __restrict__ fit, int P, int n, int* __restrict
   __shared__ uint64_t key[kRankChunk];
   const int lane = threadIdx.x & 31;
   const int i = blockIdx.x * kRankWarps + (threadIdx.x >> 5);
-  const uint64_t mine = i < P ? ga::rank_key(__ldcg(fit + i)) : kNoKey;
+  const uint64_t mine = i < P ? ga::rank_key(fit[i]) : kNoKey;
   int before = i < P ? 0 : n;
   for (int c0 = 0; c0 < P; c0 += kRankChunk) {
     const int len = min(kRankChunk, P - c0);
 #pragma unroll 8
-    for (int k = threadIdx.x; k < len; k += 32 * kRankWarps) key[k] = ga::rank_key(__ldcg(fit + c0 + k));
+    for (int k = threadIdx.x; k < len; k += 32 * kRankWarps) key[k] = ga::rank_key(fit[c0 + k]);
     __syncthreads();
     for (int k0 = 0; k0 < len && before < n; k0 += 32) {
       const int k = k0 + lane;
@@ -133,13 +133,22 @@ select_rank_kernel(const double* __restrict__ fit, int P, int n, int* __restrict
 
 }  // namespace
 
-cudaError_t launch_select_top(const double* fit, int P, int n, int* cand, cudaStream_t st) {
+cudaError_t launch_select_top(const double* fit, int P, int n, int* cand, bool callers,
+                              cudaStream_t st) {
   if (n < 1) return cudaSuccess;
   if (n > kMaxRescore || n > P) return cudaErrorInvalidValue;
-  if (P <= kRankMax)
-    return launch_behind(select_rank_kernel, ceil_div(P, kRankWarps), 32 * kRankWarps, 0, st, fit, P,
-                         n, cand);
-  return launch_behind(select_top_kernel, 1, kSelThreads, 0, st, fit, P, n, cand);
+  const int grid = P <= kRankMax ? ceil_div(P, kRankWarps) : 1;
+  const auto kern = P <= kRankMax ? select_rank_kernel : select_top_kernel;
+  constexpr int threads = 32 * kRankWarps;
+  static_assert(threads == kSelThreads, "both selections");
+  // The fitness is read through L1 (past it, P = 16,384 takes 82 us for 60), so behind
+  // a caller's kernel, which may release its successor while it still writes, the
+  // launch is an ordinary one.
+  if (callers) {
+    kern<<<grid, threads, 0, st>>>(fit, P, n, cand);
+    return cudaGetLastError();
+  }
+  return launch_behind(kern, grid, threads, 0, st, fit, P, n, cand);
 }
 
 }  // namespace game
