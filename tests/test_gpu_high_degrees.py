@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 
 from emulation import model
-from helpers import CHEB, TRIG
+from helpers import CHEB, TRIG, fp32_tol
 from paper_1211_5481_gb300 import datagen as dg
 from paper_1211_5481_gb300 import game
 
@@ -54,3 +54,16 @@ def test_high_degrees_in_a_batch():
             pop, fit, _ = b.run(r)
             want, tol = model("bf16", X, y, pop, d, basis)
             assert np.all(np.abs(fit - want) <= tol)
+
+
+# runs of degrees that end in every place of a 16-column chunk, one feature, columns
+# past the last feature
+@pytest.mark.parametrize("d", [11, 12, 14, 15, 16, 17, 19, 24, 31, 33])
+@pytest.mark.parametrize("basis", [CHEB, TRIG])
+def test_plain_fp32(orc, basis, d):
+    for N, P in ((1, 5), (3, 64), (5, 130), (7, 257)):
+        pr, pop = problem(N, d, basis, P)
+        ref = orc.fitness(pr.X, pr.y, pop, d, basis)
+        with game.Game(pr.X, pr.y, d, basis, P=max(P, 4)) as g:
+            got = g.eval_fitness(pop)
+        assert np.all(np.abs(got - ref) <= fp32_tol(ref, pr.y))
